@@ -36,6 +36,7 @@
 
 #include "common.cuh"
 #include "dalitz.cuh"
+#include "fp64.cuh"
 #include "timeterms.cuh"
 #include "model.cuh"
 
@@ -152,38 +153,6 @@ struct CohAcc {
   unsigned bad = 0;
 };
 
-// One event: S = sum_k c_k A_k, log |S|^2 and the lanes Re / Im of A_k conj(S) / |S|^2.
-template <typename T, int KB, bool GRAD>
-__device__ __forceinline__ void coh_event(const T (&cr)[KB + 1], const T (&ci)[KB + 1], const T (&ar)[KB + 1],
-                                          const T (&ai)[KB + 1], CohAcc<T, KB>& acc) {
-  constexpr int KA = KB + 1;
-  T sr = T(0), si = T(0);
-#pragma unroll
-  for (int k = 0; k < KA; ++k) {
-    sr += cr[k] * ar[k] - ci[k] * ai[k];
-    si += cr[k] * ai[k] + ci[k] * ar[k];
-  }
-  const T s2 = sr * sr + si * si;
-  if (s2 > T(0)) {
-    if constexpr (sizeof(T) == 4) {
-      acc.lf32.add(__logf(s2));
-    } else {
-      acc.lf64 += log(s2);
-    }
-    if constexpr (GRAD) {
-      const T inv = T(1) / s2;
-      const T tr = sr * inv, ti = -si * inv;  // conj(S) / |S|^2
-#pragma unroll
-      for (int k = 0; k < KA; ++k) {
-        acc.gre[k] += ar[k] * tr - ai[k] * ti;
-        acc.gim[k] += ar[k] * ti + ai[k] * tr;
-      }
-    }
-  } else {
-    acc.bad++;
-  }
-}
-
 // Block and last-block reductions of the lanes, then the FP64 combination with the
 // normalisation terms the host formed from the Gram matrix at the coefficients the kernel used
 // (they depend on theta and the MC sample only: an O(K^2) quadratic form that would otherwise
@@ -271,33 +240,73 @@ __device__ __forceinline__ void coh_coeffs(const CohArgs<T>& a, T (&cr)[KB + 1],
   ci[KB] = a.has_nr ? a.ci[nbw] : T(0);
 }
 
-// Direct form (one event per thread per grid-stride step); the FP64 path uses it.
-template <typename T, int KB, bool GRAD>
-__global__ void __launch_bounds__(kBlock, 2) coh_nll_kernel(const __grid_constant__ CohArgs<T> a, const void* cache_v,
-                                                            int64_t begin, int64_t end, float2* partials,
-                                                            unsigned* counters, double* result, int out_mode) {
-  constexpr int NS = CohLanes<T, KB, GRAD>::NS;
+// FP64 form: one event per thread per grid-stride step, amplitudes read directly.  Bound by the
+// FP64 pipe (fp64.cuh), so what counts is its slots per event: 8 per resonance (every product
+// sum is a chain of FMAs), the logarithm as a running product, the reciprocal by one third-order
+// step, the sign test on the integer pipe; absent resonance slots and the constant amplitude
+// (A = 1) cost no multiplication.  8 resonances with the gradient take 78 slots per event; 2M
+// events: 549 -> 293 us (the slots alone: 249 us at the measured 6.27e11 FMA/s).
+template <int KB, bool GRAD>
+__global__ void __launch_bounds__(kBlock, 2)
+    coh_nll_f64_kernel(const __grid_constant__ CohArgs<double> a, const double2* __restrict__ cache, int64_t begin,
+                       int64_t end, float2* partials, unsigned* counters, double* result, int out_mode) {
+  constexpr int NS = CohLanes<double, KB, GRAD>::NS;
   constexpr int KA = KB + 1;  // BW slots + NR slot
+  // the amplitudes of an event stay in registers between the sum and the gradient lanes; the
+  // 15-resonance form reads them again (its lanes alone take 64 registers)
+  constexpr bool KEEP = KB <= 8;
   __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
   __shared__ unsigned s_bad[kBlock / 32];
-  using Vec = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
-  const Vec* cache = (const Vec*)cache_v;
   const int nbw = a.nbw;
-  T cr[KA], ci[KA];
-  coh_coeffs<T, KB>(a, cr, ci);
-  CohAcc<T, KB> acc;
+  const double nr_re = a.has_nr ? a.cr[nbw] : 0.0, nr_im = a.has_nr ? a.ci[nbw] : 0.0;
+  CohAcc<double, KB> acc;
+  LogProduct lp;
 #pragma unroll
-  for (int k = 0; k < KA; ++k) acc.gre[k] = acc.gim[k] = T(0);
+  for (int k = 0; k < KA; ++k) acc.gre[k] = acc.gim[k] = 0.0;
   const int64_t n = a.n_total;
   for (int64_t i = begin + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < end;
        i += (int64_t)gridDim.x * blockDim.x) {
-    T ar[KA], ai[KA];
-    load_amps<KB>(cache, n, i, nbw, ar, ai);
-    ar[KB] = T(1);
-    ai[KB] = T(0);
-    coh_event<T, KB, GRAD>(cr, ci, ar, ai, acc);
+    double2 amp[KEEP ? KB : 1];
+    if constexpr (KEEP) {
+      // every load of the event before its first use (predicated, not a loop exit between them)
+#pragma unroll
+      for (int k = 0; k < KB; ++k) amp[k] = k < nbw ? cache[(int64_t)k * n + i] : make_double2(0.0, 0.0);
+    }
+    double sr = nr_re, si = nr_im;
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      if (k >= nbw) break;
+      const double2 v = KEEP ? amp[k] : cache[(int64_t)k * n + i];
+      sr = fma(a.cr[k], v.x, fma(-a.ci[k], v.y, sr));
+      si = fma(a.cr[k], v.y, fma(a.ci[k], v.x, si));
+    }
+    const double s2 = fma(sr, sr, si * si);
+    double inv;
+    if (positive_normal(s2)) {
+      lp.mul(s2);
+      inv = rcp64(s2);
+    } else if (s2 > 0.0) {  // subnormal or infinite
+      acc.lf64 += log(s2);
+      inv = 1.0 / s2;
+    } else {
+      acc.bad++;
+      continue;
+    }
+    if constexpr (GRAD) {
+      const double tr = sr * inv, ti = -si * inv;  // conj(S) / |S|^2
+#pragma unroll
+      for (int k = 0; k < KB; ++k) {
+        if (k >= nbw) break;
+        const double2 v = KEEP ? amp[k] : cache[(int64_t)k * n + i];
+        acc.gre[k] = fma(v.x, tr, fma(-v.y, ti, acc.gre[k]));
+        acc.gim[k] = fma(v.x, ti, fma(v.y, tr, acc.gim[k]));
+      }
+      acc.gre[KB] += tr;  // A = 1
+      acc.gim[KB] += ti;
+    }
   }
-  coh_finish<T, KB, GRAD>(a, acc, begin, end, partials, counters, result, out_mode, s_red, s_bad);
+  acc.lf64 += lp.log_value();
+  coh_finish<double, KB, GRAD>(a, acc, begin, end, partials, counters, result, out_mode, s_red, s_bad);
 }
 
 // FP32 form with the amplitude-cache tiles staged in shared memory.  A tile holds
@@ -1212,32 +1221,23 @@ static int launch_coh_staged(goo_model* m, const void* cache, const goo_dataset*
   return GOO_OK;
 }
 
-template <typename T, int KB, bool GRAD>
-static int launch_coh(goo_model* m, const void* cache, const goo_dataset* ds, int64_t begin, int64_t end,
-                      const double* theta, int out_mode, int pi) {
-  if constexpr (sizeof(T) == 4) return launch_coh_staged<KB, GRAD>(m, cache, ds, begin, end, theta, out_mode, pi);
+template <int KB, bool GRAD>
+static int launch_coh_f64(goo_model* m, const void* cache, const goo_dataset* ds, int64_t begin, int64_t end,
+                          const double* theta, int out_mode, int pi) {
   DalitzModel& d = *m->dalitz;
   goo_ctx* ctx = m->ctx;
-  static int occ = 0;
-  if (occ == 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, coh_nll_kernel<T, KB, GRAD>, kBlock, 0) != cudaSuccess ||
-        occ < 1) {
-      cudaGetLastError();
-      occ = 1;
-    }
-  }
+  const int occ = cached_occupancy((const void*)coh_nll_f64_kernel<KB, GRAD>, ctx->device, kBlock, 0);
   const int nb = grid_blocks(ctx, end - begin, occ);
-  constexpr int NS = CohLanes<T, KB, GRAD>::NS;
+  constexpr int NS = CohLanes<double, KB, GRAD>::NS;
   GOO_TRY(ensure_partials(ctx, (size_t)nb * NS));
-  CohArgs<T> a;
-  fill_args<T>(d, theta, m->n_params, ds->n, a);
-  coh_norm_terms<T>(d, d.gram_host[pi], a);
+  CohArgs<double> a;
+  fill_args<double>(d, theta, m->n_params, ds->n, a);
+  coh_norm_terms<double>(d, d.gram_host[pi], a);
   {
-    LaunchScope ls(ctx, sizeof(T) == 4 ? (GRAD ? "coh_nll_grad_f32" : "coh_nll_f32")
-                                       : (GRAD ? "coh_nll_grad_f64" : "coh_nll_f64"));
-    coh_nll_kernel<T, KB, GRAD><<<nb, kBlock, 0, ctx->stream>>>(a, cache, begin, end, ctx->scratch.partials,
-                                                                ctx->scratch.counters, ctx->scratch.result_out,
-                                                                out_mode);
+    LaunchScope ls(ctx, GRAD ? "coh_nll_grad_f64" : "coh_nll_f64");
+    coh_nll_f64_kernel<KB, GRAD><<<nb, kBlock, 0, ctx->stream>>>(a, (const double2*)cache, begin, end,
+                                                                 ctx->scratch.partials, ctx->scratch.counters,
+                                                                 ctx->scratch.result_out, out_mode);
   }
   GOO_CUDA_TRY(cudaGetLastError());
   return GOO_OK;
@@ -1246,8 +1246,13 @@ static int launch_coh(goo_model* m, const void* cache, const goo_dataset* ds, in
 template <typename T, bool GRAD>
 static int launch_coh_sel(goo_model* m, const void* cache, const goo_dataset* ds, int64_t begin, int64_t end,
                           const double* theta, int out_mode, int pi) {
-  if (m->dalitz->nbw <= 8) return launch_coh<T, 8, GRAD>(m, cache, ds, begin, end, theta, out_mode, pi);
-  return launch_coh<T, 15, GRAD>(m, cache, ds, begin, end, theta, out_mode, pi);
+  const bool small = m->dalitz->nbw <= 8;
+  if constexpr (sizeof(T) == 4)
+    return small ? launch_coh_staged<8, GRAD>(m, cache, ds, begin, end, theta, out_mode, pi)
+                 : launch_coh_staged<15, GRAD>(m, cache, ds, begin, end, theta, out_mode, pi);
+  else
+    return small ? launch_coh_f64<8, GRAD>(m, cache, ds, begin, end, theta, out_mode, pi)
+                 : launch_coh_f64<15, GRAD>(m, cache, ds, begin, end, theta, out_mode, pi);
 }
 
 // Constants of the floating-lineshape kernels at theta (FP64 on the host, rounded to T):
