@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(kBlock)
 //   R = (|A|^2+|B|^2)/2 T_ch + (|A|^2-|B|^2)/2 T_c + Re(AB*) T_sh + Im(AB*) T_s,
 // and the gradient lanes Re / -Im of (a_k V_A + abar_k V_B) / R with
 //   V_A = (T_ch + T_c) A* + (T_sh - i T_s) B*,  V_B = (T_ch - T_c) B* + (T_sh + i T_s) A*,
-// plus d R / d(x, y, tau, sigma_t) / R.  N comes from three MC Gram matrices,
+// plus the four decay-time lanes of timeterms.cuh.  N comes from three MC Gram matrices,
 //   <|A|^2> = c^T G_aa c*, <|B|^2> = c^T G_bb c*, <AB*> = c^T G_ab c*,
 // and the closed-form time integrals.
 // ---------------------------------------------------------------------------------------
@@ -886,10 +886,9 @@ __global__ void __launch_bounds__(kBlock, 2)
     }
     TimeTerms<T> tt;
     time_terms_g<T>(a.tc, a.wa, a.wN, a.wL, t, tt);
-    const T AA = Ar * Ar + Ai * Ai, BB = Br * Br + Bi * Bi;
-    const T ABr = Ar * Br + Ai * Bi, ABi = Ai * Br - Ar * Bi;  // A conj(B)
-    // R = |A|^2 P + |B|^2 Q + Re(A B*) T_sh + Im(A B*) T_s with P, Q = (T_ch +- T_c)/2
-    const T R = AA * tt.P + BB * tt.Q + ABr * tt.Tsh + ABi * tt.Ts;
+    const T AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
+    const T ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
+    const T R = td_rate(tt, AA, BB, ABr, ABi);
     if (!(R > T(0))) {
       ++bad;
       continue;
@@ -916,9 +915,7 @@ __global__ void __launch_bounds__(kBlock, 2)
       }
       lre[KB] += VAr + VBr;  // the NR slot (a = abar = 1)
       lim[KB] -= VAi + VBi;
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        lt[j] += (AA * tt.d[j][0] + BB * tt.d[j][1] + ABr * tt.d[j][2] + ABi * tt.d[j][3]) * invR;
+      time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, lt);
     }
   }
   ddf v[NS];
@@ -968,7 +965,9 @@ __global__ void __launch_bounds__(kBlock, 2)
       }
       const int o = 1 + 2 * KA;
       for (int j = 0; j < 4; ++j)
-        if (a.par_t[j] == p) g += -s_out[o + j] + (j < 3 ? nev * a.nrm_dt[j] : 0.0);
+        if (a.par_t[j] == p)
+          g += (j < 3 ? nev * a.nrm_dt[j] : 0.0) -
+               time_gradient(j, (double)a.G, (double)a.x, (double)a.y, (double)a.s, s_out + o, nev);
     }
     out[off + p] = g;
   }

@@ -26,7 +26,7 @@
 //
 // Gradient lanes per event: log R; Re, Im of a_k V / R with
 // V = (T_ch + T_c) A* + (T_sh - i T_s) B* (dR/dRe c_k = Re(a_k V), dR/dIm c_k = -Im(a_k V));
-// and dR/d(x, y, tau, sigma_t) / R.  The last block forms the NLL and its gradient in FP64.
+// and the four decay-time lanes of timeterms.cuh.  The last block forms the NLL and its gradient in FP64.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -190,10 +190,9 @@ __device__ __forceinline__ void td4_event(const Td4Args<T>& a, const T (&ar)[KB]
   }
   TimeTerms<T> tt;
   time_terms<T>(a, t, tt);
-  const T AA = Ar * Ar + Ai * Ai, BB = Br * Br + Bi * Bi;
-  const T ABr = Ar * Br + Ai * Bi, ABi = Ai * Br - Ar * Bi;  // A conj(B)
-  // R = |A|^2 P + |B|^2 Q + Re(A B*) T_sh + Im(A B*) T_s with P, Q = (T_ch +- T_c)/2
-  const T R = AA * tt.P + BB * tt.Q + ABr * tt.Tsh + ABi * tt.Ts;
+  const T AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
+  const T ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
+  const T R = td_rate(tt, AA, BB, ABr, ABi);
   if (!(R > T(0))) {
     acc.bad++;
     return;
@@ -211,9 +210,7 @@ __device__ __forceinline__ void td4_event(const Td4Args<T>& a, const T (&ar)[KB]
       acc.lre[k] += ar[k] * Vr - ai[k] * Vi;     // Re(a_k V) / R
       acc.lim[k] += -(ar[k] * Vi + ai[k] * Vr);  // -Im(a_k V) / R
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      acc.lt[j] += (AA * tt.d[j][0] + BB * tt.d[j][1] + ABr * tt.d[j][2] + ABi * tt.d[j][3]) * invR;
+    time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, acc.lt);
   }
 }
 
@@ -237,9 +234,9 @@ __device__ __forceinline__ void td4_event_f32(const Td4Args<float>& a, const flo
   const float Ar = P1.x - P2.y, Ai = P1.y + P2.x, Br = Q1.x - Q2.y, Bi = Q1.y + Q2.x;
   TimeTerms<float> tt;
   time_terms<float>(a, t, tt);
-  const float AA = Ar * Ar + Ai * Ai, BB = Br * Br + Bi * Bi;
-  const float ABr = Ar * Br + Ai * Bi, ABi = Ai * Br - Ar * Bi;  // A conj(B)
-  const float R = AA * tt.P + BB * tt.Q + ABr * tt.Tsh + ABi * tt.Ts;
+  const float AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
+  const float ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
+  const float R = td_rate(tt, AA, BB, ABr, ABi);
   if (!(R > 0.f)) {
     acc.bad++;
     return;
@@ -255,9 +252,7 @@ __device__ __forceinline__ void td4_event_f32(const Td4Args<float>& a, const flo
       acc.lre[k] += am[k].x * Vr - am[k].y * Vi;     // Re(a_k V) / R
       acc.lim[k] += -(am[k].x * Vi + am[k].y * Vr);  // -Im(a_k V) / R
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      acc.lt[j] += (AA * tt.d[j][0] + BB * tt.d[j][1] + ABr * tt.d[j][2] + ABi * tt.d[j][3]) * invR;
+    time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, acc.lt);
   }
 }
 
@@ -314,7 +309,9 @@ __device__ __forceinline__ void td4_finish(const Td4Args<T>& a, TdAcc<T, KB>& ac
       }
       const int o = 1 + 2 * KB;
       for (int j = 0; j < 4; ++j)
-        if (a.par_t[j] == p) g += -s_out[o + j] + (j < 3 ? nev * a.nrm_dt[j] : 0.0);
+        if (a.par_t[j] == p)
+          g += (j < 3 ? nev * a.nrm_dt[j] : 0.0) -
+               time_gradient(j, (double)a.G, (double)a.x, (double)a.y, (double)a.s, s_out + o, nev);
     }
     result[off + p] = g;
   }

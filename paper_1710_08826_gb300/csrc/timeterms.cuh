@@ -11,25 +11,41 @@
 // i.e. the convolutions of e^{-G t'} [cosh(y G t') +- cos(x G t')]/2, e^{-G t'} sinh(y G t')
 // and e^{-G t'} sin(x G t').  For small mixing Q, T_sh and T_s are tiny differences of nearly
 // equal convolved exponentials (Q = O(x^2 + y^2), T_sh = O(y)): formed as such differences in
-// FP32 they keep only a few significant digits, and so do their derivatives.  Where
+// FP32 they keep only a few significant digits.  Where
 // z = max(|x|, |y|) G (max(t, 0) + 6 s) is small they are therefore summed as power series in
 // the moments of the resolution-convolved exponential,
-//   M_n(t) = int_0^inf t'^n e^{-G t'} N(t - t'; 0, s) dt',
-//   u_n = G^n M_n / n!,
-//   P = sum_m a_m u_2m,  Q = sum_m b_m u_2m,  T_sh = sum_m y^(2m+1) u_(2m+1),
-//   T_s = sum_m (-1)^m x^(2m+1) u_(2m+1),
-//   a_m, b_m = (y^2m +- (-1)^m x^2m) / 2,
+//   M_n(t) = int_0^inf t'^n e^{-G t'} N(t - t'; 0, s) dt',  w_n = G^n M_n,
+//   P = sum_m a_m w_2m,  Q = sum_m b_m w_2m,  T_sh = sum_m y^(2m+1) / (2m+1)! w_(2m+1),
+//   T_s = sum_m (-1)^m x^(2m+1) / (2m+1)! w_(2m+1),
+//   a_m, b_m = (y^2m +- (-1)^m x^2m) / (2 (2m)!),
 // from the Taylor series of cosh and cos, with every term of one sign for t > G s^2.  The
 // moments follow from M_0 = E(G) (one erfcx) by the recurrence obtained by integrating
 // t' N(t - t') by parts,
-//   M_1 = (t - G s^2) M_0 + s^2 N(t),  M_(n+1) = (t - G s^2) M_n + n s^2 M_(n-1),
-// i.e. u_(n+1) = (G (t - G s^2) u_n + G^2 s^2 u_(n-1)) / (n + 1).  Derivatives:
-//   G d u_n / d G = n u_n - (n + 1) u_(n+1)        (d M_n / d G = -M_(n+1)),
-//   d u_n / d s = s d^2 u_n / d t^2                 (heat equation of the Gaussian)
-//              = s [G^2 (u_n - 2 u_(n-1) + u_(n-2)) + c_n],
-//   c_0 = N'(t) - G N(t), c_1 = G N(t), c_n = 0 for n >= 2 (from d M_n / d t = n M_(n-1)
-//   - G M_n + [n = 0] N(t)).  Elsewhere (large mixing) the terms come from the Faddeeva path,
-// where the differences are not small.
+//   w_1 = G (v M_0 + s^2 N(t)),  w_(n+1) = G v w_n + n G^2 s^2 w_(n-1),  v = t - G s^2.
+// Elsewhere (large mixing) the terms come from the Faddeeva path, where the differences are
+// not small.
+//
+// Derivatives.  The four functions f = e^{-G t'} (...) are closed under d / d t',
+//   f_P'  = -G f_P + G (y f_sh - x f_s)/2,   f_Q' = -G f_Q + G (y f_sh + x f_s)/2,
+//   f_sh' = -G f_sh + G y (f_P + f_Q),       f_s' = -G f_s + G x (f_P - f_Q),
+// with f_P(0) = 1 and the others 0 there, so every derivative of the terms is a combination of
+// the terms themselves; no series is summed for it.  Integrating t' N(t - t') by parts once
+// more, the convolutions C_f of t' f(t') are
+//   C_P  = v P + s^2 N(t) + s^2 G (y T_sh - x T_s)/2,  C_Q = v Q + s^2 G (y T_sh + x T_s)/2,
+//   C_sh = v T_sh + s^2 G y (P + Q),                   C_s = v T_s + s^2 G x (P - Q),
+// and for the event's weights (|A|^2, |B|^2, Re AB*, Im AB*) = (a, b, r, i)
+//   dR/dx = G X,  X = (b - a)/2 C_s + i (C_P - C_Q),
+//   dR/dy = G Y,  Y = (a + b)/2 C_sh + r (C_P + C_Q),
+//   G dR/dG = -G Z + G (y Y + x X),  Z = a C_P + b C_Q + r C_sh + i C_s   (G d f / d G = t' f'),
+//   dR/ds = s d^2 R / dt^2   (heat equation of the Gaussian)
+//         = s [G^2 (R - 2 (y E_y + x E_x) + y^2 R_y - x^2 R_x) + N(t) (G (y r + x i - a) - t a / s^2)],
+//   E_y = (a + b)/2 T_sh + r T_ch,  E_x = (b - a)/2 T_s + i T_c,
+//   R_y = (a + b)/2 T_ch + r T_sh,  R_x = (a - b)/2 T_c + i T_s.
+// The lanes per event are X, Y, Z and the bracket without its G^2 R, each over R; the last block
+// applies the constant factors (time_gradient).  The kernels are bound by their instructions (FP32)
+// or FP64 slots: summing the derivatives as series too and branching between two erfcx calls cost
+// 2M events FP32 64.1 us (four-body) and 114.5 us (three-body), now 59.3 and 97.3 us; 1M events
+// FP64 four-body 1222 us, now 872 us.
 #pragma once
 
 #include <cmath>
@@ -104,11 +120,11 @@ static const WeidemanTables& weideman() {
 template <typename T>
 struct TimeTerms {
   T P, Q, Tsh, Ts;
-  T d[4][4];  // d[param][term], param = x, y, tau, sigma_t; term = P, Q, sh, s
+  T phi;  // N(t; 0, s)
 };
 
-// Orders of the moment series: u_0 .. u_(2K+2) (the G-derivative of u_(2K+1) needs
-// u_(2K+2)), and the largest z = max(|x|,|y|) G (max(t,0) + 6 s) at which the truncated
+// Orders of the moment series (w_0 .. w_(2K+1)), and the largest
+// z = max(|x|,|y|) G (max(t,0) + 6 s) at which the truncated
 // series is used.  FP32: K = 4, z <= 0.5 (first omitted term of Q below 1e-8 of Q);
 // FP64: K = 6, z <= 0.35 (below 1e-16 of Q).
 template <typename T>
@@ -117,22 +133,25 @@ struct SeriesOrder {
   static constexpr double zmax = sizeof(T) == 4 ? 0.5 : 0.35;
 };
 
-// Per-theta constants of the decay-time terms in the path's precision: the series
-// coefficients and their derivatives, prepared on the host in FP64 from the rounded x, y.
+// Per-theta constants of the decay-time terms in the path's precision, prepared on the host in
+// FP64 from the rounded x, y, G and s.
 template <typename T>
 struct TimeCoef {
   static constexpr int K = SeriesOrder<T>::K;
   T G, x, y, s;
   T zs;                        // max(|x|, |y|) G
-  T a[K + 1], b[K + 1];        // P, Q coefficients of u_2m (a_0 = 1, b_0 = 0)
-  T ysh[K + 1], xs[K + 1];     // T_sh, T_s coefficients of u_(2m+1)
-  T dax[K + 1], day[K + 1];    // d a_m / dx (= -d b_m / dx), d a_m / dy (= d b_m / dy)
-  T dshy[K + 1], dsx[K + 1];   // d ysh_m / dy, d xs_m / dx
+  T a[K + 1], b[K + 1];        // P, Q coefficients of w_2m (a_0 = 1, b_0 = 0)
+  T ysh[K + 1], xs[K + 1];     // T_sh, T_s coefficients of w_(2m+1)
   // the order in use, K - 1 or K, and the largest z at which it meets the truncation
   // criterion: K - 1 when that covers every event the dataset's time range admits
   int ku;
   T zmax_ku;
-  T is2, is2h;  // 1 / s^2 and 1 / (2 s^2), so that no event divides by them
+  T is2, is2h, ir2s;           // 1 / s^2, 1 / (2 s^2), 1 / (s sqrt 2): no event divides by them
+  T k_phi;                     // 1 / (s sqrt(2 pi))
+  T s2, Gs2, hG2s2;            // s^2, G s^2, G^2 s^2 / 2
+  T nG2s2[2 * K + 1];          // n G^2 s^2
+  T hx, hy;                    // s^2 G x / 2, s^2 G y / 2
+  T y2, x2, G2;                // y^2, x^2, G^2
 };
 
 #ifndef __CUDACC_RTC__
@@ -146,21 +165,31 @@ inline void fill_time_coef(TimeCoef<T>& c, double x64, double y64, double tau, d
   c.x = (T)x64;
   c.y = (T)y64;
   c.s = (T)s64;
-  const double x = (double)c.x, y = (double)c.y, G = (double)c.G;
+  const double x = (double)c.x, y = (double)c.y, G = (double)c.G, s = (double)c.s;
   c.zs = (T)(std::fmax(std::fabs(x), std::fabs(y)) * G);
-  c.is2 = (T)(1.0 / ((double)c.s * (double)c.s));
-  c.is2h = (T)(0.5 / ((double)c.s * (double)c.s));
+  c.is2 = (T)(1.0 / (s * s));
+  c.is2h = (T)(0.5 / (s * s));
+  c.ir2s = (T)(0.70710678118654752440 / s);
+  c.k_phi = (T)(0.39894228040143267794 / s);
+  c.s2 = (T)(s * s);
+  c.Gs2 = (T)(G * s * s);
+  for (int n = 0; n <= 2 * K; ++n) c.nG2s2[n] = (T)(n * G * G * s * s);
+  c.hG2s2 = (T)(0.5 * G * G * s * s);
+  c.hx = (T)(0.5 * s * s * G * x);
+  c.hy = (T)(0.5 * s * s * G * y);
+  c.y2 = (T)(y * y);
+  c.x2 = (T)(x * x);
+  c.G2 = (T)(G * G);
+  double fact = 1.0;  // (2m)!
   for (int m = 0; m <= K; ++m) {
     const double sg = (m & 1) ? -1.0 : 1.0;
     const double y2m = std::pow(y, 2 * m), x2m = std::pow(x, 2 * m);
-    c.a[m] = (T)(0.5 * (y2m + sg * x2m));
-    c.b[m] = (T)(0.5 * (y2m - sg * x2m));
-    c.day[m] = (T)(m > 0 ? m * std::pow(y, 2 * m - 1) : 0.0);
-    c.dax[m] = (T)(m > 0 ? sg * m * std::pow(x, 2 * m - 1) : 0.0);
-    c.ysh[m] = (T)(y2m * y);
-    c.xs[m] = (T)(sg * x2m * x);
-    c.dshy[m] = (T)((2 * m + 1) * y2m);
-    c.dsx[m] = (T)(sg * (2 * m + 1) * x2m);
+    c.a[m] = (T)(0.5 * (y2m + sg * x2m) / fact);
+    c.b[m] = (T)(0.5 * (y2m - sg * x2m) / fact);
+    fact *= 2 * m + 1;
+    c.ysh[m] = (T)(y2m * y / fact);
+    c.xs[m] = (T)(sg * x2m * x / fact);
+    fact *= 2 * m + 2;
   }
   c.b[0] = (T)0;
   // the first omitted term against the leading one is about z^(2k) 2 / (2k + 2)! at order k;
@@ -168,11 +197,27 @@ inline void fill_time_coef(TimeCoef<T>& c, double x64, double y64, double tau, d
   auto ratio = [](double z, int k) { return std::pow(z, 2.0 * k) * 2.0 / std::tgamma(2.0 * k + 3.0); };
   const double eps = ratio(SeriesOrder<T>::zmax, K);
   const double zk1 = std::pow(eps * std::tgamma(2.0 * (K - 1) + 3.0) / 2.0, 1.0 / (2.0 * (K - 1)));
-  const double zdata = (double)c.zs * (std::fmax(t_hi, 0.0) + 6.0 * (double)c.s);
+  const double zdata = (double)c.zs * (std::fmax(t_hi, 0.0) + 6.0 * s);
   c.ku = zdata < zk1 ? K - 1 : K;
   c.zmax_ku = (T)(zdata < zk1 ? zk1 : SeriesOrder<T>::zmax);
 }
 #endif
+
+// Products, sums and fused multiply-adds that the compiler neither fuses nor splits: the terms
+// that enter log R are formed with them, so that an evaluation without the gradient (another
+// instantiation of the kernels) returns the same NLL.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+
+// R = |A|^2 P + |B|^2 Q + Re(A B*) T_sh + Im(A B*) T_s
+template <typename T>
+__device__ __forceinline__ T td_rate(const TimeTerms<T>& tt, T AA, T BB, T ABr, T ABi) {
+  return fma_rn(ABi, tt.Ts, fma_rn(ABr, tt.Tsh, fma_rn(BB, tt.Q, mul_rn(AA, tt.P))));
+}
 
 template <typename T>
 __device__ __forceinline__ T td_erfcx(T u) {
@@ -186,24 +231,20 @@ __device__ __forceinline__ T td_exp(T v) {
   else return exp(v);
 }
 
-// E(g) for real g, with dE/dg and dE/ds (gauss = exp(-t^2/2s^2), k = 1/(sqrt(2 pi)))
+// E(g) for real g (gauss = exp(-t^2/2s^2)): with h = gauss erfcx(|u|) / 2, u = (g s^2 - t) / (s sqrt 2),
+// E = h for u >= 0 and exp(g^2 s^2 / 2 - g t) - h below, selected, so that a warp whose events
+// lie on both sides evaluates erfcx once.  hg2s2 = g^2 s^2 / 2.
 template <typename T>
-__device__ __forceinline__ void conv_real(T g, T t, T s, T gauss, T& E, T& dEg, T& dEs) {
-  const T u = (g * s * s - t) * (T(0.70710678118654752440) / s);
-  if (u >= T(0)) {
-    E = T(0.5) * gauss * td_erfcx<T>(u);
-  } else {
-    E = td_exp<T>(T(0.5) * g * g * s * s - g * t) - T(0.5) * gauss * td_erfcx<T>(-u);
-  }
-  const T k = T(0.39894228040143267794);
-  dEg = (g * s * s - t) * E - s * k * gauss;
-  dEs = g * g * s * E - (g * s * s + t) / (s * s) * k * gauss;
+__device__ __forceinline__ T conv_real(T g, T gs2, T hg2s2, T ir2s, T t, T gauss) {
+  const T u = mul_rn(sub_rn(gs2, t), ir2s);
+  const T h = mul_rn(mul_rn(T(0.5), gauss), td_erfcx<T>(u < T(0) ? -u : u));
+  const T x = sub_rn(td_exp<T>(fma_rn(-g, t, hg2s2)), h);
+  return u >= T(0) ? h : x;
 }
 
-// E(g) for complex g = (gr, gi), with dE/dg and dE/ds
+// E(g) for complex g = (gr, gi)
 template <typename T>
-__device__ __forceinline__ void conv_complex(T gr, T gi, T t, T s, T gauss, const T* wa, int wN, T wL, T& Er, T& Ei,
-                                             T& dgr, T& dgi, T& dsr, T& dsi) {
+__device__ __forceinline__ void conv_complex(T gr, T gi, T t, T s, T gauss, const T* wa, int wN, T wL, T& Er, T& Ei) {
   const T c = T(0.70710678118654752440) / s;
   const T ur = (gr * s * s - t) * c, ui = gi * s * s * c;
   T wr, wi;
@@ -221,157 +262,93 @@ __device__ __forceinline__ void conv_complex(T gr, T gi, T t, T s, T gauss, cons
     Er = mag * cs - T(0.5) * gauss * wr;
     Ei = mag * sn - T(0.5) * gauss * wi;
   }
-  const T k = T(0.39894228040143267794);
-  // dE/dg = (g s^2 - t) E - s k gauss
-  const T ar = gr * s * s - t, ai = gi * s * s;
-  dgr = ar * Er - ai * Ei - s * k * gauss;
-  dgi = ar * Ei + ai * Er;
-  // dE/ds = g^2 s E - (g s^2 + t)/s^2 k gauss
-  const T g2r = (gr * gr - gi * gi) * s, g2i = T(2) * gr * gi * s;
-  dsr = g2r * Er - g2i * Ei - (gr * s * s + t) / (s * s) * k * gauss;
-  dsi = g2r * Ei + g2i * Er - gi * k * gauss;
 }
 
 // The decay-time terms at the observed time t from the convolved exponentials (Faddeeva
-// path, any mixing) and their derivatives with respect to (x, y, tau, sigma_t), for
-// Gamma = G, mixing (x, y), resolution s; gauss = exp(-t^2 / 2 s^2).
+// path, any mixing); gauss = exp(-t^2 / 2 s^2).
 template <typename T>
-__device__ __forceinline__ void time_terms_direct(T G, T x, T y, T s, const T* wa, int wN, T wL, T t, T gauss,
+__device__ __forceinline__ void time_terms_direct(const TimeCoef<T>& c, const T* wa, int wN, T wL, T t, T gauss,
                                                   TimeTerms<T>& R) {
-  const T gp = G * (T(1) - y), gm = G * (T(1) + y);
-  T Ep, dEgp, dEsp, Em, dEgm, dEsm;
-  conv_real<T>(gp, t, s, gauss, Ep, dEgp, dEsp);
-  conv_real<T>(gm, t, s, gauss, Em, dEgm, dEsm);
-  T Ecr, Eci, dgr, dgi, dsr, dsi;
-  conv_complex<T>(G, -G * x, t, s, gauss, wa, wN, wL, Ecr, Eci, dgr, dgi, dsr, dsi);
+  const T gp = c.G * (T(1) - c.y), gm = c.G * (T(1) + c.y);
+  const T Ep = conv_real<T>(gp, gp * c.s2, T(0.5) * gp * gp * c.s2, c.ir2s, t, gauss);
+  const T Em = conv_real<T>(gm, gm * c.s2, T(0.5) * gm * gm * c.s2, c.ir2s, t, gauss);
+  T Ecr, Eci;
+  conv_complex<T>(c.G, -c.G * c.x, t, c.s, gauss, wa, wN, wL, Ecr, Eci);
   const T Tch = T(0.5) * (Ep + Em);
   R.P = T(0.5) * (Tch + Ecr);
   R.Q = T(0.5) * (Tch - Ecr);
   R.Tsh = T(0.5) * (Ep - Em);
   R.Ts = Eci;
-  // per parameter the derivatives of (T_ch, T_c) map to P, Q as the terms do
-  T dch[4], dc[4];
-  // x: dgc/dx = -i G  ->  (-iG)(dgr + i dgi) = G dgi - i G dgr
-  dch[0] = T(0);
-  dc[0] = G * dgi;
-  R.d[0][2] = T(0);
-  R.d[0][3] = -G * dgr;
-  // y: dg+/dy = -G, dg-/dy = +G
-  dch[1] = T(0.5) * G * (dEgm - dEgp);
-  dc[1] = T(0);
-  R.d[1][2] = -T(0.5) * G * (dEgp + dEgm);
-  R.d[1][3] = T(0);
-  // tau: dg/dtau = -g G
-  dch[2] = -T(0.5) * G * (dEgp * gp + dEgm * gm);
-  dc[2] = -G * (dgr * G - dgi * (-G * x));  // Re((dgr + i dgi)(-gc G)), gc = (G, -G x)
-  R.d[2][2] = -T(0.5) * G * (dEgp * gp - dEgm * gm);
-  R.d[2][3] = -G * (dgr * (-G * x) + dgi * G);
-  // sigma_t
-  dch[3] = T(0.5) * (dEsp + dEsm);
-  dc[3] = dsr;
-  R.d[3][2] = T(0.5) * (dEsp - dEsm);
-  R.d[3][3] = dsi;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    R.d[j][0] = T(0.5) * (dch[j] + dc[j]);
-    R.d[j][1] = T(0.5) * (dch[j] - dc[j]);
-  }
 }
 
 // The decay-time terms by the moment series of order KU (small mixing; see the top of this
 // file).
 template <typename T, int KU>
 __device__ __forceinline__ void time_terms_series(const TimeCoef<T>& c, T t, T gauss, TimeTerms<T>& R) {
-  constexpr int K = KU;
-  constexpr int NU = 2 * K + 3;
-  const T G = c.G, s = c.s;
-  const T s2 = s * s;
-  T E0, dEg_unused, dEs_unused;
-  conv_real<T>(G, t, s, gauss, E0, dEg_unused, dEs_unused);
-  const T phi = T(0.39894228040143267794) / s * gauss;  // N(t; 0, s)
-  const T v = t - G * s2;
-  const T Gv = G * v, G2s2 = G * G * s2;
-  T u[NU];
-  u[0] = E0;
-  u[1] = G * (v * E0 + s2 * phi);
+  constexpr int NW = 2 * KU + 2;
+  const T v = sub_rn(t, c.Gs2), Gv = mul_rn(c.G, v);
+  T w[NW];
+  w[0] = conv_real<T>(c.G, c.Gs2, c.hG2s2, c.ir2s, t, gauss);
+  w[1] = mul_rn(c.G, fma_rn(v, w[0], mul_rn(c.s2, R.phi)));
 #pragma unroll
-  for (int n = 1; n < NU - 1; ++n) u[n + 1] = (Gv * u[n] + G2s2 * u[n - 1]) * T(1.0 / (n + 1));
-  // d u_n / d s (heat equation) and G d u_n / d G
-  const T G2 = G * G;
-  auto su = [&](int n) -> T {
-    const T um1 = n >= 1 ? u[n - 1] : T(0), um2 = n >= 2 ? u[n - 2] : T(0);
-    const T cn = n == 0 ? (-t * c.is2 - G) * phi : (n == 1 ? G * phi : T(0));
-    return s * (G2 * ((u[n] - um1) - (um1 - um2)) + cn);
-  };
-  auto gu = [&](int n) -> T { return T(n) * u[n] - T(n + 1) * u[n + 1]; };
-  T P = u[0], Q = T(0), Tsh = T(0), Ts = T(0);
-  T Px = T(0), Py = T(0), PG = gu(0), Ps = su(0), QG = T(0), Qs = T(0);
-  T Shy = T(0), ShG = T(0), Shs = T(0), Sx = T(0), SG = T(0), Ss = T(0);
+  for (int n = 1; n < NW - 1; ++n) w[n + 1] = fma_rn(Gv, w[n], mul_rn(c.nG2s2[n], w[n - 1]));
+  R.P = w[0];
+  R.Q = mul_rn(c.b[1], w[2]);
+  R.Tsh = mul_rn(c.ysh[0], w[1]);
+  R.Ts = mul_rn(c.xs[0], w[1]);
 #pragma unroll
-  for (int m = 1; m <= K; ++m) {
-    const T ue = u[2 * m];
-    P += c.a[m] * ue;
-    Q += c.b[m] * ue;
-    Px += c.dax[m] * ue;
-    Py += c.day[m] * ue;
-    const T ge = gu(2 * m), se = su(2 * m);
-    PG += c.a[m] * ge;
-    QG += c.b[m] * ge;
-    Ps += c.a[m] * se;
-    Qs += c.b[m] * se;
+  for (int m = 1; m <= KU; ++m) {
+    R.P = fma_rn(c.a[m], w[2 * m], R.P);
+    if (m > 1) R.Q = fma_rn(c.b[m], w[2 * m], R.Q);
+    R.Tsh = fma_rn(c.ysh[m], w[2 * m + 1], R.Tsh);
+    R.Ts = fma_rn(c.xs[m], w[2 * m + 1], R.Ts);
   }
-#pragma unroll
-  for (int m = 0; m <= K; ++m) {
-    const T uo = u[2 * m + 1];
-    Tsh += c.ysh[m] * uo;
-    Ts += c.xs[m] * uo;
-    Shy += c.dshy[m] * uo;
-    Sx += c.dsx[m] * uo;
-    const T go = gu(2 * m + 1), so = su(2 * m + 1);
-    ShG += c.ysh[m] * go;
-    SG += c.xs[m] * go;
-    Shs += c.ysh[m] * so;
-    Ss += c.xs[m] * so;
-  }
-  R.P = P;
-  R.Q = Q;
-  R.Tsh = Tsh;
-  R.Ts = Ts;
-  // x: P and Q move oppositely; T_sh does not depend on x, T_s not on y
-  R.d[0][0] = Px;
-  R.d[0][1] = -Px;
-  R.d[0][2] = T(0);
-  R.d[0][3] = Sx;
-  R.d[1][0] = Py;
-  R.d[1][1] = Py;
-  R.d[1][2] = Shy;
-  R.d[1][3] = T(0);
-  // tau: d / d tau = -G (G d / d G)
-  R.d[2][0] = -G * PG;
-  R.d[2][1] = -G * QG;
-  R.d[2][2] = -G * ShG;
-  R.d[2][3] = -G * SG;
-  R.d[3][0] = Ps;
-  R.d[3][1] = Qs;
-  R.d[3][2] = Shs;
-  R.d[3][3] = Ss;
 }
 
-// The decay-time terms at the observed time t and their derivatives: the moment series of the
+// The decay-time terms at the observed time t: the moment series of the
 // order in use where z = max(|x|, |y|) G (max(t, 0) + 6 s) is below its limit (c.zmax_ku),
 // else the Faddeeva path.
 template <typename T>
 __device__ __forceinline__ void time_terms_g(const TimeCoef<T>& c, const T* wa, int wN, T wL, T t, TimeTerms<T>& R) {
-  const T gauss = td_exp<T>(-t * t * c.is2h);
+  const T gauss = td_exp<T>(mul_rn(mul_rn(-t, t), c.is2h));
+  R.phi = mul_rn(c.k_phi, gauss);
   const T z = c.zs * ((t > T(0) ? t : T(0)) + T(6) * c.s);
   if (z < c.zmax_ku) {
     // the same order for every event of a launch (a uniform branch)
     if (c.ku == TimeCoef<T>::K) time_terms_series<T, TimeCoef<T>::K>(c, t, gauss, R);
     else time_terms_series<T, TimeCoef<T>::K - 1>(c, t, gauss, R);
   } else {
-    time_terms_direct<T>(c.G, c.x, c.y, c.s, wa, wN, wL, t, gauss, R);
+    time_terms_direct<T>(c, wa, wN, wL, t, gauss, R);
   }
 }
 
+// Adds one event's lanes X / R, Y / R, Z / R and the d^2 / dt^2 bracket / R (see the top of this
+// file) to lt; AA = |A|^2, BB = |B|^2, (ABr, ABi) = A conj(B).
+template <typename T>
+__device__ __forceinline__ void time_lanes(const TimeCoef<T>& c, T t, const TimeTerms<T>& tt, T AA, T BB, T ABr,
+                                           T ABi, T invR, T (&lt)[4]) {
+  const T v = t - c.Gs2;
+  const T Tch = tt.P + tt.Q, Tc = tt.P - tt.Q;
+  const T ysh = c.hy * tt.Tsh, xs = c.hx * tt.Ts;
+  const T CP = v * tt.P + (c.s2 * tt.phi + (ysh - xs)), CQ = v * tt.Q + (ysh + xs);
+  const T Csh = v * tt.Tsh + (T(2) * c.hy) * Tch, Cs = v * tt.Ts + (T(2) * c.hx) * Tc;
+  const T hp = T(0.5) * (AA + BB), hm = T(0.5) * (BB - AA);
+  lt[0] += (hm * Cs + ABi * (CP - CQ)) * invR;
+  lt[1] += (hp * Csh + ABr * (CP + CQ)) * invR;
+  lt[2] += (AA * CP + BB * CQ + ABr * Csh + ABi * Cs) * invR;
+  const T Ey = hp * tt.Tsh + ABr * Tch, Ex = hm * tt.Ts + ABi * Tc;
+  const T Ry = hp * Tch + ABr * tt.Tsh, Rx = ABi * tt.Ts - hm * Tc;
+  const T q = c.G2 * (c.y2 * Ry - c.x2 * Rx - T(2) * (c.y * Ey + c.x * Ex));
+  lt[3] += (q + tt.phi * (c.G * (c.y * ABr + c.x * ABi) - (c.G + t * c.is2) * AA)) * invR;
+}
+
+// sum_i (dR_i / dp_j) / R_i of j = x, y, tau, sigma_t from the lane sums of n events (FP64).
+__device__ __forceinline__ double time_gradient(int j, double G, double x, double y, double s, const double* lanes,
+                                                double n) {
+  if (j == 0) return G * lanes[0];
+  if (j == 1) return G * lanes[1];
+  if (j == 2) return G * G * (lanes[2] - y * lanes[1] - x * lanes[0]);  // -G (G d / dG)
+  return s * (G * G * n + lanes[3]);
+}
 
 }  // namespace goo
