@@ -106,6 +106,7 @@ struct Scratch {
   double* chunk_records = nullptr;
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t chunk_events[65] = {};
+  void* fp64_tables = nullptr;      // device copy of the FP64 function tables (fp64.cuh), on first use
 };
 constexpr int kStreamChunks = 64;  // chunks of one goo_nll_grad_streamed call, at most
 

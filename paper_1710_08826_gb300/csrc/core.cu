@@ -452,6 +452,7 @@ int goo_finalize(goo_ctx* ctx) {
   if (s.partials) cudaFree(s.partials);
   if (s.counters) cudaFree(s.counters);
   if (s.result) cudaFree(s.result);
+  if (s.fp64_tables) cudaFree(s.fp64_tables);
   if (s.theta) cudaFree(s.theta);
   if (s.host_pinned) cudaFreeHost(s.host_pinned);
   if (s.result_host) cudaFreeHost(s.result_host);

@@ -784,142 +784,20 @@ struct Td3Lanes {
   static constexpr int NS = GRAD ? 1 + 2 * (kTd3KB + 1) + 4 : 1;
 };
 
+// Block and last-block reductions of the lanes and the FP64 combination with the normalisation
+// terms the host formed from the three Gram matrices (they depend on theta and the MC sample
+// only).  lf: the thread's sum of log R as a double-float.
 template <typename T, bool GRAD>
-__global__ void __launch_bounds__(kBlock, 2)
-    td3_nll_kernel(const __grid_constant__ Td3Args<T> a, const void* __restrict__ cache_a,
-                   const void* __restrict__ cache_b, const T* __restrict__ tcol, int64_t begin, int64_t end,
-                   float2* partials, unsigned* counters, double* out, int out_mode) {
+__device__ __forceinline__ void td3_finish(const Td3Args<T>& a, ddf lf, const T (&lre)[kTd3KB + 1],
+                                           const T (&lim)[kTd3KB + 1], const T (&lt)[4], unsigned bad, int64_t begin,
+                                           int64_t end, float2* partials, unsigned* counters, double* out, int out_mode,
+                                           ddf* s_red, unsigned* s_bad) {
   constexpr int KB = kTd3KB, KA = KB + 1;
   constexpr int NS = Td3Lanes<GRAD>::NS;
-  __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
-  __shared__ unsigned s_bad[kBlock / 32];
   __shared__ double s_out[NS];
-  const int64_t n = a.n_total;
   const int nbw = a.nbw;
-  // the amplitude pair of slot k (< nbw) at event i: a_k and abar_k
-  auto load = [&](int k, int64_t i, T& ar, T& ai, T& br, T& bi) {
-    if constexpr (sizeof(T) == 4) {
-      const float4 va = __ldg((const float4*)cache_a + (int64_t)(k / 2) * n + i);
-      const float4 vb = __ldg((const float4*)cache_b + (int64_t)(k / 2) * n + i);
-      ar = (k & 1) ? va.z : va.x;
-      ai = (k & 1) ? va.w : va.y;
-      br = (k & 1) ? vb.z : vb.x;
-      bi = (k & 1) ? vb.w : vb.y;
-    } else {
-      const double2 va = __ldg((const double2*)cache_a + (int64_t)k * n + i);
-      const double2 vb = __ldg((const double2*)cache_b + (int64_t)k * n + i);
-      ar = va.x;
-      ai = va.y;
-      br = vb.x;
-      bi = vb.y;
-    }
-  };
-  // FP32: all amplitude planes of the event are requested before any is used (loads
-  // predicated on the plane count rather than a loop exit, so none waits on the arithmetic of
-  // the one before), and kept for the gradient lanes
-  constexpr int NP = sizeof(T) == 4 ? (KB + 1) / 2 : 1;
-  float4 pa[NP], pb[NP];
-#pragma unroll
-  for (int q = 0; q < NP; ++q) pa[q] = pb[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto get = [&](int k, int64_t i, T& ar, T& ai, T& br, T& bi) {
-    if constexpr (sizeof(T) == 4) {
-      const float4 va = pa[k / 2], vb = pb[k / 2];
-      ar = (k & 1) ? va.z : va.x;
-      ai = (k & 1) ? va.w : va.y;
-      br = (k & 1) ? vb.z : vb.x;
-      bi = (k & 1) ? vb.w : vb.y;
-    } else {
-      load(k, i, ar, ai, br, bi);
-    }
-  };
-  Kahan lf32;
-  double lf64 = 0.0;
-  T lre[KA], lim[KA], lt[4];
-#pragma unroll
-  for (int k = 0; k < KA; ++k) lre[k] = lim[k] = T(0);
-#pragma unroll
-  for (int j = 0; j < 4; ++j) lt[j] = T(0);
-  unsigned bad = 0;
-  for (int64_t i = begin + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < end;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const T t = tcol[i];
-    if constexpr (sizeof(T) == 4) {
-#pragma unroll
-      for (int q = 0; q < NP; ++q)
-        if (2 * q < nbw) {
-          pa[q] = __ldg((const float4*)cache_a + (int64_t)q * n + i);
-          pb[q] = __ldg((const float4*)cache_b + (int64_t)q * n + i);
-        }
-    }
-    T Ar = a.cr[KB], Ai = a.ci[KB], Br = a.cr[KB], Bi = a.ci[KB];  // the NR amplitude is 1 for both
-    if constexpr (sizeof(T) == 4) {
-      // FP32: the sums as packed (re, im) FMAs on the planes' halves, (sum cr_k a_k) and
-      // (sum ci_k a_k) per cache, combined once: four packed FMAs per amplitude, not eight
-      using namespace pk;
-      float2 P1 = make_float2(Ar, Ai), P2 = splat(0.f), Q1 = make_float2(Br, Bi), Q2 = splat(0.f);
-#pragma unroll
-      for (int k = 0; k < KB; ++k) {
-        if (k >= nbw) break;
-        const float4 va = pa[k / 2], vb = pb[k / 2];
-        const float2 ak = (k & 1) ? make_float2(va.z, va.w) : make_float2(va.x, va.y);
-        const float2 bk = (k & 1) ? make_float2(vb.z, vb.w) : make_float2(vb.x, vb.y);
-        P1 = fma(splat(a.cr[k]), ak, P1);
-        P2 = fma(splat(a.ci[k]), ak, P2);
-        Q1 = fma(splat(a.cr[k]), bk, Q1);
-        Q2 = fma(splat(a.ci[k]), bk, Q2);
-      }
-      Ar = P1.x - P2.y;
-      Ai = P1.y + P2.x;
-      Br = Q1.x - Q2.y;
-      Bi = Q1.y + Q2.x;
-    } else {
-#pragma unroll
-      for (int k = 0; k < KB; ++k) {
-        if (k >= nbw) break;
-        T ar, ai, br, bi;
-        get(k, i, ar, ai, br, bi);
-        Ar += a.cr[k] * ar - a.ci[k] * ai;
-        Ai += a.cr[k] * ai + a.ci[k] * ar;
-        Br += a.cr[k] * br - a.ci[k] * bi;
-        Bi += a.cr[k] * bi + a.ci[k] * br;
-      }
-    }
-    TimeTerms<T> tt;
-    time_terms_g<T>(a.tc, a.wa, a.wN, a.wL, t, tt);
-    const T AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
-    const T ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
-    const T R = td_rate(tt, AA, BB, ABr, ABi);
-    if (!(R > T(0))) {
-      ++bad;
-      continue;
-    }
-    if constexpr (sizeof(T) == 4) lf32.add(pk::lg2(R));  // log2 R, scaled by ln 2 at the end
-    else lf64 += log(R);
-    if constexpr (GRAD) {
-      T invR;
-      if constexpr (sizeof(T) == 4) invR = pk::rcp(R);
-      else invR = T(1) / R;
-      const T cp = T(2) * tt.P * invR, cm = T(2) * tt.Q * invR, sh = tt.Tsh * invR, ss = tt.Ts * invR;
-      // V_A / R = cp A* + (sh - i ss) B*,  V_B / R = cm B* + (sh + i ss) A*
-      const T VAr = cp * Ar + sh * Br - ss * Bi, VAi = -cp * Ai - sh * Bi - ss * Br;
-      const T VBr = cm * Br + sh * Ar + ss * Ai, VBi = -cm * Bi - sh * Ai + ss * Ar;
-#pragma unroll
-      for (int k = 0; k < KB; ++k) {
-        if (k >= nbw) break;
-        T ar, ai, br, bi;
-        get(k, i, ar, ai, br, bi);
-        const T qr = ar * VAr - ai * VAi + br * VBr - bi * VBi;  // Re(a V_A + abar V_B) / R
-        const T qi = ar * VAi + ai * VAr + br * VBi + bi * VBr;
-        lre[k] += qr;
-        lim[k] -= qi;
-      }
-      lre[KB] += VAr + VBr;  // the NR slot (a = abar = 1)
-      lim[KB] -= VAi + VBi;
-      time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, lt);
-    }
-  }
   ddf v[NS];
-  v[0] = (sizeof(T) == 4) ? dd_mul(lf32.value(), ddf{kLn2Hi, kLn2Lo}) : dd_from_double(lf64);
+  v[0] = lf;
   if constexpr (GRAD) {
 #pragma unroll
     for (int k = 0; k < KA; ++k) {
@@ -939,8 +817,6 @@ __global__ void __launch_bounds__(kBlock, 2)
     if (b) atomicAdd(counters + 1, b);
   }
   if (!last_block_ticket(counters, gridDim.x)) return;
-  // The last block reduces the lanes and combines them with the normalisation terms the host
-  // formed from the three Gram matrices (they depend on theta and the MC sample only).
   // Every other block added to the counter words before its ticket (and a fence): plain L2
   // reads, issued before the reduction so that their latency overlaps it.
   unsigned nbad = 0u, status = 0u;
@@ -986,6 +862,170 @@ __global__ void __launch_bounds__(kBlock, 2)
     }
   }
   result_complete(out, P > 1 ? P : 1);
+}
+
+// FP32: all amplitude planes of the event are requested before any is used (loads
+// predicated on the plane count rather than a loop exit, so none waits on the arithmetic of
+// the one before), and kept for the gradient lanes; the sums run as packed (re, im) FMAs on the
+// planes' halves, (sum cr_k a_k) and (sum ci_k a_k) per cache, combined once: four packed FMAs per
+// amplitude, not eight.
+template <bool GRAD>
+__global__ void __launch_bounds__(kBlock, 2)
+    td3_nll_f32_kernel(const __grid_constant__ Td3Args<float> a, const float4* __restrict__ cache_a,
+                       const float4* __restrict__ cache_b, const float* __restrict__ tcol, int64_t begin, int64_t end,
+                       float2* partials, unsigned* counters, double* out, int out_mode) {
+  using namespace pk;
+  constexpr int KB = kTd3KB, KA = KB + 1;
+  constexpr int NS = Td3Lanes<GRAD>::NS;
+  __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
+  __shared__ unsigned s_bad[kBlock / 32];
+  const int64_t n = a.n_total;
+  const int nbw = a.nbw;
+  constexpr int NP = (KB + 1) / 2;
+  float4 pa[NP], pb[NP];
+#pragma unroll
+  for (int q = 0; q < NP; ++q) pa[q] = pb[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto amp_a = [&](int k) { return (k & 1) ? make_float2(pa[k / 2].z, pa[k / 2].w) : make_float2(pa[k / 2].x, pa[k / 2].y); };
+  auto amp_b = [&](int k) { return (k & 1) ? make_float2(pb[k / 2].z, pb[k / 2].w) : make_float2(pb[k / 2].x, pb[k / 2].y); };
+  Kahan lf32;
+  float lre[KA], lim[KA], lt[4];
+#pragma unroll
+  for (int k = 0; k < KA; ++k) lre[k] = lim[k] = 0.f;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) lt[j] = 0.f;
+  unsigned bad = 0;
+  for (int64_t i = begin + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < end;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const float t = tcol[i];
+#pragma unroll
+    for (int q = 0; q < NP; ++q)
+      if (2 * q < nbw) {
+        pa[q] = __ldg(cache_a + (int64_t)q * n + i);
+        pb[q] = __ldg(cache_b + (int64_t)q * n + i);
+      }
+    // the NR amplitude is 1 for both
+    float2 P1 = make_float2(a.cr[KB], a.ci[KB]), P2 = splat(0.f), Q1 = P1, Q2 = splat(0.f);
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      if (k >= nbw) break;
+      const float2 ak = amp_a(k), bk = amp_b(k);
+      P1 = fma(splat(a.cr[k]), ak, P1);
+      P2 = fma(splat(a.ci[k]), ak, P2);
+      Q1 = fma(splat(a.cr[k]), bk, Q1);
+      Q2 = fma(splat(a.ci[k]), bk, Q2);
+    }
+    const float Ar = P1.x - P2.y, Ai = P1.y + P2.x, Br = Q1.x - Q2.y, Bi = Q1.y + Q2.x;
+    TimeTerms<float> tt;
+    time_terms_g<float>(TdMath<float>{}, a.tc, a.wa, a.wN, a.wL, t, tt);
+    const float AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
+    const float ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
+    const float R = td_rate(tt, AA, BB, ABr, ABi);
+    if (!(R > 0.f)) {
+      ++bad;
+      continue;
+    }
+    lf32.add(lg2(R));  // log2 R, scaled by ln 2 at the end
+    if constexpr (GRAD) {
+      const float invR = rcp(R);
+      const float cp = 2.f * tt.P * invR, cm = 2.f * tt.Q * invR, sh = tt.Tsh * invR, ss = tt.Ts * invR;
+      // V_A / R = cp A* + (sh - i ss) B*,  V_B / R = cm B* + (sh + i ss) A*
+      const float VAr = cp * Ar + sh * Br - ss * Bi, VAi = -cp * Ai - sh * Bi - ss * Br;
+      const float VBr = cm * Br + sh * Ar + ss * Ai, VBi = -cm * Bi - sh * Ai + ss * Ar;
+#pragma unroll
+      for (int k = 0; k < KB; ++k) {
+        if (k >= nbw) break;
+        const float2 ak = amp_a(k), bk = amp_b(k);
+        const float qr = ak.x * VAr - ak.y * VAi + bk.x * VBr - bk.y * VBi;  // Re(a V_A + abar V_B) / R
+        const float qi = ak.x * VAi + ak.y * VAr + bk.x * VBi + bk.y * VBr;
+        lre[k] += qr;
+        lim[k] -= qi;
+      }
+      lre[KB] += VAr + VBr;  // the NR slot (a = abar = 1)
+      lim[KB] -= VAi + VBi;
+      time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, lt);
+    }
+  }
+  td3_finish<float, GRAD>(a, dd_mul(lf32.value(), ddf{kLn2Hi, kLn2Lo}), lre, lim, lt, bad, begin, end, partials, counters,
+                          out, out_mode, s_red, s_bad);
+}
+
+// FP64: bound by the FP64 pipe's slots (fp64.cuh), as the four-body kernel: FMA chains, exp and
+// erfcx from tables in shared memory, the logarithm as a running product, tests on the integer
+// pipe, the amplitudes read again for the gradient lanes.  0.4M events with the gradient: 751 -> 369 us
+// per call (with the derivatives' closed form of timeterms.cuh).
+template <bool GRAD>
+__global__ void __launch_bounds__(kBlock, 2)
+    td3_nll_f64_kernel(const __grid_constant__ Td3Args<double> a, const double2* __restrict__ cache_a,
+                       const double2* __restrict__ cache_b, const double* __restrict__ tcol,
+                       const Fp64Tables* __restrict__ tables, int64_t begin, int64_t end, float2* partials,
+                       unsigned* counters, double* out, int out_mode) {
+  constexpr int KB = kTd3KB, KA = KB + 1;
+  constexpr int NS = Td3Lanes<GRAD>::NS;
+  __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
+  __shared__ unsigned s_bad[kBlock / 32];
+  __shared__ __align__(16) Fp64Tables s_tab;
+  load_fp64_tables(s_tab, tables);
+  const TdMath<double> F{s_tab};
+  const int64_t n = a.n_total;
+  const int nbw = a.nbw;
+  LogProduct lp;
+  double lf64 = 0.0;
+  double lre[KA], lim[KA], lt[4];
+#pragma unroll
+  for (int k = 0; k < KA; ++k) lre[k] = lim[k] = 0.0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) lt[j] = 0.0;
+  unsigned bad = 0;
+  __syncthreads();
+  for (int64_t i = begin + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < end;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const double t = tcol[i];
+    double Ar = a.cr[KB], Ai = a.ci[KB], Br = a.cr[KB], Bi = a.ci[KB];  // the NR amplitude is 1 for both
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      if (k >= nbw) break;
+      const double2 va = __ldg(cache_a + (int64_t)k * n + i), vb = __ldg(cache_b + (int64_t)k * n + i);
+      Ar = fma(a.cr[k], va.x, fma(-a.ci[k], va.y, Ar));
+      Ai = fma(a.cr[k], va.y, fma(a.ci[k], va.x, Ai));
+      Br = fma(a.cr[k], vb.x, fma(-a.ci[k], vb.y, Br));
+      Bi = fma(a.cr[k], vb.y, fma(a.ci[k], vb.x, Bi));
+    }
+    TimeTerms<double> tt;
+    time_terms_g<double>(F, a.tc, a.wa, a.wN, a.wL, t, tt);
+    const double AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
+    const double ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
+    const double R = td_rate(tt, AA, BB, ABr, ABi);
+    double invR;
+    if (positive_normal(R)) {
+      lp.mul(R);
+      invR = rcp64(R);
+    } else if (R > 0.0) {  // subnormal or infinite
+      lf64 += log(R);
+      invR = 1.0 / R;
+    } else {
+      ++bad;
+      continue;
+    }
+    if constexpr (GRAD) {
+      const double cp = 2.0 * tt.P * invR, cm = 2.0 * tt.Q * invR, sh = tt.Tsh * invR, ss = tt.Ts * invR;
+      // V_A / R = cp A* + (sh - i ss) B*,  V_B / R = cm B* + (sh + i ss) A*; m...i: minus the imaginary part
+      const double VAr = fma(cp, Ar, fma(sh, Br, -ss * Bi)), mVAi = fma(cp, Ai, fma(sh, Bi, ss * Br));
+      const double VBr = fma(cm, Br, fma(sh, Ar, ss * Ai)), mVBi = fma(cm, Bi, fma(sh, Ai, -ss * Ar));
+#pragma unroll
+      for (int k = 0; k < KB; ++k) {
+        if (k >= nbw) break;
+        const double2 va = __ldg(cache_a + (int64_t)k * n + i), vb = __ldg(cache_b + (int64_t)k * n + i);
+        lre[k] = fma(va.x, VAr, fma(va.y, mVAi, fma(vb.x, VBr, fma(vb.y, mVBi, lre[k]))));
+        lim[k] = fma(va.x, mVAi, fma(-va.y, VAr, fma(vb.x, mVBi, fma(-vb.y, VBr, lim[k]))));
+      }
+      lre[KB] += VAr + VBr;  // the NR slot (a = abar = 1)
+      lim[KB] += mVAi + mVBi;
+      time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, lt);
+    }
+  }
+  lf64 += lp.log_value();
+  td3_finish<double, GRAD>(a, dd_from_double(lf64), lre, lim, lt, bad, begin, end, partials, counters, out, out_mode,
+                           s_red, s_bad);
 }
 
 static int dalitz_constants(goo_model* m, const double* theta) {
@@ -1487,27 +1527,29 @@ static int launch_td3(goo_model* m, const goo_dataset* ds, int64_t begin, int64_
   DalitzModel& d = *m->dalitz;
   goo_ctx* ctx = m->ctx;
   const int pi = sizeof(T) == 4 ? 0 : 1;
-  static int occ[2] = {0, 0};
-  int& o = occ[pi];
-  if (o == 0) {
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, td3_nll_kernel<T, GRAD>, kBlock, 0) != cudaSuccess || o < 1) {
-      cudaGetLastError();
-      o = 1;
-    }
-  }
-  const int nb = grid_blocks(ctx, end - begin, o);
+  const void* fn;
+  if constexpr (sizeof(T) == 4) fn = (const void*)td3_nll_f32_kernel<GRAD>;
+  else fn = (const void*)td3_nll_f64_kernel<GRAD>;
+  const int nb = grid_blocks(ctx, end - begin, cached_occupancy(fn, ctx->device, kBlock, 0));
   constexpr int NS = Td3Lanes<GRAD>::NS;
   GOO_TRY(ensure_partials(ctx, (size_t)nb * NS));
+  const Fp64Tables* tables = nullptr;
+  if (sizeof(T) == 8) GOO_TRY(fp64_tables(ctx, &tables));
   Td3Args<T> a;
   fill_td3<T>(d, theta, m->n_params, ds->n, a, m->hi[d.col_t]);
   td3_norm_terms<T>(d, d.gram3_host[pi], a);
-  const T* tcol = sizeof(T) == 4 ? (const T*)ds->d32[d.col_t] : (const T*)ds->d64[d.col_t];
   {
     LaunchScope ls(ctx, sizeof(T) == 4 ? (GRAD ? "td3_nll_grad_f32" : "td3_nll_f32")
                                        : (GRAD ? "td3_nll_grad_f64" : "td3_nll_f64"));
-    td3_nll_kernel<T, GRAD><<<nb, kBlock, 0, ctx->stream>>>(a, ca, cb, tcol, begin, end, ctx->scratch.partials,
-                                                            ctx->scratch.counters, ctx->scratch.result_out,
-                                                            out_mode);
+    if constexpr (sizeof(T) == 4)
+      td3_nll_f32_kernel<GRAD><<<nb, kBlock, 0, ctx->stream>>>(a, (const float4*)ca, (const float4*)cb, ds->d32[d.col_t],
+                                                               begin, end, ctx->scratch.partials, ctx->scratch.counters,
+                                                               ctx->scratch.result_out, out_mode);
+    else
+      td3_nll_f64_kernel<GRAD><<<nb, kBlock, 0, ctx->stream>>>(a, (const double2*)ca, (const double2*)cb,
+                                                               ds->d64[d.col_t], tables, begin, end,
+                                                               ctx->scratch.partials, ctx->scratch.counters,
+                                                               ctx->scratch.result_out, out_mode);
   }
   GOO_CUDA_TRY(cudaGetLastError());
   return GOO_OK;

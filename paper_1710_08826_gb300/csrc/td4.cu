@@ -155,11 +155,6 @@ __global__ void td4_cache_kernel(const Td4Dev* __restrict__ tdp, Td4Cols<T> cols
   }
 }
 
-template <typename T>
-__device__ __forceinline__ void time_terms(const Td4Args<T>& a, T t, TimeTerms<T>& R) {
-  time_terms_g<T>(a.tc, a.wa, a.wN, a.wL, t, R);
-}
-
 // ---------------------------------------------------------------------------------------
 // NLL kernels
 // ---------------------------------------------------------------------------------------
@@ -176,52 +171,14 @@ struct TdAcc {
   unsigned bad = 0;
 };
 
-// One event from its amplitudes (ar, ai) and observed time t.
-template <typename T, int KB, bool GRAD>
-__device__ __forceinline__ void td4_event(const Td4Args<T>& a, const T (&ar)[KB], const T (&ai)[KB], T t,
-                                          TdAcc<T, KB>& acc) {
-  T Ar = T(0), Ai = T(0), Br = T(0), Bi = T(0);
-#pragma unroll
-  for (int k = 0; k < KB; ++k) {
-    Ar += a.cr[k] * ar[k] - a.ci[k] * ai[k];
-    Ai += a.cr[k] * ai[k] + a.ci[k] * ar[k];
-    Br += a.br[k] * ar[k] - a.bi[k] * ai[k];
-    Bi += a.br[k] * ai[k] + a.bi[k] * ar[k];
-  }
-  TimeTerms<T> tt;
-  time_terms<T>(a, t, tt);
-  const T AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
-  const T ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
-  const T R = td_rate(tt, AA, BB, ABr, ABi);
-  if (!(R > T(0))) {
-    acc.bad++;
-    return;
-  }
-  if constexpr (sizeof(T) == 4) acc.lf32.add(logf(R));
-  else acc.lf64 += log(R);
-  if constexpr (GRAD) {
-    const T invR = T(1) / R;
-    // V / R, V = (T_ch + T_c) A* + (T_sh - i T_s) B* = 2 P A* + (T_sh - i T_s) B*
-    const T c1 = T(2) * tt.P * invR, sh = tt.Tsh * invR, ss = tt.Ts * invR;
-    const T Vr = c1 * Ar + sh * Br - ss * Bi;
-    const T Vi = -c1 * Ai - sh * Bi - ss * Br;
-#pragma unroll
-    for (int k = 0; k < KB; ++k) {
-      acc.lre[k] += ar[k] * Vr - ai[k] * Vi;     // Re(a_k V) / R
-      acc.lim[k] += -(ar[k] * Vi + ai[k] * Vr);  // -Im(a_k V) / R
-    }
-    time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, acc.lt);
-  }
-}
-
-// The FP32 form of td4_event in the staged kernel.  The amplitudes come as (re, im) pairs
+// One event of the FP32 kernel.  The amplitudes come as (re, im) pairs
 // straight from the float4 planes, and A = sum c_k a_k is formed from two packed sums,
 // (sum cr_k re_k, sum cr_k im_k) and (sum ci_k re_k, sum ci_k im_k), B likewise: four packed
 // FMAs per amplitude instead of eight scalar ones.  log2 R is accumulated (td4_finish scales
 // the FP32 sum by ln 2 once per thread) and 1/R is the hardware reciprocal.
-template <int KB, bool GRAD>
-__device__ __forceinline__ void td4_event_f32(const Td4Args<float>& a, const float2 (&am)[KB], float t,
-                                              TdAcc<float, KB>& acc) {
+template <int KB>
+__device__ __forceinline__ void td4_sums_f32(const Td4Args<float>& a, const float2 (&am)[KB], float& Ar, float& Ai,
+                                             float& Br, float& Bi) {
   using namespace pk;
   float2 P1 = splat(0.f), P2 = splat(0.f), Q1 = splat(0.f), Q2 = splat(0.f);
 #pragma unroll
@@ -231,9 +188,20 @@ __device__ __forceinline__ void td4_event_f32(const Td4Args<float>& a, const flo
     Q1 = fma(splat(a.br[k]), am[k], Q1);
     Q2 = fma(splat(a.bi[k]), am[k], Q2);
   }
-  const float Ar = P1.x - P2.y, Ai = P1.y + P2.x, Br = Q1.x - Q2.y, Bi = Q1.y + Q2.x;
+  Ar = P1.x - P2.y;
+  Ai = P1.y + P2.x;
+  Br = Q1.x - Q2.y;
+  Bi = Q1.y + Q2.x;
+}
+
+template <int KB, bool GRAD>
+__device__ __forceinline__ void td4_event_f32(const Td4Args<float>& a, const float2 (&am)[KB], float t,
+                                              TdAcc<float, KB>& acc) {
+  using namespace pk;
+  float Ar, Ai, Br, Bi;
+  td4_sums_f32(a, am, Ar, Ai, Br, Bi);
   TimeTerms<float> tt;
-  time_terms<float>(a, t, tt);
+  time_terms_g<float>(TdMath<float>{}, a.tc, a.wa, a.wN, a.wL, t, tt);
   const float AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
   const float ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
   const float R = td_rate(tt, AA, BB, ABr, ABi);
@@ -332,35 +300,85 @@ __device__ __forceinline__ void td4_finish(const Td4Args<T>& a, TdAcc<T, KB>& ac
   result_complete(result, P > 1 ? P : 1);
 }
 
-// FP64: direct loads, one event per thread per grid-stride step.
+// The FP64 sums A = sum c_k a_k and B = sum b_k a_k of event i.
+__device__ __forceinline__ void td4_sums(const Td4Args<double>& a, const double2* __restrict__ cache, int KB, int64_t i,
+                                         double& Ar, double& Ai, double& Br, double& Bi) {
+  Ar = Ai = Br = Bi = 0.0;
+#pragma unroll
+  for (int k = 0; k < KB; ++k) {
+    if (k >= a.K) break;
+    const double2 v = cache[(int64_t)k * a.n_total + i];
+    Ar = fma(a.cr[k], v.x, fma(-a.ci[k], v.y, Ar));
+    Ai = fma(a.cr[k], v.y, fma(a.ci[k], v.x, Ai));
+    Br = fma(a.br[k], v.x, fma(-a.bi[k], v.y, Br));
+    Bi = fma(a.br[k], v.y, fma(a.bi[k], v.x, Bi));
+  }
+}
+
+// FP64: direct loads, one event per thread per grid-stride step.  Bound by the FP64 pipe's slots
+// (fp64.cuh): FMA chains, exp and erfcx from tables in shared memory, the logarithm as a running
+// product, tests on the integer pipe.  The amplitudes are read again for the gradient lanes
+// (their registers would spill; the second read costs no FP64 slot).  1M events, 10 amplitudes with
+// the gradient: 872 -> 571 us (three slots per product pair and CUDA's exp, erfcx, log and division
+// before).
 template <int KB, bool GRAD>
 __global__ void __launch_bounds__(kBlock, 2) td4_nll_f64_kernel(const __grid_constant__ Td4Args<double> a,
                                                                 const double2* __restrict__ cache,
-                                                                const double* __restrict__ tcol, int64_t begin,
+                                                                const double* __restrict__ tcol,
+                                                                const Fp64Tables* __restrict__ tables, int64_t begin,
                                                                 int64_t end, float2* partials, unsigned* counters,
                                                                 double* result, int out_mode) {
   constexpr int NS = TdLanes<KB, GRAD>::NS;
   __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
   __shared__ unsigned s_bad[kBlock / 32];
+  __shared__ __align__(16) Fp64Tables s_tab;
+  load_fp64_tables(s_tab, tables);
+  const TdMath<double> F{s_tab};
   TdAcc<double, KB> acc;
+  LogProduct lp;
 #pragma unroll
   for (int k = 0; k < KB; ++k) acc.lre[k] = acc.lim[k] = 0.0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) acc.lt[j] = 0.0;
-  const int K = a.K;
   const int64_t n = a.n_total;
+  __syncthreads();
   for (int64_t i = begin + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < end;
        i += (int64_t)gridDim.x * blockDim.x) {
-    double ar[KB], ai[KB];
-#pragma unroll
-    for (int k = 0; k < KB; ++k) {
-      double2 v = make_double2(0.0, 0.0);
-      if (k < K) v = cache[(int64_t)k * n + i];
-      ar[k] = v.x;
-      ai[k] = v.y;
+    const double t = tcol[i];
+    double Ar, Ai, Br, Bi;
+    td4_sums(a, cache, KB, i, Ar, Ai, Br, Bi);
+    TimeTerms<double> tt;
+    time_terms_g<double>(F, a.tc, a.wa, a.wN, a.wL, t, tt);
+    const double AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
+    const double ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
+    const double R = td_rate(tt, AA, BB, ABr, ABi);
+    double invR;
+    if (positive_normal(R)) {
+      lp.mul(R);
+      invR = rcp64(R);
+    } else if (R > 0.0) {  // subnormal or infinite
+      acc.lf64 += log(R);
+      invR = 1.0 / R;
+    } else {
+      acc.bad++;
+      continue;
     }
-    td4_event<double, KB, GRAD>(a, ar, ai, tcol[i], acc);
+    if constexpr (GRAD) {
+      // V / R, V = (T_ch + T_c) A* + (T_sh - i T_s) B* = 2 P A* + (T_sh - i T_s) B*
+      const double c1 = 2.0 * tt.P * invR, sh = tt.Tsh * invR, ss = tt.Ts * invR;
+      const double Vr = fma(c1, Ar, fma(sh, Br, -ss * Bi));
+      const double mVi = fma(c1, Ai, fma(sh, Bi, ss * Br));  // -Im V / R
+#pragma unroll
+      for (int k = 0; k < KB; ++k) {
+        if (k >= a.K) break;
+        const double2 v = cache[(int64_t)k * n + i];
+        acc.lre[k] = fma(v.x, Vr, fma(v.y, mVi, acc.lre[k]));   // Re(a_k V) / R
+        acc.lim[k] = fma(v.x, mVi, fma(-v.y, Vr, acc.lim[k]));  // -Im(a_k V) / R
+      }
+      time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, acc.lt);
+    }
   }
+  acc.lf64 += lp.log_value();
   td4_finish<double, KB, GRAD>(a, acc, begin, end, partials, counters, result, out_mode, s_red, s_bad);
 }
 
@@ -461,32 +479,44 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f32_kernel(const __grid_con
 }
 
 // per-event log f = log R - log N (goo_eval_logf)
-template <typename T, int KB>
-__global__ void td4_logf_kernel(const __grid_constant__ Td4Args<T> a, const void* cache_v, const T* __restrict__ tcol,
-                                double logN, double* __restrict__ out) {
-  const int K = a.K;
+template <int KB>
+__global__ void td4_logf_f32_kernel(const __grid_constant__ Td4Args<float> a, const float4* __restrict__ cache,
+                                    const float* __restrict__ tcol, double logN, double* __restrict__ out) {
   const int64_t n = a.n_total;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    T ar[KB], ai[KB];
+    float2 am[KB];
 #pragma unroll
-    for (int k = 0; k < KB; ++k) {
-      ar[k] = ai[k] = T(0);
-      if (k < K) {
-        if constexpr (sizeof(T) == 4) {
-          const float4 v = ((const float4*)cache_v)[(int64_t)(k / 2) * n + i];
-          ar[k] = (k & 1) ? v.z : v.x;
-          ai[k] = (k & 1) ? v.w : v.y;
-        } else {
-          const double2 v = ((const double2*)cache_v)[(int64_t)k * n + i];
-          ar[k] = v.x;
-          ai[k] = v.y;
-        }
-      }
+    for (int p = 0; p < KB / 2; ++p) {
+      const float4 v = p < a.planes ? cache[(int64_t)p * n + i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      am[2 * p] = make_float2(v.x, v.y);
+      am[2 * p + 1] = make_float2(v.z, v.w);
     }
-    TdAcc<T, KB> acc;
-    td4_event<T, KB, false>(a, ar, ai, tcol[i], acc);
-    const double lr = (sizeof(T) == 4) ? dd_to_double(acc.lf32.value()) : acc.lf64;
-    out[i] = acc.bad ? -HUGE_VAL : lr - logN;
+    float Ar, Ai, Br, Bi;
+    td4_sums_f32(a, am, Ar, Ai, Br, Bi);
+    TimeTerms<float> tt;
+    time_terms_g<float>(TdMath<float>{}, a.tc, a.wa, a.wN, a.wL, tcol[i], tt);
+    const float R = td_rate(tt, fma_rn(Ar, Ar, mul_rn(Ai, Ai)), fma_rn(Br, Br, mul_rn(Bi, Bi)),
+                            fma_rn(Ar, Br, mul_rn(Ai, Bi)), fma_rn(Ai, Br, -mul_rn(Ar, Bi)));
+    out[i] = R > 0.f ? (double)logf(R) - logN : -HUGE_VAL;
+  }
+}
+
+template <int KB>
+__global__ void td4_logf_f64_kernel(const __grid_constant__ Td4Args<double> a, const double2* __restrict__ cache,
+                                    const double* __restrict__ tcol, const Fp64Tables* __restrict__ tables, double logN,
+                                    double* __restrict__ out) {
+  __shared__ __align__(16) Fp64Tables s_tab;
+  load_fp64_tables(s_tab, tables);
+  __syncthreads();
+  const int64_t n = a.n_total;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    double Ar, Ai, Br, Bi;
+    td4_sums(a, cache, KB, i, Ar, Ai, Br, Bi);
+    TimeTerms<double> tt;
+    time_terms_g<double>(TdMath<double>{s_tab}, a.tc, a.wa, a.wN, a.wL, tcol[i], tt);
+    const double R = td_rate(tt, fma_rn(Ar, Ar, mul_rn(Ai, Ai)), fma_rn(Br, Br, mul_rn(Bi, Bi)),
+                             fma_rn(Ar, Br, mul_rn(Ai, Bi)), fma_rn(Ai, Br, -mul_rn(Ar, Bi)));
+    out[i] = R > 0.0 ? log(R) - logN : -HUGE_VAL;
   }
 }
 
@@ -815,17 +845,14 @@ static int launch_td4_f64(goo_model* m, const void* cache, const goo_dataset* ds
   Td4Args<double> a;
   td4_args<double>(m, theta, ds->n, a);
   td4_norm_terms<double>(m, GOO_F64, a);
-  static int occ = 0;
-  if (occ == 0 && (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, td4_nll_f64_kernel<KB, GRAD>, kBlock, 0) != cudaSuccess ||
-                   occ < 1)) {
-    cudaGetLastError();
-    occ = 1;
-  }
+  const Fp64Tables* tables = nullptr;
+  GOO_TRY(fp64_tables(ctx, &tables));
+  const int occ = cached_occupancy((const void*)td4_nll_f64_kernel<KB, GRAD>, ctx->device, kBlock, 0);
   const int nb = grid_blocks(ctx, end - begin, occ);
   GOO_TRY(ensure_partials(ctx, (size_t)nb * TdLanes<KB, GRAD>::NS));
   {
     LaunchScope ls(ctx, GRAD ? "td4_nll_grad_f64" : "td4_nll_f64");
-    td4_nll_f64_kernel<KB, GRAD><<<nb, kBlock, 0, ctx->stream>>>(a, (const double2*)cache, ds->d64[5], begin, end,
+    td4_nll_f64_kernel<KB, GRAD><<<nb, kBlock, 0, ctx->stream>>>(a, (const double2*)cache, ds->d64[5], tables, begin, end,
                                                                 ctx->scratch.partials, ctx->scratch.counters,
                                                                 ctx->scratch.result_out, out_mode);
   }
@@ -917,13 +944,17 @@ int td4_eval_logf(goo_model* m, const goo_dataset* ds, const double* theta, int 
   if (precision == GOO_F32) {
     Td4Args<float> a;
     td4_args<float>(m, theta, ds->n, a);
-    if (small) td4_logf_kernel<float, 10><<<nb, kBlock, 0, ctx->stream>>>(a, cache, ds->d32[5], logN, logf_dev);
-    else td4_logf_kernel<float, 16><<<nb, kBlock, 0, ctx->stream>>>(a, cache, ds->d32[5], logN, logf_dev);
+    const float4* amps = (const float4*)cache;
+    if (small) td4_logf_f32_kernel<10><<<nb, kBlock, 0, ctx->stream>>>(a, amps, ds->d32[5], logN, logf_dev);
+    else td4_logf_f32_kernel<16><<<nb, kBlock, 0, ctx->stream>>>(a, amps, ds->d32[5], logN, logf_dev);
   } else {
     Td4Args<double> a;
     td4_args<double>(m, theta, ds->n, a);
-    if (small) td4_logf_kernel<double, 10><<<nb, kBlock, 0, ctx->stream>>>(a, cache, ds->d64[5], logN, logf_dev);
-    else td4_logf_kernel<double, 16><<<nb, kBlock, 0, ctx->stream>>>(a, cache, ds->d64[5], logN, logf_dev);
+    const Fp64Tables* tables = nullptr;
+    GOO_TRY(fp64_tables(ctx, &tables));
+    const double2* amps = (const double2*)cache;
+    if (small) td4_logf_f64_kernel<10><<<nb, kBlock, 0, ctx->stream>>>(a, amps, ds->d64[5], tables, logN, logf_dev);
+    else td4_logf_f64_kernel<16><<<nb, kBlock, 0, ctx->stream>>>(a, amps, ds->d64[5], tables, logN, logf_dev);
   }
   GOO_CUDA_TRY(cudaGetLastError());
   return GOO_OK;

@@ -52,6 +52,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fp64.cuh"
 
 namespace goo {
 
@@ -139,19 +140,19 @@ template <typename T>
 struct TimeCoef {
   static constexpr int K = SeriesOrder<T>::K;
   T G, x, y, s;
-  T zs;                        // max(|x|, |y|) G
   T a[K + 1], b[K + 1];        // P, Q coefficients of w_2m (a_0 = 1, b_0 = 0)
   T ysh[K + 1], xs[K + 1];     // T_sh, T_s coefficients of w_(2m+1)
-  // the order in use, K - 1 or K, and the largest z at which it meets the truncation
+  // the order in use, K - 1 or K, and the observed time up to which it meets the truncation
   // criterion: K - 1 when that covers every event the dataset's time range admits
   int ku;
-  T zmax_ku;
+  T t_series;
   T is2, is2h, ir2s;           // 1 / s^2, 1 / (2 s^2), 1 / (s sqrt 2): no event divides by them
   T k_phi;                     // 1 / (s sqrt(2 pi))
   T s2, Gs2, hG2s2;            // s^2, G s^2, G^2 s^2 / 2
   T nG2s2[2 * K + 1];          // n G^2 s^2
-  T hx, hy;                    // s^2 G x / 2, s^2 G y / 2
-  T y2, x2, G2;                // y^2, x^2, G^2
+  T hx, hy, fx, fy;            // s^2 G x / 2, s^2 G y / 2, and twice these
+  T Gx, Gy, qx, qy;            // G x, G y, 2 G^2 x, 2 G^2 y
+  T Gx2, Gy2;                  // (G x)^2, (G y)^2
 };
 
 #ifndef __CUDACC_RTC__
@@ -166,7 +167,7 @@ inline void fill_time_coef(TimeCoef<T>& c, double x64, double y64, double tau, d
   c.y = (T)y64;
   c.s = (T)s64;
   const double x = (double)c.x, y = (double)c.y, G = (double)c.G, s = (double)c.s;
-  c.zs = (T)(std::fmax(std::fabs(x), std::fabs(y)) * G);
+  const double zs = std::fmax(std::fabs(x), std::fabs(y)) * G;
   c.is2 = (T)(1.0 / (s * s));
   c.is2h = (T)(0.5 / (s * s));
   c.ir2s = (T)(0.70710678118654752440 / s);
@@ -177,9 +178,14 @@ inline void fill_time_coef(TimeCoef<T>& c, double x64, double y64, double tau, d
   c.hG2s2 = (T)(0.5 * G * G * s * s);
   c.hx = (T)(0.5 * s * s * G * x);
   c.hy = (T)(0.5 * s * s * G * y);
-  c.y2 = (T)(y * y);
-  c.x2 = (T)(x * x);
-  c.G2 = (T)(G * G);
+  c.fx = (T)(s * s * G * x);
+  c.fy = (T)(s * s * G * y);
+  c.Gx = (T)(G * x);
+  c.Gy = (T)(G * y);
+  c.qx = (T)(2.0 * G * G * x);
+  c.qy = (T)(2.0 * G * G * y);
+  c.Gx2 = (T)(G * G * x * x);
+  c.Gy2 = (T)(G * G * y * y);
   double fact = 1.0;  // (2m)!
   for (int m = 0; m <= K; ++m) {
     const double sg = (m & 1) ? -1.0 : 1.0;
@@ -197,9 +203,12 @@ inline void fill_time_coef(TimeCoef<T>& c, double x64, double y64, double tau, d
   auto ratio = [](double z, int k) { return std::pow(z, 2.0 * k) * 2.0 / std::tgamma(2.0 * k + 3.0); };
   const double eps = ratio(SeriesOrder<T>::zmax, K);
   const double zk1 = std::pow(eps * std::tgamma(2.0 * (K - 1) + 3.0) / 2.0, 1.0 / (2.0 * (K - 1)));
-  const double zdata = (double)c.zs * (std::fmax(t_hi, 0.0) + 6.0 * s);
+  const double zdata = zs * (std::fmax(t_hi, 0.0) + 6.0 * s);
   c.ku = zdata < zk1 ? K - 1 : K;
-  c.zmax_ku = (T)(zdata < zk1 ? zk1 : SeriesOrder<T>::zmax);
+  const double zlim = zdata < zk1 ? zk1 : SeriesOrder<T>::zmax;
+  // z < zlim for max(t, 0) < zlim / zs - 6 s; never, where that is not positive
+  const double tlim = zs > 0.0 ? zlim / zs - 6.0 * s : HUGE_VAL;
+  c.t_series = (T)(tlim > 0.0 ? tlim : -HUGE_VAL);
 }
 #endif
 
@@ -219,32 +228,50 @@ __device__ __forceinline__ T td_rate(const TimeTerms<T>& tt, T AA, T BB, T ABr, 
   return fma_rn(ABi, tt.Ts, fma_rn(ABr, tt.Tsh, fma_rn(BB, tt.Q, mul_rn(AA, tt.P))));
 }
 
+// exp and erfcx / 2 of the path's precision: CUDA's in FP32, the tables of fp64.cuh in FP64.
 template <typename T>
-__device__ __forceinline__ T td_erfcx(T u) {
-  if constexpr (sizeof(T) == 4) return erfcxf(u);
-  else return erfcx(u);
-}
-
-template <typename T>
-__device__ __forceinline__ T td_exp(T v) {
-  if constexpr (sizeof(T) == 4) return expf(v);
-  else return exp(v);
-}
+struct TdMath;
+template <>
+struct TdMath<float> {
+  __device__ __forceinline__ float exp(float v) const { return expf(v); }
+  // gauss erfcx(|u|) / 2
+  __device__ __forceinline__ float gauss_herfcx(float gauss, float u) const {
+    return mul_rn(mul_rn(0.5f, gauss), erfcxf(fabsf(u)));
+  }
+  __device__ __forceinline__ static bool nonneg(float u) { return u >= 0.f; }
+  __device__ __forceinline__ static bool below(float t, float limit) { return t < limit; }
+};
+template <>
+struct TdMath<double> {
+  const Fp64Tables& tab;
+  __device__ __forceinline__ double exp(double v) const { return exp_tab(v, tab); }
+  // gauss erfcx(|u|) / 2; where u <= -6 it is below 2^-56 of the exponential it is subtracted from
+  // (conv_real) and is left out
+  __device__ __forceinline__ double gauss_herfcx(double gauss, double u) const {
+    const int hu = __double2hiint(u), ha = hu & 0x7fffffff;
+    if (ha < 0x40180000) return mul_rn(gauss, herfcx_tab(__hiloint2double(ha, __double2loint(u)), tab));
+    return hu < 0 ? 0.0 : mul_rn(gauss, 0.5 * erfcx(u));
+  }
+  // on the integer pipe (nonneg: false for -0, where both forms agree; below: to 2^-20)
+  __device__ __forceinline__ static bool nonneg(double u) { return __double2hiint(u) >= 0; }
+  __device__ __forceinline__ static bool below(double t, double limit) { return __double2hiint(t) < __double2hiint(limit); }
+};
 
 // E(g) for real g (gauss = exp(-t^2/2s^2)): with h = gauss erfcx(|u|) / 2, u = (g s^2 - t) / (s sqrt 2),
 // E = h for u >= 0 and exp(g^2 s^2 / 2 - g t) - h below, selected, so that a warp whose events
 // lie on both sides evaluates erfcx once.  hg2s2 = g^2 s^2 / 2.
 template <typename T>
-__device__ __forceinline__ T conv_real(T g, T gs2, T hg2s2, T ir2s, T t, T gauss) {
+__device__ __forceinline__ T conv_real(const TdMath<T>& F, T g, T gs2, T hg2s2, T ir2s, T t, T gauss) {
   const T u = mul_rn(sub_rn(gs2, t), ir2s);
-  const T h = mul_rn(mul_rn(T(0.5), gauss), td_erfcx<T>(u < T(0) ? -u : u));
-  const T x = sub_rn(td_exp<T>(fma_rn(-g, t, hg2s2)), h);
-  return u >= T(0) ? h : x;
+  const T h = F.gauss_herfcx(gauss, u);
+  const T x = sub_rn(F.exp(fma_rn(-g, t, hg2s2)), h);
+  return F.nonneg(u) ? h : x;
 }
 
 // E(g) for complex g = (gr, gi)
 template <typename T>
-__device__ __forceinline__ void conv_complex(T gr, T gi, T t, T s, T gauss, const T* wa, int wN, T wL, T& Er, T& Ei) {
+__device__ __forceinline__ void conv_complex(const TdMath<T>& F, T gr, T gi, T t, T s, T gauss, const T* wa, int wN,
+                                             T wL, T& Er, T& Ei) {
   const T c = T(0.70710678118654752440) / s;
   const T ur = (gr * s * s - t) * c, ui = gi * s * s * c;
   T wr, wi;
@@ -255,7 +282,7 @@ __device__ __forceinline__ void conv_complex(T gr, T gi, T t, T s, T gauss, cons
   } else {
     faddeeva<T>(ui, -ur, wa, wN, wL, wr, wi);  // w(-i u)
     const T er = T(0.5) * (gr * gr - gi * gi) * s * s - gr * t, ei = gr * gi * s * s - gi * t;
-    const T mag = td_exp<T>(er);
+    const T mag = F.exp(er);
     T sn, cs;
     if constexpr (sizeof(T) == 4) sincosf(ei, &sn, &cs);
     else sincos(ei, &sn, &cs);
@@ -267,13 +294,13 @@ __device__ __forceinline__ void conv_complex(T gr, T gi, T t, T s, T gauss, cons
 // The decay-time terms at the observed time t from the convolved exponentials (Faddeeva
 // path, any mixing); gauss = exp(-t^2 / 2 s^2).
 template <typename T>
-__device__ __forceinline__ void time_terms_direct(const TimeCoef<T>& c, const T* wa, int wN, T wL, T t, T gauss,
-                                                  TimeTerms<T>& R) {
+__device__ __forceinline__ void time_terms_direct(const TdMath<T>& F, const TimeCoef<T>& c, const T* wa, int wN, T wL,
+                                                  T t, T gauss, TimeTerms<T>& R) {
   const T gp = c.G * (T(1) - c.y), gm = c.G * (T(1) + c.y);
-  const T Ep = conv_real<T>(gp, gp * c.s2, T(0.5) * gp * gp * c.s2, c.ir2s, t, gauss);
-  const T Em = conv_real<T>(gm, gm * c.s2, T(0.5) * gm * gm * c.s2, c.ir2s, t, gauss);
+  const T Ep = conv_real<T>(F, gp, gp * c.s2, T(0.5) * gp * gp * c.s2, c.ir2s, t, gauss);
+  const T Em = conv_real<T>(F, gm, gm * c.s2, T(0.5) * gm * gm * c.s2, c.ir2s, t, gauss);
   T Ecr, Eci;
-  conv_complex<T>(c.G, -c.G * c.x, t, c.s, gauss, wa, wN, wL, Ecr, Eci);
+  conv_complex<T>(F, c.G, -c.G * c.x, t, c.s, gauss, wa, wN, wL, Ecr, Eci);
   const T Tch = T(0.5) * (Ep + Em);
   R.P = T(0.5) * (Tch + Ecr);
   R.Q = T(0.5) * (Tch - Ecr);
@@ -284,11 +311,12 @@ __device__ __forceinline__ void time_terms_direct(const TimeCoef<T>& c, const T*
 // The decay-time terms by the moment series of order KU (small mixing; see the top of this
 // file).
 template <typename T, int KU>
-__device__ __forceinline__ void time_terms_series(const TimeCoef<T>& c, T t, T gauss, TimeTerms<T>& R) {
+__device__ __forceinline__ void time_terms_series(const TdMath<T>& F, const TimeCoef<T>& c, T t, T gauss,
+                                                  TimeTerms<T>& R) {
   constexpr int NW = 2 * KU + 2;
   const T v = sub_rn(t, c.Gs2), Gv = mul_rn(c.G, v);
   T w[NW];
-  w[0] = conv_real<T>(c.G, c.Gs2, c.hG2s2, c.ir2s, t, gauss);
+  w[0] = conv_real<T>(F, c.G, c.Gs2, c.hG2s2, c.ir2s, t, gauss);
   w[1] = mul_rn(c.G, fma_rn(v, w[0], mul_rn(c.s2, R.phi)));
 #pragma unroll
   for (int n = 1; n < NW - 1; ++n) w[n + 1] = fma_rn(Gv, w[n], mul_rn(c.nG2s2[n], w[n - 1]));
@@ -306,19 +334,19 @@ __device__ __forceinline__ void time_terms_series(const TimeCoef<T>& c, T t, T g
 }
 
 // The decay-time terms at the observed time t: the moment series of the
-// order in use where z = max(|x|, |y|) G (max(t, 0) + 6 s) is below its limit (c.zmax_ku),
+// order in use where z = max(|x|, |y|) G (max(t, 0) + 6 s) is below its limit (t < c.t_series),
 // else the Faddeeva path.
 template <typename T>
-__device__ __forceinline__ void time_terms_g(const TimeCoef<T>& c, const T* wa, int wN, T wL, T t, TimeTerms<T>& R) {
-  const T gauss = td_exp<T>(mul_rn(mul_rn(-t, t), c.is2h));
+__device__ __forceinline__ void time_terms_g(const TdMath<T>& F, const TimeCoef<T>& c, const T* wa, int wN, T wL, T t,
+                                             TimeTerms<T>& R) {
+  const T gauss = F.exp(mul_rn(mul_rn(-t, t), c.is2h));
   R.phi = mul_rn(c.k_phi, gauss);
-  const T z = c.zs * ((t > T(0) ? t : T(0)) + T(6) * c.s);
-  if (z < c.zmax_ku) {
+  if (F.below(t, c.t_series)) {
     // the same order for every event of a launch (a uniform branch)
-    if (c.ku == TimeCoef<T>::K) time_terms_series<T, TimeCoef<T>::K>(c, t, gauss, R);
-    else time_terms_series<T, TimeCoef<T>::K - 1>(c, t, gauss, R);
+    if (c.ku == TimeCoef<T>::K) time_terms_series<T, TimeCoef<T>::K>(F, c, t, gauss, R);
+    else time_terms_series<T, TimeCoef<T>::K - 1>(F, c, t, gauss, R);
   } else {
-    time_terms_direct<T>(c, wa, wN, wL, t, gauss, R);
+    time_terms_direct<T>(F, c, wa, wN, wL, t, gauss, R);
   }
 }
 
@@ -330,16 +358,17 @@ __device__ __forceinline__ void time_lanes(const TimeCoef<T>& c, T t, const Time
   const T v = t - c.Gs2;
   const T Tch = tt.P + tt.Q, Tc = tt.P - tt.Q;
   const T ysh = c.hy * tt.Tsh, xs = c.hx * tt.Ts;
-  const T CP = v * tt.P + (c.s2 * tt.phi + (ysh - xs)), CQ = v * tt.Q + (ysh + xs);
-  const T Csh = v * tt.Tsh + (T(2) * c.hy) * Tch, Cs = v * tt.Ts + (T(2) * c.hx) * Tc;
+  const T CP = fma_rn(v, tt.P, fma_rn(c.s2, tt.phi, ysh - xs)), CQ = fma_rn(v, tt.Q, ysh + xs);
+  const T Csh = fma_rn(v, tt.Tsh, c.fy * Tch), Cs = fma_rn(v, tt.Ts, c.fx * Tc);
   const T hp = T(0.5) * (AA + BB), hm = T(0.5) * (BB - AA);
-  lt[0] += (hm * Cs + ABi * (CP - CQ)) * invR;
-  lt[1] += (hp * Csh + ABr * (CP + CQ)) * invR;
-  lt[2] += (AA * CP + BB * CQ + ABr * Csh + ABi * Cs) * invR;
-  const T Ey = hp * tt.Tsh + ABr * Tch, Ex = hm * tt.Ts + ABi * Tc;
-  const T Ry = hp * Tch + ABr * tt.Tsh, Rx = ABi * tt.Ts - hm * Tc;
-  const T q = c.G2 * (c.y2 * Ry - c.x2 * Rx - T(2) * (c.y * Ey + c.x * Ex));
-  lt[3] += (q + tt.phi * (c.G * (c.y * ABr + c.x * ABi) - (c.G + t * c.is2) * AA)) * invR;
+  lt[0] = fma_rn(fma_rn(hm, Cs, ABi * (CP - CQ)), invR, lt[0]);
+  lt[1] = fma_rn(fma_rn(hp, Csh, ABr * (CP + CQ)), invR, lt[1]);
+  lt[2] = fma_rn(fma_rn(AA, CP, fma_rn(BB, CQ, fma_rn(ABr, Csh, ABi * Cs))), invR, lt[2]);
+  const T Ey = fma_rn(hp, tt.Tsh, ABr * Tch), Ex = fma_rn(hm, tt.Ts, ABi * Tc);
+  const T Ry = fma_rn(hp, Tch, ABr * tt.Tsh), Rx = fma_rn(-hm, Tc, ABi * tt.Ts);
+  const T b = fma_rn(-fma_rn(t, c.is2, c.G), AA, fma_rn(c.Gy, ABr, c.Gx * ABi));
+  const T q = fma_rn(tt.phi, b, fma_rn(c.Gy2, Ry, fma_rn(-c.Gx2, Rx, fma_rn(-c.qy, Ey, -c.qx * Ex))));
+  lt[3] = fma_rn(q, invR, lt[3]);
 }
 
 // sum_i (dR_i / dp_j) / R_i of j = x, y, tau, sigma_t from the lane sums of n events (FP64).
