@@ -11,6 +11,10 @@ static const Fp64Tables& host_tables() {
   static const Fp64Tables t = [] {
     Fp64Tables h;
     for (int j = 0; j < kExpTab; ++j) h.exp2j[j] = (double)std::exp2((long double)j / kExpTab);
+    for (int j = 0; j < kLogTab; ++j) {
+      h.log_inv[j] = (double)(1.0L / (1.0L + (j + 0.5L) / kLogTab));
+      h.log_ref[j] = (double)-std::log((long double)h.log_inv[j]);
+    }
     constexpr int N = kErfcxDeg + 1;
     const long double pi = 3.14159265358979323846264338327950288L, half = 0.5L / kErfcxStep;
     for (int i = 0; i < kErfcxTab; ++i) {

@@ -24,6 +24,13 @@ __device__ __forceinline__ double rcp64(double x) {
   return ::fma(y, ::fma(e, e, e), y);
 }
 
+// 1 / x for any x: the step above where x and 1 / x are normal (tested on the integer pipe), else a
+// division.
+__device__ __forceinline__ double recip(double x) {
+  const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+  return h - 0x00300000u < 0x7fa00000u - 0x00300000u ? rcp64(x) : 1.0 / x;
+}
+
 // True for a positive, normal, finite x: one integer test on the high word (a comparison of
 // doubles takes a slot of the FP64 pipe).
 __device__ __forceinline__ bool positive_normal(double x) {
@@ -62,8 +69,11 @@ constexpr int kErfcxMax = 6;        // table range [0, 6]
 constexpr int kErfcxTab = kErfcxStep * kErfcxMax + 1;
 constexpr int kErfcxDeg = 7;
 
+constexpr int kLogTab = 256;
+
 struct Fp64Tables {
   double exp2j[kExpTab];
+  double log_inv[kLogTab], log_ref[kLogTab];  // about 1 / (1 + (j + 1/2) / 256), and minus its logarithm
   double node[kErfcxTab];                 // i / 32
   double herfcx[kErfcxDeg + 1][kErfcxTab];  // erfcx(node + r) / 2 = sum_d herfcx[d][i] r^d, |r| <= 1 / 64
 };
@@ -103,6 +113,25 @@ __device__ __forceinline__ double exp_tab(double x, const Fp64Tables& tab) {
   const double t = tab.exp2j[n & (kExpTab - 1)];
   const double s = __hiloint2double(__double2hiint(t) + ((n >> 8) << 20), __double2loint(t));
   return ::fma(s, q, s);
+}
+
+// log(x) for x > 0, table-driven (P. T. P. Tang, ACM TOMS 16 (1990) 378): x = 2^e m, j the top 8 bits of m's
+// fraction, r = m inv_j - 1 with |r| < 2^-8.9, log x = e ln2 - log inv_j + log1p(r) with log1p to degree 5
+// (truncation 2e-17): 9 slots, the error about one unit of the last place of e ln2 - log inv_j (so
+// absolute, not relative, for x near 1), where log() takes some twenty-five.  Subnormal, infinite and NaN
+// arguments go to log().
+__device__ __forceinline__ double log_tab(double x, const Fp64Tables& tab) {
+  if (!positive_normal(x)) return log(x);
+  const int hx = __double2hiint(x);
+  const int j = (hx >> 12) & (kLogTab - 1), e = (hx >> 20) - 1023;
+  const double m = __hiloint2double((hx & 0x000fffff) | 0x3ff00000, __double2loint(x));
+  const double r = ::fma(m, tab.log_inv[j], -1.0);
+  const double de = __hiloint2double(0x43380000 + (e >> 31), e) - 6755399441055744.0;
+  double p = ::fma(r, 0.2, -0.25);
+  p = ::fma(r, p, 1.0 / 3.0);
+  p = ::fma(r, p, -0.5);
+  const double q = ::fma(r * r, p, r);
+  return ::fma(de, 0.693147180559945309417, tab.log_ref[j]) + q;
 }
 
 // erfcx(u) / 2 for 0 <= u < 6: the degree-7 interpolant of the nearest node (relative error of the

@@ -427,6 +427,9 @@ struct EventOcc {
   static constexpr int value = (sizeof(T) == 4 && K * L <= 6) ? 3 : 2;
 };
 
+// The scalar kernel: weighted FP32 datasets, FP32 shapes the pair kernel does not take, and both precisions
+// of goo_nll_grad_static (whose calls have no context to keep the FP64 function tables of the
+// faster sop_event64_kernel in).
 // wcol (nullable): per-event weights w_i (a binned dataset: bin centres with their counts);
 // the lanes then sum w_i log f_i and w_i times the gradient terms, and events of weight 0 are
 // skipped.

@@ -42,6 +42,7 @@
 #include "model.cuh"
 #include "jit.cuh"
 #include "sop_kernels.cuh"
+#include "sop64.cuh"
 
 namespace goo {
 
@@ -890,26 +891,57 @@ static EvConst<T, K, L> make_evconst(const ModelDev& h) {
   return P;
 }
 
-template <typename T, int K, int L, bool GRAD>
-static int launch_event_T(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, int out_mode,
-                          double* result) {
-  const T* wcol = sizeof(T) == 4 ? (const T*)(const void*)ds->w32 : (const T*)(const void*)ds->w64;
+// The scalar FP32 kernel: weighted datasets, and the shapes the pair kernel does not take.
+template <int K, int L, bool GRAD>
+static int launch_event_f32(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, int out_mode,
+                            double* result) {
   goo_ctx* ctx = m->ctx;
-  static int occ = 0;
-  const int bps = blocks_per_sm(sop_event_kernel<T, K, L, GRAD>, &occ);
+  const int bps = cached_occupancy((const void*)sop_event_kernel<float, K, L, GRAD>, ctx->device, kBlock, 0);
   const int nb = grid_blocks(ctx, end - begin, bps);
-  constexpr int NS = EventLanes<T, K, L, GRAD>::NS;
-  GOO_TRY(ensure_partials(ctx, (size_t)nb * NS));
-  Cols<T> cols{};
-  for (int c = 0; c < kMaxObs; ++c) {
-    if (sizeof(T) == 4) cols.c[c] = (const T*)(c < ds->ncols ? (const void*)ds->d32[c] : (const void*)ds->d32[0]);
-    else cols.c[c] = (const T*)(c < ds->ncols ? (const void*)ds->d64[c] : (const void*)ds->d64[0]);
-  }
+  GOO_TRY(ensure_partials(ctx, (size_t)nb * EventLanes<float, K, L, GRAD>::NS));
+  Cols<float> cols{};
+  for (int c = 0; c < kMaxObs; ++c) cols.c[c] = ds->d32[c < ds->ncols ? c : 0];
   {
-    LaunchScope ls(ctx, sizeof(T) == 4 ? (GRAD ? "sop_nll_grad_f32" : "sop_nll_f32") : (GRAD ? "sop_nll_grad_f64" : "sop_nll_f64"));
-    sop_event_kernel<T, K, L, GRAD><<<nb, kBlock, 0, ctx->stream>>>(m->dev, make_evconst<T, K, L>(*m->stage), cols,
-                                                                   begin, end, ctx->scratch.partials,
-                                                                   ctx->scratch.counters, result, out_mode, wcol);
+    LaunchScope ls(ctx, GRAD ? "sop_nll_grad_f32" : "sop_nll_f32");
+    sop_event_kernel<float, K, L, GRAD><<<nb, kBlock, 0, ctx->stream>>>(
+        m->dev, make_evconst<float, K, L>(*m->stage), cols, begin, end, ctx->scratch.partials, ctx->scratch.counters,
+        result, out_mode, ds->w32);
+  }
+  GOO_CUDA_TRY(cudaGetLastError());
+  return GOO_OK;
+}
+
+// The FP64 kernel, launched as a programmatic dependent of the normalisation kernel before it: its
+// blocks load their tables and first columns while that kernel finishes.
+template <int K, int L, bool GRAD>
+static int launch_event_f64(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, int out_mode,
+                            double* result) {
+  goo_ctx* ctx = m->ctx;
+  const void* fn = (const void*)sop_event64_kernel<K, L, GRAD>;
+  const int nb = grid_blocks(ctx, end - begin, cached_occupancy(fn, ctx->device, kBlock, 0));
+  GOO_TRY(ensure_partials(ctx, (size_t)nb * EventLanes<double, K, L, GRAD>::NS));
+  const Fp64Tables* tables = nullptr;
+  GOO_TRY(fp64_tables(ctx, &tables));
+  Cols<double> cols{};
+  for (int c = 0; c < kMaxObs; ++c) cols.c[c] = ds->d64[c < ds->ncols ? c : 0];
+  {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(nb);
+    cfg.blockDim = dim3(kBlock);
+    cfg.stream = ctx->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    LaunchScope ls(ctx, GRAD ? "sop_nll_grad_f64" : "sop_nll_f64");
+    const ModelDev* md = m->dev;
+    EvConst<double, K, L> P = make_evconst<double, K, L>(*m->stage);
+    float2* partials = ctx->scratch.partials;
+    unsigned* counters = ctx->scratch.counters;
+    const double* w = ds->w64;
+    void* args[] = {&md, &P, &cols, &tables, &begin, &end, &partials, &counters, &result, &out_mode, &w};
+    GOO_CUDA_TRY(cudaLaunchKernelExC(&cfg, fn, args));
   }
   GOO_CUDA_TRY(cudaGetLastError());
   return GOO_OK;
@@ -1061,8 +1093,13 @@ static int launch_event_sel(goo_model* m, const goo_dataset* ds, int64_t begin, 
     return set_error(GOO_ERR_UNSUPPORTED, "a GOO_BORROW_HOST dataset is read by the packed-pair FP32 kernel only "
                                           "(at most 2 products of 3 leaves with the gradient, 4 of 4 without)");
   if (fused_norm) return set_error(GOO_ERR_STATE, "sop_events: in-kernel normalisation needs the pair kernel");
-  if (m->host.nK <= 2 && m->max_leaf <= 3) return launch_event_T<T, 2, 3, GRAD>(m, ds, begin, end, out_mode, result);
-  return launch_event_T<T, 4, 4, GRAD>(m, ds, begin, end, out_mode, result);
+  const bool small = m->host.nK <= 2 && m->max_leaf <= 3;
+  if constexpr (sizeof(T) == 4)
+    return small ? launch_event_f32<2, 3, GRAD>(m, ds, begin, end, out_mode, result)
+                 : launch_event_f32<4, 4, GRAD>(m, ds, begin, end, out_mode, result);
+  else
+    return small ? launch_event_f64<2, 3, GRAD>(m, ds, begin, end, out_mode, result)
+                 : launch_event_f64<4, 4, GRAD>(m, ds, begin, end, out_mode, result);
 }
 
 int sop_events(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, int precision, bool grad, int out_mode,
