@@ -90,7 +90,8 @@ struct Scratch {
   size_t partials_cap = 0;          // in float2 elements
   // [0]: ticket, [1]: non-positive events, [kStatusWord]: a device wait gave up,
   // [kWaitLimitWord]: the tile-wait limit (goo_set_wait_limit), [kWithholdWord]: the
-  // failure-detection test hook (goo_debug_withhold_tile), [5..]: spare
+  // failure-detection test hook (goo_debug_withhold_tile), [kRangeWord]: see below, [8..9]: the
+  // upload's range check, [16..39]: the Gram tiles' tickets (gram.cuh)
   unsigned* counters = nullptr;
   double* result = nullptr;         // kResultDoubles doubles
   double* theta = nullptr;          // kMaxParams doubles
@@ -106,8 +107,10 @@ struct Scratch {
   double* chunk_records = nullptr;
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t chunk_events[65] = {};
+  double* gram_host = nullptr;      // mapped record of the Gram matrices (kGramRecord doubles), on first use
   void* fp64_tables = nullptr;      // device copy of the FP64 function tables (fp64.cuh), on first use
 };
+constexpr int kGramRecord = 3 * 2 * 16 * 16;  // three 16 x 16 complex matrices
 constexpr int kStreamChunks = 64;  // chunks of one goo_nll_grad_streamed call, at most
 
 }  // namespace goo
@@ -198,6 +201,9 @@ int cached_occupancy(const void* kernel, int device, int block, size_t smem);
 int read_result_mapped(goo_ctx* ctx, int n, double* dst);
 // Fills the mapped record with kResultSentinel before a launch that writes to it.
 void arm_result_mapped(goo_ctx* ctx);
+// The same for any mapped record of n fields.
+void arm_mapped(double* record, int n);
+int read_mapped(goo_ctx* ctx, const double* record, int n, double* dst);
 // For the lifetime of the guard, the amplitude kernels write their record to the mapped host
 // copy (scratch.result_out = scratch.result_host), armed with kResultSentinel.
 struct MappedResult {

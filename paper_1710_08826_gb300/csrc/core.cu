@@ -110,14 +110,13 @@ static void fold_timings(goo_ctx* ctx) {
 // with kResultSentinel before its launch) all hold values, then copies them.  Each field is
 // one aligned 8-byte store of the kernel, so a field read without the sentinel is final.  The
 // host polls for up to 2 ms, then waits on the stream, which also reports a failed launch.
-void arm_result_mapped(goo_ctx* ctx) {
-  volatile unsigned long long* rec = reinterpret_cast<volatile unsigned long long*>(ctx->scratch.result_host);
-  for (int i = 0; i < kResultDoubles; ++i) rec[i] = kResultSentinel;
-  ctx->scratch.result_host[kResultFlag] = 0.0;
+void arm_mapped(double* record, int n) {
+  volatile unsigned long long* rec = reinterpret_cast<volatile unsigned long long*>(record);
+  for (int i = 0; i < n; ++i) rec[i] = kResultSentinel;
 }
 
-int read_result_mapped(goo_ctx* ctx, int n, double* dst) {
-  volatile unsigned long long* rec = reinterpret_cast<volatile unsigned long long*>(ctx->scratch.result_host);
+int read_mapped(goo_ctx* ctx, const double* record, int n, double* dst) {
+  const volatile unsigned long long* rec = reinterpret_cast<const volatile unsigned long long*>(record);
   const auto t0 = std::chrono::steady_clock::now();
   int i = 0;
   for (unsigned it = 0;; ++it) {
@@ -132,9 +131,16 @@ int read_result_mapped(goo_ctx* ctx, int n, double* dst) {
     }
   }
   std::atomic_thread_fence(std::memory_order_acquire);
-  std::memcpy(dst, (const double*)ctx->scratch.result_host, n * sizeof(double));
+  std::memcpy(dst, record, n * sizeof(double));
   return GOO_OK;
 }
+
+void arm_result_mapped(goo_ctx* ctx) {
+  arm_mapped(ctx->scratch.result_host, kResultDoubles);
+  ctx->scratch.result_host[kResultFlag] = 0.0;
+}
+
+int read_result_mapped(goo_ctx* ctx, int n, double* dst) { return read_mapped(ctx, ctx->scratch.result_host, n, dst); }
 
 MappedResult::MappedResult(goo_ctx* c) : ctx(c) {
   arm_result_mapped(ctx);
@@ -453,6 +459,7 @@ int goo_finalize(goo_ctx* ctx) {
   if (s.counters) cudaFree(s.counters);
   if (s.result) cudaFree(s.result);
   if (s.fp64_tables) cudaFree(s.fp64_tables);
+  if (s.gram_host) cudaFreeHost(s.gram_host);
   if (s.theta) cudaFree(s.theta);
   if (s.host_pinned) cudaFreeHost(s.host_pinned);
   if (s.result_host) cudaFreeHost(s.result_host);

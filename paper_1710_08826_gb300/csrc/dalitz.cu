@@ -37,6 +37,7 @@
 #include "common.cuh"
 #include "dalitz.cuh"
 #include "fp64.cuh"
+#include "gram.cuh"
 #include "lineshape.cuh"
 #include "timeterms.cuh"
 #include "model.cuh"
@@ -70,8 +71,7 @@ struct DalitzModel {
   bool td = false;
   int col_t = 2;
   int par_t[4] = {-1, -1, -1, -1};  // x, y, tau, sigma_t
-  double* gram3_dev[2] = {nullptr, nullptr};  // per precision: G_aa, G_bb, G_ab (K x K complex each)
-  double gram3_host[2][3 * kMaxAmp * kMaxAmp * 2];
+  double gram3_host[2][3 * kMaxAmp * kMaxAmp * 2];  // per precision: G_aa, G_bb, G_ab (K x K complex each)
   uint64_t gram3_key[2] = {0, 0};
 };
 
@@ -467,9 +467,6 @@ __global__ void coh_logf_kernel(const __grid_constant__ CohArgs<T> a, const void
 }
 
 // ---------------------------------------------------------------------------------------
-// Gram matrix over an MC cache: block (x, k) accumulates row k, G_kl for all l, over its
-// share of the MC events.  Lanes: 2 per l (re, im).  K <= kMaxAmp incl. the NR amplitude.
-// ---------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------
 static double kallen(double a, double b, double c) { return a * a + b * b + c * c - 2 * a * b - 2 * a * c - 2 * b * c; }
@@ -722,55 +719,6 @@ __global__ void __launch_bounds__(kBlock)
 //   <|A|^2> = c^T G_aa c*, <|B|^2> = c^T G_bb c*, <AB*> = c^T G_ab c*,
 // and the closed-form time integrals.
 // ---------------------------------------------------------------------------------------
-
-// G_kl = mean over the events of X_k conj(Y_l) (k, l < K; the amplitude nbw is the constant
-// NR amplitude 1 when present), one block per (k, l), FP64 sums in a fixed order.
-template <typename T>
-__global__ void __launch_bounds__(kBlock) gram_cross_kernel(const void* xv, const void* yv, int64_t n, int nbw, int K,
-                                                            double* out) {
-  const int k = blockIdx.x / K, l = blockIdx.x % K;
-  auto amp = [&](const void* c, int j, int64_t i, double& re, double& im) {
-    if (j >= nbw) {
-      re = 1.0;
-      im = 0.0;
-    } else if constexpr (sizeof(T) == 4) {
-      const float4 v = ((const float4*)c)[(int64_t)(j / 2) * n + i];
-      re = (double)((j & 1) ? v.z : v.x);
-      im = (double)((j & 1) ? v.w : v.y);
-    } else {
-      const double2 v = ((const double2*)c)[(int64_t)j * n + i];
-      re = v.x;
-      im = v.y;
-    }
-  };
-  double sr = 0.0, si = 0.0;
-  for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-    double xr, xi, yr, yi;
-    amp(xv, k, i, xr, xi);
-    amp(yv, l, i, yr, yi);
-    sr += xr * yr + xi * yi;  // X conj(Y)
-    si += xi * yr - xr * yi;
-  }
-  __shared__ double s_r[kBlock / 32], s_i[kBlock / 32];
-  for (int m = 16; m > 0; m >>= 1) {
-    sr += __shfl_xor_sync(0xffffffffu, sr, m);
-    si += __shfl_xor_sync(0xffffffffu, si, m);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    s_r[threadIdx.x >> 5] = sr;
-    s_i[threadIdx.x >> 5] = si;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double tr = 0.0, ti = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      tr += s_r[w];
-      ti += s_i[w];
-    }
-    out[2 * (k * K + l)] = tr / (double)n;
-    out[2 * (k * K + l) + 1] = ti / (double)n;
-  }
-}
 
 constexpr int kTd3KB = 15;  // resonance slots of the time-dependent three-body kernels (NR in slot 15)
 
@@ -1184,31 +1132,6 @@ static int ensure_cache(goo_model* m, const goo_dataset* ds_c, int precision, co
   return GOO_OK;
 }
 
-template <typename T, int KB>
-static int launch_gram(goo_model* m, const void* cache, int64_t n, int pi) {
-  DalitzModel& d = *m->dalitz;
-  goo_ctx* ctx = m->ctx;
-  constexpr int NS = 2 * (KB + 1);
-  int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gram_kernel<T, KB>, kBlock, 0) != cudaSuccess || bps < 1) {
-    cudaGetLastError();
-    bps = 1;
-  }
-  const int K = d.K;
-  int64_t nbx = (n + kBlock - 1) / kBlock;
-  const int64_t cap = ((int64_t)ctx->num_sms * bps + K - 1) / K;
-  if (nbx > cap) nbx = cap;
-  if (nbx < 1) nbx = 1;
-  GOO_TRY(ensure_partials(ctx, (size_t)nbx * K * NS));
-  {
-    LaunchScope ls(ctx, sizeof(T) == 4 ? "gram_f32" : "gram_f64");
-    gram_kernel<T, KB><<<dim3((unsigned)nbx, K), kBlock, 0, ctx->stream>>>(
-        cache, n, d.nbw, d.has_nr ? 1 : 0, ctx->scratch.partials, ctx->scratch.counters, d.gram_dev[pi]);
-  }
-  GOO_CUDA_TRY(cudaGetLastError());
-  return GOO_OK;
-}
-
 static int ensure_gram(goo_model* m, int precision) {
   DalitzModel& d = *m->dalitz;
   const int pi = precision == GOO_F32 ? 0 : 1;
@@ -1218,14 +1141,8 @@ static int ensure_gram(goo_model* m, int precision) {
   const void* cache = nullptr;
   GOO_TRY(ensure_cache(m, d.mc, precision, &cache));
   if (d.mc->n < 1) return set_error(GOO_ERR_ARG, "the MC normalisation sample is empty");
-  if (pi == 0) {
-    GOO_TRY((d.nbw <= 8 ? launch_gram<float, 8>(m, cache, d.mc->n, pi) : launch_gram<float, 15>(m, cache, d.mc->n, pi)));
-  } else {
-    GOO_TRY((d.nbw <= 8 ? launch_gram<double, 8>(m, cache, d.mc->n, pi) : launch_gram<double, 15>(m, cache, d.mc->n, pi)));
-  }
-  GOO_CUDA_TRY(cudaMemcpyAsync(d.gram_host[pi], d.gram_dev[pi], sizeof(double) * 2 * d.K * d.K, cudaMemcpyDeviceToHost,
-                               m->ctx->stream));
-  GOO_CUDA_TRY(cudaStreamSynchronize(m->ctx->stream));
+  GOO_TRY(gram_matrices(m->ctx, precision, false, 1, &cache, &cache, d.mc->n, d.nbw, d.K, d.gram_dev[pi],
+                        d.gram_host[pi], pi == 0 ? "gram_f32" : "gram_f64"));
   d.gram_key[pi] = key;
   return GOO_OK;
 }
@@ -1453,22 +1370,9 @@ static int ensure_td_grams(goo_model* m, int precision) {
   const void *ca = nullptr, *cb = nullptr;
   GOO_TRY(ensure_cache(m, d.mc, precision, &ca));
   GOO_TRY(ensure_cache(m, d.mc, precision, &cb, true));
-  const int K = d.K;
-  double* g = d.gram3_dev[pi];
-  const void* pairs[3][2] = {{ca, ca}, {cb, cb}, {ca, cb}};
-  for (int q = 0; q < 3; ++q) {
-    LaunchScope ls(ctx, pi == 0 ? "td3_gram_f32" : "td3_gram_f64");
-    if (pi == 0)
-      gram_cross_kernel<float><<<K * K, kBlock, 0, ctx->stream>>>(pairs[q][0], pairs[q][1], d.mc->n, d.nbw, K,
-                                                                 g + (size_t)q * 2 * K * K);
-    else
-      gram_cross_kernel<double><<<K * K, kBlock, 0, ctx->stream>>>(pairs[q][0], pairs[q][1], d.mc->n, d.nbw, K,
-                                                                  g + (size_t)q * 2 * K * K);
-  }
-  GOO_CUDA_TRY(cudaGetLastError());
-  GOO_CUDA_TRY(cudaMemcpyAsync(d.gram3_host[pi], g, sizeof(double) * 3 * 2 * K * K, cudaMemcpyDeviceToHost,
-                               ctx->stream));
-  GOO_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  const void *x[3] = {ca, cb, ca}, *y[3] = {ca, cb, cb};
+  GOO_TRY(gram_matrices(ctx, precision, true, 3, x, y, d.mc->n, d.nbw, d.K, nullptr, d.gram3_host[pi],
+                        pi == 0 ? "td3_gram_f32" : "td3_gram_f64"));
   d.gram3_key[pi] = key;
   return GOO_OK;
 }
@@ -1705,13 +1609,6 @@ int build_dalitz_model(goo_ctx* ctx, const goo_node* nodes, int n_nodes, int n_p
   if (d->td && std::fabs(d->m2 - d->m3) > 1e-12 * d->M)
     return set_error(GOO_ERR_ARG, "GOO_OP_TD3: the CP-conjugate particles 2 and 3 need equal masses (%g, %g)", d->m2,
                      d->m3);
-  if (d->td) {
-    for (int i = 0; i < 2; ++i)
-      if (cudaMalloc(&d->gram3_dev[i], sizeof(double) * 3 * 2 * kMaxAmp * kMaxAmp) != cudaSuccess) {
-        cudaGetLastError();
-        return set_error(GOO_ERR_OOM, "cannot allocate the amplitude model");
-      }
-  }
   (void)lo;
   (void)hi;
   if (cudaMalloc(&d->dev, sizeof(DalitzDev)) != cudaSuccess ||
@@ -1746,8 +1643,6 @@ void dalitz_free(goo_model* m) {
   for (int i = 0; i < 2; ++i)
     if (d->gram_dev[i]) cudaFree(d->gram_dev[i]);
   if (d->ls_mc) cudaFree(d->ls_mc);
-  for (int i = 0; i < 2; ++i)
-    if (d->gram3_dev[i]) cudaFree(d->gram3_dev[i]);
   delete d;
   m->dalitz = nullptr;
 }

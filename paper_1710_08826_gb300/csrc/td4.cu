@@ -33,7 +33,7 @@
 #include <vector>
 
 #include "common.cuh"
-#include "dalitz.cuh"
+#include "gram.cuh"
 #include "model.cuh"
 #include "timeterms.cuh"
 
@@ -679,31 +679,6 @@ static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, const
   return GOO_OK;
 }
 
-template <typename T>
-static int td4_gram_launch(goo_model* m, const void* cache, int64_t n, int pi) {
-  Td4Model& d = *m->td4;
-  goo_ctx* ctx = m->ctx;
-  constexpr int KB = 15;
-  constexpr int NS = 2 * (KB + 1);
-  int bps = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, gram_kernel<T, KB>, kBlock, 0) != cudaSuccess || bps < 1) {
-    cudaGetLastError();
-    bps = 1;
-  }
-  int64_t nbx = (n + kBlock - 1) / kBlock;
-  const int64_t cap = ((int64_t)ctx->num_sms * bps + d.K - 1) / d.K;
-  if (nbx > cap) nbx = cap;
-  if (nbx < 1) nbx = 1;
-  GOO_TRY(ensure_partials(ctx, (size_t)nbx * d.K * NS));
-  {
-    LaunchScope ls(ctx, sizeof(T) == 4 ? "td4_gram_f32" : "td4_gram_f64");
-    gram_kernel<T, KB><<<dim3((unsigned)nbx, d.K), kBlock, 0, ctx->stream>>>(cache, n, d.K, 0, ctx->scratch.partials,
-                                                                            ctx->scratch.counters, d.gram_dev[pi]);
-  }
-  GOO_CUDA_TRY(cudaGetLastError());
-  return GOO_OK;
-}
-
 static int td4_ensure_gram(goo_model* m, int precision) {
   Td4Model& d = *m->td4;
   const int pi = precision == GOO_F32 ? 0 : 1;
@@ -714,11 +689,8 @@ static int td4_ensure_gram(goo_model* m, int precision) {
   if (d.mc->n < 1) return set_error(GOO_ERR_ARG, "the MC normalisation sample is empty");
   const void* cache = nullptr;
   GOO_TRY(td4_cache(m, d.mc, precision, &cache));
-  if (pi == 0) GOO_TRY(td4_gram_launch<float>(m, cache, d.mc->n, pi));
-  else GOO_TRY(td4_gram_launch<double>(m, cache, d.mc->n, pi));
-  GOO_CUDA_TRY(cudaMemcpyAsync(d.gram_host[pi], d.gram_dev[pi], sizeof(double) * 2 * d.K * d.K, cudaMemcpyDeviceToHost,
-                               m->ctx->stream));
-  GOO_CUDA_TRY(cudaStreamSynchronize(m->ctx->stream));
+  GOO_TRY(gram_matrices(m->ctx, precision, false, 1, &cache, &cache, d.mc->n, d.K, d.K, d.gram_dev[pi], d.gram_host[pi],
+                        pi == 0 ? "td4_gram_f32" : "td4_gram_f64"));
   d.gram_key[pi] = key;
   return GOO_OK;
 }
