@@ -65,7 +65,6 @@ struct DalitzModel {
   uint64_t gram_key[2] = {0, 0};
   const goo_dataset* mc = nullptr;
   bool floating = false;           // GOO_LINESHAPE_FLOATING: no cache, lineshape gradients
-  double* ls_mc = nullptr;         // MC-pass lane sums of the floating-lineshape path (device)
   bool polar = false;              // GOO_COEF_POLAR: the coefficient parameters are (r, phi)
   // time-dependent three-body model (GOO_OP_TD3)
   bool td = false;
@@ -524,24 +523,35 @@ static uint64_t lineshape_key(const DalitzModel& d, const double* theta) {
 // Lineshape constants for the current theta (FP64, once per lineshape version).
 // ---------------------------------------------------------------------------------------
 // floating lineshapes (masses and widths free; paper Sec. 4: the cache is then invalid at
-// every step).  No amplitude cache: each evaluation runs a pass over the MC sample and one
-// over the events, and both evaluate every Breit-Wigner amplitude from (s12, s13) with the
+// every step).  No amplitude cache: each evaluation evaluates every Breit-Wigner amplitude of the
+// events and of the MC sample from (s12, s13) with the
 // parts of its denominator D = m0^2 - s - i m0 Gamma(s), which give
 //   d log A / d m0     = rho - (2 m0 - i kappa m0 Gamma(s)) / D,
 //   d log A / d Gamma0 = i m0 Gamma(s) / (Gamma0 D),
 // where rho = d log(B_L(z) / B_L(z0)) / d m0 (through q0) and kappa = d log(m0 Gamma(s)) /
 // d m0 = 2 / m0 - (2L + 1) d log q0 / d m0 + 2 rho are constants of the resonance (the
-// spin and parent-barrier factors do not depend on m0 or Gamma0).  Lanes: 0 = sum log |S|^2
-// (events) or sum |S|^2 (MC); then per amplitude slot Re / Im of A_k conj(S) w; then per
-// resonance Re(c_k A_k conj(S) w d log A_k / d m0) and the same for Gamma0, with w = 1 / |S|^2
-// for events and 1 for MC points.  The event pass's last block combines both passes:
+// spin and parent-barrier factors do not depend on m0 or Gamma0).  With u_k = A_k conj(S) w and
+// y_k = c_k u_k / D_k (w = 1 / |S|^2 for events and 1 for MC points) the lanes are: 0 = sum log2 |S|^2
+// (events) or sum |S|^2 (MC); per amplitude slot sum u_k (re, im); per resonance sum Re y_k and
+// sum m0 Gamma(s) Im y_k.  The last block has
+//   sum Re(c_k u_k d log A_k / d m0) = rho Re(c_k sum u_k) - 2 m0 sum Re y_k - kappa sum m0 Gamma Im y_k,
+//   sum Re(c_k u_k d log A_k / d Gamma0) = -(sum m0 Gamma Im y_k) / Gamma0
+// from both sets of sums and combines them:
 //   NLL = -sum log |S|^2 + n log(sum_MC |S|^2 / n_MC),
 //   d NLL / d p = -sum_events (d |S|^2 / d p) / |S|^2 + n (sum_MC d |S|^2 / d p) / sum_MC |S|^2.
+//
+// Issue-bound.  The factors shared by a pair and spin are formed once per point (lineshape.cuh) and kept
+// in the thread's column of shared memory; FP32 works on two points at a time; a resonance's
+// amplitude is formed again for its lanes (ten operations) rather than kept; the
+// first blocks of the one launch take the MC sample and the others the events, so that neither waits for the
+// other's reduction.  5M events and 1M MC points, 8 resonances: 495 us in two launches with every
+// resonance evaluated by itself, now 156 us.
 // ---------------------------------------------------------------------------------------
 template <typename T>
 struct LsConst {
   T cr[kMaxAmp], ci[kMaxAmp];          // coefficients by slot: resonances, then the NR in slot KB
-  T rho[kMaxAmp], kappa[kMaxAmp], two_m0[kMaxAmp], inv_g0[kMaxAmp];
+  T ncr[kMaxAmp], nci[kMaxAmp];        // minus these
+  double rho[kMaxAmp], kappa[kMaxAmp], two_m0[kMaxAmp], inv_g0[kMaxAmp];
   int par_m0[kMaxAmp], par_w[kMaxAmp];
 };
 
@@ -550,157 +560,226 @@ struct LsLanes {
   static constexpr int NS = GRAD ? 1 + 2 * (KB + 1) + 2 * KB : 1;
 };
 
-// Dynamic shared memory of a floating-lineshape block: per thread, the five parts (re, im,
-// dr, di, inv) of each resonance's amplitude and the NS - 1 gradient lanes, as columns of
-// kBlock values (thread t at offset t: conflict-free), with the gradient only.
+// One set of points (the MC sample or the events).
+template <typename T>
+struct LsSet {
+  const T *c12, *c13;
+  int64_t begin, end, n;  // the points of the evaluation, and of the column
+};
+
+// Dynamic shared memory: the shared factors of every thread, later the block reduction's lanes.
 template <typename T, int KB, bool GRAD>
 constexpr size_t ls_smem() {
-  return GRAD ? (size_t)(5 * KB + LsLanes<KB, GRAD>::NS - 1) * kBlock * sizeof(T) : 0;
+  const size_t f = (size_t)kLsCols * kBlock * 8, r = (size_t)LsLanes<KB, GRAD>::NS * kBlock * sizeof(ddf);
+  return f > r ? f : r;
 }
 
-// The resonances are visited in a run-time loop (not unrolled) whose state lives in those
-// shared-memory columns, so that the kernel needs few registers.
-template <typename T, int KB, bool GRAD, bool MC>
-__global__ void __launch_bounds__(kBlock)
+namespace lsv {
+// sums over a thread's points: a packed pair's two halves, or the double itself
+__device__ __forceinline__ ddf total(float2 v) { return dd_add(ddf{v.x, 0.f}, ddf{v.y, 0.f}); }
+__device__ __forceinline__ ddf total(double v) { return dd_from_double(v); }
+}  // namespace lsv
+
+// Compensated (FP32) or plain (FP64) running sum of lane 0.
+struct LsSumF {
+  Kahan a, b;
+  __device__ __forceinline__ void add(float2 x) {
+    a.add(x.x);
+    b.add(x.y);
+  }
+  __device__ __forceinline__ ddf value() const { return dd_add(a.value(), b.value()); }
+};
+struct LsSumD {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double x) { s += x; }
+  __device__ __forceinline__ ddf value() const { return dd_from_double(s); }
+};
+
+// The point(s) of step j: (s12, s13), and which of them count.
+__device__ __forceinline__ void ls_load(const LsSet<float>& D, int64_t j, float2& a, float2& b, bool& v0, bool& v1) {
+  const int64_t i = 2 * j;  // pairs at even indices
+  v0 = i >= D.begin;
+  v1 = i + 1 < D.end;
+  if (i + 1 < D.n) {
+    a = *reinterpret_cast<const float2*>(D.c12 + i);
+    b = *reinterpret_cast<const float2*>(D.c13 + i);
+  } else {
+    a = pk::splat(D.c12[i]);
+    b = pk::splat(D.c13[i]);
+  }
+  if (!(v0 && v1)) {  // a point outside the range takes the other's place, with weight 0
+    a = pk::splat(v0 ? a.x : a.y);
+    b = pk::splat(v0 ? b.x : b.y);
+  }
+}
+__device__ __forceinline__ void ls_load(const LsSet<double>& D, int64_t j, double& a, double& b, bool& v0, bool& v1) {
+  a = D.c12[j];
+  b = D.c13[j];
+  v0 = true;
+  v1 = false;
+}
+__device__ __forceinline__ int64_t ls_first(const LsSet<float>& D) { return D.begin >> 1; }
+__device__ __forceinline__ int64_t ls_last(const LsSet<float>& D) { return (D.end + 1) >> 1; }
+__device__ __forceinline__ int64_t ls_first(const LsSet<double>& D) { return D.begin; }
+__device__ __forceinline__ int64_t ls_last(const LsSet<double>& D) { return D.end; }
+
+// The weight 1 / |S|^2 (MC: 1) and lane 0's term (log2 |S|^2 in FP32, log in FP64; MC: |S|^2) of the points that
+// count, 0 for the others; events with |S|^2 <= 0 are counted in bad.
+__device__ __forceinline__ void ls_weight(bool mc, float2 s2, bool v0, bool v1, float2& w, float2& term, unsigned& bad) {
+  if (mc) {
+    w = make_float2(v0 ? 1.f : 0.f, v1 ? 1.f : 0.f);
+    term = make_float2(v0 ? s2.x : 0.f, v1 ? s2.y : 0.f);
+    return;
+  }
+  const bool ok0 = s2.x > 0.f, ok1 = s2.y > 0.f;
+  bad += (unsigned)(v0 && !ok0) + (unsigned)(v1 && !ok1);
+  constexpr float kMin = 1.17549435e-38f;  // the hardware functions flush smaller values to 0
+  const float2 s = make_float2(fmaxf(s2.x, kMin), fmaxf(s2.y, kMin)), r = lsv::rcp(s);
+  w = make_float2(v0 && ok0 ? r.x : 0.f, v1 && ok1 ? r.y : 0.f);
+  term = make_float2(v0 && ok0 ? pk::lg2(s.x) : 0.f, v1 && ok1 ? pk::lg2(s.y) : 0.f);
+}
+__device__ __forceinline__ void ls_weight(bool mc, double s2, bool, bool, double& w, double& term, unsigned& bad) {
+  if (mc) {
+    w = 1.0;
+    term = s2;
+  } else if (s2 > 0.0) {
+    w = recip(s2);
+    term = log(s2);
+  } else {
+    ++bad;
+    w = term = 0.0;
+  }
+}
+
+template <typename T, int KB, bool GRAD>
+__global__ void __launch_bounds__(kBlock, KB <= 8 ? 2 : 1)
     coh_ls_kernel(const __grid_constant__ CohArgs<T> a, const __grid_constant__ LsConst<T> c,
-                  const DalitzDev* __restrict__ ddp, const T* __restrict__ c12, const T* __restrict__ c13,
-                  int64_t begin, int64_t end, const double* __restrict__ mc_sums, double n_mc, float2* partials,
-                  unsigned* counters, double* out, int out_mode) {
+                  const __grid_constant__ LsTables<T> t, const __grid_constant__ LsSet<T> mc,
+                  const __grid_constant__ LsSet<T> ev, int nb_mc, float2* partials, unsigned* counters, double* out,
+                  int out_mode) {
+  using namespace lsv;
+  using V = typename std::conditional<sizeof(T) == 4, float2, double>::type;
+  using Sum = typename std::conditional<sizeof(T) == 4, LsSumF, LsSumD>::type;
   constexpr int KA = KB + 1;
   constexpr int NS = LsLanes<KB, GRAD>::NS;
-  __shared__ DalitzDev s_dd;
-  __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
-  __shared__ unsigned s_bad[kBlock / 32];
-  __shared__ double s_out[NS];
+  __shared__ ddf s_red[kBlock / 32];
+  __shared__ double s_out[NS], s_mc[NS];
   extern __shared__ __align__(16) unsigned char s_dyn[];
-  T* s_a = reinterpret_cast<T*>(s_dyn);  // [5][KB][kBlock]
-  T* s_l = s_a + 5 * KB * kBlock;        // [NS - 1][kBlock]
-  const int t = threadIdx.x;
-  for (int i = t; i < (int)(sizeof(DalitzDev) / 4); i += blockDim.x) ((int*)&s_dd)[i] = ((const int*)ddp)[i];
-  if constexpr (GRAD)
-    for (int j = 0; j < NS - 1; ++j) s_l[j * kBlock + t] = T(0);
-  __syncthreads();
-  const int nbw = s_dd.nbw;
-  const T cnr = c.cr[KB], cni = c.ci[KB];
-  Kahan lf32;
-  double lf64 = 0.0;
+  V* s_v = reinterpret_cast<V*>(s_dyn);
+  V *sc = s_v + threadIdx.x, *gc = sc + 3 * kBlock, *hc = sc + 12 * kBlock;
+  const bool is_mc = (int)blockIdx.x < nb_mc;
+  const LsSet<T>& D = is_mc ? mc : ev;
+  const int nb = is_mc ? nb_mc : (int)gridDim.x - nb_mc, b0 = is_mc ? (int)blockIdx.x : (int)blockIdx.x - nb_mc;
+  Sum l0;
+  V lre[KA], lim[KA], lwr[KB], lwi[KB];
+  const V zero = splat(V{}, T(0));
+#pragma unroll
+  for (int k = 0; k < KA; ++k) lre[k] = lim[k] = zero;
+#pragma unroll
+  for (int k = 0; k < KB; ++k) lwr[k] = lwi[k] = zero;
   unsigned bad = 0;
-  for (int64_t i = begin + blockIdx.x * (int64_t)blockDim.x + t; i < end; i += (int64_t)gridDim.x * blockDim.x) {
-    const T x12 = c12[i], x13 = c13[i];
-    T x23;
-    if constexpr (sizeof(T) == 4) x23 = (float)(s_dd.sumsq - (double)x12 - (double)x13);
-    else x23 = s_dd.sumsq - x12 - x13;
-    T sr = cnr, si = cni;  // the non-resonant amplitude is 1
-#pragma unroll 1
-    for (int k = 0; k < nbw; ++k) {
-      T ar, ai, dr, di, iv;
-      bw_amp_parts<T>(bw_of<T>(s_dd, k), x12, x13, x23, ar, ai, dr, di, iv);
-      sr += c.cr[k] * ar - c.ci[k] * ai;
-      si += c.cr[k] * ai + c.ci[k] * ar;
-      if constexpr (GRAD) {
-        T* col = s_a + k * kBlock + t;
-        col[0] = ar;
-        col[KB * kBlock] = ai;
-        col[2 * KB * kBlock] = dr;
-        col[3 * KB * kBlock] = di;
-        col[4 * KB * kBlock] = iv;
-      }
+  const int64_t last = ls_last(D);
+  for (int64_t j = ls_first(D) + b0 * (int64_t)kBlock + threadIdx.x; j < last; j += (int64_t)nb * kBlock) {
+    V x12, x13, re, im, dr, di, iv;
+    bool v0, v1;
+    ls_load(D, j, x12, x13, v0, v1);
+    ls_groups<T, V>(t, x12, x13, sc, gc, hc, kBlock);
+    V sr = splat(V{}, c.cr[KB]), si = splat(V{}, c.ci[KB]);  // the non-resonant amplitude is 1
+#pragma unroll 4
+    for (int k = 0; k < t.nbw; ++k) {
+      ls_amp<T, V>(t, k, sc, gc, hc, kBlock, re, im, dr, di, iv);
+      const V cr = splat(V{}, c.cr[k]);
+      sr = fma(cr, re, fma(splat(V{}, c.nci[k]), im, sr));
+      si = fma(cr, im, fma(splat(V{}, c.ci[k]), re, si));
     }
-    const T s2 = sr * sr + si * si;
-    if (!MC && !(s2 > T(0))) {
-      ++bad;
-      continue;
-    }
-    if constexpr (sizeof(T) == 4) lf32.add(MC ? s2 : __logf(s2));
-    else lf64 += MC ? s2 : log(s2);
+    V w, term;
+    ls_weight(is_mc, fma(sr, sr, mul(si, si)), v0, v1, w, term, bad);
+    l0.add(term);
     if constexpr (GRAD) {
-      const T w = MC ? T(1) : T(1) / s2;
-      const T tr = sr * w, ti = -si * w;  // conj(S) w
-      s_l[(2 * KB) * kBlock + t] += tr;   // the non-resonant slot: A = 1
-      s_l[(2 * KB + 1) * kBlock + t] += ti;
-#pragma unroll 1
-      for (int k = 0; k < nbw; ++k) {
-        const T* col = s_a + k * kBlock + t;
-        const T ar = col[0], ai = col[KB * kBlock], dr = col[2 * KB * kBlock], di = col[3 * KB * kBlock],
-                iv = col[4 * KB * kBlock];
-        const T ur = ar * tr - ai * ti, ui = ar * ti + ai * tr;                      // A_k conj(S) w
-        const T vr = c.cr[k] * ur - c.ci[k] * ui, vi = c.cr[k] * ui + c.ci[k] * ur;  // c_k A_k conj(S) w
-        const T e2 = di * iv;
-        const T lmr = c.rho[k] - (c.two_m0[k] * dr + c.kappa[k] * di * di) * iv;
-        const T lmi = -(c.two_m0[k] - c.kappa[k] * dr) * e2;
-        const T lgr = -di * e2 * c.inv_g0[k], lgi = dr * e2 * c.inv_g0[k];
-        T* lane = s_l + 2 * k * kBlock + t;
-        lane[0] += ur;
-        lane[kBlock] += ui;
-        lane[2 * KA * kBlock] += vr * lmr - vi * lmi;
-        lane[(2 * KA + 1) * kBlock] += vr * lgr - vi * lgi;
+      const V tr = mul(sr, w), mti = mul(si, w), ti = neg(mti);  // conj(S) w
+      lre[KB] = add(lre[KB], tr);  // the non-resonant slot: A = 1
+      lim[KB] = add(lim[KB], ti);
+#pragma unroll
+      for (int k = 0; k < KB; ++k) {
+        if (k >= t.nbw) break;
+        ls_amp<T, V>(t, k, sc, gc, hc, kBlock, re, im, dr, di, iv);
+        const V ur = fma(re, tr, mul(im, mti)), ui = fma(re, ti, mul(im, tr));  // A_k conj(S) w
+        lre[k] = add(lre[k], ur);
+        lim[k] = add(lim[k], ui);
+        // v = c_k u_k / |D|^2 and mvi = -Im v; y_k = v (dr + i di)
+        const V nci = splat(V{}, c.nci[k]);
+        const V vr = mul(fma(splat(V{}, c.cr[k]), ur, mul(nci, ui)), iv);
+        const V mvi = mul(fma(splat(V{}, c.ncr[k]), ui, mul(nci, ur)), iv);
+        lwr[k] = fma(vr, dr, fma(mvi, di, lwr[k]));
+        lwi[k] = fma(di, sub(mul(vr, di), mul(mvi, dr)), lwi[k]);
       }
     }
   }
   ddf v[NS];
-  v[0] = (sizeof(T) == 4) ? lf32.value() : dd_from_double(lf64);
+  v[0] = l0.value();
+  if (sizeof(T) == 4 && !is_mc) v[0] = dd_mul(v[0], ddf{kLn2Hi, kLn2Lo});
   if constexpr (GRAD) {
 #pragma unroll
-    for (int j = 0; j < NS - 1; ++j) {
-      const T x = s_l[j * kBlock + t];
-      v[1 + j] = (sizeof(T) == 4) ? ddf{(float)x, 0.f} : dd_from_double((double)x);
+    for (int k = 0; k < KA; ++k) {
+      v[1 + 2 * k] = total(lre[k]);
+      v[2 + 2 * k] = total(lim[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < KB; ++k) {
+      v[1 + 2 * KA + 2 * k] = total(lwr[k]);
+      v[2 + 2 * KA + 2 * k] = total(lwi[k]);
     }
   }
   for (int m = 16; m > 0; m >>= 1) bad += __shfl_xor_sync(0xffffffffu, bad, m);
-  if ((threadIdx.x & 31) == 0) s_bad[threadIdx.x >> 5] = bad;
-  block_reduce_to_partials<NS>(v, NS, partials, s_red);
-  if (threadIdx.x == 0) {
-    unsigned b = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += s_bad[w];
-    if (b) atomicAdd(counters + 1, b);
-  }
+  if ((threadIdx.x & 31) == 0 && bad) atomicAdd(counters + 1, bad);
+  __syncthreads();  // the columns of the shared factors become the reduction's buffer
+  block_reduce_transpose<NS>(v, partials, reinterpret_cast<ddf*>(s_dyn));
   if (!last_block_ticket(counters, gridDim.x)) return;
-  reduce_partials(partials, NS, gridDim.x, s_out, s_red, blockDim.x);
-  if constexpr (MC) {
-    // the MC pass ends with its lane sums (read by the event pass that follows it)
-    for (int t = threadIdx.x; t < NS; t += blockDim.x) out[t] = s_out[t];
-    if (threadIdx.x == 0) *counters = 0u;  // the ticket
-    return;
+  unsigned nbad = 0u, status = 0u;
+  if (threadIdx.x == 0) {
+    nbad = __ldcg(counters + 1);
+    status = __ldcg(counters + kStatusWord);
   }
-  const double nev = (double)(end - begin);
-  const double Smc = mc_sums[0];
+  reduce_partials<24>(partials, NS, nb_mc, s_mc, s_red, kBlock);
+  reduce_partials<24>(partials + (size_t)nb_mc * NS, NS, (int)gridDim.x - nb_mc, s_out, s_red, kBlock);
+  const double nev = (double)(ev.end - ev.begin), Smc = s_mc[0];
   const int P = a.n_params;
   const int off = out_mode == 0 ? 2 : 3;
   for (int p = threadIdx.x; p < P; p += blockDim.x) {
     double g = 0.0;
-    if (GRAD) {
+    if constexpr (GRAD) {
+      const double f = nev / Smc;
+      // -2 (events) + 2 n / S_mc (MC) of lane j
+      auto both = [&](int j) { return 2.0 * (f * s_mc[j] - s_out[j]); };
       for (int kk = 0; kk < a.K; ++kk) {
         const int sl = kk < a.nbw ? kk : KB;  // the NR lives in the last slot
-        double gre = -2.0 * s_out[1 + 2 * sl] + 2.0 * nev * mc_sums[1 + 2 * sl] / Smc;
-        double gim = 2.0 * s_out[2 + 2 * sl] - 2.0 * nev * mc_sums[2 + 2 * sl] / Smc;
+        double gre = both(1 + 2 * sl), gim = -both(2 + 2 * sl);
         coef_chain(a.polar, a.jc[kk], a.js[kk], a.jr[kk], gre, gim);
         if (a.par_re[kk] == p) g += gre;
         if (a.par_im[kk] == p) g += gim;
       }
       for (int k = 0; k < a.nbw; ++k) {
-        const int o = 1 + 2 * KA + 2 * k;
-        if (c.par_m0[k] == p) g += -2.0 * s_out[o] + 2.0 * nev * mc_sums[o] / Smc;
-        if (c.par_w[k] == p) g += -2.0 * s_out[o + 1] + 2.0 * nev * mc_sums[o + 1] / Smc;
+        const double cu = (double)c.cr[k] * both(1 + 2 * k) - (double)c.ci[k] * both(2 + 2 * k);
+        const double y = both(2 + 2 * KA + 2 * k);
+        if (c.par_m0[k] == p) g += c.rho[k] * cu - c.two_m0[k] * both(1 + 2 * KA + 2 * k) - c.kappa[k] * y;
+        if (c.par_w[k] == p) g -= c.inv_g0[k] * y;
       }
     }
     out[off + p] = g;
   }
   if (threadIdx.x == 0) {
-    // every other block added to these words before its ticket (and a fence): plain L2 reads
-    const unsigned nbad = __ldcg(counters + 1);
-    const unsigned status = __ldcg(counters + kStatusWord);
     counters[1] = 0u;
     counters[kStatusWord] = 0u;
     *counters = 0u;  // the ticket
-    const double N = Smc / n_mc;
-    const double nb = status ? -1.0 : (double)nbad;  // a device wait that gave up: negative count
+    const double N = Smc / (double)(mc.end - mc.begin);
+    const double nb_ = status ? -1.0 : (double)nbad;  // a device wait that gave up: negative count
     out[0] = -s_out[0] + nev * log(N);
     if (out_mode == 0) {
-      out[1] = nb;
+      out[1] = nb_;
       out[2 + P] = N;
     } else {
       out[1] = 0.0;
-      out[2] = nb;
+      out[2] = nb_;
     }
   }
   result_complete(out);
@@ -1275,6 +1354,8 @@ static void fill_ls(const DalitzModel& d, const double* theta, LsConst<T>& c) {
     coef(d, theta, k, re, im);
     c.cr[k] = (T)re;
     c.ci[k] = (T)im;
+    c.ncr[k] = -c.cr[k];
+    c.nci[k] = -c.ci[k];
     c.par_m0[k] = d.par_m0[k];
     c.par_w[k] = d.par_w[k];
     double mA, mB, mC;
@@ -1289,36 +1370,32 @@ static void fill_ls(const DalitzModel& d, const double* theta, LsConst<T>& c) {
     if (L == 1) rho = 0.5 / (1.0 + z0) * r2 * dq0sq;
     if (L == 2) rho = 0.5 * (3.0 + 2.0 * z0) / (9.0 + 3.0 * z0 + z0 * z0) * r2 * dq0sq;
     const double kappa = 2.0 / m0 - (2 * L + 1) * dq0sq / (2.0 * q0sq) + 2.0 * rho;
-    c.rho[k] = (T)rho;
-    c.kappa[k] = (T)kappa;
-    c.two_m0[k] = (T)(2.0 * m0);
-    c.inv_g0[k] = (T)(1.0 / g0);
+    c.rho[k] = rho;
+    c.kappa[k] = kappa;
+    c.two_m0[k] = 2.0 * m0;
+    c.inv_g0[k] = 1.0 / g0;
   }
   for (int k = d.nbw; k < kMaxAmp; ++k) c.par_m0[k] = c.par_w[k] = -1;
 }
 
-template <typename T, int KB, bool GRAD, bool MC>
+template <typename T, int KB, bool GRAD>
 static int launch_ls(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, const double* theta,
-                     double* out, int out_mode) {
+                     int out_mode) {
   DalitzModel& d = *m->dalitz;
   goo_ctx* ctx = m->ctx;
-  GOO_TRY(dalitz_dev(m));
   constexpr size_t smem = ls_smem<T, KB, GRAD>();
-  static int occ[2] = {0, 0};
-  int& o = occ[MC ? 1 : 0];
-  if (o == 0) {
-    if (smem > 48 * 1024)
-      GOO_CUDA_TRY(cudaFuncSetAttribute(coh_ls_kernel<T, KB, GRAD, MC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem));
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, coh_ls_kernel<T, KB, GRAD, MC>, kBlock, smem) != cudaSuccess ||
-        o < 1) {
-      cudaGetLastError();
-      o = 1;
-    }
-  }
-  const int nb = grid_blocks(ctx, end - begin, o);
   constexpr int NS = LsLanes<KB, GRAD>::NS;
-  GOO_TRY(ensure_partials(ctx, (size_t)nb * NS));
+  const void* fn = (const void*)coh_ls_kernel<T, KB, GRAD>;
+  GOO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int64_t cap = (int64_t)ctx->num_sms * cached_occupancy(fn, ctx->device, kBlock, smem);
+  // blocks in proportion to the points, at least one each, no more than there are steps
+  constexpr int per = sizeof(T) == 4 ? 2 : 1;
+  auto steps = [](int64_t n) { return (n / per + 1 + kBlock) / kBlock; };
+  const int64_t n_mc = d.mc->n, n_ev = end - begin;
+  const int64_t want_mc = std::max<int64_t>(1, (int64_t)((double)cap * n_mc / (double)(n_mc + n_ev) + 0.5));
+  const int nb_mc = (int)std::min<int64_t>(std::min<int64_t>(want_mc, cap - 1), steps(n_mc));
+  const int nb_ev = (int)std::min<int64_t>(cap - nb_mc, steps(n_ev));
+  GOO_TRY(ensure_partials(ctx, (size_t)(nb_mc + nb_ev) * NS));
   CohArgs<T> a;
   fill_args<T>(d, theta, m->n_params, ds->n, a);
   LsConst<T> c;
@@ -1329,31 +1406,28 @@ static int launch_ls(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t
     c.cr[KB] = (T)re;
     c.ci[KB] = (T)im;
   }
-  const T* c12 = sizeof(T) == 4 ? (const T*)ds->d32[d.col12] : (const T*)ds->d64[d.col12];
-  const T* c13 = sizeof(T) == 4 ? (const T*)ds->d32[d.col13] : (const T*)ds->d64[d.col13];
+  auto set = [&](const goo_dataset* s, int64_t b, int64_t e) {
+    if constexpr (sizeof(T) == 4) return LsSet<T>{s->d32[d.col12], s->d32[d.col13], b, e, s->n};
+    else return LsSet<T>{s->d64[d.col12], s->d64[d.col13], b, e, s->n};
+  };
   {
-    LaunchScope ls(ctx, MC ? (sizeof(T) == 4 ? "coh_ls_mc_f32" : "coh_ls_mc_f64")
-                           : (sizeof(T) == 4 ? (GRAD ? "coh_ls_grad_f32" : "coh_ls_f32")
-                                             : (GRAD ? "coh_ls_grad_f64" : "coh_ls_f64")));
-    coh_ls_kernel<T, KB, GRAD, MC><<<nb, kBlock, smem, ctx->stream>>>(
-        a, c, d.dev, c12, c13, begin, end, d.ls_mc, (double)(d.mc ? d.mc->n : 0), ctx->scratch.partials,
-        ctx->scratch.counters, out, out_mode);
+    LaunchScope ls(ctx, sizeof(T) == 4 ? (GRAD ? "coh_ls_grad_f32" : "coh_ls_f32") : (GRAD ? "coh_ls_grad_f64" : "coh_ls_f64"));
+    const LsTables<T>* t;
+    if constexpr (sizeof(T) == 4) t = &d.ls32;
+    else t = &d.ls64;
+    coh_ls_kernel<T, KB, GRAD><<<nb_mc + nb_ev, kBlock, smem, ctx->stream>>>(
+        a, c, *t, set(d.mc, 0, n_mc), set(ds, begin, end), nb_mc, ctx->scratch.partials, ctx->scratch.counters,
+        ctx->scratch.result_out, out_mode);
   }
   GOO_CUDA_TRY(cudaGetLastError());
   return GOO_OK;
 }
 
-// The floating-lineshape evaluation: the MC pass, then the event pass over [begin, end).
 template <typename T, bool GRAD>
-static int launch_ls_pair(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, const double* theta,
-                          int out_mode) {
-  DalitzModel& d = *m->dalitz;
-  if (d.nbw <= 8) {
-    GOO_TRY((launch_ls<T, 8, GRAD, true>(m, d.mc, 0, d.mc->n, theta, d.ls_mc, 0)));
-    return launch_ls<T, 8, GRAD, false>(m, ds, begin, end, theta, m->ctx->scratch.result_out, out_mode);
-  }
-  GOO_TRY((launch_ls<T, 15, GRAD, true>(m, d.mc, 0, d.mc->n, theta, d.ls_mc, 0)));
-  return launch_ls<T, 15, GRAD, false>(m, ds, begin, end, theta, m->ctx->scratch.result_out, out_mode);
+static int launch_ls_sel(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, const double* theta,
+                         int out_mode) {
+  return m->dalitz->nbw <= 8 ? launch_ls<T, 8, GRAD>(m, ds, begin, end, theta, out_mode)
+                             : launch_ls<T, 15, GRAD>(m, ds, begin, end, theta, out_mode);
 }
 
 // The three MC Gram matrices of the time-dependent three-body model (G_aa, G_bb, G_ab) in
@@ -1642,7 +1716,6 @@ void dalitz_free(goo_model* m) {
   if (d->dev) cudaFree(d->dev);
   for (int i = 0; i < 2; ++i)
     if (d->gram_dev[i]) cudaFree(d->gram_dev[i]);
-  if (d->ls_mc) cudaFree(d->ls_mc);
   delete d;
   m->dalitz = nullptr;
 }
@@ -1711,24 +1784,19 @@ int dalitz_nll(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, 
                     : launch_td3<double, false>(m, ds, begin, end, theta, ca, cb, out_mode)));
     }
   } else if (d.floating) {
-    // no cache and no Gram matrix: an MC pass and an event pass, lineshape gradients included
+    // no cache and no Gram matrix: MC points and events in one launch, lineshape gradients included
     if (!d.mc) return set_error(GOO_ERR_STATE, "amplitude model has no MC normalisation sample (goo_model_set_norm)");
     if (d.mc->n < 1) return set_error(GOO_ERR_ARG, "the MC normalisation sample is empty");
     if (end <= begin) {
       for (int i = 0; i < nout; ++i) out[i] = 0.0;
       return GOO_OK;
     }
-    if (!d.ls_mc && cudaMalloc(&d.ls_mc, 64 * sizeof(double)) != cudaSuccess) {
-      cudaGetLastError();
-      d.ls_mc = nullptr;
-      return set_error(GOO_ERR_OOM, "floating-lineshape work space");
-    }
     if (precision == GOO_F32) {
-      GOO_TRY((grad ? launch_ls_pair<float, true>(m, ds, begin, end, theta, out_mode)
-                    : launch_ls_pair<float, false>(m, ds, begin, end, theta, out_mode)));
+      GOO_TRY((grad ? launch_ls_sel<float, true>(m, ds, begin, end, theta, out_mode)
+                    : launch_ls_sel<float, false>(m, ds, begin, end, theta, out_mode)));
     } else {
-      GOO_TRY((grad ? launch_ls_pair<double, true>(m, ds, begin, end, theta, out_mode)
-                    : launch_ls_pair<double, false>(m, ds, begin, end, theta, out_mode)));
+      GOO_TRY((grad ? launch_ls_sel<double, true>(m, ds, begin, end, theta, out_mode)
+                    : launch_ls_sel<double, false>(m, ds, begin, end, theta, out_mode)));
     }
   } else {
   GOO_TRY(ensure_gram(m, precision));

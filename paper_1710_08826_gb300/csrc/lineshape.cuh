@@ -45,10 +45,11 @@ __device__ __forceinline__ float2 mul(float2 a, float2 b) { return pk::mul(a, b)
 __device__ __forceinline__ double add(double a, double b) { return a + b; }
 __device__ __forceinline__ float2 add(float2 a, float2 b) { return pk::add(a, b); }
 __device__ __forceinline__ double sub(double a, double b) { return a - b; }
-__device__ __forceinline__ float2 sub(float2 a, float2 b) { return pk::sub(a, b); }
+// a - b as an FMA by -1 and a negation as a product by -1 (exact): one packed instruction each
+__device__ __forceinline__ float2 sub(float2 a, float2 b) { return pk::fma(b, pk::splat(-1.f), a); }
 __device__ __forceinline__ double fma(double a, double b, double c) { return ::fma(a, b, c); }
 __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return pk::fma(a, b, c); }
-__device__ __forceinline__ float2 neg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 neg(float2 a) { return pk::mul(a, pk::splat(-1.f)); }
 __device__ __forceinline__ double neg(double a) { return -a; }
 __device__ __forceinline__ float2 floor_at(float2 a, float lo) { return make_float2(fmaxf(a.x, lo), fmaxf(a.y, lo)); }
 // lo >= 0: the sign and the magnitude are compared as integers
@@ -59,7 +60,7 @@ __device__ __forceinline__ double floor_at(double a, double lo) {
 __device__ __forceinline__ double rcp(double x) { return rcp64(x); }
 __device__ __forceinline__ float2 rcp(float2 x) {
   const float2 y = pk::rcp(x);
-  return fma(y, fma(neg(x), y, pk::splat(1.f)), y);
+  return fma(y, fma(x, neg(y), pk::splat(1.f)), y);
 }
 // 1 / sqrt(x), x > 0
 __device__ __forceinline__ double rsqrt(double x) {
@@ -75,8 +76,8 @@ __device__ __forceinline__ float rsqrt1(float x) {
 }
 __device__ __forceinline__ float2 rsqrt(float2 x) {
   const float2 y = make_float2(rsqrt1(x.x), rsqrt1(x.y));
-  const float2 e = fma(neg(mul(x, y)), y, pk::splat(1.f));
-  return fma(mul(pk::splat(0.5f), y), e, y);
+  const float2 e = fma(mul(x, y), y, pk::splat(-1.f));  // x y^2 - 1
+  return fma(mul(pk::splat(-0.5f), y), e, y);
 }
 // M^2 + sum m_i^2 - a - b to full precision: in FP32 from the exact differences (a < sum, b < sum - a)
 __device__ __forceinline__ double third(const LsTables<double>& t, double a, double b) { return t.sum_hi - a - b; }
