@@ -107,6 +107,9 @@ struct Scratch {
   double* chunk_records = nullptr;
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t chunk_events[65] = {};
+  // goo_nll_grad_batch's work space (pinned host and device), grown on demand
+  unsigned char *batch_host = nullptr, *batch_dev = nullptr;
+  size_t batch_host_cap = 0, batch_dev_cap = 0;
   double* gram_host = nullptr;      // mapped record of the Gram matrices (kGramRecord doubles), on first use
   void* fp64_tables = nullptr;      // device copy of the FP64 function tables (fp64.cuh), on first use
 };

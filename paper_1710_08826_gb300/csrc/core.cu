@@ -460,6 +460,8 @@ int goo_finalize(goo_ctx* ctx) {
   if (s.result) cudaFree(s.result);
   if (s.fp64_tables) cudaFree(s.fp64_tables);
   if (s.gram_host) cudaFreeHost(s.gram_host);
+  if (s.batch_host) cudaFreeHost(s.batch_host);
+  if (s.batch_dev) cudaFree(s.batch_dev);
   if (s.theta) cudaFree(s.theta);
   if (s.host_pinned) cudaFreeHost(s.host_pinned);
   if (s.result_host) cudaFreeHost(s.result_host);

@@ -1869,6 +1869,10 @@ int dalitz_amplitudes(goo_model* m, const goo_dataset* ds, const double* theta, 
   return GOO_OK;
 }
 
+int dalitz_cache(goo_model* m, const goo_dataset* ds, int precision, const void** cache) {
+  return ensure_cache(m, ds, precision, cache);
+}
+
 int dalitz_server_info(goo_model* m, const double* theta, AmpModelInfo* info) {
   if (m->kind != 1) return set_error(GOO_ERR_STATE, "toy server needs an amplitude model");
   if (m->dalitz->td) return set_error(GOO_ERR_UNSUPPORTED, "toy server of the time-dependent three-body model");
@@ -1879,6 +1883,7 @@ int dalitz_server_info(goo_model* m, const double* theta, AmpModelInfo* info) {
   const DalitzModel& d = *m->dalitz;
   info->dalitz_dev = d.dev;
   info->gram_dev = d.gram_dev[0];
+  info->gram_host = d.gram_host[0];
   info->K = d.K;
   info->nbw = d.nbw;
   info->has_nr = d.has_nr ? 1 : 0;

@@ -84,6 +84,9 @@ int dalitz_eval_logf(goo_model* m, const goo_dataset* ds, const double* theta, i
 int dalitz_gram(goo_model* m, const double* theta, int precision, double* out, int* K_out);
 int dalitz_amplitudes(goo_model* m, const goo_dataset* ds, const double* theta, int precision, const void** cache,
                       int* nbw);
+// the dataset's amplitude cache at the lineshapes of the latest call that took a theta, in order on the
+// context's stream
+int dalitz_cache(goo_model* m, const goo_dataset* ds, int precision, const void** cache);
 int dalitz_set_lineshapes(goo_model* m, int mode);
 bool dalitz_lineshape_param(const goo_model* m, int p);  // p is a resonance mass or width
 bool dalitz_floating(const goo_model* m);
@@ -134,6 +137,7 @@ namespace goo {
 struct AmpModelInfo {
   const void* dalitz_dev;   // DalitzDev*
   const double* gram_dev;   // K x K complex, FP64 (from the float32 MC cache)
+  const double* gram_host;  // the same on the host
   int K, nbw, has_nr;
   int par_re[16], par_im[16];
   double lo12, hi12, lo13, hi13;

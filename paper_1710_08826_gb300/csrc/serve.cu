@@ -323,7 +323,9 @@ struct SrvModel {   // shared by every fit of a batch
 // kSrvStages sub-tiles ahead of the consumers.  Dynamic shared memory:
 // kSrvStages * (kSrvKB / 2) * kSrvSub float4.  status[0] is set when a copy wait gave up;
 // wait_limit bounds each wait for a sub-tile in SM clocks (the drain before exit allows
-// kWaitCycles).
+// kWaitCycles).  host_results (null: none): a mapped record per fit (kSrvRecord doubles: nll, or +inf with
+// events of no density, then (re, im) of every slot's gradient) that the host polls field by field.
+constexpr int kSrvRecord = 1 + 2 * kSrvKA;
 constexpr int kSrvSub = 768;
 constexpr int kSrvStages = 2;
 constexpr size_t kSrvSmem = (size_t)kSrvStages * (kSrvKB / 2) * kSrvSub * sizeof(float4);
@@ -333,7 +335,7 @@ __global__ void __launch_bounds__(kBlock, 2) srv_nll_kernel(const SrvEval* __res
                                                            int tile_events, const SrvModel* __restrict__ sm,
                                                            float2* tile_partials, unsigned* fit_ticket,
                                                            SrvResult* results, unsigned* status,
-                                                           long long wait_limit) {
+                                                           long long wait_limit, double* host_results) {
   __shared__ ddf s_red[(kBlock / 32) * kSrvLanes > kBlock ? (kBlock / 32) * kSrvLanes : kBlock];
   __shared__ unsigned s_bad[kBlock / 32];
   __shared__ bool s_last;
@@ -519,12 +521,21 @@ __global__ void __launch_bounds__(kBlock, 2) srv_nll_kernel(const SrvEval* __res
       for (int m = 16; m > 0; m >>= 1) Nk += __shfl_xor_sync(0xffffffffu, Nk, m);
       const double nev = (double)e.n;
       SrvResult& R = results[fit];
+      volatile double* H = host_results ? host_results + (size_t)fit * kSrvRecord : nullptr;
       if (k < kSrvKA) {
-        R.gre[k] = live ? -2.0 * s_fin[1 + 2 * k] + nev * 2.0 * vr / Nk : 0.0;
-        R.gim[k] = live ? 2.0 * s_fin[2 + 2 * k] - nev * 2.0 * vi / Nk : 0.0;
+        const double gre = live ? -2.0 * s_fin[1 + 2 * k] + nev * 2.0 * vr / Nk : 0.0;
+        const double gim = live ? 2.0 * s_fin[2 + 2 * k] - nev * 2.0 * vi / Nk : 0.0;
+        R.gre[k] = gre;
+        R.gim[k] = gim;
+        if (H) {
+          H[1 + 2 * k] = gre;
+          H[2 + 2 * k] = gim;
+        }
       }
       if (k == 0) {
         R.nll = -s_fin[0] + nev * log(Nk);
+        // every tile counted its events of no density before its ticket
+        if (H) H[0] = __ldcg(&R.bad) ? HUGE_VAL : R.nll;
         R.norm = Nk;
         fit_ticket[fit] = 0u;
       }
@@ -1035,6 +1046,35 @@ struct goo_server {
 namespace goo {
 
 static size_t al256(size_t b) { return (b + 255) / 256 * 256; }
+
+// goo_nll_grad_batch's work space: at least host_bytes pinned and dev_bytes on the device, kept by
+// the context for the next call (no launch that uses it is in flight between calls).
+static int ensure_batch(goo_ctx* ctx, size_t host_bytes, size_t dev_bytes) {
+  Scratch& s = ctx->scratch;
+  if (s.batch_host_cap < host_bytes) {
+    if (s.batch_host) cudaFreeHost(s.batch_host);
+    s.batch_host = nullptr;
+    s.batch_host_cap = 0;
+    if (cudaMallocHost(&s.batch_host, 2 * host_bytes) != cudaSuccess) {
+      cudaGetLastError();
+      s.batch_host = nullptr;
+      return set_error(GOO_ERR_OOM, "goo_nll_grad_batch: work space");
+    }
+    s.batch_host_cap = 2 * host_bytes;
+  }
+  if (s.batch_dev_cap < dev_bytes) {
+    if (s.batch_dev) cudaFree(s.batch_dev);
+    s.batch_dev = nullptr;
+    s.batch_dev_cap = 0;
+    if (cudaMalloc(&s.batch_dev, 2 * dev_bytes) != cudaSuccess) {
+      cudaGetLastError();
+      s.batch_dev = nullptr;
+      return set_error(GOO_ERR_OOM, "goo_nll_grad_batch: work space");
+    }
+    s.batch_dev_cap = 2 * dev_bytes;
+  }
+  return GOO_OK;
+}
 
 static int arena_alloc(goo_server* s, size_t bytes, size_t* off) {
   bytes = al256(bytes);
@@ -1577,7 +1617,8 @@ int goo_server_step(goo_server* s, int* n_queued, int* n_active, int* n_done) {
       srv_nll_kernel<<<nb, kBlock, kSrvSmem, ctx->stream>>>(s->d_evals, s->d_tiles, s->d_fit_tiles, (int)s->ntiles,
                                                             s->opt.tile_events, s->d_model, s->d_tile_partials,
                                                             s->d_tickets, s->d_results, s->d_done_count + 1,
-                                                            ctx->wait_limit ? (long long)ctx->wait_limit : kWaitCycles);
+                                                            ctx->wait_limit ? (long long)ctx->wait_limit : kWaitCycles,
+                                                            nullptr);
     }
     GOO_CUDA_TRY(cudaGetLastError());
     {
@@ -1759,22 +1800,38 @@ int goo_nll_grad_batch(goo_model* m, int n_fits, const goo_dataset* const* ds, c
     return set_error(GOO_ERR_UNSUPPORTED, "goo_nll_grad_batch: needs <= %d resonances and a reference amplitude", kSrvKB);
   // one Gram matrix serves the batch: every fit must share the lineshape (non-coefficient)
   // parameters
-  for (int f = 1; f < n_fits; ++f)
-    for (int p = 0; p < P; ++p) {
-      bool coef = false;
-      for (int k = 0; k < info.K; ++k) coef = coef || p == info.par_re[k] || p == info.par_im[k];
-      if (!coef && theta[(size_t)f * P + p] != theta[p])
+  std::vector<char> is_coef(P, 0);
+  for (int k = 0; k < info.K; ++k) is_coef[info.par_re[k]] = is_coef[info.par_im[k]] = 1;
+  for (int p = 0; p < P; ++p) {
+    if (is_coef[p]) continue;
+    for (int f = 1; f < n_fits; ++f)
+      if (theta[(size_t)f * P + p] != theta[p])
         return set_error(GOO_ERR_ARG, "goo_nll_grad_batch: fit %d differs from fit 0 in lineshape parameter %d", f, p);
-    }
+  }
   const int T = 16384;
-  std::vector<SrvEval> ev(n_fits);
-  std::vector<int2> tiles, fit_tiles(n_fits);
+  size_t ntiles = 0;
+  for (int f = 0; f < n_fits; ++f) ntiles += (size_t)std::max<int64_t>(1, (ds[f]->n + T - 1) / T);
+  // The call's work space, kept by the context: what the kernel reads and what it expects zeroed is
+  // laid out in pinned host memory and goes up in one copy; the tiles' partial sums follow on
+  // the device only; the results come back through the pinned memory behind the upload.  64 toys: an
+  // allocation, eight copies and fills and a synchronise per toy cost 155 us beside the kernel's 118.
+  const size_t o_ev = 0, o_tiles = al256(o_ev + sizeof(SrvEval) * n_fits), o_ft = al256(o_tiles + sizeof(int2) * ntiles),
+               o_sm = al256(o_ft + sizeof(int2) * n_fits), o_tk = al256(o_sm + sizeof(SrvModel)),
+               o_res = al256(o_tk + sizeof(unsigned) * n_fits), o_status = o_res + sizeof(SrvResult) * n_fits,
+               up = al256(o_status + sizeof(unsigned)), bytes = up + sizeof(float2) * kSrvLanes * ntiles;
+  const int fields = n_fits * kSrvRecord;
+  GOO_TRY(ensure_batch(ctx, up + fields * sizeof(double), bytes));
+  unsigned char *h = ctx->scratch.batch_host, *w = ctx->scratch.batch_dev;
+  std::memset(h, 0, up);
+  double* res = (double*)(h + up);
+  arm_mapped(res, fields);
+  SrvEval* ev = (SrvEval*)(h + o_ev);
+  int2 *tiles = (int2*)(h + o_tiles), *fit_tiles = (int2*)(h + o_ft);
+  int nt_all = 0;
   for (int f = 0; f < n_fits; ++f) {
     const void* cache = nullptr;
-    int nres = 0;
-    GOO_TRY(dalitz_amplitudes(m, ds[f], theta + (size_t)f * P, GOO_F32, &cache, &nres));
+    GOO_TRY(dalitz_cache(m, ds[f], GOO_F32, &cache));  // every fit has dalitz_server_info's lineshapes
     SrvEval& e = ev[f];
-    std::memset(&e, 0, sizeof e);
     e.cache = (const float4*)cache;
     e.n = ds[f]->n;
     e.plane = ds[f]->n;
@@ -1785,86 +1842,48 @@ int goo_nll_grad_batch(goo_model* m, int n_fits, const goo_dataset* const* ds, c
     e.cr[kSrvKB] = (float)theta[(size_t)f * P + info.par_re[info.nbw]];
     e.ci[kSrvKB] = (float)theta[(size_t)f * P + info.par_im[info.nbw]];
     const int nt = (int)std::max<int64_t>(1, (e.n + T - 1) / T);
-    fit_tiles[f] = make_int2(nt, (int)tiles.size());
-    for (int t = 0; t < nt; ++t) tiles.push_back(make_int2(f, t));
+    fit_tiles[f] = make_int2(nt, nt_all);
+    for (int t = 0; t < nt; ++t) tiles[nt_all++] = make_int2(f, t);
   }
-  SrvModel sm{};
+  SrvModel& sm = *(SrvModel*)(h + o_sm);
   sm.nbw = info.nbw;
   sm.has_ref = 1;
-  std::vector<double> G(2 * info.K * info.K);
-  GOO_CUDA_TRY(cudaMemcpy(G.data(), info.gram_dev, G.size() * sizeof(double), cudaMemcpyDeviceToHost));
   auto slot_of = [&](int a) { return a < info.nbw ? a : kSrvKB; };
   for (int a = 0; a < info.K; ++a)
     for (int b = 0; b < info.K; ++b)
-      for (int c = 0; c < 2; ++c) sm.G[2 * (slot_of(a) * kSrvKA + slot_of(b)) + c] = G[2 * (a * info.K + b) + c];
-  // one allocation for the work space of this call
-  const size_t bytes = sizeof(SrvEval) * n_fits + sizeof(int2) * (tiles.size() + n_fits) + sizeof(SrvModel) +
-                       sizeof(SrvResult) * n_fits + sizeof(unsigned) * n_fits + sizeof(float2) * kSrvLanes * tiles.size() +
-                       sizeof(unsigned) + 9 * 256;
-  unsigned char* w = nullptr;
-  if (cudaMalloc(&w, bytes) != cudaSuccess) {
-    cudaGetLastError();
-    return set_error(GOO_ERR_OOM, "goo_nll_grad_batch: work space");
+      for (int c = 0; c < 2; ++c)
+        sm.G[2 * (slot_of(a) * kSrvKA + slot_of(b)) + c] = info.gram_host[2 * (a * info.K + b) + c];
+  GOO_CUDA_TRY(cudaMemcpyAsync(w, h, up, cudaMemcpyHostToDevice, ctx->stream));
+  GOO_CUDA_TRY(cudaFuncSetAttribute(srv_nll_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSrvSmem));
+  const int occ = cached_occupancy((const void*)srv_nll_kernel, ctx->device, kBlock, kSrvSmem);
+  const int nb = (int)std::min<size_t>(ntiles, (size_t)ctx->num_sms * occ);
+  {
+    LaunchScope ls(ctx, "srv_nll_grad");
+    srv_nll_kernel<<<nb, kBlock, kSrvSmem, ctx->stream>>>(
+        (const SrvEval*)(w + o_ev), (const int2*)(w + o_tiles), (const int2*)(w + o_ft), (int)ntiles, T,
+        (const SrvModel*)(w + o_sm), (float2*)(w + up), (unsigned*)(w + o_tk), (SrvResult*)(w + o_res),
+        (unsigned*)(w + o_status), ctx->wait_limit ? (long long)ctx->wait_limit : kWaitCycles, res);
   }
-  size_t o = 0;
-  auto take = [&](size_t b) {
-    unsigned char* p = w + o;
-    o = al256(o + b);
-    return p;
-  };
-  SrvEval* d_ev = (SrvEval*)take(sizeof(SrvEval) * n_fits);
-  int2* d_tiles = (int2*)take(sizeof(int2) * tiles.size());
-  int2* d_ft = (int2*)take(sizeof(int2) * n_fits);
-  SrvModel* d_sm = (SrvModel*)take(sizeof(SrvModel));
-  SrvResult* d_res = (SrvResult*)take(sizeof(SrvResult) * n_fits);
-  unsigned* d_tk = (unsigned*)take(sizeof(unsigned) * n_fits);
-  float2* d_part = (float2*)take(sizeof(float2) * kSrvLanes * tiles.size());
-  unsigned* d_status = (unsigned*)take(sizeof(unsigned));
-  int rc = GOO_OK;
-  unsigned status = 0;
-  std::vector<SrvResult> res(n_fits);
-  do {
-    if (cudaMemcpyAsync(d_ev, ev.data(), sizeof(SrvEval) * n_fits, cudaMemcpyHostToDevice, ctx->stream) ||
-        cudaMemcpyAsync(d_tiles, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice, ctx->stream) ||
-        cudaMemcpyAsync(d_ft, fit_tiles.data(), sizeof(int2) * n_fits, cudaMemcpyHostToDevice, ctx->stream) ||
-        cudaMemcpyAsync(d_sm, &sm, sizeof sm, cudaMemcpyHostToDevice, ctx->stream) ||
-        cudaMemsetAsync(d_res, 0, sizeof(SrvResult) * n_fits, ctx->stream) ||
-        cudaMemsetAsync(d_tk, 0, sizeof(unsigned) * n_fits, ctx->stream) ||
-        cudaMemsetAsync(d_status, 0, sizeof(unsigned), ctx->stream)) {
-      rc = set_error(GOO_ERR_CUDA, "goo_nll_grad_batch: copy failed");
-      break;
-    }
-    int occ = 0;
-    if (cudaFuncSetAttribute(srv_nll_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSrvSmem) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, srv_nll_kernel, kBlock, kSrvSmem) != cudaSuccess || occ < 1)
-      occ = 1;
-    cudaGetLastError();
-    const int nb = (int)std::min<size_t>(tiles.size(), (size_t)ctx->num_sms * occ);
-    {
-      LaunchScope ls(ctx, "srv_nll_grad");
-      srv_nll_kernel<<<nb, kBlock, kSrvSmem, ctx->stream>>>(d_ev, d_tiles, d_ft, (int)tiles.size(), T, d_sm, d_part, d_tk,
-                                                            d_res, d_status,
-                                                            ctx->wait_limit ? (long long)ctx->wait_limit : kWaitCycles);
-    }
-    if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpyAsync(res.data(), d_res, sizeof(SrvResult) * n_fits, cudaMemcpyDeviceToHost, ctx->stream) ||
-        cudaMemcpyAsync(&status, d_status, sizeof status, cudaMemcpyDeviceToHost, ctx->stream) ||
-        cudaStreamSynchronize(ctx->stream)) {
-      rc = set_error(GOO_ERR_CUDA, "goo_nll_grad_batch: kernel failed");
-      break;
-    }
-  } while (false);
-  cudaFree(w);
-  if (rc != GOO_OK) return rc;
-  if (status) return set_error(GOO_ERR_TIMEOUT, "goo_nll_grad_batch: a device wait for amplitude data gave up");
+  GOO_CUDA_TRY(cudaGetLastError());
+  std::vector<double> rec(fields);
+  const int rc = read_mapped(ctx, res, fields, rec.data());
+  if (rc != GOO_OK) {
+    // a fit without a result: a block whose wait gave up left its tiles out
+    unsigned status = 0;
+    GOO_CUDA_TRY(cudaMemcpyAsync(&status, w + o_status, sizeof status, cudaMemcpyDeviceToHost, ctx->stream));
+    GOO_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    if (status) return set_error(GOO_ERR_TIMEOUT, "goo_nll_grad_batch: a device wait for amplitude data gave up");
+    return rc;
+  }
   for (int f = 0; f < n_fits; ++f) {
+    const double* r = rec.data() + (size_t)f * kSrvRecord;
     double* g = grad_out + (size_t)f * P;
     for (int p = 0; p < P; ++p) g[p] = 0.0;
-    nll_out[f] = res[f].bad ? HUGE_VAL : res[f].nll;
+    nll_out[f] = r[0];
     for (int k = 0; k <= info.nbw; ++k) {
       const int sl = slot_of(k);
-      g[info.par_re[k]] = res[f].gre[sl];
-      g[info.par_im[k]] = res[f].gim[sl];
+      g[info.par_re[k]] = r[1 + 2 * sl];
+      g[info.par_im[k]] = r[2 + 2 * sl];
     }
   }
   return GOO_OK;
