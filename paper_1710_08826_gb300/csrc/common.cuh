@@ -483,22 +483,41 @@ __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.w
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------------------
-// Block reduction of `nslots` double-float lanes held per thread in `v[]` (compile-time
-// count NS, runtime count nslots <= NS).  Lane results of block b go to
-// partials[b * nslots + s].  Fixed order: warp xor-tree, then warps in index order.
+// Warp sums of NS double-float lanes by an exchanging butterfly: at each of the five levels a thread
+// keeps one half of its lanes and sends the other half to its partner, so that the warp performs
+// about NS + 5 additions per thread (5 NS when every lane runs its own tree: 95 against 21 for 19
+// lanes).  Afterwards the thread holds the sums of lanes first .. first + count - 1 in v[0 .. count).
+// Fixed order, so bitwise repeatable.
 // ---------------------------------------------------------------------------------------
+template <int C, int M, int NS>
+__device__ __forceinline__ void dd_warp_exchange(ddf (&v)[NS], int& first, int& count) {
+  if constexpr (M > 0) {
+    constexpr int H = (C + 1) / 2;  // lanes kept (the upper half may have one less)
+    const bool up = (threadIdx.x & M) != 0;
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      const ddf lo = v[j], hi = H + j < C ? v[H + j] : ddf{0.f, 0.f};
+      const ddf keep = up ? hi : lo, send = up ? lo : hi;
+      v[j] = dd_add(keep, dd_shfl_xor(send, M));
+    }
+    first += up ? H : 0;
+    count = up ? count - H : (count < H ? count : H);
+    dd_warp_exchange<H, M / 2, NS>(v, first, count);
+  }
+}
+
+// Block reduction of `nslots` = NS double-float lanes held per thread in `v[]`.  Lane results of block b
+// go to partials[b * nslots + s].  Fixed order: the warp exchange, then the warps in index order.
 template <int NS>
 __device__ __forceinline__ void block_reduce_to_partials(ddf (&v)[NS], int nslots, float2* partials,
-                                                         ddf* smem /* [kBlock/32][NS] */) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+                                                         ddf* smem /* [blockDim / 32][NS] */) {
+  const int warp = threadIdx.x >> 5;
   const int nwarps = blockDim.x >> 5;
+  int first = 0, count = NS;
+  dd_warp_exchange<NS, 16, NS>(v, first, count);
 #pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    if (s < nslots) {
-      ddf w = dd_warp_sum(v[s]);
-      if (lane == 0) smem[warp * NS + s] = w;
-    }
-  }
+  for (int j = 0; j < (NS + 31) / 32; ++j)
+    if (j < count) smem[warp * NS + first + j] = v[j];
   __syncthreads();
   if (threadIdx.x < nslots) {
     ddf acc = smem[threadIdx.x];

@@ -327,7 +327,8 @@ __global__ void __launch_bounds__(kBlock, 2)
 // tb0 + b, tb0 + b + gridDim.x, ...  Ragged first / last tiles are read from global memory.
 // Dynamic shared memory: kCohStages * n_planes * kCohTile float4.
 constexpr int kCohTile = kStagedBlock;  // one event per thread per tile
-constexpr int kCohStages = 3;
+template <int KB>
+constexpr int kCohStages = KB <= 8 ? 4 : 3;
 
 template <int KB, bool GRAD>
 __global__ void __launch_bounds__(kStagedBlock, 1) coh_nll_staged_kernel(const __grid_constant__ CohArgs<float> a,
@@ -337,7 +338,7 @@ __global__ void __launch_bounds__(kStagedBlock, 1) coh_nll_staged_kernel(const _
   constexpr int NS = CohLanes<float, KB, GRAD>::NS;
   constexpr int KA = KB + 1;
   constexpr int TE = kCohTile;
-  constexpr int NST = kCohStages;
+  constexpr int NST = kCohStages<KB>;
   __shared__ ddf s_red[(kStagedBlock / 32) * NS > kStagedBlock ? (kStagedBlock / 32) * NS : kStagedBlock];
   __shared__ unsigned s_bad[kStagedBlock / 32];
   __shared__ __align__(8) uint64_t s_bar[NST];
@@ -1280,12 +1281,12 @@ static int launch_coh_staged(goo_model* m, const void* cache, const goo_dataset*
   DalitzModel& d = *m->dalitz;
   goo_ctx* ctx = m->ctx;
   const int planes = (d.nbw + 1) / 2;
-  const size_t smem = (size_t)kCohStages * planes * kCohTile * sizeof(float4);
+  const size_t smem = (size_t)kCohStages<KB> * planes * kCohTile * sizeof(float4);
   static bool configured[kMaxDevicesCoh] = {};
   if (ctx->device < 0 || ctx->device >= kMaxDevicesCoh) return set_error(GOO_ERR_ARG, "device %d", ctx->device);
   if (!configured[ctx->device]) {
     GOO_CUDA_TRY(cudaFuncSetAttribute(coh_nll_staged_kernel<KB, GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((size_t)kCohStages * ((KB + 1) / 2) * kCohTile * sizeof(float4))));
+                                      (int)((size_t)kCohStages<KB> * ((KB + 1) / 2) * kCohTile * sizeof(float4))));
     configured[ctx->device] = true;
   }
   const int occ = cached_occupancy((const void*)coh_nll_staged_kernel<KB, GRAD>, ctx->device, kStagedBlock, smem);

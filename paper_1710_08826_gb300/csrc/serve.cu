@@ -457,12 +457,10 @@ __global__ void __launch_bounds__(kBlock, 2) srv_nll_kernel(const SrvEval* __res
     __syncthreads();  // s_red / s_bad reuse across tiles
     if ((threadIdx.x & 31) == 0) s_bad[threadIdx.x >> 5] = bad;
     {
-      const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-      for (int s = 0; s < kSrvLanes; ++s) {
-        const ddf w = dd_warp_sum(v[s]);
-        if (lane == 0) s_red[warp * kSrvLanes + s] = w;
-      }
+      static_assert(kSrvLanes <= 32, "one lane per thread after the exchange");
+      int first = 0, count = kSrvLanes;
+      dd_warp_exchange<kSrvLanes, 16, kSrvLanes>(v, first, count);
+      if (count > 0) s_red[(threadIdx.x >> 5) * kSrvLanes + first] = v[0];
       __syncthreads();
       if (threadIdx.x < kSrvLanes) {
         ddf a = s_red[threadIdx.x];
