@@ -475,6 +475,60 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, unsigned b
                : "memory");
 }
 
+// A ring of NST staged tiles that the warps of a block consume independently: a warp waits for
+// tile j's copies on its stage's mbarrier, and when it has read the tile counts itself done with the
+// stage; the warp that completes the count refills it with tile j + NST.  No block barrier separates
+// tiles, so a warp that is fast on one tile runs ahead on the next.
+template <int NST>
+struct TileRing {
+  uint64_t bar[NST];
+  unsigned done[NST];  // warps done with each stage's tile, counted over all its tiles
+  int last[NST];       // the last tile issued into each stage (-1: none)
+  unsigned fail;       // a warp's wait gave up
+  // thread 0; the caller then issues the first tiles and the block synchronises
+  __device__ __forceinline__ void init() {
+    for (int st = 0; st < NST; ++st) {
+      mbar_init(&bar[st], 1);
+      done[st] = 0u;
+      last[st] = -1;
+    }
+    fail = 0u;
+    mbar_init_fence();
+  }
+  // whether tile j arrived in time; the whole warp agrees
+  __device__ __forceinline__ bool wait(int j, long long limit) {
+    return __all_sync(0xffffffffu, mbar_wait(&bar[j % NST], (unsigned)(j / NST) & 1u, limit));
+  }
+  // the warp has read tile j: every warp's reads precede its count (block-scope fences around the
+  // shared atomic), and the refilling thread orders them before the asynchronous copies of issue(j + NST)
+  template <typename Issue>
+  __device__ __forceinline__ void release(int j, Issue issue) {
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) {
+      __threadfence_block();
+      if (atomicAdd(&done[j % NST], 1u) + 1u == (unsigned)(j / NST + 1) * (blockDim.x >> 5)) {
+        __threadfence_block();
+        fence_proxy_async();
+        issue(j + NST);
+      }
+    }
+  }
+  // every thread, after its last tile (gave_up: its warp's wait ran out): when some wait did, records it
+  // in the status word and waits, with the default limit, for the block's copies in flight
+  __device__ __forceinline__ void finish(bool gave_up, unsigned* counters) {
+    if (gave_up && (threadIdx.x & 31) == 0) atomicOr(&fail, 1u);
+    __syncthreads();
+    if (fail) {
+      if (threadIdx.x == 0) {
+        atomicOr(counters + kStatusWord, 1u);
+        for (int st = 0; st < NST; ++st)
+          if (last[st] >= 0) mbar_wait(&bar[st], (unsigned)(last[st] / NST) & 1u);
+      }
+      __syncthreads();
+    }
+  }
+};
+
 // Programmatic dependent launch: a kernel launched with the programmatic-serialisation
 // attribute may start while the previous kernel in the stream runs; grid_dep_wait() blocks
 // until that kernel has completed and its writes are visible.  grid_dep_launch() lets the

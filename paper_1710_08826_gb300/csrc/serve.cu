@@ -389,6 +389,9 @@ __global__ void __launch_bounds__(kBlock, 2) srv_nll_kernel(const SrvEval* __res
   __syncthreads();  // barriers initialised before any thread waits on them
   int j = 0;  // consumer job number
   bool failed = false;
+  float4 v4[NP];  // the event's planes; those the model lacks stay zero
+#pragma unroll
+  for (int p = 0; p < NP; ++p) v4[p] = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int t = blockIdx.x; t < ntiles && !failed; t += gridDim.x) {
     const int fit = tiles[t].x;
     const SrvEval& e = ev[fit];
@@ -416,16 +419,14 @@ __global__ void __launch_bounds__(kBlock, 2) srv_nll_kernel(const SrvEval* __res
       if (ok_wait) {
         const float4* sb = s_amp + (size_t)st * NP * TE;  // plane p at sb + p * TE
         for (int q = threadIdx.x; q < cnt; q += blockDim.x) {
-          float2 amp[kSrvKA];
+          float2 amp[kSrvKB];
 #pragma unroll
           for (int p = 0; p < NP; ++p) {
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (p < planes) v = sb[p * TE + q];
-            amp[2 * p] = make_float2(v.x, v.y);
-            amp[2 * p + 1] = make_float2(v.z, v.w);
+            if (p < planes) v4[p] = sb[p * TE + q];
+            amp[2 * p] = make_float2(v4[p].x, v4[p].y);
+            amp[2 * p + 1] = make_float2(v4[p].z, v4[p].w);
           }
-          amp[kSrvKB] = make_float2(1.f, 0.f);
-          coh_event_pk<kSrvKA, true>(cre, cim, amp, acc, G1, G2, bad);
+          coh_event_pk<kSrvKB, true>(cre, cim, amp, acc, G1, G2, bad);
         }
       }
       // every thread is done with buffer st (and agrees on whether a wait gave up) before

@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f32_kernel(const __grid_con
   constexpr int TE = kTdTile, NST = kTdStages;
   __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
   __shared__ unsigned s_bad[kBlock / 32];
-  __shared__ __align__(8) uint64_t s_bar[NST];
+  __shared__ __align__(8) TileRing<NST> s_ring;
   extern __shared__ __align__(128) float4 s_tile[];  // per stage: planes x TE float4, then TE float
   const int planes = a.planes;
   const int64_t n = a.n_total;
@@ -410,7 +410,8 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f32_kernel(const __grid_con
   auto issue = [&](int j) {
     const int64_t t = tile_of(j);
     if (t >= tb1) return;
-    uint64_t* bar = &s_bar[j % NST];
+    uint64_t* bar = &s_ring.bar[j % NST];
+    s_ring.last[j % NST] = j;
     float4* base = s_tile + (size_t)(j % NST) * stage_f4;
     if (full(t)) {
       mbar_arrive_expect_tx(bar, (unsigned)(planes * TE * sizeof(float4) + TE * sizeof(float)));
@@ -421,8 +422,7 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f32_kernel(const __grid_con
     }
   };
   if (threadIdx.x == 0) {
-    for (int st = 0; st < NST; ++st) mbar_init(&s_bar[st], 1);
-    mbar_init_fence();
+    s_ring.init();
     for (int j = 0; j < NST; ++j) issue(j);
   }
   TdAcc<float, KB> acc;
@@ -432,49 +432,36 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f32_kernel(const __grid_con
   for (int j = 0; j < 4; ++j) acc.lt[j] = 0.f;
   __syncthreads();  // barriers initialised before any thread waits on them
   const long long wlim = tile_wait_limit(counters);
-  int j = 0;
-  bool failed = false;
-  for (; tile_of(j) < tb1; ++j) {
-    const int64_t t = tile_of(j);
-    const int st = j % NST;
-    const bool ok_wait = mbar_wait(&s_bar[st], (unsigned)(j / NST) & 1u, wlim);
-    if (ok_wait) {
-      const float4* sb = s_tile + (size_t)st * stage_f4;
-      const float* stt = (const float*)(sb + (size_t)planes * TE);
-      const bool staged = full(t);
-      for (int e = threadIdx.x; e < TE; e += blockDim.x) {
-        const int64_t i = t * TE + e;
-        if (!staged && (i < begin || i >= end)) continue;
-        float2 am[KB];
+  // absent planes stay zero: only the model's planes are loaded over these
+  float4 v[KB / 2];
 #pragma unroll
-        for (int p = 0; p < KB / 2; ++p) {
-          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (p < planes) v = staged ? sb[(size_t)p * TE + e] : __ldg(cache + (int64_t)p * n + i);
-          am[2 * p] = make_float2(v.x, v.y);
-          am[2 * p + 1] = make_float2(v.z, v.w);
-        }
-        const float tv = staged ? stt[e] : __ldg(tcol + i);
-        td4_event_f32<KB, GRAD>(a, am, tv, acc);
-      }
-    }
-    if (__syncthreads_or(!ok_wait)) {
-      failed = true;
+  for (int p = 0; p < KB / 2; ++p) v[p] = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto event = [&](float tv) {
+    float2 am[KB];
+#pragma unroll
+    for (int k = 0; k < KB; ++k) am[k] = (k & 1) ? make_float2(v[k / 2].z, v[k / 2].w) : make_float2(v[k / 2].x, v[k / 2].y);
+    td4_event_f32<KB, GRAD>(a, am, tv, acc);
+  };
+  bool gave_up = false;
+  for (int j = 0; tile_of(j) < tb1; ++j) {
+    const int64_t t = tile_of(j);
+    if (!s_ring.wait(j, wlim)) {
+      gave_up = true;
       break;
     }
-    if (threadIdx.x == 0) {
-      fence_proxy_async();
-      issue(j + NST);
+    const bool staged = full(t);
+    const int64_t i = t * TE + threadIdx.x;
+    if (staged || (i >= begin && i < end)) {
+      const float4* sb = s_tile + (size_t)(j % NST) * stage_f4 + threadIdx.x;
+#pragma unroll
+      for (int p = 0; p < KB / 2; ++p)
+        if (p < planes) v[p] = staged ? sb[(size_t)p * TE] : __ldg(cache + (int64_t)p * n + i);
+      event(staged ? reinterpret_cast<const float*>(s_tile + (size_t)(j % NST) * stage_f4 + (size_t)planes * TE)[threadIdx.x]
+                   : __ldg(tcol + i));
     }
+    s_ring.release(j, issue);
   }
-  if (failed) {
-    // a copy did not arrive in time: record it, then wait (again bounded) for this block's
-    // copies still in flight before the block's shared memory is released
-    if (threadIdx.x == 0) {
-      atomicOr(counters + kStatusWord, 1u);
-      for (int jj = j; jj < j + NST && tile_of(jj) < tb1; ++jj) mbar_wait(&s_bar[jj % NST], (unsigned)(jj / NST) & 1u);
-    }
-    __syncthreads();
-  }
+  s_ring.finish(gave_up, counters);
   td4_finish<float, KB, GRAD>(a, acc, begin, end, partials, counters, result, out_mode, s_red, s_bad);
 }
 
