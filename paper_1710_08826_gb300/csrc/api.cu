@@ -55,7 +55,7 @@ int nll_common(goo_model* m, const goo_dataset* ds, const double* theta, int pre
   } else if (m->kind == 2) {
     GOO_TRY(td4_nll(m, ds, 0, ds->n, theta, precision, grad, res, 0));
   } else {
-    const bool fuse = ds->n > 0 && !ds->w64 && sop_norm_in_event(m, precision, grad);
+    const bool fuse = ds->n > 0 && sop_norm_in_event(m, precision, grad);
     GOO_TRY(sop_prepare(m, theta, precision, fuse));
     arm_result_mapped(ctx);
     if (ds->n > 0) GOO_TRY(sop_events(m, ds, 0, ds->n, precision, grad, 0, fuse, ctx->scratch.result_host));
@@ -231,7 +231,7 @@ int goo_nll_partial(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t 
   } else if (m->kind == 1) {
     GOO_TRY(dalitz_nll(m, ds, begin, end, theta, precision, want_grad != 0, res, 1));
   } else {
-    const bool fuse = end > begin && !ds->w64 && sop_norm_in_event(m, precision, want_grad != 0);
+    const bool fuse = end > begin && sop_norm_in_event(m, precision, want_grad != 0);
     GOO_TRY(sop_prepare(m, theta, precision, fuse));
     if (end > begin) {
       arm_result_mapped(ctx);
@@ -292,7 +292,7 @@ int goo_model_set_jit(goo_model* m, int mode) {
   if (mode != 0 && mode != 1) return set_error(GOO_ERR_ARG, "goo_model_set_jit: mode=%d", mode);
   m->jit_mode = mode;
   m->jit_status = mode;
-  m->ev2_fn[0] = m->ev2_fn[1] = m->ev2_fn[2] = m->ev2_fn[3] = nullptr;
+  for (const void*& f : m->ev2_fn) f = nullptr;
   return GOO_OK;
 }
 

@@ -15,6 +15,7 @@ struct LeafDev {
   float f[6];          // FP32 constants (offsets as hi/lo pairs)
   double d[6];         // FP64 constants
   double a_ref;        // grid reference exponent of this leaf (upper bound of a over its range)
+  double dlog[3];      // ANALYTIC: d log N / d par_j of this leaf's closed-form integral
   float a_ref_hi, a_ref_lo;
 };
 
@@ -63,7 +64,8 @@ int sop_set_norm(goo_model* m, const goo_norm_spec* spec);
 // Uploads the prepared model block and launches the grid normalisation, unless norm_in_event
 // (sop_norm_in_event true, and the following sop_events call passes it too).
 int sop_prepare(goo_model* m, const double* theta_host, int precision, bool norm_in_event = false);
-// True when the FP32 event kernel for this model normalises a separable grid itself.
+// True when the FP32 event kernel for this model takes its normalisation by value (closed forms) or
+// normalises a separable grid itself.
 bool sop_norm_in_event(const goo_model* m, int precision, bool grad);
 void host_prep(ModelDev& h, const double* theta, int precision);
 // result: the record's destination (kResultDoubles + 1 doubles; null: the context's device
@@ -126,9 +128,9 @@ struct goo_model {
   // the packed-pair event kernel resolved for this model (index: gradient form) and the
   // jit_status it came with; reset by goo_model_set_jit
   // the pair kernel per gradient form (index gi) and column source (+2: host columns read
-  // directly), resolved on first use
-  const void* ev2_fn[4] = {nullptr, nullptr, nullptr, nullptr};
-  int ev2_status[4] = {0, 0, 0, 0};
+  // directly, +4: weighted), resolved on first use
+  const void* ev2_fn[6] = {};
+  int ev2_status[6] = {};
 };
 
 namespace goo {

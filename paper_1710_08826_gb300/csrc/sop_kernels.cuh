@@ -52,6 +52,7 @@ __host__ __device__ constexpr int leaf_nder(int op) {
 template <typename T>
 struct Cols {
   const T* c[kMaxObs];
+  const T* w;  // the pair kernel's weighted form: per-event weights
   // for the pair kernel's direct form (a GOO_BORROW_HOST dataset: c are device-mapped host
   // columns, read straight into registers): the float limits that admit exactly the values
   // inside the double limits
@@ -306,6 +307,10 @@ struct EvNorm {
   float lo_hi[K * L], lo_lo[K * L], h_hi[K * L], h_lo[K * L], aref_hi[K * L], aref_lo[K * L];
   double h64[K * L];
   int nb[K * L];                                   // bins (0: no leaf in the slot)
+  // closed-form normalisation: -log N_k and the leaves' d log N / d par_j, instead of the grid
+  int analytic;
+  float off_hi[K], off_lo[K];
+  double dlog[K * L][3];
   double w[K];                                     // w_k
   int n_params;
   signed char par[K][L][3];                        // parameter of leaf constant j (-1: none)
@@ -427,7 +432,7 @@ struct EventOcc {
   static constexpr int value = (sizeof(T) == 4 && K * L <= 6) ? 3 : 2;
 };
 
-// The scalar kernel: weighted FP32 datasets, FP32 shapes the pair kernel does not take, and both precisions
+// The scalar kernel: FP32 shapes the pair kernel does not take, and both precisions
 // of goo_nll_grad_static (whose calls have no context to keep the FP64 function tables of the
 // faster sop_event64_kernel in).
 // wcol (nullable): per-event weights w_i (a binned dataset: bin centres with their counts);
@@ -886,7 +891,9 @@ __device__ __forceinline__ void event_finish_fused(const ddf (&v)[EventLanes<flo
     // quotient in double-float, then FP64)
     for (int t = threadIdx.x; t < K * L * 3; t += blockDim.x) {
       const int sl = t / 3, jj = t % 3;
-      s_t[sl][jj] = N.nb[sl] ? dd_to_double(dd_div(s_raw[sl][1 + jj], s_raw[sl][0])) : 0.0;
+      s_t[sl][jj] = N.analytic ? N.dlog[sl][jj]
+                    : N.nb[sl] ? dd_to_double(dd_div(s_raw[sl][1 + jj], s_raw[sl][0]))
+                               : 0.0;
     }
   }
   reduce_partials<24>(partials, NS, gridDim.x, s_out, s_red, blockDim.x);
@@ -953,18 +960,30 @@ struct PairAcc {
   unsigned bad;
 };
 
-// One event pair: evaluate and accumulate the lanes that are in range (v0, v1) with f > 0.
-template <int K, int L, bool GRAD, unsigned long long SIG = 0>
+// One event pair: evaluate and accumulate the lanes that are in range (v0, v1) with f > 0, each
+// times its weight w when WEIGHTED (an event of weight 0 may have f = 0).
+template <int K, int L, bool GRAD, unsigned long long SIG = 0, bool WEIGHTED = false>
 __device__ __forceinline__ void pair_step(const EvConst<float, K, L>& P, const float (&off_hi)[K],
                                           const float (&off_lo)[K], const float2 (&xl)[K][L], bool v0, bool v1,
-                                          PairAcc<K, L>& S) {
+                                          float2 w, PairAcc<K, L>& S) {
   float2 logf, ck[K], qk[K], dk[K][L][3];
   bool ok0, ok1;
   eval_event2<K, L, GRAD, SIG>(P, off_hi, off_lo, xl, logf, ok0, ok1, ck, qk, dk);
   const bool m0 = v0 && ok0, m1 = v1 && ok1;
-  S.bad += (unsigned)(v0 && !ok0) + (unsigned)(v1 && !ok1);
+  S.bad += (unsigned)(v0 && !ok0 && (!WEIGHTED || w.x != 0.f)) + (unsigned)(v1 && !ok1 && (!WEIGHTED || w.y != 0.f));
+  if constexpr (WEIGHTED && GRAD) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      ck[k] = pk::mul(ck[k], w);
+      qk[k] = sig_product_poly_q(SIG, k, L) ? pk::mul(qk[k], w) : ck[k];
+    }
+  }
+  if (WEIGHTED) {
+    // compensated pair by pair: weighted terms vary in size more than a tile's log2 f do
+    S.lf.add(make_float2(m0 ? w.x * logf.x : 0.f, m1 ? w.y * logf.y : 0.f));
+  }
   if (m0 && m1) {
-    S.lt = pk::add(S.lt, logf);
+    if (!WEIGHTED) S.lt = pk::add(S.lt, logf);
     if constexpr (GRAD) {
 #pragma unroll
       for (int k = 0; k < K; ++k) {
@@ -982,7 +1001,7 @@ __device__ __forceinline__ void pair_step(const EvConst<float, K, L>& P, const f
 #pragma unroll
     for (int lane = 0; lane < 2; ++lane) {
       if (!(lane ? m1 : m0)) continue;
-      (lane ? S.lt.y : S.lt.x) += lane ? logf.y : logf.x;
+      if (!WEIGHTED) (lane ? S.lt.y : S.lt.x) += lane ? logf.y : logf.x;
       if constexpr (GRAD) {
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -1023,11 +1042,14 @@ __host__ __device__ constexpr int cols_col(unsigned long long cols, int slot) { 
 // warp that completes the count refills the buffer with the tile kEventStages ahead.  No
 // block barrier separates tiles, so a warp that is fast on one tile runs ahead on the next
 // instead of waiting for the slowest warp.
-// Dynamic shared memory: kEventStages * n_obs * TE floats.
-template <int K, int L, bool GRAD, unsigned long long SIG = 0, unsigned long long COLS = 0, bool DIRECT = false>
+// WEIGHTED (the interpreter only: a fit's evaluations would not pay for a compilation): the
+// weights are staged as one more column behind the observables.
+// Dynamic shared memory: kEventStages * n_obs (+ 1 when weighted) * TE floats.
+template <int K, int L, bool GRAD, unsigned long long SIG = 0, unsigned long long COLS = 0, bool DIRECT = false,
+          bool WEIGHTED = false>
 __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
     sop_event2_kernel(const ModelDev* __restrict__ md, const EvConst<float, K, L> P,
-                      const __grid_constant__ EvNorm<K, L, GRAD> N, Cols<float> cols, int64_t begin, int64_t end,
+                      const __grid_constant__ EvNorm<K, L, GRAD> N, const __grid_constant__ Cols<float> cols, int64_t begin, int64_t end,
                       float2* partials, unsigned* counters, double* result, int out_mode, int fused_norm) {
   using namespace pk;
   constexpr int NS = EventLanes<float, K, L, GRAD, SIG>::NS;
@@ -1045,6 +1067,8 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
   __shared__ float s_off[K][2];
   extern __shared__ __align__(128) float s_col[];  // [NST][nobs][TE]
   const int nobs = P.nobs;
+  const int ncol = nobs + (WEIGHTED ? 1 : 0);
+  auto column = [&](int c) { return WEIGHTED && c == nobs ? cols.w : cols.c[c]; };
   const int lane = threadIdx.x & 31;
   const int64_t A = min(end, (begin + 7) & ~(int64_t)7);
   const int64_t B = max(A, end & ~(int64_t)7);
@@ -1052,7 +1076,7 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
   const int64_t r0 = min(B, A + (int64_t)blockIdx.x * chunk), r1 = min(B, r0 + chunk);
   const int ntile = (int)((r1 - r0 + TE - 1) / TE);
   auto tile_count = [&](int j) { return (int)min((int64_t)TE, r1 - (r0 + (int64_t)j * TE)); };
-  auto buf = [&](int st, int c) { return s_col + ((size_t)st * nobs + c) * TE; };
+  auto buf = [&](int st, int c) { return s_col + ((size_t)st * ncol + c) * TE; };
   const unsigned withhold = withheld_tile(counters);
   // one thread stages tile j in buffer j % NST (a withheld tile's copies are never issued, so
   // its waits run out: the failure-detection test hook)
@@ -1062,8 +1086,8 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
     const unsigned bytes = (unsigned)tile_count(j) * (unsigned)sizeof(float);
     const int64_t t0 = r0 + (int64_t)j * TE;
     s_last[st] = j;
-    mbar_arrive_expect_tx(&s_bar[st], (unsigned)nobs * bytes);
-    for (int c = 0; c < nobs; ++c) bulk_load(buf(st, c), cols.c[c] + t0, bytes, &s_bar[st]);
+    mbar_arrive_expect_tx(&s_bar[st], (unsigned)ncol * bytes);
+    for (int c = 0; c < ncol; ++c) bulk_load(buf(st, c), column(c) + t0, bytes, &s_bar[st]);
   };
   // DIRECT (a GOO_BORROW_HOST dataset): the columns are read straight from host memory, so
   // no copies are staged; a separate instantiation, so that the staged kernel carries none of
@@ -1084,14 +1108,14 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
       for (int j = 0; j < NST && j < ntile && !direct; ++j) {
         if (withhold && j == (int)withhold - 1) continue;
         s_last[j] = j;
-        mbar_arrive_expect_tx(&s_bar[j], (unsigned)nobs * (unsigned)tile_count(j) * (unsigned)sizeof(float));
+        mbar_arrive_expect_tx(&s_bar[j], (unsigned)ncol * (unsigned)tile_count(j) * (unsigned)sizeof(float));
       }
     }
     __syncwarp();
-    for (int q = lane; q < NST * nobs && !direct; q += 32) {
-      const int j = q / nobs, c = q % nobs;
+    for (int q = lane; q < NST * ncol && !direct; q += 32) {
+      const int j = q / ncol, c = q % ncol;
       if (j < ntile && !(withhold && j == (int)withhold - 1))
-        bulk_load(buf(j, c), cols.c[c] + r0 + (int64_t)j * TE, (unsigned)tile_count(j) * (unsigned)sizeof(float),
+        bulk_load(buf(j, c), column(c) + r0 + (int64_t)j * TE, (unsigned)tile_count(j) * (unsigned)sizeof(float),
                   &s_bar[j]);
     }
   }
@@ -1100,7 +1124,14 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
   grid_dep_wait();
   float off_hi[K], off_lo[K];
   const int nK = P.nK;
-  if (fused_norm) {
+  if (fused_norm && N.analytic) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      off_hi[k] = N.off_hi[k];
+      off_lo[k] = N.off_lo[k];
+    }
+    __syncthreads();  // barriers initialised before any thread waits on them
+  } else if (fused_norm) {
     fused_grid_norm<K, L, GRAD>(P, N, s_raw, s_off, off_hi, off_lo);  // synchronises the block
   } else {
     load_offsets<float, K>(md, off_hi, off_lo);
@@ -1171,7 +1202,7 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
 #pragma unroll
     for (int k = 0; k < K; ++k)
 #pragma unroll
-      for (int l = 0; l < L; ++l) coff[k][l] = (st * nobs + leaf_col(k, l)) * TE;
+      for (int l = 0; l < L; ++l) coff[k][l] = (st * ncol + leaf_col(k, l)) * TE;
 #pragma unroll 1
     for (int u = 0; u < PPT; ++u) {
       const int pr = threadIdx.x + u * kBlock;
@@ -1183,7 +1214,8 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
       for (int k = 0; k < K; ++k)
 #pragma unroll
         for (int l = 0; l < L; ++l) xl[k][l] = reinterpret_cast<const float2*>(s_col + coff[k][l])[pr];
-      pair_step<K, L, GRAD, SIG>(P, off_hi, off_lo, xl, true, true, S);
+      const float2 w = WEIGHTED ? reinterpret_cast<const float2*>(buf(st, nobs))[pr] : splat(1.f);
+      pair_step<K, L, GRAD, SIG, WEIGHTED>(P, off_hi, off_lo, xl, true, true, w, S);
     }
     S.lf.add(S.lt);
     S.lt = splat(0.f);
@@ -1221,12 +1253,14 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
       }
     }
     if (direct) nout += (v0 && !ok0 ? 1u : 0u) + (v1 && !ok1 ? 1u : 0u);
+    float2 w = splat(1.f);
+    if (WEIGHTED) w = make_float2(v0 ? cols.w[i] : 0.f, v1 ? cols.w[i + 1] : 0.f);
     float2 xl[K][L];
 #pragma unroll
     for (int k = 0; k < K; ++k)
 #pragma unroll
       for (int l = 0; l < L; ++l) xl[k][l] = pk::pick(leaf_col(k, l), x[0], x[1], x[2], x[3]);
-    pair_step<K, L, GRAD, SIG>(P, off_hi, off_lo, xl, v0, v1, S);
+    pair_step<K, L, GRAD, SIG, WEIGHTED>(P, off_hi, off_lo, xl, v0, v1, w, S);
   };
   if (!failed) {
     if (blockIdx.x == 0 && A > begin) ragged(begin, A);

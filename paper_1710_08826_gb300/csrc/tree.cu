@@ -187,6 +187,9 @@ void host_prep(ModelDev& h, const double* theta, int precision) {
       }
       dlog_leaf[t][0] = g0;
       dlog_leaf[t][1] = g1;
+      L.dlog[0] = g0;
+      L.dlog[1] = g1;
+      L.dlog[2] = 0.0;
       L.a_ref = amax_leaf[t];
       L.a_ref_hi = (float)amax_leaf[t];
       L.a_ref_lo = (float)(amax_leaf[t] - (double)L.a_ref_hi);
@@ -828,8 +831,9 @@ constexpr int kFusedNormBins = 4096;
 
 bool sop_norm_in_event(const goo_model* m, int precision, bool grad) {
   const ModelDev& h = m->host;
-  if (precision != GOO_F32 || h.norm_kind != GOO_NORM_GRID || !h.grid_separable) return false;
+  if (precision != GOO_F32 || (h.norm_kind == GOO_NORM_GRID && !h.grid_separable)) return false;
   if (grad && !(h.nK <= 2 && m->max_leaf <= 3)) return false;  // the scalar kernel takes that shape
+  if (h.norm_kind == GOO_NORM_ANALYTIC) return true;
   int64_t bins = 0;
   for (int k = 0; k < h.nK; ++k)
     for (int l = 0; l < h.comp[k].n_leaf; ++l) {
@@ -891,7 +895,7 @@ static EvConst<T, K, L> make_evconst(const ModelDev& h) {
   return P;
 }
 
-// The scalar FP32 kernel: weighted datasets, and the shapes the pair kernel does not take.
+// The scalar FP32 kernel: the shapes the pair kernel does not take.
 template <int K, int L, bool GRAD>
 static int launch_event_f32(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, int out_mode,
                             double* result) {
@@ -954,13 +958,21 @@ template <int K, int L, bool GRAD>
 static EvNorm<K, L, GRAD> make_evnorm(const ModelDev& h) {
   EvNorm<K, L, GRAD> N;
   std::memset(&N, 0, sizeof N);
+  N.analytic = h.norm_kind == GOO_NORM_ANALYTIC;
   for (int k = 0; k < K; ++k) {
     N.w[k] = k < h.nK ? h.comp[k].w : 0.0;
+    N.off_hi[k] = k < h.nK ? h.comp[k].off_hi : 0.f;
+    N.off_lo[k] = k < h.nK ? h.comp[k].off_lo : 0.f;
     for (int l = 0; l < L; ++l) {
       const int sl = k * L + l;
       for (int j = 0; j < 3; ++j) N.par[k][l][j] = -1;
       if (k >= h.nK || l >= h.comp[k].n_leaf) continue;
       const LeafDev& LD = h.leaf[k * kMaxLeaf + l];
+      for (int j = 0; j < 3; ++j) {
+        N.par[k][l][j] = (signed char)LD.par[j];
+        N.dlog[sl][j] = LD.dlog[j];
+      }
+      if (N.analytic) continue;
       const GridDev& G = h.grid[k];
       const int d = G.dim_of_col[LD.col];
       N.nb[sl] = G.bins[d];
@@ -971,7 +983,6 @@ static EvNorm<K, L, GRAD> make_evnorm(const ModelDev& h) {
       N.h64[sl] = G.h64[d];
       N.aref_hi[sl] = LD.a_ref_hi;
       N.aref_lo[sl] = LD.a_ref_lo;
-      for (int j = 0; j < 3; ++j) N.par[k][l][j] = (signed char)LD.par[j];
     }
   }
   N.n_params = h.n_params;
@@ -989,22 +1000,25 @@ static int launch_event2(goo_model* m, const goo_dataset* ds, int64_t begin, int
   // the column tiles, and room for the final block reduction (event_finish_fused), which reuses
   // the tile buffers: every lane of every thread as a double-float
   constexpr size_t red_bytes = (size_t)EventLanes<float, K, L, GRAD>::NS * kBlock * sizeof(ddf);
-  const size_t smem = std::max((size_t)kEventStages * m->host.n_obs * TE * sizeof(float), red_bytes);
+  const bool direct = ds->host_borrowed, weighted = ds->w32 != nullptr;
+  const size_t smem = std::max((size_t)kEventStages * (m->host.n_obs + (weighted ? 1 : 0)) * TE * sizeof(float), red_bytes);
   // room for the largest column count, so one setting serves every model on this device
-  const size_t smem_max = std::max((size_t)kEventStages * kMaxObs * TE * sizeof(float), red_bytes);
-  static bool configured[kMaxDevicesEv][2] = {};
+  const size_t smem_max = std::max((size_t)kEventStages * (kMaxObs + (weighted ? 1 : 0)) * TE * sizeof(float), red_bytes);
+  static bool configured[kMaxDevicesEv][3] = {};
   if (ctx->device < 0 || ctx->device >= kMaxDevicesEv) return set_error(GOO_ERR_ARG, "device %d", ctx->device);
   // the kernel for this model, gradient form and column source, resolved on its first
   // evaluation: the one specialised for the model's leaf signature (jit.cu), else the
-  // interpreter; host columns (GOO_BORROW_HOST) take the direct-read instantiation
-  const bool direct = ds->host_borrowed;
-  const int gi = (GRAD ? 1 : 0) + (direct ? 2 : 0);
+  // interpreter; host columns (GOO_BORROW_HOST) take the direct-read instantiation, weighted
+  // datasets the interpreter's weighted one
+  const int form = direct ? 1 : weighted ? 2 : 0;
+  const int gi = (GRAD ? 1 : 0) + 2 * form;
   if (!m->ev2_fn[gi]) {
-    const void* interp = direct ? (const void*)sop_event2_kernel<K, L, GRAD, 0, 0, true>
-                                : (const void*)sop_event2_kernel<K, L, GRAD>;
+    const void* interp = direct     ? (const void*)sop_event2_kernel<K, L, GRAD, 0, 0, true>
+                         : weighted ? (const void*)sop_event2_kernel<K, L, GRAD, 0, 0, false, true>
+                                    : (const void*)sop_event2_kernel<K, L, GRAD>;
     const void* fn = interp;
     int st = m->jit_mode;
-    if (m->jit_mode) {
+    if (m->jit_mode && !weighted) {
       unsigned long long sig = 0, colmap = 0;
       for (int k = 0; k < m->host.nK && k < K; ++k)
         for (int l = 0; l < m->host.comp[k].n_leaf && l < L; ++l) {
@@ -1015,15 +1029,15 @@ static int launch_event2(goo_model* m, const goo_dataset* ds, int64_t begin, int
       const void* jf = jit_event2_kernel(ctx->device, K, L, GRAD, sig, colmap, direct, smem_max, &st);
       if (jf) fn = jf;
     }
-    if (fn == interp && !configured[ctx->device][direct ? 1 : 0]) {
+    if (fn == interp && !configured[ctx->device][form]) {
       GOO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max));
-      configured[ctx->device][direct ? 1 : 0] = true;
+      configured[ctx->device][form] = true;
     }
     m->ev2_fn[gi] = fn;
     m->ev2_status[gi] = st;
   }
   const void* fn = m->ev2_fn[gi];
-  m->jit_status = m->ev2_status[gi];
+  if (!weighted) m->jit_status = m->ev2_status[gi];  // a weighted evaluation leaves it as it is
   const int bps = cached_occupancy(fn, ctx->device, kBlock, smem);
   // every block takes an equal contiguous share of the events (sop_event2_kernel), at most
   // one tile's worth when the range is small
@@ -1033,6 +1047,7 @@ static int launch_event2(goo_model* m, const goo_dataset* ds, int64_t begin, int
   GOO_TRY(ensure_partials(ctx, (size_t)nb * NS));
   Cols<float> cols{};
   for (int c = 0; c < kMaxObs; ++c) cols.c[c] = ds->d32[c < ds->ncols ? c : 0];
+  cols.w = ds->w32;
   if (ds->host_borrowed) {
     // read over the host link by the kernel itself, each value checked against the float
     // limits that admit exactly the float values inside the double limits
@@ -1082,12 +1097,10 @@ static int launch_event_sel(goo_model* m, const goo_dataset* ds, int64_t begin, 
                             bool fused_norm, double* result) {
   if constexpr (sizeof(T) == 4) {
     // packed pairs, except the largest shape with gradient lanes (its pair accumulators do
-    // not fit in registers) and weighted datasets (the scalar kernel carries the weights)
-    if (!ds->w32) {
-      if (m->host.nK <= 2 && m->max_leaf <= 3)
-        return launch_event2<2, 3, GRAD>(m, ds, begin, end, out_mode, fused_norm, result);
-      if constexpr (!GRAD) return launch_event2<4, 4, GRAD>(m, ds, begin, end, out_mode, fused_norm, result);
-    }
+    // not fit in registers)
+    if (m->host.nK <= 2 && m->max_leaf <= 3)
+      return launch_event2<2, 3, GRAD>(m, ds, begin, end, out_mode, fused_norm, result);
+    if constexpr (!GRAD) return launch_event2<4, 4, GRAD>(m, ds, begin, end, out_mode, fused_norm, result);
   }
   if (ds->host_borrowed)
     return set_error(GOO_ERR_UNSUPPORTED, "a GOO_BORROW_HOST dataset is read by the packed-pair FP32 kernel only "
