@@ -603,6 +603,35 @@ __device__ __forceinline__ void block_reduce_transpose(const ddf (&v)[NS], float
   if (s < NS && g == 0) partials[(size_t)blockIdx.x * NS + s] = make_float2(acc.hi, acc.lo);
 }
 
+// Which of N gradient terms belong to each parameter, as lists threaded through the terms in their
+// order (host-built, passed by value): in the final FP64 combination one thread forms one term and
+// one thread per parameter adds its own few, where a thread that ran over every term for its
+// parameter kept the last block busy for one to two microseconds (an FP64 instruction takes a
+// warp 64 cycles).
+template <int N>
+struct GradMap {
+  static_assert(N <= 127, "terms are numbered in a signed char");
+  signed char head[kMaxParams];  // first term of the parameter (-1: none)
+  signed char next[N > 0 ? N : 1];
+#ifndef __CUDACC_RTC__
+  __host__ void clear() {
+    for (int p = 0; p < kMaxParams; ++p) head[p] = -1;
+    for (int t = 0; t < N; ++t) next[t] = -1;
+  }
+  // terms are added in descending order, so that each list runs upwards
+  __host__ void add(int t, int p) {
+    if (p < 0) return;
+    next[t] = head[p];
+    head[p] = (signed char)t;
+  }
+#endif
+  __device__ __forceinline__ double gather(int p, const double* terms) const {
+    double g = 0.0;
+    for (int t = head[p]; t >= 0; t = next[t]) g += terms[t];
+    return g;
+  }
+};
+
 // Completion word of a result record (kResultFlag): every thread of the last block calls
 // this after its last write to `result`; thread 0 sets the word.  A host that polls a mapped
 // record watches its fields (kResultSentinel), so no system-scope fence is needed here (one

@@ -131,7 +131,8 @@ template <typename T>
 struct CohArgs {
   T cr[kMaxAmp], ci[kMaxAmp];  // coefficients (BWs first, then NR)
   int nbw, K, has_nr;
-  int par_re[kMaxAmp], par_im[kMaxAmp];
+  GradMap<4 * kMaxAmp> map;    // terms 2k, 2k + 1: amplitude k's two coefficient parameters; floating
+                               // lineshapes: 2K + 2k, + 1: resonance k's mass and width
   int n_params;
   int64_t n_total;             // events of the dataset (cache plane length)
   int polar;                   // the coefficient parameters are (r, phi): c = r e^{i phi}
@@ -207,19 +208,22 @@ __device__ __forceinline__ void coh_finish(const CohArgs<T>& a, CohAcc<T, KB>& a
   const int K = a.K;
   const int P = a.n_params;
   const int off = out_mode == 0 ? 2 : 3;
-  // thread p gathers the gradient of parameter p (parameters may be shared) in a fixed order
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    double g = 0.0;
-    if (GRAD)
-      for (int k = 0; k < K; ++k) {
-        const int slot = (k < a.nbw) ? k : KB;  // NR lives in the last slot
-        double gre = -2.0 * s_out[1 + 2 * slot] + nev * a.nrm_vr[k];
-        double gim = 2.0 * s_out[2 + 2 * slot] - nev * a.nrm_vi[k];
-        coef_chain(a.polar, a.jc[k], a.js[k], a.jr[k], gre, gim);
-        if (a.par_re[k] == p) g += gre;
-        if (a.par_im[k] == p) g += gim;
-      }
-    result[off + p] = g;
+  // one thread per amplitude forms its two terms, then one per parameter gathers (GradMap)
+  if constexpr (GRAD) {
+    __shared__ double s_term[2 * kMaxAmp];
+    if ((int)threadIdx.x < K) {
+      const int k = threadIdx.x;
+      const int slot = (k < a.nbw) ? k : KB;  // NR lives in the last slot
+      double gre = fma(nev, a.nrm_vr[k], -2.0 * s_out[1 + 2 * slot]);
+      double gim = fma(-nev, a.nrm_vi[k], 2.0 * s_out[2 + 2 * slot]);
+      coef_chain(a.polar, a.jc[k], a.js[k], a.jr[k], gre, gim);
+      s_term[2 * k] = gre;
+      s_term[2 * k + 1] = gim;
+    }
+    __syncthreads();
+    for (int p = threadIdx.x; p < P; p += blockDim.x) result[off + p] = a.map.gather(p, s_term);
+  } else {
+    for (int p = threadIdx.x; p < P; p += blockDim.x) result[off + p] = 0.0;
   }
   if (threadIdx.x == 0) {
     counters[1] = 0u;
@@ -548,7 +552,6 @@ struct LsConst {
   T cr[kMaxAmp], ci[kMaxAmp];          // coefficients by slot: resonances, then the NR in slot KB
   T ncr[kMaxAmp], nci[kMaxAmp];        // minus these
   double rho[kMaxAmp], kappa[kMaxAmp], two_m0[kMaxAmp], inv_g0[kMaxAmp];
-  int par_m0[kMaxAmp], par_w[kMaxAmp];
 };
 
 template <int KB, bool GRAD>
@@ -741,27 +744,28 @@ __global__ void __launch_bounds__(kBlock, KB <= 8 ? 2 : 1)
   const double nev = (double)(ev.end - ev.begin), Smc = s_mc[0];
   const int P = a.n_params;
   const int off = out_mode == 0 ? 2 : 3;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    double g = 0.0;
-    if constexpr (GRAD) {
-      const double f = nev / Smc;
-      // -2 (events) + 2 n / S_mc (MC) of lane j
-      auto both = [&](int j) { return 2.0 * (f * s_mc[j] - s_out[j]); };
-      for (int kk = 0; kk < a.K; ++kk) {
-        const int sl = kk < a.nbw ? kk : KB;  // the NR lives in the last slot
-        double gre = both(1 + 2 * sl), gim = -both(2 + 2 * sl);
-        coef_chain(a.polar, a.jc[kk], a.js[kk], a.jr[kk], gre, gim);
-        if (a.par_re[kk] == p) g += gre;
-        if (a.par_im[kk] == p) g += gim;
-      }
-      for (int k = 0; k < a.nbw; ++k) {
-        const double cu = (double)c.cr[k] * both(1 + 2 * k) - (double)c.ci[k] * both(2 + 2 * k);
-        const double y = both(2 + 2 * KA + 2 * k);
-        if (c.par_m0[k] == p) g += c.rho[k] * cu - c.two_m0[k] * both(1 + 2 * KA + 2 * k) - c.kappa[k] * y;
-        if (c.par_w[k] == p) g -= c.inv_g0[k] * y;
-      }
+  if constexpr (GRAD) {
+    __shared__ double s_term[4 * kMaxAmp];
+    const double f = nev / Smc;
+    // -2 (events) + 2 n / S_mc (MC) of lane j
+    auto both = [&](int j) { return 2.0 * fma(f, s_mc[j], -s_out[j]); };
+    if ((int)threadIdx.x < a.K) {
+      const int k = threadIdx.x, sl = k < a.nbw ? k : KB;  // the NR lives in the last slot
+      double gre = both(1 + 2 * sl), gim = -both(2 + 2 * sl);
+      coef_chain(a.polar, a.jc[k], a.js[k], a.jr[k], gre, gim);
+      s_term[2 * k] = gre;
+      s_term[2 * k + 1] = gim;
+    } else if (threadIdx.x >= 32 && (int)threadIdx.x < 32 + a.nbw) {
+      const int k = threadIdx.x - 32;
+      const double cu = (double)c.cr[k] * both(1 + 2 * k) - (double)c.ci[k] * both(2 + 2 * k);
+      const double y = both(2 + 2 * KA + 2 * k);
+      s_term[2 * (a.K + k)] = c.rho[k] * cu - c.two_m0[k] * both(1 + 2 * KA + 2 * k) - c.kappa[k] * y;
+      s_term[2 * (a.K + k) + 1] = -c.inv_g0[k] * y;
     }
-    out[off + p] = g;
+    __syncthreads();
+    for (int p = threadIdx.x; p < P; p += blockDim.x) out[off + p] = a.map.gather(p, s_term);
+  } else {
+    for (int p = threadIdx.x; p < P; p += blockDim.x) out[off + p] = 0.0;
   }
   if (threadIdx.x == 0) {
     counters[1] = 0u;
@@ -805,7 +809,9 @@ struct Td3Args {
   T wa[kWMax];                       // Weideman coefficients
   T wL;
   int wN, nbw, K, n_params;
-  int par_re[kMaxAmp], par_im[kMaxAmp], par_t[4];  // parameter of each amplitude (tree order)
+  // terms 2k, 2k + 1: the coefficient parameters of amplitude k (tree order); 2 kMaxAmp + j: the time
+  // parameters
+  GradMap<2 * kMaxAmp + 4> map;
   int64_t n_total;                   // events of the dataset (cache plane length)
   int polar;                         // the coefficient parameters are (r, phi)
   double jc[kMaxAmp], js[kMaxAmp], jr[kMaxAmp];  // cos phi, sin phi, r per amplitude (polar)
@@ -865,23 +871,23 @@ __device__ __forceinline__ void td3_finish(const Td3Args<T>& a, ddf lf, const T 
   const double nev = (double)(end - begin);
   const int P = a.n_params;
   const int off = out_mode == 0 ? 2 : 3;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    double g = 0.0;
-    if (GRAD) {
-      for (int kk = 0; kk < K; ++kk) {
-        const int sl = kk < nbw ? kk : KB;
-        double gre = -s_out[1 + 2 * sl] + nev * a.nrm_re[kk], gim = -s_out[2 + 2 * sl] + nev * a.nrm_im[kk];
-        coef_chain(a.polar, a.jc[kk], a.js[kk], a.jr[kk], gre, gim);
-        if (a.par_re[kk] == p) g += gre;
-        if (a.par_im[kk] == p) g += gim;
-      }
-      const int o = 1 + 2 * KA;
-      for (int j = 0; j < 4; ++j)
-        if (a.par_t[j] == p)
-          g += (j < 3 ? nev * a.nrm_dt[j] : 0.0) -
-               time_gradient(j, (double)a.G, (double)a.x, (double)a.y, (double)a.s, s_out + o, nev);
+  if constexpr (GRAD) {
+    __shared__ double s_term[2 * kMaxAmp + 4];
+    if ((int)threadIdx.x < K) {
+      const int k = threadIdx.x, sl = k < nbw ? k : KB;
+      double gre = fma(nev, a.nrm_re[k], -s_out[1 + 2 * sl]), gim = fma(nev, a.nrm_im[k], -s_out[2 + 2 * sl]);
+      coef_chain(a.polar, a.jc[k], a.js[k], a.jr[k], gre, gim);
+      s_term[2 * k] = gre;
+      s_term[2 * k + 1] = gim;
+    } else if (threadIdx.x >= 32 && threadIdx.x < 36) {
+      const int j = threadIdx.x - 32;
+      s_term[2 * kMaxAmp + j] = (j < 3 ? nev * a.nrm_dt[j] : 0.0) -
+                                time_gradient(j, (double)a.G, (double)a.x, (double)a.y, (double)a.s, s_out + 1 + 2 * KA, nev);
     }
-    out[off + p] = g;
+    __syncthreads();
+    for (int p = threadIdx.x; p < P; p += blockDim.x) out[off + p] = a.map.gather(p, s_term);
+  } else {
+    for (int p = threadIdx.x; p < P; p += blockDim.x) out[off + p] = 0.0;
   }
   if (threadIdx.x == 0) {
     counters[1] = 0u;
@@ -1222,6 +1228,15 @@ static int ensure_gram(goo_model* m, int precision) {
   return GOO_OK;
 }
 
+// Terms 2k, 2k + 1 of a gradient map: the coefficient parameters of amplitude k.
+template <int N>
+static void map_coefficients(const DalitzModel& d, GradMap<N>& map) {
+  for (int k = d.K - 1; k >= 0; --k) {
+    map.add(2 * k + 1, d.par_im[k]);
+    map.add(2 * k, d.par_re[k]);
+  }
+}
+
 template <typename T>
 static void fill_args(const DalitzModel& d, const double* theta, int n_params, int64_t n_total, CohArgs<T>& a) {
   std::memset(&a, 0, sizeof a);
@@ -1235,9 +1250,14 @@ static void fill_args(const DalitzModel& d, const double* theta, int n_params, i
     coef(d, theta, k, re, im);
     a.cr[k] = (T)re;
     a.ci[k] = (T)im;
-    a.par_re[k] = d.par_re[k];
-    a.par_im[k] = d.par_im[k];
   }
+  a.map.clear();
+  if (d.floating)
+    for (int k = d.nbw - 1; k >= 0; --k) {
+      a.map.add(2 * (d.K + k) + 1, d.par_w[k]);
+      a.map.add(2 * (d.K + k), d.par_m0[k]);
+    }
+  map_coefficients(d, a.map);
   fill_jacobian(d, theta, a);
 }
 
@@ -1352,8 +1372,6 @@ static void fill_ls(const DalitzModel& d, const double* theta, LsConst<T>& c) {
     c.ci[k] = (T)im;
     c.ncr[k] = -c.cr[k];
     c.nci[k] = -c.ci[k];
-    c.par_m0[k] = d.par_m0[k];
-    c.par_w[k] = d.par_w[k];
     double mA, mB, mC;
     pair_masses(d, d.pair[k], mA, mB, mC);
     const int L = d.spin[k];
@@ -1371,7 +1389,6 @@ static void fill_ls(const DalitzModel& d, const double* theta, LsConst<T>& c) {
     c.two_m0[k] = 2.0 * m0;
     c.inv_g0[k] = 1.0 / g0;
   }
-  for (int k = d.nbw; k < kMaxAmp; ++k) c.par_m0[k] = c.par_w[k] = -1;
 }
 
 template <typename T, int KB, bool GRAD>
@@ -1457,15 +1474,15 @@ static void fill_td3(const DalitzModel& d, const double* theta, int n_params, in
     coef(d, theta, k, re, im);
     a.cr[sl] = (T)re;
     a.ci[sl] = (T)im;
-    a.par_re[k] = d.par_re[k];
-    a.par_im[k] = d.par_im[k];
   }
+  a.map.clear();
+  for (int j = 3; j >= 0; --j) a.map.add(2 * kMaxAmp + j, d.par_t[j]);
+  map_coefficients(d, a.map);
   fill_time_coef<T>(a.tc, theta[d.par_t[0]], theta[d.par_t[1]], theta[d.par_t[2]], theta[d.par_t[3]], t_hi);
   a.x = a.tc.x;
   a.y = a.tc.y;
   a.G = a.tc.G;
   a.s = a.tc.s;
-  for (int j = 0; j < 4; ++j) a.par_t[j] = d.par_t[j];
   const WeidemanTables& w = weideman();
   a.wN = sizeof(T) == 4 ? kWN32 : kWN64;
   for (int j = 0; j < a.wN; ++j) a.wa[j] = (T)(sizeof(T) == 4 ? w.a32[j] : w.a64[j]);

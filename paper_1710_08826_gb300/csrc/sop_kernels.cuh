@@ -313,7 +313,8 @@ struct EvNorm {
   double dlog[K * L][3];
   double w[K];                                     // w_k
   int n_params;
-  signed char par[K][L][3];                        // parameter of leaf constant j (-1: none)
+  // the gradient terms of leaf constants, term (k L + l) 3 + j, by parameter
+  GradMap<K * L * 3> map;
   double dw[GRAD ? K : 1][GRAD ? kMaxParams : 1];  // d w_k / d theta_p
 };
 
@@ -840,9 +841,7 @@ __device__ __forceinline__ void fused_grid_norm(const EvConst<float, K, L>& P, c
 // Block reduction, last-block reduction over the blocks and the final FP64 combination of the
 // self-normalising pair kernel:
 //   d NLL / d theta_p = - sum_k C_k dw_kp + sum_{k,l,j: par = p} w_k (C_k D_klj / S_kl - A_klj),
-// the normalisation terms D_klj / S_kl formed here from the block's own grid sums.  Thread p
-// takes parameter p; its terms are formed independently and added by a fixed pairwise tree
-// (the combination is bound by FP64 latency, not throughput).  buf: NS * blockDim
+// the normalisation terms D_klj / S_kl formed here from the block's own grid sums.  buf: NS * blockDim
 // double-floats of shared memory (the tile buffers, idle now) for the block reduction.
 template <int K, int L, bool GRAD, unsigned long long SIG>
 __device__ __forceinline__ void event_finish_fused(const ddf (&v)[EventLanes<float, K, L, GRAD, SIG>::NS],
@@ -851,11 +850,8 @@ __device__ __forceinline__ void event_finish_fused(const ddf (&v)[EventLanes<flo
                                                    unsigned* counters, double* result, int out_mode, ddf* buf,
                                                    unsigned* s_bad) {
   constexpr int NS = EventLanes<float, K, L, GRAD, SIG>::NS;
-  constexpr int NT = GRAD ? K + K * L * 3 : 1;  // terms of one parameter's gradient
   __shared__ double s_out[NS];
-  __shared__ double s_w[K];
-  __shared__ double s_t[K * L][3];
-  __shared__ int s_par[K][L][3];
+  __shared__ double s_t[K * L * 3];
   __shared__ ddf s_red[kBlock / 32];
   const int p = threadIdx.x;
   const int P = N.n_params;
@@ -863,11 +859,6 @@ __device__ __forceinline__ void event_finish_fused(const ddf (&v)[EventLanes<flo
   if constexpr (GRAD) {
 #pragma unroll
     for (int k = 0; k < K; ++k) dwp[k] = (p < P && k < nK) ? N.dw[k][p] : 0.0;
-    for (int t = threadIdx.x; t < K * L * 3; t += blockDim.x) {
-      const int k = t / (L * 3), l = (t / 3) % L, jj = t % 3;
-      s_par[k][l][jj] = k < nK ? N.par[k][l][jj] : -1;
-    }
-    if (threadIdx.x < K) s_w[threadIdx.x] = N.w[threadIdx.x];
   }
   for (int m = 16; m > 0; m >>= 1) bad += __shfl_xor_sync(0xffffffffu, bad, m);
   if ((threadIdx.x & 31) == 0) s_bad[threadIdx.x >> 5] = bad;
@@ -888,43 +879,44 @@ __device__ __forceinline__ void event_finish_fused(const ddf (&v)[EventLanes<flo
   }
   if constexpr (GRAD) {
     // the normalisation terms D_j / S of every leaf slot, from this block's grid sums (the
-    // quotient in double-float, then FP64)
+    // quotient in double-float, then FP64) or the closed forms
     for (int t = threadIdx.x; t < K * L * 3; t += blockDim.x) {
       const int sl = t / 3, jj = t % 3;
-      s_t[sl][jj] = N.analytic ? N.dlog[sl][jj]
-                    : N.nb[sl] ? dd_to_double(dd_div(s_raw[sl][1 + jj], s_raw[sl][0]))
-                               : 0.0;
+      s_t[t] = N.analytic ? N.dlog[sl][jj]
+               : N.nb[sl] ? dd_to_double(dd_div(s_raw[sl][1 + jj], s_raw[sl][0]))
+                          : 0.0;
     }
   }
   reduce_partials<24>(partials, NS, gridDim.x, s_out, s_red, blockDim.x);
 
-  // ---- final combination (last block, FP64) ----
+  // ---- final combination (last block, FP64): one thread per leaf term, then one per parameter, which
+  // gathers its terms (an FP64 instruction takes a warp 64 cycles, so a parameter's thread that ran
+  // over every term cost 1.9 us) ----
   const int off = out_mode == 0 ? 2 : 3;
-  if (p < P) {
-    double tm[NT];
-    if constexpr (GRAD) {
+  if constexpr (GRAD) {
+    if (threadIdx.x < K * L * 3) {
+      const int t = threadIdx.x, k = t / (L * 3);
+      double a = 0.0, w = 0.0;
 #pragma unroll
-      for (int k = 0; k < K; ++k) tm[k] = k < nK ? -s_out[1 + k] * dwp[k] : 0.0;
+      for (int q = 0; q < K * L * 3; ++q)
+        if (q == t && a_present<K, L, SIG>(q / (L * 3), (q / 3) % L, q % 3))
+          a = s_out[a_lane<K, L, SIG>(q / (L * 3), (q / 3) % L, q % 3)];
+#pragma unroll
+      for (int q = 0; q < K; ++q)
+        if (q == k) w = N.w[q];
+      s_t[t] = w * (s_out[1 + k] * s_t[t] - a);
+    }
+    __syncthreads();
+  }
+  if (p < P) {
+    double g = 0.0;
+    if constexpr (GRAD) {
+      g = N.map.gather(p, s_t);
 #pragma unroll
       for (int k = 0; k < K; ++k)
-#pragma unroll
-        for (int l = 0; l < L; ++l)
-#pragma unroll
-          for (int jj = 0; jj < 3; ++jj) {
-            double term = 0.0;
-            if (a_present<K, L, SIG>(k, l, jj) && s_par[k][l][jj] == p)
-              term = s_w[k] * (s_out[1 + k] * s_t[k * L + l][jj] - s_out[a_lane<K, L, SIG>(k, l, jj)]);
-            tm[K + (k * L + l) * 3 + jj] = term;
-          }
-      // fixed pairwise tree over the NT terms
-#pragma unroll
-      for (int w = 1; w < NT; w *= 2)
-#pragma unroll
-        for (int i = 0; i + w < NT; i += 2 * w) tm[i] += tm[i + w];
-    } else {
-      tm[0] = 0.0;
+        if (k < nK && (__double_as_longlong(dwp[k]) << 1) != 0) g = fma(-s_out[1 + k], dwp[k], g);
     }
-    result[off + p] = tm[0];
+    result[off + p] = g;
   }
   if (threadIdx.x == 0) {
     counters[0] = 0u;  // the ticket

@@ -61,7 +61,8 @@ struct Td4Args {
   T wa[kWMax];   // Weideman coefficients (constant term first)
   T wL;
   int wN, K, n_params, planes;
-  int par_re[kTdMaxAmp], par_im[kTdMaxAmp], par_t[4];
+  // terms 2k, 2k + 1: the coefficient parameters of amplitude k; 2 kTdMaxAmp + j: the time parameters
+  GradMap<2 * kTdMaxAmp + 4> map;
   int64_t n_total;  // events of the dataset (cache plane length)
   // the normalisation at theta, formed on the host in FP64 from the cached Gram matrix
   // (td4_norm_terms): N, log N, (dN / d Re c_k) / N, (dN / d Im c_k) / N and (dN / dx) / N,
@@ -268,20 +269,22 @@ __device__ __forceinline__ void td4_finish(const Td4Args<T>& a, TdAcc<T, KB>& ac
   const int K = a.K;
   const int P = a.n_params;
   const int off = out_mode == 0 ? 2 : 3;
-  for (int p = threadIdx.x; p < P; p += blockDim.x) {
-    double g = 0.0;
-    if (GRAD) {
-      for (int k = 0; k < K; ++k) {
-        if (a.par_re[k] == p) g += -s_out[1 + 2 * k] + nev * a.nrm_ur[k];
-        if (a.par_im[k] == p) g += -s_out[2 + 2 * k] - nev * a.nrm_ui[k];
-      }
-      const int o = 1 + 2 * KB;
-      for (int j = 0; j < 4; ++j)
-        if (a.par_t[j] == p)
-          g += (j < 3 ? nev * a.nrm_dt[j] : 0.0) -
-               time_gradient(j, (double)a.G, (double)a.x, (double)a.y, (double)a.s, s_out + o, nev);
+  // one thread per amplitude and time parameter forms its terms, then one per parameter gathers
+  if constexpr (GRAD) {
+    __shared__ double s_term[2 * kTdMaxAmp + 4];
+    if ((int)threadIdx.x < K) {
+      const int k = threadIdx.x;
+      s_term[2 * k] = fma(nev, a.nrm_ur[k], -s_out[1 + 2 * k]);
+      s_term[2 * k + 1] = fma(-nev, a.nrm_ui[k], -s_out[2 + 2 * k]);
+    } else if (threadIdx.x >= 32 && threadIdx.x < 36) {
+      const int j = threadIdx.x - 32;
+      s_term[2 * kTdMaxAmp + j] = (j < 3 ? nev * a.nrm_dt[j] : 0.0) -
+                                  time_gradient(j, (double)a.G, (double)a.x, (double)a.y, (double)a.s, s_out + 1 + 2 * KB, nev);
     }
-    result[off + p] = g;
+    __syncthreads();
+    for (int p = threadIdx.x; p < P; p += blockDim.x) result[off + p] = a.map.gather(p, s_term);
+  } else {
+    for (int p = threadIdx.x; p < P; p += blockDim.x) result[off + p] = 0.0;
   }
   if (threadIdx.x == 0) {
     counters[1] = 0u;
@@ -695,10 +698,13 @@ static void td4_args(const goo_model* m, const double* theta, int64_t n_total, T
     a.ci[k] = (T)theta[d.par_im[k]];
     a.br[k] = (T)d.br[k];
     a.bi[k] = (T)d.bi[k];
-    a.par_re[k] = d.par_re[k];
-    a.par_im[k] = d.par_im[k];
   }
-  for (int j = 0; j < 4; ++j) a.par_t[j] = d.par_t[j];
+  a.map.clear();
+  for (int j = 3; j >= 0; --j) a.map.add(2 * kTdMaxAmp + j, d.par_t[j]);
+  for (int k = d.K - 1; k >= 0; --k) {
+    a.map.add(2 * k + 1, d.par_im[k]);
+    a.map.add(2 * k, d.par_re[k]);
+  }
   fill_time_coef<T>(a.tc, theta[d.par_t[0]], theta[d.par_t[1]], theta[d.par_t[2]], theta[d.par_t[3]], m->hi[5]);
   a.x = a.tc.x;
   a.y = a.tc.y;

@@ -959,19 +959,20 @@ static EvNorm<K, L, GRAD> make_evnorm(const ModelDev& h) {
   EvNorm<K, L, GRAD> N;
   std::memset(&N, 0, sizeof N);
   N.analytic = h.norm_kind == GOO_NORM_ANALYTIC;
+  N.map.clear();
+  for (int t = K * L * 3 - 1; t >= 0; --t) {
+    const int k = t / (L * 3), l = (t / 3) % L;
+    if (k < h.nK && l < h.comp[k].n_leaf) N.map.add(t, h.leaf[k * kMaxLeaf + l].par[t % 3]);
+  }
   for (int k = 0; k < K; ++k) {
     N.w[k] = k < h.nK ? h.comp[k].w : 0.0;
     N.off_hi[k] = k < h.nK ? h.comp[k].off_hi : 0.f;
     N.off_lo[k] = k < h.nK ? h.comp[k].off_lo : 0.f;
     for (int l = 0; l < L; ++l) {
       const int sl = k * L + l;
-      for (int j = 0; j < 3; ++j) N.par[k][l][j] = -1;
       if (k >= h.nK || l >= h.comp[k].n_leaf) continue;
       const LeafDev& LD = h.leaf[k * kMaxLeaf + l];
-      for (int j = 0; j < 3; ++j) {
-        N.par[k][l][j] = (signed char)LD.par[j];
-        N.dlog[sl][j] = LD.dlog[j];
-      }
+      for (int j = 0; j < 3; ++j) N.dlog[sl][j] = LD.dlog[j];
       if (N.analytic) continue;
       const GridDev& G = h.grid[k];
       const int d = G.dim_of_col[LD.col];
