@@ -545,7 +545,7 @@ static uint64_t lineshape_key(const DalitzModel& d, const double* theta) {
 // amplitude is formed again for its lanes (ten operations) rather than kept; the
 // first blocks of the one launch take the MC sample and the others the events, so that neither waits for the
 // other's reduction.  5M events and 1M MC points, 8 resonances: 495 us in two launches with every
-// resonance evaluated by itself, now 156 us.
+// resonance evaluated by itself, now 144 us (150 with two blocks of 256 threads per SM).
 // ---------------------------------------------------------------------------------------
 template <typename T>
 struct LsConst {
@@ -566,10 +566,15 @@ struct LsSet {
   int64_t begin, end, n;  // the points of the evaluation, and of the column
 };
 
+// Threads per block: 16 warps per SM in one block (half as many partial sums for the last block as with two of
+// 8), 8 where 15 resonances' lanes fill the register file.
+template <int KB>
+constexpr int kLsBlockOf = KB <= 8 ? kStagedBlock : kBlock;
+
 // Dynamic shared memory: the shared factors of every thread, later the block reduction's lanes.
 template <typename T, int KB, bool GRAD>
 constexpr size_t ls_smem() {
-  const size_t f = (size_t)kLsCols * kBlock * 8, r = (size_t)LsLanes<KB, GRAD>::NS * kBlock * sizeof(ddf);
+  const size_t f = (size_t)kLsCols * kLsBlockOf<KB> * 8, r = (size_t)LsLanes<KB, GRAD>::NS * kLsBlockOf<KB> * sizeof(ddf);
   return f > r ? f : r;
 }
 
@@ -651,7 +656,7 @@ __device__ __forceinline__ void ls_weight(bool mc, double s2, bool, bool, double
 }
 
 template <typename T, int KB, bool GRAD>
-__global__ void __launch_bounds__(kBlock, KB <= 8 ? 2 : 1)
+__global__ void __launch_bounds__(kLsBlockOf<KB>, 1)
     coh_ls_kernel(const __grid_constant__ CohArgs<T> a, const __grid_constant__ LsConst<T> c,
                   const __grid_constant__ LsTables<T> t, const __grid_constant__ LsSet<T> mc,
                   const __grid_constant__ LsSet<T> ev, int nb_mc, float2* partials, unsigned* counters, double* out,
@@ -660,12 +665,13 @@ __global__ void __launch_bounds__(kBlock, KB <= 8 ? 2 : 1)
   using V = typename std::conditional<sizeof(T) == 4, float2, double>::type;
   using Sum = typename std::conditional<sizeof(T) == 4, LsSumF, LsSumD>::type;
   constexpr int KA = KB + 1;
+  constexpr int NT = kLsBlockOf<KB>;
   constexpr int NS = LsLanes<KB, GRAD>::NS;
-  __shared__ ddf s_red[kBlock / 32];
+  __shared__ ddf s_red[NT / 32];
   __shared__ double s_out[NS], s_mc[NS];
   extern __shared__ __align__(16) unsigned char s_dyn[];
   V* s_v = reinterpret_cast<V*>(s_dyn);
-  V *sc = s_v + threadIdx.x, *gc = sc + 3 * kBlock, *hc = sc + 12 * kBlock;
+  V *sc = s_v + threadIdx.x, *gc = sc + 3 * NT, *hc = sc + 12 * NT;
   const bool is_mc = (int)blockIdx.x < nb_mc;
   const LsSet<T>& D = is_mc ? mc : ev;
   const int nb = is_mc ? nb_mc : (int)gridDim.x - nb_mc, b0 = is_mc ? (int)blockIdx.x : (int)blockIdx.x - nb_mc;
@@ -678,15 +684,15 @@ __global__ void __launch_bounds__(kBlock, KB <= 8 ? 2 : 1)
   for (int k = 0; k < KB; ++k) lwr[k] = lwi[k] = zero;
   unsigned bad = 0;
   const int64_t last = ls_last(D);
-  for (int64_t j = ls_first(D) + b0 * (int64_t)kBlock + threadIdx.x; j < last; j += (int64_t)nb * kBlock) {
+  for (int64_t j = ls_first(D) + b0 * (int64_t)NT + threadIdx.x; j < last; j += (int64_t)nb * NT) {
     V x12, x13, re, im, dr, di, iv;
     bool v0, v1;
     ls_load(D, j, x12, x13, v0, v1);
-    ls_groups<T, V>(t, x12, x13, sc, gc, hc, kBlock);
+    ls_groups<T, V>(t, x12, x13, sc, gc, hc, NT);
     V sr = splat(V{}, c.cr[KB]), si = splat(V{}, c.ci[KB]);  // the non-resonant amplitude is 1
 #pragma unroll 4
     for (int k = 0; k < t.nbw; ++k) {
-      ls_amp<T, V>(t, k, sc, gc, hc, kBlock, re, im, dr, di, iv);
+      ls_amp<T, V>(t, k, sc, gc, hc, NT, re, im, dr, di, iv);
       const V cr = splat(V{}, c.cr[k]);
       sr = fma(cr, re, fma(splat(V{}, c.nci[k]), im, sr));
       si = fma(cr, im, fma(splat(V{}, c.ci[k]), re, si));
@@ -701,7 +707,7 @@ __global__ void __launch_bounds__(kBlock, KB <= 8 ? 2 : 1)
 #pragma unroll
       for (int k = 0; k < KB; ++k) {
         if (k >= t.nbw) break;
-        ls_amp<T, V>(t, k, sc, gc, hc, kBlock, re, im, dr, di, iv);
+        ls_amp<T, V>(t, k, sc, gc, hc, NT, re, im, dr, di, iv);
         const V ur = fma(re, tr, mul(im, mti)), ui = fma(re, ti, mul(im, tr));  // A_k conj(S) w
         lre[k] = add(lre[k], ur);
         lim[k] = add(lim[k], ui);
@@ -739,8 +745,8 @@ __global__ void __launch_bounds__(kBlock, KB <= 8 ? 2 : 1)
     nbad = __ldcg(counters + 1);
     status = __ldcg(counters + kStatusWord);
   }
-  reduce_partials<24>(partials, NS, nb_mc, s_mc, s_red, kBlock);
-  reduce_partials<24>(partials + (size_t)nb_mc * NS, NS, (int)gridDim.x - nb_mc, s_out, s_red, kBlock);
+  reduce_partials<24>(partials, NS, nb_mc, s_mc, s_red, NT);
+  reduce_partials<24>(partials + (size_t)nb_mc * NS, NS, (int)gridDim.x - nb_mc, s_out, s_red, NT);
   const double nev = (double)(ev.end - ev.begin), Smc = s_mc[0];
   const int P = a.n_params;
   const int off = out_mode == 0 ? 2 : 3;
@@ -1398,12 +1404,13 @@ static int launch_ls(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t
   goo_ctx* ctx = m->ctx;
   constexpr size_t smem = ls_smem<T, KB, GRAD>();
   constexpr int NS = LsLanes<KB, GRAD>::NS;
+  constexpr int NT = kLsBlockOf<KB>;
   const void* fn = (const void*)coh_ls_kernel<T, KB, GRAD>;
   GOO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const int64_t cap = (int64_t)ctx->num_sms * cached_occupancy(fn, ctx->device, kBlock, smem);
+  const int64_t cap = (int64_t)ctx->num_sms * cached_occupancy(fn, ctx->device, NT, smem);
   // blocks in proportion to the points, at least one each, no more than there are steps
   constexpr int per = sizeof(T) == 4 ? 2 : 1;
-  auto steps = [](int64_t n) { return (n / per + 1 + kBlock) / kBlock; };
+  auto steps = [](int64_t n) { return (n / per + 1 + NT) / NT; };
   const int64_t n_mc = d.mc->n, n_ev = end - begin;
   const int64_t want_mc = std::max<int64_t>(1, (int64_t)((double)cap * n_mc / (double)(n_mc + n_ev) + 0.5));
   const int nb_mc = (int)std::min<int64_t>(std::min<int64_t>(want_mc, cap - 1), steps(n_mc));
@@ -1428,7 +1435,7 @@ static int launch_ls(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t
     const LsTables<T>* t;
     if constexpr (sizeof(T) == 4) t = &d.ls32;
     else t = &d.ls64;
-    coh_ls_kernel<T, KB, GRAD><<<nb_mc + nb_ev, kBlock, smem, ctx->stream>>>(
+    coh_ls_kernel<T, KB, GRAD><<<nb_mc + nb_ev, NT, smem, ctx->stream>>>(
         a, c, *t, set(d.mc, 0, n_mc), set(ds, begin, end), nb_mc, ctx->scratch.partials, ctx->scratch.counters,
         ctx->scratch.result_out, out_mode);
   }
