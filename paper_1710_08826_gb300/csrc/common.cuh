@@ -111,7 +111,7 @@ struct Scratch {
   unsigned char *batch_host = nullptr, *batch_dev = nullptr;
   size_t batch_host_cap = 0, batch_dev_cap = 0;
   double* gram_host = nullptr;      // mapped record of the Gram matrices (kGramRecord doubles), on first use
-  void* fp64_tables = nullptr;      // device copy of the FP64 function tables (fp64.cuh), on first use
+  void *fp64_tables = nullptr, *fp32_tables = nullptr;  // device copies of the function tables (fp64.cuh), on first use
 };
 constexpr int kGramRecord = 3 * 2 * 16 * 16;  // three 16 x 16 complex matrices
 constexpr int kStreamChunks = 64;  // chunks of one goo_nll_grad_streamed call, at most
@@ -366,6 +366,18 @@ __device__ __forceinline__ float rcp(float x) {
 constexpr float kLn2 = 0.6931471805599453f;
 __device__ __forceinline__ float2 rcp(float2 x) { return make_float2(rcp(x.x), rcp(x.y)); }
 }  // namespace pk
+
+// Compensated FP32 accumulator of an event pair (one Kahan sum per lane, packed).
+struct Kahan2 {
+  float2 s = {0.f, 0.f}, c = {0.f, 0.f};
+  __device__ __forceinline__ void add(float2 x) {
+    const float2 y = pk::sub(x, c);
+    const float2 t = pk::add(s, y);
+    c = pk::sub(pk::sub(t, s), y);
+    s = t;
+  }
+  __device__ __forceinline__ ddf value() const { return dd_add(dd_make(s.x, -c.x), dd_make(s.y, -c.y)); }
+};
 
 // ---------------------------------------------------------------------------------------
 // Bulk asynchronous copies global -> shared (the non-tensor TMA form, cp.async.bulk) that

@@ -459,6 +459,7 @@ int goo_finalize(goo_ctx* ctx) {
   if (s.counters) cudaFree(s.counters);
   if (s.result) cudaFree(s.result);
   if (s.fp64_tables) cudaFree(s.fp64_tables);
+  if (s.fp32_tables) cudaFree(s.fp32_tables);
   if (s.gram_host) cudaFreeHost(s.gram_host);
   if (s.batch_host) cudaFreeHost(s.batch_host);
   if (s.batch_dev) cudaFree(s.batch_dev);

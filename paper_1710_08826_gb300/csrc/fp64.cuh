@@ -145,10 +145,17 @@ __device__ __forceinline__ double herfcx_tab(double u, const Fp64Tables& tab) {
   return p;
 }
 
+// The same interpolants of erfcx(u) / 2 in FP32: degree 3 (error of the interpolation 4e-9).
+constexpr int kErfcxDeg32 = 3;
+struct Fp32Tables {
+  float herfcx[kErfcxDeg32 + 1][kErfcxTab];
+};
+
 #ifndef __CUDACC_RTC__
-// The context's device copy of the tables, built on first use (host pointer arithmetic only
+// The context's device copies of the tables, built on first use (host pointer arithmetic only
 // afterwards) and freed with the context.
 int fp64_tables(goo_ctx* ctx, const Fp64Tables** dev);
+int fp32_tables(goo_ctx* ctx, const Fp32Tables** dev);
 #endif
 
 }  // namespace goo

@@ -712,18 +712,6 @@ __device__ __forceinline__ void eval_event2(const EvConst<float, K, L>& P, const
   }
 }
 
-// Compensated FP32 accumulator of an event pair (one Kahan sum per lane, packed).
-struct Kahan2 {
-  float2 s = {0.f, 0.f}, c = {0.f, 0.f};
-  __device__ __forceinline__ void add(float2 x) {
-    const float2 y = pk::sub(x, c);
-    const float2 t = pk::add(s, y);
-    c = pk::sub(pk::sub(t, s), y);
-    s = t;
-  }
-};
-
-
 // Midpoint coordinate of bin idx of a 1-D grid as a double-float (the FP32 path's grid_coord).
 __device__ __forceinline__ void grid_coord_f(float lo_hi, float lo_lo, float h_hi, float h_lo, int64_t idx, float& x,
                                              float& xlo) {
@@ -1280,7 +1268,7 @@ __global__ void __launch_bounds__(kBlock, EventOcc2<K, L, GRAD>::value)
   // lanes: the two Kahan sums as one double-float (log2 f, turned into natural logarithms),
   // the gradient lanes as the lane sums, each times its constant factor (leaf_eval2)
   ddf v[NS];
-  v[0] = dd_mul(dd_add(dd_make(S.lf.s.x, -S.lf.c.x), dd_make(S.lf.s.y, -S.lf.c.y)), ddf{kLn2Hi, kLn2Lo});
+  v[0] = dd_mul(S.lf.value(), ddf{kLn2Hi, kLn2Lo});
   if constexpr (GRAD) {
 #pragma unroll
     for (int k = 0; k < K; ++k) {

@@ -166,17 +166,15 @@ struct TdLanes {
 
 template <typename T, int KB>
 struct TdAcc {
-  Kahan lf32;
-  double lf64 = 0.0;
+  ddf lf;  // the thread's sum of log R
   T lre[KB], lim[KB], lt[4];
   unsigned bad = 0;
 };
 
-// One event of the FP32 kernel.  The amplitudes come as (re, im) pairs
+// The FP32 sums of one event.  The amplitudes come as (re, im) pairs
 // straight from the float4 planes, and A = sum c_k a_k is formed from two packed sums,
 // (sum cr_k re_k, sum cr_k im_k) and (sum ci_k re_k, sum ci_k im_k), B likewise: four packed
-// FMAs per amplitude instead of eight scalar ones.  log2 R is accumulated (td4_finish scales
-// the FP32 sum by ln 2 once per thread) and 1/R is the hardware reciprocal.
+// FMAs per amplitude instead of eight scalar ones.
 template <int KB>
 __device__ __forceinline__ void td4_sums_f32(const Td4Args<float>& a, const float2 (&am)[KB], float& Ar, float& Ai,
                                              float& Br, float& Bi) {
@@ -195,36 +193,6 @@ __device__ __forceinline__ void td4_sums_f32(const Td4Args<float>& a, const floa
   Bi = Q1.y + Q2.x;
 }
 
-template <int KB, bool GRAD>
-__device__ __forceinline__ void td4_event_f32(const Td4Args<float>& a, const float2 (&am)[KB], float t,
-                                              TdAcc<float, KB>& acc) {
-  using namespace pk;
-  float Ar, Ai, Br, Bi;
-  td4_sums_f32(a, am, Ar, Ai, Br, Bi);
-  TimeTerms<float> tt;
-  time_terms_g<float>(TdMath<float>{}, a.tc, a.wa, a.wN, a.wL, t, tt);
-  const float AA = fma_rn(Ar, Ar, mul_rn(Ai, Ai)), BB = fma_rn(Br, Br, mul_rn(Bi, Bi));
-  const float ABr = fma_rn(Ar, Br, mul_rn(Ai, Bi)), ABi = fma_rn(Ai, Br, -mul_rn(Ar, Bi));  // A conj(B)
-  const float R = td_rate(tt, AA, BB, ABr, ABi);
-  if (!(R > 0.f)) {
-    acc.bad++;
-    return;
-  }
-  acc.lf32.add(lg2(R));
-  if constexpr (GRAD) {
-    const float invR = rcp(R);
-    const float c1 = 2.f * tt.P * invR, sh = tt.Tsh * invR, ss = tt.Ts * invR;
-    const float Vr = c1 * Ar + sh * Br - ss * Bi;
-    const float Vi = -c1 * Ai - sh * Bi - ss * Br;
-#pragma unroll
-    for (int k = 0; k < KB; ++k) {
-      acc.lre[k] += am[k].x * Vr - am[k].y * Vi;     // Re(a_k V) / R
-      acc.lim[k] += -(am[k].x * Vi + am[k].y * Vr);  // -Im(a_k V) / R
-    }
-    time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, acc.lt);
-  }
-}
-
 // Block and last-block reductions, then the FP64 combination with the normalisation terms the
 // host formed from the Gram matrix (they depend on theta and the MC sample only, not on the
 // events: an O(K^2) quadratic form, whose FP64 latency chain had been the last block's tail).
@@ -234,8 +202,7 @@ __device__ __forceinline__ void td4_finish(const Td4Args<T>& a, TdAcc<T, KB>& ac
                                            ddf* s_red, unsigned* s_bad) {
   constexpr int NS = TdLanes<KB, GRAD>::NS;
   ddf v[NS];
-  // the FP32 kernel sums log2 R (td4_event_f32)
-  v[0] = (sizeof(T) == 4) ? dd_mul(acc.lf32.value(), ddf{kLn2Hi, kLn2Lo}) : dd_from_double(acc.lf64);
+  v[0] = acc.lf;
   if constexpr (GRAD) {
 #pragma unroll
     for (int k = 0; k < KB; ++k) {
@@ -339,6 +306,7 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f64_kernel(const __grid_con
   const TdMath<double> F{s_tab};
   TdAcc<double, KB> acc;
   LogProduct lp;
+  double lf64 = 0.0;
 #pragma unroll
   for (int k = 0; k < KB; ++k) acc.lre[k] = acc.lim[k] = 0.0;
 #pragma unroll
@@ -360,7 +328,7 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f64_kernel(const __grid_con
       lp.mul(R);
       invR = rcp64(R);
     } else if (R > 0.0) {  // subnormal or infinite
-      acc.lf64 += log(R);
+      lf64 += log(R);
       invR = 1.0 / R;
     } else {
       acc.bad++;
@@ -381,28 +349,39 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f64_kernel(const __grid_con
       time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, acc.lt);
     }
   }
-  acc.lf64 += lp.log_value();
+  acc.lf = dd_from_double(lf64 + lp.log_value());
   td4_finish<double, KB, GRAD>(a, acc, begin, end, partials, counters, result, out_mode, s_red, s_bad);
 }
 
 // FP32: tiles of kTdTile events (aligned to multiples of kTdTile) of every amplitude plane
-// and of the time column staged in shared memory by bulk copies, kTdStages tiles ahead;
+// and of the time column staged in shared memory by bulk copies, kTdStages tiles ahead, the warps
+// releasing the stages one by one (TileRing);
 // block b takes tiles tb0 + b, + gridDim.x, ...; ragged first / last tiles read global
-// memory.  Dynamic shared memory: kTdStages * (planes * kTdTile float4 + kTdTile float).
-constexpr int kTdTile = kBlock;  // one event per thread per tile
-constexpr int kTdStages = 4;
+// memory.  A thread takes events e and e + kBlock of a tile: what depends on the time (exp, erfcx, the
+// moment series, the rate and its derivatives, 280 of the 500 instructions an event took one at
+// a time) runs once for both in packed FP32, and two events' independent sums overlap.  The
+// amplitudes are read from the tile again for the gradient lanes, as packed
+//   G1_k += Re(V/R) a_k,  G2_k += Im(V/R) a_k   (Re(a_k V)/R = G1.x - G2.y, Im = G1.y + G2.x).
+// log2 R is summed, scaled by ln 2 once per thread; 1/R is the hardware reciprocal.
+// 2M events, 10 amplitudes: 52.4 us one event at a time, now 45.6 us (84 bytes per event: 24.8 us of HBM).
+// Dynamic shared memory: kTdStages * (planes * kTdTile float4 + kTdTile float).
+constexpr int kTdTile = 2 * kBlock;
+// stages by slot count: two blocks per SM at 10 amplitudes (43 KB a stage), one at 16 (68 KB)
+template <int KB>
+constexpr int kTdStages = KB <= 10 ? 2 : 3;
 
 template <int KB, bool GRAD>
-__global__ void __launch_bounds__(kBlock, 2) td4_nll_f32_kernel(const __grid_constant__ Td4Args<float> a,
-                                                                const float4* __restrict__ cache,
-                                                                const float* __restrict__ tcol, int64_t begin,
-                                                                int64_t end, float2* partials, unsigned* counters,
-                                                                double* result, int out_mode) {
+__global__ void __launch_bounds__(kBlock, KB <= 10 ? 2 : 1)
+    td4_nll_f32_kernel(const __grid_constant__ Td4Args<float> a, const float4* __restrict__ cache,
+                       const float* __restrict__ tcol, const Fp32Tables* __restrict__ tables, int64_t begin, int64_t end,
+                       float2* partials, unsigned* counters, double* result, int out_mode) {
+  using namespace pk;
   constexpr int NS = TdLanes<KB, GRAD>::NS;
-  constexpr int TE = kTdTile, NST = kTdStages;
+  constexpr int TE = kTdTile, NST = kTdStages<KB>;
   __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
   __shared__ unsigned s_bad[kBlock / 32];
   __shared__ __align__(8) TileRing<NST> s_ring;
+  __shared__ Fp32Tables s_tab;
   extern __shared__ __align__(128) float4 s_tile[];  // per stage: planes x TE float4, then TE float
   const int planes = a.planes;
   const int64_t n = a.n_total;
@@ -428,23 +407,72 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f32_kernel(const __grid_con
     s_ring.init();
     for (int j = 0; j < NST; ++j) issue(j);
   }
-  TdAcc<float, KB> acc;
+  for (int i = threadIdx.x; i < (int)(sizeof(Fp32Tables) / 4); i += kBlock)
+    ((float*)&s_tab)[i] = __ldg((const float*)tables + i);
+  const TdMath<float2> F{s_tab};
+  Kahan2 lf;
+  float2 G1[KB], G2[KB], lt[4];
 #pragma unroll
-  for (int k = 0; k < KB; ++k) acc.lre[k] = acc.lim[k] = 0.f;
+  for (int k = 0; k < KB; ++k) G1[k] = G2[k] = splat(0.f);
 #pragma unroll
-  for (int j = 0; j < 4; ++j) acc.lt[j] = 0.f;
-  __syncthreads();  // barriers initialised before any thread waits on them
-  const long long wlim = tile_wait_limit(counters);
-  // absent planes stay zero: only the model's planes are loaded over these
-  float4 v[KB / 2];
+  for (int j = 0; j < 4; ++j) lt[j] = splat(0.f);
+  unsigned bad = 0;
+  // two events: load(e, p) is plane p of event e (0, 1), t their times, v0, v1 whether they count
+  auto pair = [&](auto load, float2 t, bool v0, bool v1) {
+    float Ar[2], Ai[2], Br[2], Bi[2];
 #pragma unroll
-  for (int p = 0; p < KB / 2; ++p) v[p] = make_float4(0.f, 0.f, 0.f, 0.f);
-  auto event = [&](float tv) {
-    float2 am[KB];
+    for (int e = 0; e < 2; ++e) {
+      float2 P1 = splat(0.f), P2 = splat(0.f), Q1 = splat(0.f), Q2 = splat(0.f);
 #pragma unroll
-    for (int k = 0; k < KB; ++k) am[k] = (k & 1) ? make_float2(v[k / 2].z, v[k / 2].w) : make_float2(v[k / 2].x, v[k / 2].y);
-    td4_event_f32<KB, GRAD>(a, am, tv, acc);
+      for (int p = 0; p < KB / 2; ++p) {
+        if (p >= planes) break;
+        const float4 v = load(e, p);
+        const float2 a0 = make_float2(v.x, v.y), a1 = make_float2(v.z, v.w);
+        P1 = fma(splat(a.cr[2 * p + 1]), a1, fma(splat(a.cr[2 * p]), a0, P1));
+        P2 = fma(splat(a.ci[2 * p + 1]), a1, fma(splat(a.ci[2 * p]), a0, P2));
+        Q1 = fma(splat(a.br[2 * p + 1]), a1, fma(splat(a.br[2 * p]), a0, Q1));
+        Q2 = fma(splat(a.bi[2 * p + 1]), a1, fma(splat(a.bi[2 * p]), a0, Q2));
+      }
+      Ar[e] = P1.x - P2.y;
+      Ai[e] = P1.y + P2.x;
+      Br[e] = Q1.x - Q2.y;
+      Bi[e] = Q1.y + Q2.x;
+    }
+    const float2 A2r = make_float2(Ar[0], Ar[1]), A2i = make_float2(Ai[0], Ai[1]);
+    const float2 B2r = make_float2(Br[0], Br[1]), B2i = make_float2(Bi[0], Bi[1]);
+    TimeTerms<float2> tt;
+    time_terms_pair(F, a.tc, a.wa, a.wN, a.wL, t, tt);
+    const float2 AA = fma_rn(A2r, A2r, mul_rn(A2i, A2i)), BB = fma_rn(B2r, B2r, mul_rn(B2i, B2i));
+    const float2 ABr = fma_rn(A2r, B2r, mul_rn(A2i, B2i)), ABi = sub_rn(mul_rn(A2i, B2r), mul_rn(A2r, B2i));  // A conj(B)
+    const float2 R = td_rate(tt, AA, BB, ABr, ABi);
+    const bool ok0 = v0 && R.x > 0.f, ok1 = v1 && R.y > 0.f;
+    bad += (unsigned)(v0 && !ok0) + (unsigned)(v1 && !ok1);
+    lf.add(make_float2(ok0 ? lg2(R.x) : 0.f, ok1 ? lg2(R.y) : 0.f));
+    if constexpr (GRAD) {
+      const float2 invR = make_float2(ok0 ? rcp(R.x) : 0.f, ok1 ? rcp(R.y) : 0.f);
+      // V / R, V = (T_ch + T_c) A* + (T_sh - i T_s) B* = 2 P A* + (T_sh - i T_s) B*; mVi = -Im V / R
+      const float2 c1 = mul_rn(mul_rn(splat(2.f), tt.P), invR), sh = mul_rn(tt.Tsh, invR), ss = mul_rn(tt.Ts, invR);
+      const float2 Vr = sub_rn(fma_rn(c1, A2r, mul_rn(sh, B2r)), mul_rn(ss, B2i));
+      const float2 mVi = fma_rn(c1, A2i, fma_rn(sh, B2i, mul_rn(ss, B2r)));
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float2 vr = splat(e ? Vr.y : Vr.x), vi = splat(e ? -mVi.y : -mVi.x);
+#pragma unroll
+        for (int p = 0; p < KB / 2; ++p) {
+          if (p >= planes) break;
+          const float4 v = load(e, p);
+          const float2 a0 = make_float2(v.x, v.y), a1 = make_float2(v.z, v.w);
+          G1[2 * p] = fma(vr, a0, G1[2 * p]);
+          G2[2 * p] = fma(vi, a0, G2[2 * p]);
+          G1[2 * p + 1] = fma(vr, a1, G1[2 * p + 1]);
+          G2[2 * p + 1] = fma(vi, a1, G2[2 * p + 1]);
+        }
+      }
+      time_lanes(a.tc, t, tt, AA, BB, ABr, ABi, invR, lt);
+    }
   };
+  __syncthreads();  // barriers initialised and the table copied before any thread uses them
+  const long long wlim = tile_wait_limit(counters);
   bool gave_up = false;
   for (int j = 0; tile_of(j) < tb1; ++j) {
     const int64_t t = tile_of(j);
@@ -452,19 +480,33 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f32_kernel(const __grid_con
       gave_up = true;
       break;
     }
-    const bool staged = full(t);
-    const int64_t i = t * TE + threadIdx.x;
-    if (staged || (i >= begin && i < end)) {
+    if (full(t)) {
       const float4* sb = s_tile + (size_t)(j % NST) * stage_f4 + threadIdx.x;
-#pragma unroll
-      for (int p = 0; p < KB / 2; ++p)
-        if (p < planes) v[p] = staged ? sb[(size_t)p * TE] : __ldg(cache + (int64_t)p * n + i);
-      event(staged ? reinterpret_cast<const float*>(s_tile + (size_t)(j % NST) * stage_f4 + (size_t)planes * TE)[threadIdx.x]
-                   : __ldg(tcol + i));
+      const float* st = reinterpret_cast<const float*>(s_tile + (size_t)(j % NST) * stage_f4 + (size_t)planes * TE) + threadIdx.x;
+      pair([&](int e, int p) { return sb[(size_t)p * TE + e * kBlock]; }, make_float2(st[0], st[kBlock]), true, true);
+    } else {
+      const int64_t i0 = t * TE + threadIdx.x, i1 = i0 + kBlock;
+      const bool v0 = i0 >= begin && i0 < end, v1 = i1 >= begin && i1 < end;
+      // an event outside the range takes the other's place, with weight 0
+      if (v0 || v1) {
+        const int64_t j0 = v0 ? i0 : i1, j1 = v1 ? i1 : i0;
+        pair([&](int e, int p) { return __ldg(cache + (int64_t)p * n + (e ? j1 : j0)); },
+             make_float2(__ldg(tcol + j0), __ldg(tcol + j1)), v0, v1);
+      }
     }
     s_ring.release(j, issue);
   }
   s_ring.finish(gave_up, counters);
+  TdAcc<float, KB> acc;
+  acc.lf = dd_mul(lf.value(), ddf{kLn2Hi, kLn2Lo});
+  acc.bad = bad;
+#pragma unroll
+  for (int k = 0; k < KB; ++k) {
+    acc.lre[k] = G1[k].x - G2[k].y;
+    acc.lim[k] = -(G1[k].y + G2[k].x);
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) acc.lt[j] = lt[j].x + lt[j].y;
   td4_finish<float, KB, GRAD>(a, acc, begin, end, partials, counters, result, out_mode, s_red, s_bad);
 }
 
@@ -781,12 +823,14 @@ static int launch_td4_f32(goo_model* m, const void* cache, const goo_dataset* ds
   Td4Args<float> a;
   td4_args<float>(m, theta, ds->n, a);
   td4_norm_terms<float>(m, GOO_F32, a);
-  const size_t smem = (size_t)kTdStages * ((size_t)a.planes * kTdTile * sizeof(float4) + kTdTile * sizeof(float));
+  const Fp32Tables* tables = nullptr;
+  GOO_TRY(fp32_tables(ctx, &tables));
+  const size_t smem = (size_t)kTdStages<KB> * ((size_t)a.planes * kTdTile * sizeof(float4) + kTdTile * sizeof(float));
   static bool configured[kMaxDevicesTd] = {};
   if (ctx->device < 0 || ctx->device >= kMaxDevicesTd) return set_error(GOO_ERR_ARG, "device %d", ctx->device);
   if (!configured[ctx->device]) {
     GOO_CUDA_TRY(cudaFuncSetAttribute(td4_nll_f32_kernel<KB, GRAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)((size_t)kTdStages * ((KB / 2) * kTdTile * sizeof(float4) + kTdTile * sizeof(float)))));
+                                      (int)((size_t)kTdStages<KB> * ((KB / 2) * kTdTile * sizeof(float4) + kTdTile * sizeof(float)))));
     configured[ctx->device] = true;
   }
   const int occ = cached_occupancy((const void*)td4_nll_f32_kernel<KB, GRAD>, ctx->device, kBlock, smem);
@@ -795,7 +839,7 @@ static int launch_td4_f32(goo_model* m, const void* cache, const goo_dataset* ds
   GOO_TRY(ensure_partials(ctx, (size_t)nb * TdLanes<KB, GRAD>::NS));
   {
     LaunchScope ls(ctx, GRAD ? "td4_nll_grad_f32" : "td4_nll_f32");
-    td4_nll_f32_kernel<KB, GRAD><<<nb, kBlock, smem, ctx->stream>>>(a, (const float4*)cache, ds->d32[5], begin, end,
+    td4_nll_f32_kernel<KB, GRAD><<<nb, kBlock, smem, ctx->stream>>>(a, (const float4*)cache, ds->d32[5], tables, begin, end,
                                                                    ctx->scratch.partials, ctx->scratch.counters,
                                                                    ctx->scratch.result_out, out_mode);
   }

@@ -118,10 +118,19 @@ static const WeidemanTables& weideman() {
 // ---------------------------------------------------------------------------------------
 // decay-time terms
 // ---------------------------------------------------------------------------------------
-template <typename T>
+// V: float or double (one event), float2 (two events, packed FP32).
+template <typename V>
 struct TimeTerms {
-  T P, Q, Tsh, Ts;
-  T phi;  // N(t; 0, s)
+  V P, Q, Tsh, Ts;
+  V phi;  // N(t; 0, s)
+};
+template <typename V>
+struct ScalarOf {
+  using type = V;
+};
+template <>
+struct ScalarOf<float2> {
+  using type = float;
 };
 
 // Orders of the moment series (w_0 .. w_(2K+1)), and the largest
@@ -221,15 +230,26 @@ __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, 
 __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float2 mul_rn(float2 a, float2 b) { return pk::mul(a, b); }
+__device__ __forceinline__ float2 sub_rn(float2 a, float2 b) { return pk::fma(b, pk::splat(-1.f), a); }
+__device__ __forceinline__ float2 fma_rn(float2 a, float2 b, float2 c) { return pk::fma(a, b, c); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ float2 add_rn(float2 a, float2 b) { return pk::add(a, b); }
+// a scalar constant in every element of V
+__device__ __forceinline__ float in(float, float c) { return c; }
+__device__ __forceinline__ double in(double, double c) { return c; }
+__device__ __forceinline__ float2 in(float2, float c) { return pk::splat(c); }
 
 // R = |A|^2 P + |B|^2 Q + Re(A B*) T_sh + Im(A B*) T_s
-template <typename T>
-__device__ __forceinline__ T td_rate(const TimeTerms<T>& tt, T AA, T BB, T ABr, T ABi) {
+template <typename V>
+__device__ __forceinline__ V td_rate(const TimeTerms<V>& tt, V AA, V BB, V ABr, V ABi) {
   return fma_rn(ABi, tt.Ts, fma_rn(ABr, tt.Tsh, fma_rn(BB, tt.Q, mul_rn(AA, tt.P))));
 }
 
-// exp and erfcx / 2 of the path's precision: CUDA's in FP32, the tables of fp64.cuh in FP64.
-template <typename T>
+// exp and erfcx / 2 of the path's precision: CUDA's for one FP32 event, the tables of fp64.cuh in FP64 and
+// for two FP32 events.
+template <typename V>
 struct TdMath;
 template <>
 struct TdMath<float> {
@@ -240,6 +260,34 @@ struct TdMath<float> {
   }
   __device__ __forceinline__ static bool nonneg(float u) { return u >= 0.f; }
   __device__ __forceinline__ static bool below(float t, float limit) { return t < limit; }
+};
+// Two events: exp from the hardware's 2^x of x log2(e) rounded once, the product's rounding error (an FMA gives
+// it) applied as a factor; erfcx from its table in shared memory.
+template <>
+struct TdMath<float2> {
+  const Fp32Tables& tab;
+  __device__ __forceinline__ float2 exp(float2 v) const {
+    const float2 np = mul_rn(v, pk::splat(-kLog2eHi));  // - v log2 e
+    const float2 e = fma_rn(v, pk::splat(kLog2eLo), fma_rn(v, pk::splat(kLog2eHi), np));
+    const float2 y = make_float2(pk::ex2(-np.x), pk::ex2(-np.y));
+    return fma_rn(mul_rn(y, e), pk::splat(kLn2Hi), y);
+  }
+  // gauss erfcx(|u|) / 2; where u <= -6 it is below 2^-52 of the exponential it is subtracted from
+  // (conv_real) and is left out
+  __device__ __forceinline__ float2 gauss_herfcx(float2 gauss, float2 u) const {
+    const float2 a = make_float2(fminf(fabsf(u.x), (float)kErfcxMax), fminf(fabsf(u.y), (float)kErfcxMax));
+    const float2 m = fma_rn(a, pk::splat((float)kErfcxStep), pk::splat(12582912.f));  // 1.5 2^23: the node in the low bits
+    const float2 r = fma_rn(add_rn(m, pk::splat(-12582912.f)), pk::splat(-1.f / kErfcxStep), a);
+    const int i0 = __float_as_int(m.x) & 0xff, i1 = __float_as_int(m.y) & 0xff;
+    float2 p = make_float2(tab.herfcx[kErfcxDeg32][i0], tab.herfcx[kErfcxDeg32][i1]);
+#pragma unroll
+    for (int d = kErfcxDeg32 - 1; d >= 0; --d)
+      p = fma_rn(p, r, make_float2(tab.herfcx[d][i0], tab.herfcx[d][i1]));
+    float2 h = mul_rn(gauss, p);
+    if (fabsf(u.x) > (float)kErfcxMax) h.x = u.x < 0.f ? 0.f : mul_rn(gauss.x, 0.5f * erfcxf(u.x));
+    if (fabsf(u.y) > (float)kErfcxMax) h.y = u.y < 0.f ? 0.f : mul_rn(gauss.y, 0.5f * erfcxf(u.y));
+    return h;
+  }
 };
 template <>
 struct TdMath<double> {
@@ -260,12 +308,14 @@ struct TdMath<double> {
 // E(g) for real g (gauss = exp(-t^2/2s^2)): with h = gauss erfcx(|u|) / 2, u = (g s^2 - t) / (s sqrt 2),
 // E = h for u >= 0 and exp(g^2 s^2 / 2 - g t) - h below, selected, so that a warp whose events
 // lie on both sides evaluates erfcx once.  hg2s2 = g^2 s^2 / 2.
-template <typename T>
-__device__ __forceinline__ T conv_real(const TdMath<T>& F, T g, T gs2, T hg2s2, T ir2s, T t, T gauss) {
-  const T u = mul_rn(sub_rn(gs2, t), ir2s);
-  const T h = F.gauss_herfcx(gauss, u);
-  const T x = sub_rn(F.exp(fma_rn(-g, t, hg2s2)), h);
-  return F.nonneg(u) ? h : x;
+template <typename V, typename T>
+__device__ __forceinline__ V conv_real(const TdMath<V>& F, T g, T gs2, T hg2s2, T ir2s, V t, V gauss) {
+  const V z{};
+  const V u = mul_rn(sub_rn(in(z, gs2), t), in(z, ir2s));
+  const V h = F.gauss_herfcx(gauss, u);
+  const V x = sub_rn(F.exp(fma_rn(in(z, -g), t, in(z, hg2s2))), h);
+  if constexpr (sizeof(V) > sizeof(T)) return make_float2(u.x >= 0.f ? h.x : x.x, u.y >= 0.f ? h.y : x.y);
+  else return F.nonneg(u) ? h : x;
 }
 
 // E(g) for complex g = (gr, gi)
@@ -297,8 +347,8 @@ template <typename T>
 __device__ __forceinline__ void time_terms_direct(const TdMath<T>& F, const TimeCoef<T>& c, const T* wa, int wN, T wL,
                                                   T t, T gauss, TimeTerms<T>& R) {
   const T gp = c.G * (T(1) - c.y), gm = c.G * (T(1) + c.y);
-  const T Ep = conv_real<T>(F, gp, gp * c.s2, T(0.5) * gp * gp * c.s2, c.ir2s, t, gauss);
-  const T Em = conv_real<T>(F, gm, gm * c.s2, T(0.5) * gm * gm * c.s2, c.ir2s, t, gauss);
+  const T Ep = conv_real(F, gp, gp * c.s2, T(0.5) * gp * gp * c.s2, c.ir2s, t, gauss);
+  const T Em = conv_real(F, gm, gm * c.s2, T(0.5) * gm * gm * c.s2, c.ir2s, t, gauss);
   T Ecr, Eci;
   conv_complex<T>(F, c.G, -c.G * c.x, t, c.s, gauss, wa, wN, wL, Ecr, Eci);
   const T Tch = T(0.5) * (Ep + Em);
@@ -310,26 +360,27 @@ __device__ __forceinline__ void time_terms_direct(const TdMath<T>& F, const Time
 
 // The decay-time terms by the moment series of order KU (small mixing; see the top of this
 // file).
-template <typename T, int KU>
-__device__ __forceinline__ void time_terms_series(const TdMath<T>& F, const TimeCoef<T>& c, T t, T gauss,
-                                                  TimeTerms<T>& R) {
+template <typename V, typename T, int KU>
+__device__ __forceinline__ void time_terms_series(const TdMath<V>& F, const TimeCoef<T>& c, V t, V gauss,
+                                                  TimeTerms<V>& R) {
   constexpr int NW = 2 * KU + 2;
-  const T v = sub_rn(t, c.Gs2), Gv = mul_rn(c.G, v);
-  T w[NW];
-  w[0] = conv_real<T>(F, c.G, c.Gs2, c.hG2s2, c.ir2s, t, gauss);
-  w[1] = mul_rn(c.G, fma_rn(v, w[0], mul_rn(c.s2, R.phi)));
+  const V z{};
+  const V v = sub_rn(t, in(z, c.Gs2)), Gv = mul_rn(in(z, c.G), v);
+  V w[NW];
+  w[0] = conv_real(F, c.G, c.Gs2, c.hG2s2, c.ir2s, t, gauss);
+  w[1] = mul_rn(in(z, c.G), fma_rn(v, w[0], mul_rn(in(z, c.s2), R.phi)));
 #pragma unroll
-  for (int n = 1; n < NW - 1; ++n) w[n + 1] = fma_rn(Gv, w[n], mul_rn(c.nG2s2[n], w[n - 1]));
+  for (int n = 1; n < NW - 1; ++n) w[n + 1] = fma_rn(Gv, w[n], mul_rn(in(z, c.nG2s2[n]), w[n - 1]));
   R.P = w[0];
-  R.Q = mul_rn(c.b[1], w[2]);
-  R.Tsh = mul_rn(c.ysh[0], w[1]);
-  R.Ts = mul_rn(c.xs[0], w[1]);
+  R.Q = mul_rn(in(z, c.b[1]), w[2]);
+  R.Tsh = mul_rn(in(z, c.ysh[0]), w[1]);
+  R.Ts = mul_rn(in(z, c.xs[0]), w[1]);
 #pragma unroll
   for (int m = 1; m <= KU; ++m) {
-    R.P = fma_rn(c.a[m], w[2 * m], R.P);
-    if (m > 1) R.Q = fma_rn(c.b[m], w[2 * m], R.Q);
-    R.Tsh = fma_rn(c.ysh[m], w[2 * m + 1], R.Tsh);
-    R.Ts = fma_rn(c.xs[m], w[2 * m + 1], R.Ts);
+    R.P = fma_rn(in(z, c.a[m]), w[2 * m], R.P);
+    if (m > 1) R.Q = fma_rn(in(z, c.b[m]), w[2 * m], R.Q);
+    R.Tsh = fma_rn(in(z, c.ysh[m]), w[2 * m + 1], R.Tsh);
+    R.Ts = fma_rn(in(z, c.xs[m]), w[2 * m + 1], R.Ts);
   }
 }
 
@@ -343,31 +394,57 @@ __device__ __forceinline__ void time_terms_g(const TdMath<T>& F, const TimeCoef<
   R.phi = mul_rn(c.k_phi, gauss);
   if (F.below(t, c.t_series)) {
     // the same order for every event of a launch (a uniform branch)
-    if (c.ku == TimeCoef<T>::K) time_terms_series<T, TimeCoef<T>::K>(F, c, t, gauss, R);
-    else time_terms_series<T, TimeCoef<T>::K - 1>(F, c, t, gauss, R);
+    if (c.ku == TimeCoef<T>::K) time_terms_series<T, T, TimeCoef<T>::K>(F, c, t, gauss, R);
+    else time_terms_series<T, T, TimeCoef<T>::K - 1>(F, c, t, gauss, R);
   } else {
     time_terms_direct<T>(F, c, wa, wN, wL, t, gauss, R);
   }
 }
 
+// The same for two events, packed; an event above the series' limit goes through the scalar code.
+__device__ __forceinline__ void time_terms_pair(const TdMath<float2>& F, const TimeCoef<float>& c, const float* wa,
+                                                int wN, float wL, float2 t, TimeTerms<float2>& R) {
+  const float2 gauss = F.exp(mul_rn(mul_rn(mul_rn(t, pk::splat(-1.f)), t), pk::splat(c.is2h)));
+  R.phi = mul_rn(pk::splat(c.k_phi), gauss);
+  if (c.ku == TimeCoef<float>::K) time_terms_series<float2, float, TimeCoef<float>::K>(F, c, t, gauss, R);
+  else time_terms_series<float2, float, TimeCoef<float>::K - 1>(F, c, t, gauss, R);
+  if (!(t.x < c.t_series && t.y < c.t_series)) {
+#pragma unroll 1
+    for (int e = 0; e < 2; ++e) {
+      const float te = e ? t.y : t.x;
+      if (te < c.t_series) continue;
+      TimeTerms<float> S;
+      time_terms_direct<float>(TdMath<float>{}, c, wa, wN, wL, te, expf(mul_rn(mul_rn(-te, te), c.is2h)), S);
+      (e ? R.P.y : R.P.x) = S.P;
+      (e ? R.Q.y : R.Q.x) = S.Q;
+      (e ? R.Tsh.y : R.Tsh.x) = S.Tsh;
+      (e ? R.Ts.y : R.Ts.x) = S.Ts;
+    }
+  }
+}
+
 // Adds one event's lanes X / R, Y / R, Z / R and the d^2 / dt^2 bracket / R (see the top of this
 // file) to lt; AA = |A|^2, BB = |B|^2, (ABr, ABi) = A conj(B).
-template <typename T>
-__device__ __forceinline__ void time_lanes(const TimeCoef<T>& c, T t, const TimeTerms<T>& tt, T AA, T BB, T ABr,
-                                           T ABi, T invR, T (&lt)[4]) {
-  const T v = t - c.Gs2;
-  const T Tch = tt.P + tt.Q, Tc = tt.P - tt.Q;
-  const T ysh = c.hy * tt.Tsh, xs = c.hx * tt.Ts;
-  const T CP = fma_rn(v, tt.P, fma_rn(c.s2, tt.phi, ysh - xs)), CQ = fma_rn(v, tt.Q, ysh + xs);
-  const T Csh = fma_rn(v, tt.Tsh, c.fy * Tch), Cs = fma_rn(v, tt.Ts, c.fx * Tc);
-  const T hp = T(0.5) * (AA + BB), hm = T(0.5) * (BB - AA);
-  lt[0] = fma_rn(fma_rn(hm, Cs, ABi * (CP - CQ)), invR, lt[0]);
-  lt[1] = fma_rn(fma_rn(hp, Csh, ABr * (CP + CQ)), invR, lt[1]);
-  lt[2] = fma_rn(fma_rn(AA, CP, fma_rn(BB, CQ, fma_rn(ABr, Csh, ABi * Cs))), invR, lt[2]);
-  const T Ey = fma_rn(hp, tt.Tsh, ABr * Tch), Ex = fma_rn(hm, tt.Ts, ABi * Tc);
-  const T Ry = fma_rn(hp, Tch, ABr * tt.Tsh), Rx = fma_rn(-hm, Tc, ABi * tt.Ts);
-  const T b = fma_rn(-fma_rn(t, c.is2, c.G), AA, fma_rn(c.Gy, ABr, c.Gx * ABi));
-  const T q = fma_rn(tt.phi, b, fma_rn(c.Gy2, Ry, fma_rn(-c.Gx2, Rx, fma_rn(-c.qy, Ey, -c.qx * Ex))));
+template <typename V, typename T>
+__device__ __forceinline__ void time_lanes(const TimeCoef<T>& c, V t, const TimeTerms<V>& tt, V AA, V BB, V ABr, V ABi,
+                                           V invR, V (&lt)[4]) {
+  const V z{};
+  auto K = [&](T x) { return in(z, x); };
+  const V v = sub_rn(t, K(c.Gs2));
+  const V Tch = add_rn(tt.P, tt.Q), Tc = sub_rn(tt.P, tt.Q);
+  const V ysh = mul_rn(K(c.hy), tt.Tsh), xs = mul_rn(K(c.hx), tt.Ts);
+  const V CP = fma_rn(v, tt.P, fma_rn(K(c.s2), tt.phi, sub_rn(ysh, xs))), CQ = fma_rn(v, tt.Q, add_rn(ysh, xs));
+  const V Csh = fma_rn(v, tt.Tsh, mul_rn(K(c.fy), Tch)), Cs = fma_rn(v, tt.Ts, mul_rn(K(c.fx), Tc));
+  const V hp = mul_rn(K(T(0.5)), add_rn(AA, BB)), hm = mul_rn(K(T(0.5)), sub_rn(BB, AA));
+  lt[0] = fma_rn(fma_rn(hm, Cs, mul_rn(ABi, sub_rn(CP, CQ))), invR, lt[0]);
+  lt[1] = fma_rn(fma_rn(hp, Csh, mul_rn(ABr, add_rn(CP, CQ))), invR, lt[1]);
+  lt[2] = fma_rn(fma_rn(AA, CP, fma_rn(BB, CQ, fma_rn(ABr, Csh, mul_rn(ABi, Cs)))), invR, lt[2]);
+  // E_y, E_x, R_y and R_x each times its factor: G^2 (y^2 R_y - x^2 R_x - 2 (y E_y + x E_x))
+  const V Ey = fma_rn(hp, tt.Tsh, mul_rn(ABr, Tch)), Ex = fma_rn(hm, tt.Ts, mul_rn(ABi, Tc));
+  const V Ry = fma_rn(hp, Tch, mul_rn(ABr, tt.Tsh)), mRx = fma_rn(hm, Tc, mul_rn(K(T(-1)), mul_rn(ABi, tt.Ts)));
+  const V b = fma_rn(fma_rn(t, K(-c.is2), K(-c.G)), AA, fma_rn(K(c.Gy), ABr, mul_rn(K(c.Gx), ABi)));
+  const V q = fma_rn(tt.phi, b,
+                     fma_rn(K(c.Gy2), Ry, fma_rn(K(c.Gx2), mRx, fma_rn(K(-c.qy), Ey, mul_rn(K(-c.qx), Ex)))));
   lt[3] = fma_rn(q, invR, lt[3]);
 }
 
