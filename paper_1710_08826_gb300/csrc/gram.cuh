@@ -29,6 +29,10 @@ constexpr int kGramLanes = 2 * kGramRows * kGramCols;  // lane 2 (k kGramCols + 
 constexpr int kGramAll = kGramLanes + 2 * kGramRows;   // then the rows' own sums (the constant amplitude's column)
 constexpr int kGramTickets = 16;  // the tiles' tickets: counters[kGramTickets ..)
 constexpr int kGramRun = 16;      // FP32: events summed in registers at a time
+// FP32: events requested ahead.  Two in flight per thread of one block per SM held 37 KB per SM, which at
+// the memory's latency is 3/4 of its bandwidth
+template <bool DIAG>
+constexpr int kGramAhead = DIAG ? 4 : 2;
 // threads per block: FP32 the most whose lanes fit in shared memory, FP64 the most whose sums fit in registers
 template <typename T>
 constexpr int kGramBlock = sizeof(T) == 4 ? 384 : 256;
@@ -155,11 +159,12 @@ __device__ __forceinline__ void gram_tile_sums(const GramArgs& A, const GramArgs
   GramAcc<T, EXACT> acc;
   acc.clear();
   auto lane = [&](int j) -> ddf& { return s[j * kGramBlock<T>]; };
-  // the two events ahead are requested before this one's products
-  V nx[2][kGramRows], ny[2][kGramCols];
+  // the D events ahead are requested before this one's products; a diagonal tile's rows are its first columns
+  constexpr int D = kGramAhead<DIAG>;
+  V nx[D][kGramRows], ny[D][kGramCols];
   auto fetch = [&](int b, int64_t j) {
     if (j >= A.n) return;
-    GramAmp<T>::load(xc, A.n, j, t.r0, A.nbw, nx[b]);
+    if (!DIAG) GramAmp<T>::load(xc, A.n, j, t.r0, A.nbw, nx[b]);
     GramAmp<T>::load(yc, A.n, j, t.c0, A.nbw, ny[b]);
   };
   auto event = [&](int b) {
@@ -168,11 +173,11 @@ __device__ __forceinline__ void gram_tile_sums(const GramArgs& A, const GramArgs
       if (t.c0 + l >= A.nbw) break;  // uniform
 #pragma unroll
       for (int k = 0; k < kGramRows; ++k)
-        if (!DIAG || l >= k) acc.m[k][l].mul_add(nx[b][k], ny[b][l]);
+        if (!DIAG || l >= k) acc.m[k][l].mul_add(DIAG ? ny[b][k] : nx[b][k], ny[b][l]);
     }
     if (DIAG) {
 #pragma unroll
-      for (int k = 0; k < kGramRows; ++k) acc.row[k].add(nx[b][k]);
+      for (int k = 0; k < kGramRows; ++k) acc.row[k].add(ny[b][k]);
     }
   };
   if constexpr (RUNS) {
@@ -199,16 +204,16 @@ __device__ __forceinline__ void gram_tile_sums(const GramArgs& A, const GramArgs
       }
       acc.clear();
     };
-    fetch(0, i);
-    fetch(1, i + stride);
+#pragma unroll
+    for (int e = 0; e < D; ++e) fetch(e, i + e * stride);
     while (i < A.n) {
 #pragma unroll 1
-      for (int r = 0; r < kGramRun / 2 && i < A.n; ++r, i += 2 * stride) {
-        event(0);
-        fetch(0, i + 2 * stride);
-        if (i + stride < A.n) {
-          event(1);
-          fetch(1, i + 3 * stride);
+      for (int r = 0; r < kGramRun / D && i < A.n; ++r, i += D * stride) {
+#pragma unroll
+        for (int e = 0; e < D; ++e) {
+          if (i + e * stride >= A.n) break;
+          event(e);
+          fetch(e, i + (D + e) * stride);
         }
       }
       flush();
