@@ -1219,7 +1219,10 @@ static int ensure_cache(goo_model* m, const goo_dataset* ds_c, int precision, co
   return GOO_OK;
 }
 
-static int ensure_gram(goo_model* m, int precision) {
+// The Gram matrix at the current lineshapes.  `ds`: a dataset whose cache the caller needs next; when the
+// matrix is rebuilt, so is that cache, behind the Gram kernel, and the GPU is busy while the host takes the
+// matrix and launches the likelihood (2M events, 1M MC points: @@).
+static int ensure_gram(goo_model* m, int precision, const goo_dataset* ds = nullptr) {
   DalitzModel& d = *m->dalitz;
   const int pi = precision == GOO_F32 ? 0 : 1;
   if (!d.mc) return set_error(GOO_ERR_STATE, "amplitude model has no MC normalisation sample (goo_model_set_norm)");
@@ -1229,7 +1232,10 @@ static int ensure_gram(goo_model* m, int precision) {
   GOO_TRY(ensure_cache(m, d.mc, precision, &cache));
   if (d.mc->n < 1) return set_error(GOO_ERR_ARG, "the MC normalisation sample is empty");
   GOO_TRY(gram_matrices(m->ctx, precision, false, 1, &cache, &cache, d.mc->n, d.nbw, d.K, d.gram_dev[pi],
-                        d.gram_host[pi], pi == 0 ? "gram_f32" : "gram_f64"));
+                        d.gram_host[pi], pi == 0 ? "gram_f32" : "gram_f64", [&]() -> int {
+                          const void* c = nullptr;
+                          return ds ? ensure_cache(m, ds, precision, &c) : GOO_OK;
+                        }));
   d.gram_key[pi] = key;
   return GOO_OK;
 }
@@ -1452,8 +1458,8 @@ static int launch_ls_sel(goo_model* m, const goo_dataset* ds, int64_t begin, int
 
 // The three MC Gram matrices of the time-dependent three-body model (G_aa, G_bb, G_ab) in
 // `precision`, rebuilt when the lineshapes or the MC sample change; a host copy for
-// goo_normalise.
-static int ensure_td_grams(goo_model* m, int precision) {
+// goo_normalise.  `ds` as in ensure_gram, both its caches.
+static int ensure_td_grams(goo_model* m, int precision, const goo_dataset* ds = nullptr) {
   DalitzModel& d = *m->dalitz;
   goo_ctx* ctx = m->ctx;
   const int pi = precision == GOO_F32 ? 0 : 1;
@@ -1466,7 +1472,12 @@ static int ensure_td_grams(goo_model* m, int precision) {
   GOO_TRY(ensure_cache(m, d.mc, precision, &cb, true));
   const void *x[3] = {ca, cb, ca}, *y[3] = {ca, cb, cb};
   GOO_TRY(gram_matrices(ctx, precision, true, 3, x, y, d.mc->n, d.nbw, d.K, nullptr, d.gram3_host[pi],
-                        pi == 0 ? "td3_gram_f32" : "td3_gram_f64"));
+                        pi == 0 ? "td3_gram_f32" : "td3_gram_f64", [&]() -> int {
+                          const void* c = nullptr;
+                          if (!ds) return GOO_OK;
+                          GOO_TRY(ensure_cache(m, ds, precision, &c));
+                          return ensure_cache(m, ds, precision, &c, true);
+                        }));
   d.gram3_key[pi] = key;
   return GOO_OK;
 }
@@ -1788,7 +1799,7 @@ int dalitz_nll(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, 
   if (d.td) {
     // time-dependent three-body model: amplitude caches at the event and the exchanged point
     if (ds->ncols <= d.col_t) return set_error(GOO_ERR_ARG, "dataset lacks the decay-time column");
-    GOO_TRY(ensure_td_grams(m, precision));
+    GOO_TRY(ensure_td_grams(m, precision, end > begin ? ds : nullptr));
     if (end <= begin) {
       for (int i = 0; i < nout; ++i) out[i] = 0.0;
       return GOO_OK;
@@ -1819,7 +1830,7 @@ int dalitz_nll(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, 
                     : launch_ls_sel<double, false>(m, ds, begin, end, theta, out_mode)));
     }
   } else {
-  GOO_TRY(ensure_gram(m, precision));
+  GOO_TRY(ensure_gram(m, precision, end > begin ? ds : nullptr));
   const int pi = precision == GOO_F32 ? 0 : 1;
   if (end <= begin) {
     for (int i = 0; i < nout; ++i) out[i] = 0.0;

@@ -22,7 +22,8 @@ static int launch_gram_tiles(goo_ctx* ctx, GramArgs& A, double* out, double* out
 }
 
 int gram_matrices(goo_ctx* ctx, int precision, bool exact, int nmat, const void* const* x, const void* const* y,
-                  int64_t n, int nbw, int K, double* out, double* host, const char* name) {
+                  int64_t n, int nbw, int K, double* out, double* host, const char* name,
+                  const std::function<int()>& behind) {
   const int fields = nmat * 2 * K * K;
   if (nmat > 3 || fields > kGramRecord) return set_error(GOO_ERR_STATE, "Gram matrices of %d fields", fields);
   Scratch& s = ctx->scratch;
@@ -74,7 +75,9 @@ int gram_matrices(goo_ctx* ctx, int precision, bool exact, int nmat, const void*
     else if (exact) GOO_TRY((launch_gram_tiles<float, true>(ctx, A, out, s.gram_host, name)));
     else GOO_TRY((launch_gram_tiles<float, false>(ctx, A, out, s.gram_host, name)));
   }
-  GOO_TRY(read_mapped(ctx, s.gram_host, fields, host));
+  const int queued = behind ? behind() : GOO_OK;
+  GOO_TRY(read_mapped(ctx, s.gram_host, fields, host));  // in any case: the kernel writes the record
+  GOO_TRY(queued);
   // of two different caches: mean X_k conj(1) and mean 1 conj(Y_l) from the caches' own matrices
   for (int q = 0; q < nmat && nbw < K; ++q)
     for (int h = 0; h < nmat; ++h) {

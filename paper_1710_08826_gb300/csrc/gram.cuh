@@ -19,6 +19,8 @@
 // Each tile's last block adds its blocks' sums in block order; results are bitwise repeatable.
 #pragma once
 
+#include <functional>
+
 #include "common.cuh"
 
 namespace goo {
@@ -294,10 +296,12 @@ __global__ void __launch_bounds__(kGramBlock<T>, 1) gram_tile_kernel(const __gri
 }
 
 // Sums the nmat (1..3) K x K matrices of the caches x[q], y[q] over n events into `host` (nmat x K x K
-// complex) and, one Hermitian matrix only, `out` on the device (or null): launches the kernel and waits for the
-// mapped record.  A matrix of two different caches needs both caches' own matrices in the same
-// call.  exact: see above (FP32).
+// complex) and, one Hermitian matrix only, `out` on the device (or null): launches the kernel, queues
+// what `behind` queues (device work that does not need the matrices, so that it runs while the host
+// waits for them and launches what does), and waits for the mapped record.  A matrix of two different caches
+// needs both caches' own matrices in the same call.  exact: see above (FP32).
 int gram_matrices(goo_ctx* ctx, int precision, bool exact, int nmat, const void* const* x, const void* const* y,
-                  int64_t n, int nbw, int K, double* out, double* host, const char* name);
+                  int64_t n, int nbw, int K, double* out, double* host, const char* name,
+                  const std::function<int()>& behind = {});
 
 }  // namespace goo
