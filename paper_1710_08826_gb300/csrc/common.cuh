@@ -18,6 +18,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <string>
+#include <utility>
 #include <vector>
 #endif
 
@@ -192,6 +193,23 @@ struct LaunchScope {
   LaunchScope(goo_ctx* c, const char* n);
   ~LaunchScope();
 };
+// Launches `kernel` as a programmatic dependent of the kernel before it in `stream`: its blocks may
+// start while that one's last blocks run, and it calls grid_dep_wait() before it touches what the
+// other uses.
+template <typename... P, typename... A>
+cudaError_t launch_early(void (*kernel)(P...), int blocks, int threads, size_t smem, cudaStream_t stream, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 int grid_blocks(goo_ctx* ctx, int64_t work_items, int blocks_per_sm);
 // Resident blocks per SM of `kernel` (a __global__ function or a run-time compiled kernel
 // handle) with `block` threads and `smem` bytes of dynamic shared memory on the current

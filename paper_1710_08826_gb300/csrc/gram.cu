@@ -15,8 +15,8 @@ static int launch_gram_tiles(goo_ctx* ctx, GramArgs& A, double* out, double* out
   for (int t = 0; t < A.ntiles; ++t) blocks += A.tile[t].nblk;
   GOO_TRY(ensure_partials(ctx, (size_t)blocks * kGramAll));
   LaunchScope ls(ctx, name);
-  gram_tile_kernel<T, EXACT><<<blocks, kGramBlock<T>, kGramSmem<T>, ctx->stream>>>(A, ctx->scratch.partials, ctx->scratch.counters,
-                                                                         out, out_host);
+  GOO_CUDA_TRY(launch_early(gram_tile_kernel<T, EXACT>, blocks, kGramBlock<T>, kGramSmem<T>, ctx->stream, A,
+                            ctx->scratch.partials, ctx->scratch.counters, out, out_host));
   GOO_CUDA_TRY(cudaGetLastError());
   return GOO_OK;
 }

@@ -253,8 +253,10 @@ __global__ void __launch_bounds__(kGramBlock<T>, 1) gram_tile_kernel(const __gri
   const int b = blockIdx.x - t.blk0;
   ddf* buf = reinterpret_cast<ddf*>(s_gram);
   const int64_t i0 = b * (int64_t)kGramBlock<T> + threadIdx.x, stride = (int64_t)t.nblk * kGramBlock<T>;
+  grid_dep_wait();  // the caches' kernel
   if (t.diag) gram_tile_sums<T, EXACT, true>(A, t, i0, stride, buf + threadIdx.x);
   else gram_tile_sums<T, EXACT, false>(A, t, i0, stride, buf + threadIdx.x);
+  grid_dep_launch();  // what is queued behind may take the SMs that are done
   __syncthreads();
   // lane sums over the threads: one warp per lane at a time, then the warp's tree
   float2* part = partials + (size_t)t.blk0 * kGramAll;
