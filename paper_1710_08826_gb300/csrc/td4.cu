@@ -51,6 +51,7 @@ struct Td4Dev {
   int K, pad;
   double m1, m2, m3, m4, r;
   Td4Amp amp[kTdMaxAmp];
+  double br[kTdMaxAmp], bi[kTdMaxAmp];  // the model's constant coefficients of B = sum b_k a_k
 };
 
 template <typename T>
@@ -64,6 +65,7 @@ struct Td4Args {
   // terms 2k, 2k + 1: the coefficient parameters of amplitude k; 2 kTdMaxAmp + j: the time parameters
   GradMap<2 * kTdMaxAmp + 4> map;
   int64_t n_total;  // events of the dataset (cache plane length)
+  int has_b;        // FP64: the cache holds B in plane K
   // the normalisation at theta, formed on the host in FP64 from the cached Gram matrix
   // (td4_norm_terms): N, log N, (dN / d Re c_k) / N, (dN / d Im c_k) / N and (dN / dx) / N,
   // (dN / dy) / N, (tau dN / d tau) / N
@@ -120,10 +122,18 @@ struct Td4Cols {
   const T* c[5];  // m12, m34, c12, c34, phi
 };
 
+// B += b a, one order of operations wherever B is formed
+__device__ __forceinline__ void td4_add_b(double br, double bi, double2 a, double& Br, double& Bi) {
+  Br = fma_rn(br, a.x, fma_rn(-bi, a.y, Br));
+  Bi = fma_rn(br, a.y, fma_rn(bi, a.x, Bi));
+}
+
 // Cache layout as for the three-body model: FP32 ceil(K/2) planes of float4 (re_k, im_k,
-// re_k+1, im_k+1), FP64 K planes of double2; plane p of an n-event dataset at p * n.
+// re_k+1, im_k+1), FP64 K planes of double2; plane p of an n-event dataset at p * n.  FP64, with_b: B = sum b_k a_k,
+// whose coefficients are the model's constants, in plane K (16 bytes more an event where B costs the
+// evaluation 4 K slots of the FP64 pipe).
 template <typename T>
-__global__ void td4_cache_kernel(const Td4Dev* __restrict__ tdp, Td4Cols<T> cols, int64_t n, void* cache_v) {
+__global__ void td4_cache_kernel(const Td4Dev* __restrict__ tdp, Td4Cols<T> cols, int64_t n, void* cache_v, bool with_b) {
   __shared__ Td4Dev td;
   for (int i = threadIdx.x; i < (int)(sizeof(Td4Dev) / 4); i += blockDim.x) ((int*)&td)[i] = ((const int*)tdp)[i];
   __syncthreads();
@@ -131,6 +141,7 @@ __global__ void td4_cache_kernel(const Td4Dev* __restrict__ tdp, Td4Cols<T> cols
   const T r = (T)td.r;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const T m12 = cols.c[0][i], m34 = cols.c[1][i], c12 = cols.c[2][i], c34 = cols.c[3][i], phi = cols.c[4][i];
+    double Br = 0.0, Bi = 0.0;
     for (int k = 0; k < K; ++k) {
       const Td4Amp& A = td.amp[k];
       T f1r, f1i, f2r, f2i, wr, wi;
@@ -145,8 +156,10 @@ __global__ void td4_cache_kernel(const Td4Dev* __restrict__ tdp, Td4Cols<T> cols
         plane[2 * (k & 1) + 1] = ai;
       } else {
         ((double2*)cache_v)[(int64_t)k * n + i] = make_double2(ar, ai);
+        td4_add_b(td.br[k], td.bi[k], make_double2(ar, ai), Br, Bi);
       }
     }
+    if (sizeof(T) == 8 && with_b) ((double2*)cache_v)[(int64_t)K * n + i] = make_double2(Br, Bi);
     if constexpr (sizeof(T) == 4) {
       if (K & 1) {  // zero the unused half of the last plane
         float* plane = (float*)((float4*)cache_v + (int64_t)(K / 2) * n + i);
@@ -270,19 +283,25 @@ __device__ __forceinline__ void td4_finish(const Td4Args<T>& a, TdAcc<T, KB>& ac
   result_complete(result, P > 1 ? P : 1);
 }
 
-// The FP64 sums A = sum c_k a_k and B = sum b_k a_k of event i.
+// The FP64 sums A = sum c_k a_k and B = sum b_k a_k of event i; B comes from the cache where it holds it.
 __device__ __forceinline__ void td4_sums(const Td4Args<double>& a, const double2* __restrict__ cache, int KB, int64_t i,
                                          double& Ar, double& Ai, double& Br, double& Bi) {
   Ar = Ai = Br = Bi = 0.0;
+  if (a.has_b) {
+    const double2 v = cache[(int64_t)a.K * a.n_total + i];
+    Br = v.x;
+    Bi = v.y;
+  }
 #pragma unroll
   for (int k = 0; k < KB; ++k) {
     if (k >= a.K) break;
     const double2 v = cache[(int64_t)k * a.n_total + i];
     Ar = fma(a.cr[k], v.x, fma(-a.ci[k], v.y, Ar));
     Ai = fma(a.cr[k], v.y, fma(a.ci[k], v.x, Ai));
-    Br = fma(a.br[k], v.x, fma(-a.bi[k], v.y, Br));
-    Bi = fma(a.br[k], v.y, fma(a.bi[k], v.x, Bi));
   }
+  if (!a.has_b)
+#pragma unroll 1
+    for (int k = 0; k < a.K; ++k) td4_add_b(a.br[k], a.bi[k], cache[(int64_t)k * a.n_total + i], Br, Bi);
 }
 
 // FP64: direct loads, one event per thread per grid-stride step.  Bound by the FP64 pipe's slots
@@ -290,7 +309,7 @@ __device__ __forceinline__ void td4_sums(const Td4Args<double>& a, const double2
 // product, tests on the integer pipe.  The amplitudes are read again for the gradient lanes
 // (their registers would spill; the second read costs no FP64 slot).  1M events, 10 amplitudes with
 // the gradient: 872 -> 571 us (three slots per product pair and CUDA's exp, erfcx, log and division
-// before).
+// before), 500 us with B from the cache.
 template <int KB, bool GRAD>
 __global__ void __launch_bounds__(kBlock, 2) td4_nll_f64_kernel(const __grid_constant__ Td4Args<double> a,
                                                                 const double2* __restrict__ cache,
@@ -616,8 +635,8 @@ int build_td4_model(goo_ctx* ctx, const goo_node* nodes, int n_nodes, int n_para
       if (a.par[j] < 0 || a.par[j] >= n_params) return set_error(GOO_ERR_ARG, "amplitude %d coefficient index", k);
     d->par_re[k] = a.par[0];
     d->par_im[k] = a.par[1];
-    d->br[k] = a.dval[4];
-    d->bi[k] = a.dval[5];
+    h.br[k] = d->br[k] = a.dval[4];
+    h.bi[k] = d->bi[k] = a.dval[5];
     Td4Amp& A = h.amp[k];
     A.ang = a.ival[0];
     spins_of(A.ang, A.L1, A.L2);
@@ -632,7 +651,7 @@ int build_td4_model(goo_ctx* ctx, const goo_node* nodes, int n_nodes, int n_para
     A.b0a = barrier_host(A.L1, (h.r * A.q0a) * (h.r * A.q0a));
     A.b0b = barrier_host(A.L2, (h.r * A.q0b) * (h.r * A.q0b));
   }
-  uint64_t key = 1469598103934665603ull;  // FNV-1a over the lineshape constants
+  uint64_t key = 1469598103934665603ull;  // FNV-1a over the cache's constants
   const unsigned char* bytes = (const unsigned char*)&h;
   for (size_t i = 0; i < sizeof(Td4Dev); ++i) key = (key ^ bytes[i]) * 1099511628211ull;
   d->key = key;
@@ -667,6 +686,9 @@ int td4_set_norm(goo_model* m, const goo_norm_spec* spec) {
   return GOO_OK;
 }
 
+// Bytes of the FP64 cache with B's plane.
+static size_t td4_bytes_b(const Td4Model& d, int64_t n) { return (size_t)(d.K + 1) * (size_t)n * sizeof(double2); }
+
 static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, const void** out) {
   goo_dataset* ds = const_cast<goo_dataset*>(ds_c);
   Td4Model& d = *m->td4;
@@ -685,11 +707,19 @@ static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, const
     if (slot.ptr) cudaFree(slot.ptr);
     slot.ptr = nullptr;
     slot.bytes = 0;
-    if (cudaMalloc(&slot.ptr, bytes > 0 ? bytes : 16) != cudaSuccess) {
+    size_t got = pi == 1 ? td4_bytes_b(d, n) : bytes;
+    cudaError_t e = cudaMalloc(&slot.ptr, got > 0 ? got : 16);
+    if (e != cudaSuccess && got > bytes) {  // no room for B's plane: the evaluation forms B itself
       cudaGetLastError();
+      got = bytes;
+      e = cudaMalloc(&slot.ptr, got);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      slot.ptr = nullptr;
       return set_error(GOO_ERR_OOM, "amplitude cache of %zu bytes does not fit", bytes);
     }
-    slot.bytes = bytes;
+    slot.bytes = got;
   }
   if (n > 0) {
     const int nb = grid_blocks(ctx, n, 4);
@@ -697,12 +727,12 @@ static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, const
       Td4Cols<float> c{};
       for (int j = 0; j < 5; ++j) c.c[j] = ds->d32[j];
       LaunchScope ls(ctx, "td4_cache_f32");
-      td4_cache_kernel<float><<<nb, kBlock, 0, ctx->stream>>>(d.dev, c, n, slot.ptr);
+      td4_cache_kernel<float><<<nb, kBlock, 0, ctx->stream>>>(d.dev, c, n, slot.ptr, false);
     } else {
       Td4Cols<double> c{};
       for (int j = 0; j < 5; ++j) c.c[j] = ds->d64[j];
       LaunchScope ls(ctx, "td4_cache_f64");
-      td4_cache_kernel<double><<<nb, kBlock, 0, ctx->stream>>>(d.dev, c, n, slot.ptr);
+      td4_cache_kernel<double><<<nb, kBlock, 0, ctx->stream>>>(d.dev, c, n, slot.ptr, slot.bytes >= td4_bytes_b(d, n));
     }
     GOO_CUDA_TRY(cudaGetLastError());
   }
@@ -853,6 +883,7 @@ static int launch_td4_f64(goo_model* m, const void* cache, const goo_dataset* ds
   goo_ctx* ctx = m->ctx;
   Td4Args<double> a;
   td4_args<double>(m, theta, ds->n, a);
+  a.has_b = ds->cache[1].bytes >= td4_bytes_b(*m->td4, ds->n);
   td4_norm_terms<double>(m, GOO_F64, a);
   const Fp64Tables* tables = nullptr;
   GOO_TRY(fp64_tables(ctx, &tables));
@@ -959,6 +990,7 @@ int td4_eval_logf(goo_model* m, const goo_dataset* ds, const double* theta, int 
   } else {
     Td4Args<double> a;
     td4_args<double>(m, theta, ds->n, a);
+    a.has_b = ds->cache[1].bytes >= td4_bytes_b(*m->td4, ds->n);
     const Fp64Tables* tables = nullptr;
     GOO_TRY(fp64_tables(ctx, &tables));
     const double2* amps = (const double2*)cache;
