@@ -1018,7 +1018,7 @@ __global__ void __launch_bounds__(kBlock, 2)
   constexpr int NS = Td3Lanes<GRAD>::NS;
   __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
   __shared__ unsigned s_bad[kBlock / 32];
-  __shared__ __align__(16) Fp64Tables s_tab;
+  __shared__ TimeTables s_tab;
   load_fp64_tables(s_tab, tables);
   const TdMath<double> F{s_tab};
   const int64_t n = a.n_total;

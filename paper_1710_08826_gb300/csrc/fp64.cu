@@ -34,16 +34,16 @@ static void herfcx_coeffs(int i, long double (&out)[DEG + 1]) {
 static const Fp64Tables& host_tables() {
   static const Fp64Tables t = [] {
     Fp64Tables h;
-    for (int j = 0; j < kExpTab; ++j) h.exp2j[j] = (double)std::exp2((long double)j / kExpTab);
+    for (int j = 0; j < kExpTab; ++j) h.exp.exp2j[j] = (double)std::exp2((long double)j / kExpTab);
     for (int j = 0; j < kLogTab; ++j) {
-      h.log_inv[j] = (double)(1.0L / (1.0L + (j + 0.5L) / kLogTab));
-      h.log_ref[j] = (double)-std::log((long double)h.log_inv[j]);
+      h.log.inv[j] = (double)(1.0L / (1.0L + (j + 0.5L) / kLogTab));
+      h.log.ref[j] = (double)-std::log((long double)h.log.inv[j]);
     }
     for (int i = 0; i < kErfcxTab; ++i) {
-      h.node[i] = (double)i / kErfcxStep;
+      h.erfcx.node[i] = (double)i / kErfcxStep;
       long double c[kErfcxDeg + 1];
       herfcx_coeffs<kErfcxDeg>(i, c);
-      for (int d = 0; d <= kErfcxDeg; ++d) h.herfcx[d][i] = (double)c[d];
+      for (int d = 0; d <= kErfcxDeg; ++d) h.erfcx.herfcx[d][i] = (double)c[d];
     }
     return h;
   }();

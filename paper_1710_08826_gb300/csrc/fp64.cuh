@@ -61,27 +61,55 @@ struct LogProduct {
 // conflicts) cost nothing next to a 16-cycle FP64 slot, and the table index is formed on the
 // integer and FP32 pipes, so that only the polynomial is left on the FP64 pipe.
 // The tables are computed on the host (fp64.cu) in extended precision.  Largest difference from CUDA's
-// functions over 16M arguments: exp_tab 1 unit of the last place, herfcx_tab 2, rcp64 half a unit.
+// functions over 16M arguments: exp_tab 1 unit of the last place (1.5 where |x| nears 700), herfcx_tab 2, rcp64 half a unit.
 // ---------------------------------------------------------------------------------------
-constexpr int kExpTab = 256;        // 2^(j / 256)
+constexpr int kExpTab = 2048;       // 2^(j / 2048)
 constexpr int kErfcxStep = 32;      // nodes of erfcx per unit of its argument
 constexpr int kErfcxMax = 6;        // table range [0, 6]
 constexpr int kErfcxTab = kErfcxStep * kErfcxMax + 1;
 constexpr int kErfcxDeg = 7;
 
-constexpr int kLogTab = 256;
+constexpr int kLogTab = 1024;
 
-struct Fp64Tables {
-  double exp2j[kExpTab];
-  double log_inv[kLogTab], log_ref[kLogTab];  // about 1 / (1 + (j + 1/2) / 256), and minus its logarithm
+struct alignas(16) ErfcxTable {
   double node[kErfcxTab];                 // i / 32
   double herfcx[kErfcxDeg + 1][kErfcxTab];  // erfcx(node + r) / 2 = sum_d herfcx[d][i] r^d, |r| <= 1 / 64
 };
+struct alignas(16) ExpTable {
+  double exp2j[kExpTab];
+};
+struct alignas(16) LogTable {
+  double inv[kLogTab], ref[kLogTab];  // about 1 / (1 + (j + 1/2) / 1024), and minus its logarithm
+};
+struct Fp64Tables {
+  ErfcxTable erfcx;
+  ExpTable exp;
+  LogTable log;
+};
+// What a kernel keeps in shared memory: the functions that it calls.
+struct TimeTables {
+  ErfcxTable erfcx;
+  ExpTable exp;
+};
+struct SopTables {
+  ExpTable exp;
+  LogTable log;
+};
 
-// The block's copy of the tables (no barrier after).
-__device__ __forceinline__ void load_fp64_tables(Fp64Tables& s, const Fp64Tables* __restrict__ g) {
-  for (int i = threadIdx.x; i < (int)(sizeof(Fp64Tables) / sizeof(double2)); i += blockDim.x)
-    reinterpret_cast<double2*>(&s)[i] = __ldg(reinterpret_cast<const double2*>(g) + i);
+// The block's copy of a table (no barrier after).
+template <typename Table>
+__device__ __forceinline__ void load_table(Table& s, const Table& g) {
+  static_assert(sizeof(Table) % sizeof(double2) == 0, "16-byte pieces");
+  for (int i = threadIdx.x; i < (int)(sizeof(Table) / sizeof(double2)); i += blockDim.x)
+    reinterpret_cast<double2*>(&s)[i] = __ldg(reinterpret_cast<const double2*>(&g) + i);
+}
+__device__ __forceinline__ void load_fp64_tables(TimeTables& s, const Fp64Tables* __restrict__ g) {
+  load_table(s.erfcx, g->erfcx);
+  load_table(s.exp, g->exp);
+}
+__device__ __forceinline__ void load_fp64_tables(SopTables& s, const Fp64Tables* __restrict__ g) {
+  load_table(s.exp, g->exp);
+  load_table(s.log, g->log);
 }
 
 // |x| (x normal, 2^-126 <= |x| < 2^128) as a float, truncated, without the FP64 pipe: the exponent
@@ -93,50 +121,49 @@ __device__ __forceinline__ float abs_float_trunc(double x) {
   return h < (897 << 20) ? 0.f : __int_as_float(f);
 }
 
-// exp(x), table-driven (P. T. P. Tang, ACM TOMS 15 (1989) 144): x = n ln2 / 256 + r, exp(x) = 2^(n / 256) exp(r)
-// with n / 256 split into an exponent and a table index, |r| <= ln2 / 512 and a degree-4 polynomial
-// (truncation 4e-17): 8 slots of the FP64 pipe and within one unit of the last place, where exp()
-// takes about twenty.  |x| > 704 (and NaN) goes to exp().
-__device__ __forceinline__ double exp_tab(double x, const Fp64Tables& tab) {
+// exp(x), table-driven (P. T. P. Tang, ACM TOMS 15 (1989) 144): x = n ln2 / 2048 + r, exp(x) = 2^(n / 2048) exp(r)
+// with n / 2048 split into an exponent and a table index, |r| <= ln2 / 4096 = h and a degree-3 polynomial
+// (the series with its r^4 replaced by h^2 r^2, which leaves h^4 / 192 = 4e-18): 7 slots of the FP64
+// pipe and within one unit of the last place, where exp() takes about twenty.  |x| > 704 (and NaN) goes
+// to exp().  A table of 256 entries needs degree 4.
+__device__ __forceinline__ double exp_tab(double x, const ExpTable& tab) {
   const int hx = __double2hiint(x);
   if ((hx & 0x7fffffff) >= 0x40860000) return exp(x);
-  const float f = abs_float_trunc(x) * 369.329930467574634f;  // 256 / ln 2
+  const float f = abs_float_trunc(x) * 2954.639443740597f;  // 2048 / ln 2
   const int na = __float2int_rn(f), n = hx < 0 ? -na : na;
   // n as a double: 2^52 + 2^51 + n holds n in its low word
   const double dn = __hiloint2double(0x43380000 + (n >> 31), n) - 6755399441055744.0;
-  // ln2 / 256 as a 34-bit head (n times it is exact) and the rest
-  double r = ::fma(dn, -0.002707606173999011, x);
-  r = ::fma(dn, -6.327543041662719e-14, r);
-  double p = ::fma(r, 1.0 / 24.0, 1.0 / 6.0);
-  p = ::fma(r, p, 0.5);
+  // ln2 / 2048 as a 31-bit head (n times it is exact) and the rest
+  double r = ::fma(dn, -0.0003384507717782981, x);
+  r = ::fma(dn, 2.0512280628325608e-14, r);
+  const double p = ::fma(r, 1.0 / 6.0, 0.500000001193218);  // 1/2 + h^2 / 24
   const double q = ::fma(r * r, p, r);
   const double t = tab.exp2j[n & (kExpTab - 1)];
-  const double s = __hiloint2double(__double2hiint(t) + ((n >> 8) << 20), __double2loint(t));
+  const double s = __hiloint2double(__double2hiint(t) + ((n >> 11) << 20), __double2loint(t));
   return ::fma(s, q, s);
 }
 
-// log(x) for x > 0, table-driven (P. T. P. Tang, ACM TOMS 16 (1990) 378): x = 2^e m, j the top 8 bits of m's
-// fraction, r = m inv_j - 1 with |r| < 2^-8.9, log x = e ln2 - log inv_j + log1p(r) with log1p to degree 5
-// (truncation 2e-17): 9 slots, the error about one unit of the last place of e ln2 - log inv_j (so
+// log(x) for x > 0, table-driven (P. T. P. Tang, ACM TOMS 16 (1990) 378): x = 2^e m, j the top 10 bits of m's
+// fraction, r = m inv_j - 1 with |r| < 2^-10.9, log x = e ln2 - log inv_j + log1p(r) with log1p to degree 4
+// (truncation 8e-18): 8 slots, the error about one unit of the last place of e ln2 - log inv_j (so
 // absolute, not relative, for x near 1), where log() takes some twenty-five.  Subnormal, infinite and NaN
 // arguments go to log().
-__device__ __forceinline__ double log_tab(double x, const Fp64Tables& tab) {
+__device__ __forceinline__ double log_tab(double x, const LogTable& tab) {
   if (!positive_normal(x)) return log(x);
   const int hx = __double2hiint(x);
-  const int j = (hx >> 12) & (kLogTab - 1), e = (hx >> 20) - 1023;
+  const int j = (hx >> 10) & (kLogTab - 1), e = (hx >> 20) - 1023;
   const double m = __hiloint2double((hx & 0x000fffff) | 0x3ff00000, __double2loint(x));
-  const double r = ::fma(m, tab.log_inv[j], -1.0);
+  const double r = ::fma(m, tab.inv[j], -1.0);
   const double de = __hiloint2double(0x43380000 + (e >> 31), e) - 6755399441055744.0;
-  double p = ::fma(r, 0.2, -0.25);
-  p = ::fma(r, p, 1.0 / 3.0);
+  double p = ::fma(r, -0.25, 1.0 / 3.0);
   p = ::fma(r, p, -0.5);
   const double q = ::fma(r * r, p, r);
-  return ::fma(de, 0.693147180559945309417, tab.log_ref[j]) + q;
+  return ::fma(de, 0.693147180559945309417, tab.ref[j]) + q;
 }
 
 // erfcx(u) / 2 for 0 <= u < 6: the degree-7 interpolant of the nearest node (relative error of the
 // interpolation below 1e-17), 8 slots.
-__device__ __forceinline__ double herfcx_tab(double u, const Fp64Tables& tab) {
+__device__ __forceinline__ double herfcx_tab(double u, const ErfcxTable& tab) {
   const int i = __float2int_rn(abs_float_trunc(u) * (float)kErfcxStep);
   const double r = u - tab.node[i];
   double p = tab.herfcx[kErfcxDeg][i];

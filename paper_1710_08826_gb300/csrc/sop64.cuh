@@ -9,9 +9,11 @@
 //   - with two products one exponential, exp(-|a_1 - a_0|), serves both; with one, none is needed;
 //   - log S is a running product (LogProduct), 1/S, 1/u and 1/r are third-order reciprocals, exp
 //     and log come from shared-memory tables;
-//   - the constant factors of the lanes (1/sigma, 2/m0) are applied once per thread.
-// The three-dimensional signal + background model takes about 80 slots per event with the
-// gradient; the interpreter it replaces took about 235 (3M events: 1123 us, now 481 us).
+//   - a polynomial r that is its product's only one needs no reciprocal: c_k / r is the other factors;
+//   - the constant factors of the lanes (1/sigma, 2/m0) are applied once per thread, and the Argus endpoint's
+//     derivative is formed from the sums of c_k / u, c_k and c_k u.
+// The three-dimensional signal + background model takes about 62 slots per event with the
+// gradient; the interpreter it replaces took about 235 (3M events: 1123 us; 481 us with 71 slots, now 436 us).
 #pragma once
 
 #include "fp64.cuh"
@@ -21,13 +23,18 @@
 namespace goo {
 
 // exp(-x) for x >= 0, 0 from 704 on (below 2^-1015 of the term it is added to)
-__device__ __forceinline__ double exp_neg(double x, const Fp64Tables& tab) {
+__device__ __forceinline__ double exp_neg(double x, const ExpTable& tab) {
   return __double2hiint(x) >= 0x40860000 ? 0.0 : exp_tab(-x, tab);
 }
 
 // On the integer pipe: x is not zero; the largest exponent of an event's products is a number, not an
 // absent product's -1e30 nor infinite.
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+// a b is not zero; the product itself only where it might leave the normal range
+__device__ __forceinline__ bool nonzero_product(double a, double b) {
+  const int ea = (__double2hiint(a) >> 20) & 0x7ff, eb = (__double2hiint(b) >> 20) & 0x7ff;
+  return (ea != 0 && eb != 0 && ea + eb > 1024) || nonzero(a * b);
+}
 __device__ __forceinline__ bool usable_exponent(double M) {
   const int h = __double2hiint(M);
   return h < 0 ? (h & 0x7fffffff) < 0x45f00000 : h < 0x7ff00000;
@@ -43,7 +50,7 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
   constexpr int NS = EventLanes<double, K, L, GRAD>::NS;
   __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
   __shared__ unsigned s_bad[kBlock / 32];
-  __shared__ __align__(16) Fp64Tables s_tab;
+  __shared__ SopTables s_tab;
   load_fp64_tables(s_tab, tables);
   const int nK = P.nK, nobs = P.nobs;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -61,6 +68,14 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
   fetch(i);
   // the tables and columns depend on no earlier kernel; the offsets -log N_k do
   grid_dep_wait();
+  unsigned one_poly = 0;  // bit k: product k has exactly one polynomial
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    int np = 0;
+#pragma unroll
+    for (int l = 0; l < L; ++l) np += P.leaf[k][l].op == GOO_OP_POLY2;
+    one_poly |= (k < nK && np == 1 ? 1u : 0u) << k;
+  }
   double off[K], unused_lo[K];
   load_offsets<double, K>(md, off, unused_lo);
   double acc = 0.0, C[K], A[K][L][3];
@@ -77,13 +92,15 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
     const double x0 = nx[0], x1 = nx[1], x2 = nx[2], x3 = nx[3], wi = nw;
     fetch(i + stride);
     if (wcol && wi == 0.0) continue;  // an empty bin
-    double a[K], t[K], d0[K][L], d1[K][L];
+    // t: the product's factor without its polynomial where it has just one (q; else 1)
+    double a[K], t[K], q[K], d0[K][L], d1[K][L];
 #pragma unroll
     for (int k = 0; k < K; ++k) {
       a[k] = -1e30;  // an absent product
       t[k] = 0.0;
+      q[k] = 1.0;
       if (k >= nK) continue;
-      double ak = off[k], r = 1.0;
+      double ak = off[k], r = 1.0, rq = 1.0;
       bool present = true, has_r = false;
 #pragma unroll
       for (int l = 0; l < L; ++l) {
@@ -104,10 +121,14 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
             break;
           case GOO_OP_POLY2: {
             const double rp = fma(x, fma(F.c[1], x, F.c[0]), 1.0);
-            r = has_r ? r * rp : rp;
-            has_r = true;
+            if (one_poly >> k & 1) {
+              rq = rp;
+            } else {
+              r = has_r ? r * rp : rp;
+              has_r = true;
+              d1[k][l] = rp;
+            }
             d0[k][l] = x;
-            d1[k][l] = rp;
             break;
           }
           case GOO_OP_ARGUS: {
@@ -115,7 +136,7 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
             r = has_r ? r * x : x;
             has_r = true;
             if (__double_as_longlong(u) > 0) {
-              const double lu = log_tab(u, s_tab);
+              const double lu = log_tab(u, s_tab.log);
               ak = fma(F.c[3], lu, fma(F.c[2], u, ak));
               d0[k][l] = u;
               d1[k][l] = lu;
@@ -129,18 +150,21 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
         }
       }
       // r == 0: the product vanishes, whatever its exponent
-      if (has_r) present = present && nonzero(r);
+      if (one_poly >> k & 1) present = present && nonzero_product(r, rq);
+      else if (has_r) present = present && nonzero(r);
       a[k] = present ? ak : -1e30;
       t[k] = present ? r : 0.0;
+      q[k] = present ? rq : 1.0;
     }
     double M = a[0];
     if (K == 2) {
       if (nK == 2) {
         const double d = a[1] - a[0];
         const int hd = __double2hiint(d);
-        const double e = exp_neg(__hiloint2double(hd & 0x7fffffff, __double2loint(d)), s_tab);
-        t[0] *= hd < 0 ? 1.0 : e;
-        t[1] *= hd < 0 ? e : 1.0;
+        const double e = exp_neg(__hiloint2double(hd & 0x7fffffff, __double2loint(d)), s_tab.exp);
+        const double te = (hd < 0 ? t[1] : t[0]) * e;
+        t[0] = hd < 0 ? t[0] : te;
+        t[1] = hd < 0 ? te : t[1];
         M = hd < 0 ? a[0] : a[1];
       }
     } else if (nK > 1) {
@@ -148,7 +172,13 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
       for (int k = 1; k < K; ++k) M = a[k] > M ? a[k] : M;
 #pragma unroll
       for (int k = 0; k < K; ++k)
-        if (k < nK) t[k] *= exp_neg(M - a[k], s_tab);
+        if (k < nK) t[k] *= exp_neg(M - a[k], s_tab.exp);
+    }
+    double tr[K];  // t without the polynomial
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      tr[k] = t[k];
+      if (one_poly >> k & 1) t[k] *= q[k];
     }
     double S = P.w_hi[0] * t[0];
 #pragma unroll
@@ -157,7 +187,7 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
     double invS;
     if (positive_normal(S) && usable_exponent(M)) {
       if (wcol) {
-        acc = fma(wi, M + log_tab(S, s_tab), acc);
+        acc = fma(wi, M + log_tab(S, s_tab.log), acc);
       } else {
         acc += M;
         lp.mul(S);
@@ -190,19 +220,18 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
               A[k][l][0] = fma(ck, p, A[k][l][0]);
               break;
             case GOO_OP_POLY2: {  // x / r, x^2 / r
-              // r = 0 only where the product vanishes (ck = 0); its reciprocal is not used there
-              const double cq = ck * (nonzero(ck) ? recip(q) : 0.0), cx = cq * p;
+              // t / r is the product's other factors; with several polynomials r = 0 only where the product
+              // vanishes (ck = 0) and its reciprocal is not used there
+              const double cq = one_poly >> k & 1 ? tr[k] * invS : ck * (nonzero(ck) ? recip(q) : 0.0), cx = cq * p;
               A[k][l][0] += cx;
               A[k][l][1] = fma(cx, p, A[k][l][1]);
               break;
             }
-            case GOO_OP_ARGUS: {  // (1 - u) (p / u + c) (times 2 / m0 at the end), u, log u
-              const double v = ck * (1.0 - p);
-              A[k][l][0] = fma(v, fma(F.c[3], nonzero(ck) ? recip(p) : 0.0, F.c[2]), A[k][l][0]);
+            case GOO_OP_ARGUS:  // 1 / u, u, log u
+              A[k][l][0] = fma(ck, nonzero(ck) ? recip(p) : 0.0, A[k][l][0]);
               A[k][l][1] = fma(ck, p, A[k][l][1]);
               A[k][l][2] = fma(ck, q, A[k][l][2]);
               break;
-            }
             default:
               break;
           }
@@ -221,6 +250,9 @@ __global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
       for (int l = 0; l < L; ++l) {
         const LeafReg<double>& F = P.leaf[k][l];
         const double s0 = F.op == GOO_OP_GAUSS ? F.c[1] : F.op == GOO_OP_ARGUS ? F.c[4] : 1.0;
+        // Argus, d / d m0: sum c_k (1 - u) (p / u + c) from the sums of c_k / u, c_k and c_k u
+        if (F.op == GOO_OP_ARGUS)
+          A[k][l][0] = fma(F.c[3], A[k][l][0], fma(F.c[2] - F.c[3], C[k], -F.c[2] * A[k][l][1]));
         const double s1 = F.op == GOO_OP_GAUSS ? F.c[1] : 1.0;
         v[1 + K + (k * L + l) * 3] = dd_from_double(A[k][l][0] * s0);
         v[1 + K + (k * L + l) * 3 + 1] = dd_from_double(A[k][l][1] * s1);

@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kBlock, 2) td4_nll_f64_kernel(const __grid_con
   constexpr int NS = TdLanes<KB, GRAD>::NS;
   __shared__ ddf s_red[(kBlock / 32) * NS > kBlock ? (kBlock / 32) * NS : kBlock];
   __shared__ unsigned s_bad[kBlock / 32];
-  __shared__ __align__(16) Fp64Tables s_tab;
+  __shared__ TimeTables s_tab;
   load_fp64_tables(s_tab, tables);
   const TdMath<double> F{s_tab};
   TdAcc<double, KB> acc;
@@ -556,7 +556,7 @@ template <int KB>
 __global__ void td4_logf_f64_kernel(const __grid_constant__ Td4Args<double> a, const double2* __restrict__ cache,
                                     const double* __restrict__ tcol, const Fp64Tables* __restrict__ tables, double logN,
                                     double* __restrict__ out) {
-  __shared__ __align__(16) Fp64Tables s_tab;
+  __shared__ TimeTables s_tab;
   load_fp64_tables(s_tab, tables);
   __syncthreads();
   const int64_t n = a.n_total;

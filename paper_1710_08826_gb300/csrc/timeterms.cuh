@@ -291,13 +291,13 @@ struct TdMath<float2> {
 };
 template <>
 struct TdMath<double> {
-  const Fp64Tables& tab;
-  __device__ __forceinline__ double exp(double v) const { return exp_tab(v, tab); }
+  const TimeTables& tab;
+  __device__ __forceinline__ double exp(double v) const { return exp_tab(v, tab.exp); }
   // gauss erfcx(|u|) / 2; where u <= -6 it is below 2^-56 of the exponential it is subtracted from
   // (conv_real) and is left out
   __device__ __forceinline__ double gauss_herfcx(double gauss, double u) const {
     const int hu = __double2hiint(u), ha = hu & 0x7fffffff;
-    if (ha < 0x40180000) return mul_rn(gauss, herfcx_tab(__hiloint2double(ha, __double2loint(u)), tab));
+    if (ha < 0x40180000) return mul_rn(gauss, herfcx_tab(__hiloint2double(ha, __double2loint(u)), tab.erfcx));
     return hu < 0 ? 0.0 : mul_rn(gauss, 0.5 * erfcx(u));
   }
   // on the integer pipe (nonneg: false for -0, where both forms agree; below: to 2^-20)

@@ -72,3 +72,33 @@ def test_no_density_is_reported(goo, ctx):
     with pytest.raises(goo.GooError) as e:
         goo.Model(ctx, spec).nll_grad(goo.Dataset.from_spec(ctx, spec, cols), theta, "f64")
     assert e.value.code == goo.GOO_ERR_NONPOSITIVE_PDF
+
+
+@pytest.mark.parametrize("n_poly", [1, 2])
+@pytest.mark.parametrize("zero", [False, True])
+def test_polynomials_of_a_product(goo, ctx, n_poly, zero):
+    # one polynomial in a product takes 1 / r from the other factors, two take reciprocals; where
+    # the polynomial is zero the product vanishes and the others remain
+    spec = synth.c2_spec(bins=32)
+    _, _, (sig, bkg) = spec["pdf"]
+    extra = [("q1", 0.05, False, 0.01), ("q2", 0.01, False, 0.01)]
+    leaves = list(bkg[1])
+    if n_poly == 2:
+        leaves = [("poly2", "t", "q1", "q2") if l[0] == "expo" else l for l in leaves]
+    spec = dict(spec, params=spec["params"] + (extra if n_poly == 2 else []),
+                pdf=("add", spec["pdf"][1], [sig, ("prod", leaves)]))
+    cols = {k: v[:20_001] for k, v in synth.gen_c2(n=20_001, seed=33).items()}
+    theta = np.array(synth.param_values(spec))
+    poly = next(l for l in leaves if l[0] == "poly2" and l[1] == "dE")
+    names = [p[0] for p in spec["params"]]
+    lanes = np.ones(len(names), bool)
+    if zero:   # (1 - 8 dE)^2, zero for every ninth event; the lanes x / r leave out a vanished product
+        theta[names.index(poly[2])], theta[names.index(poly[3])] = -16.0, 64.0
+        cols["dE"][::9] = 0.125
+        lanes[[names.index(poly[2]), names.index(poly[3])]] = False
+    ref, model = om.TreeModel(spec), goo.Model(ctx, spec)
+    nll, g = model.nll_grad(goo.Dataset.from_spec(ctx, spec, cols), theta, "f64")
+    rnll, rg = ref.nll_grad(cols, theta)
+    assert abs(nll - rnll) <= TOL_NLL * max(abs(rnll), 20_001), (nll, rnll)
+    assert np.max(np.abs(g - rg)[lanes]) <= TOL_GRAD * max(np.max(np.abs(rg[lanes])), 20_001), (g, rg)
+    assert np.all(np.isfinite(g))
