@@ -267,9 +267,11 @@ __device__ __forceinline__ void coh_coeffs(const CohArgs<T>& a, T (&cr)[KB + 1],
 // sum is a chain of FMAs), the logarithm as a running product, the reciprocal by one third-order
 // step, the sign test on the integer pipe; absent resonance slots and the constant amplitude
 // (A = 1) cost no multiplication.  8 resonances with the gradient take 78 slots per event; 2M
-// events: 549 -> 293 us (the slots alone: 249 us at the measured 6.27e11 FMA/s).
+// events: 549 -> 286 us (the slots alone: 249 us at the measured 6.27e11 FMA/s).  One block per SM: with the
+// registers of 16 warps to interleave independent chains 8 warps fill the pipe (286 us; 290 us with two
+// blocks, 303 with 20 warps), and a small dataset's events spread over the SMs more evenly (100k: 41 -> 33 us).
 template <int KB, bool GRAD>
-__global__ void __launch_bounds__(kBlock, 2)
+__global__ void __launch_bounds__(kBlock, 1)
     coh_nll_f64_kernel(const __grid_constant__ CohArgs<double> a, const double2* __restrict__ cache, int64_t begin,
                        int64_t end, float2* partials, unsigned* counters, double* result, int out_mode) {
   constexpr int NS = CohLanes<double, KB, GRAD>::NS;

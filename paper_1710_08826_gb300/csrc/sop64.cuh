@@ -12,8 +12,9 @@
 //   - a polynomial r that is its product's only one needs no reciprocal: c_k / r is the other factors;
 //   - the constant factors of the lanes (1/sigma, 2/m0) are applied once per thread, and the Argus endpoint's
 //     derivative is formed from the sums of c_k / u, c_k and c_k u.
-// The three-dimensional signal + background model takes about 62 slots per event with the
-// gradient; the interpreter it replaces took about 235 (3M events: 1123 us; 481 us with 71 slots, now 436 us).
+// The three-dimensional signal + background model takes 76 slots per event (counted) with the
+// gradient; the interpreter it replaces took about 235 (3M events: 1123 us; 481 us with
+// nine slots more and two blocks per SM, 436 us with two blocks, now 426 us; 100k events: 50 -> 39 us).
 #pragma once
 
 #include "fp64.cuh"
@@ -42,7 +43,7 @@ __device__ __forceinline__ bool usable_exponent(double M) {
 
 // Per leaf slot, kept for the gradient: Gauss (z, z^2), Expo (x, -), Poly2 (x, r), Argus (u, log u).
 template <int K, int L, bool GRAD>
-__global__ void __launch_bounds__(kBlock, K * L <= 6 ? 2 : 1)
+__global__ void __launch_bounds__(kBlock, 1)
     sop_event64_kernel(const ModelDev* __restrict__ md, const __grid_constant__ EvConst<double, K, L> P,
                        Cols<double> cols, const Fp64Tables* __restrict__ tables, int64_t begin, int64_t end,
                        float2* partials, unsigned* counters, double* result, int out_mode,
