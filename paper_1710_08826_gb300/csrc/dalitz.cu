@@ -102,9 +102,9 @@ __global__ void __launch_bounds__(kLsBlock)
     }
     ls_groups<float, float2>(t, a, b, sc, gc, hc, kLsBlock);
     for (int p = 0; p < planes; ++p) {
-      float2 r0, i0, r1 = pk::splat(0.f), i1 = pk::splat(0.f), dr, di, inv;
-      ls_amp<float, float2>(t, 2 * p, sc, gc, hc, kLsBlock, r0, i0, dr, di, inv);
-      if (2 * p + 1 < t.nbw) ls_amp<float, float2>(t, 2 * p + 1, sc, gc, hc, kLsBlock, r1, i1, dr, di, inv);
+      float2 r0, i0, r1 = pk::splat(0.f), i1 = pk::splat(0.f);
+      ls_amp<float, float2>(t, 2 * p, sc, gc, hc, kLsBlock, r0, i0);
+      if (2 * p + 1 < t.nbw) ls_amp<float, float2>(t, 2 * p + 1, sc, gc, hc, kLsBlock, r1, i1);
       float4* out = cache + (int64_t)p * n + i;
       out[0] = make_float4(r0.x, i0.x, r1.x, i1.x);
       if (two) out[1] = make_float4(r0.y, i0.y, r1.y, i1.y);
@@ -122,8 +122,8 @@ __global__ void __launch_bounds__(kLsBlock)
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     ls_groups<double, double>(t, s12c[i], s13c[i], sc, gc, hc, kLsBlock);
     for (int k = 0; k < t.nbw; ++k) {
-      double re, im, dr, di, inv;
-      ls_amp<double, double>(t, k, sc, gc, hc, kLsBlock, re, im, dr, di, inv);
+      double re, im;
+      ls_amp<double, double>(t, k, sc, gc, hc, kLsBlock, re, im);
       cache[(int64_t)k * n + i] = make_double2(re, im);
     }
   }
@@ -550,11 +550,12 @@ static uint64_t lineshape_key(const DalitzModel& d, const double* theta) {
 //   d NLL / d p = -sum_events (d |S|^2 / d p) / |S|^2 + n (sum_MC d |S|^2 / d p) / sum_MC |S|^2.
 //
 // Issue-bound.  The factors shared by a pair and spin are formed once per point (lineshape.cuh) and kept
-// in the thread's column of shared memory; FP32 works on two points at a time; a resonance's
-// amplitude is formed again for its lanes (ten operations) rather than kept; the
-// first blocks of the one launch take the MC sample and the others the events, so that neither waits for the
+// in the thread's column of shared memory, and so are g_k = 1 / D_k and c_k g_k of every resonance for
+// its lanes (A_k = h g_k with a real h, so u_k = h (g_k conj(S) w) and y_k = h (g_k conj(S) w) (c_k g_k)); FP32
+// works on two points at a time; the first blocks of the one launch take the MC sample and the others the events, so that neither waits for the
 // other's reduction.  5M events and 1M MC points, 8 resonances: 495 us in two launches with every
-// resonance evaluated by itself, now 144 us (150 with two blocks of 256 threads per SM).
+// resonance evaluated by itself, 144 us with the amplitudes formed a second time for the lanes, now
+// 131 us (217 KB of shared memory; issue slots 59 %, FMA pipe 54 %, shared memory 53 % busy).
 // ---------------------------------------------------------------------------------------
 template <typename T>
 struct LsConst {
@@ -583,7 +584,7 @@ constexpr int kLsBlockOf = KB <= 8 ? kStagedBlock : kBlock;
 // Dynamic shared memory: the shared factors of every thread, later the block reduction's lanes.
 template <typename T, int KB, bool GRAD>
 constexpr size_t ls_smem() {
-  const size_t f = (size_t)kLsCols * kLsBlockOf<KB> * 8, r = (size_t)LsLanes<KB, GRAD>::NS * kLsBlockOf<KB> * sizeof(ddf);
+  const size_t f = (size_t)(kLsCols + (GRAD ? 4 * KB : 0)) * kLsBlockOf<KB> * 8, r = (size_t)LsLanes<KB, GRAD>::NS * kLsBlockOf<KB> * sizeof(ddf);
   return f > r ? f : r;
 }
 
@@ -680,7 +681,7 @@ __global__ void __launch_bounds__(kLsBlockOf<KB>, 1)
   __shared__ double s_out[NS], s_mc[NS];
   extern __shared__ __align__(16) unsigned char s_dyn[];
   V* s_v = reinterpret_cast<V*>(s_dyn);
-  V *sc = s_v + threadIdx.x, *gc = sc + 3 * NT, *hc = sc + 12 * NT;
+  V *sc = s_v + threadIdx.x, *gc = sc + 3 * NT, *hc = sc + 12 * NT, *ac = sc + kLsCols * NT;
   const bool is_mc = (int)blockIdx.x < nb_mc;
   const LsSet<T>& D = is_mc ? mc : ev;
   const int nb = is_mc ? nb_mc : (int)gridDim.x - nb_mc, b0 = is_mc ? (int)blockIdx.x : (int)blockIdx.x - nb_mc;
@@ -694,17 +695,26 @@ __global__ void __launch_bounds__(kLsBlockOf<KB>, 1)
   unsigned bad = 0;
   const int64_t last = ls_last(D);
   for (int64_t j = ls_first(D) + b0 * (int64_t)NT + threadIdx.x; j < last; j += (int64_t)nb * NT) {
-    V x12, x13, re, im, dr, di, iv;
+    V x12, x13;
     bool v0, v1;
     ls_load(D, j, x12, x13, v0, v1);
     ls_groups<T, V>(t, x12, x13, sc, gc, hc, NT);
     V sr = splat(V{}, c.cr[KB]), si = splat(V{}, c.ci[KB]);  // the non-resonant amplitude is 1
 #pragma unroll 4
     for (int k = 0; k < t.nbw; ++k) {
-      ls_amp<T, V>(t, k, sc, gc, hc, NT, re, im, dr, di, iv);
-      const V cr = splat(V{}, c.cr[k]);
-      sr = fma(cr, re, fma(splat(V{}, c.nci[k]), im, sr));
-      si = fma(cr, im, fma(splat(V{}, c.ci[k]), re, si));
+      // g = 1 / D, A_k = h g with a real h; c_k g serves the sum and the mass and width lanes
+      V gr, gi, di;
+      ls_propagator<T, V>(t, k, sc, gc, NT, gr, gi, di);
+      const V h = ls_numerator<T, V>(t, k, hc, NT), cr = splat(V{}, c.cr[k]);
+      const V qr = fma(cr, gr, mul(splat(V{}, c.nci[k]), gi)), qi = fma(cr, gi, mul(splat(V{}, c.ci[k]), gr));
+      sr = fma(h, qr, sr);
+      si = fma(h, qi, si);
+      if constexpr (GRAD) {
+        ac[4 * k * NT] = gr;
+        ac[(4 * k + 1) * NT] = gi;
+        ac[(4 * k + 2) * NT] = qr;
+        ac[(4 * k + 3) * NT] = qi;
+      }
     }
     V w, term;
     ls_weight(is_mc, fma(sr, sr, mul(si, si)), v0, v1, w, term, bad);
@@ -716,16 +726,14 @@ __global__ void __launch_bounds__(kLsBlockOf<KB>, 1)
 #pragma unroll
       for (int k = 0; k < KB; ++k) {
         if (k >= t.nbw) break;
-        ls_amp<T, V>(t, k, sc, gc, hc, NT, re, im, dr, di, iv);
-        const V ur = fma(re, tr, mul(im, mti)), ui = fma(re, ti, mul(im, tr));  // A_k conj(S) w
-        lre[k] = add(lre[k], ur);
-        lim[k] = add(lim[k], ui);
-        // v = c_k u_k / |D|^2 and mvi = -Im v; y_k = v (dr + i di)
-        const V nci = splat(V{}, c.nci[k]);
-        const V vr = mul(fma(splat(V{}, c.cr[k]), ur, mul(nci, ui)), iv);
-        const V mvi = mul(fma(splat(V{}, c.ncr[k]), ui, mul(nci, ur)), iv);
-        lwr[k] = fma(vr, dr, fma(mvi, di, lwr[k]));
-        lwi[k] = fma(di, sub(mul(vr, di), mul(mvi, dr)), lwi[k]);
+        const V gr = ac[4 * k * NT], gi = ac[(4 * k + 1) * NT], qr = ac[(4 * k + 2) * NT], qi = ac[(4 * k + 3) * NT];
+        const V h = ls_numerator<T, V>(t, k, hc, NT);
+        const V ur = fma(gr, tr, mul(gi, mti)), ui = fma(gr, ti, mul(gi, tr));  // conj(S) w / D_k
+        lre[k] = fma(h, ur, lre[k]);
+        lim[k] = fma(h, ui, lim[k]);
+        // y_k = c_k A_k conj(S) w / D_k
+        lwr[k] = fma(h, sub(mul(ur, qr), mul(ui, qi)), lwr[k]);
+        lwi[k] = fma(mul(h, ls_width<T, V>(t, k, gc, NT)), fma(ur, qi, mul(ui, qr)), lwi[k]);
       }
     }
   }

@@ -114,7 +114,10 @@ __device__ __forceinline__ void ls_groups(const LsTables<T>& t, V a, V b, V* sc,
     const V q2 = floor_at(mul(mul(lam1, is), splat(V{}, T(0.25))), ls_q2_floor<T>());
     const V qrs = mul(mul(q2, rsqrt(q2)), rs);  // q / sqrt(s)
     sc[p * stride] = s;
-    if (used & 1) gc[3 * p * stride] = qrs;
+    if (used & 1) {
+      gc[3 * p * stride] = qrs;
+      hc[3 * p * stride] = one;
+    }
     if (!(used & 6)) continue;
     const V z = mul(splat(V{}, t.r2), q2);
     const V lam2 = mul(sub(s, splat(V{}, P.pthrP)), sub(s, splat(V{}, P.pthrM)));
@@ -137,19 +140,39 @@ __device__ __forceinline__ void ls_groups(const LsTables<T>& t, V a, V b, V* sc,
   }
 }
 
-// Amplitude k from the shared factors, with the parts of its denominator: D = dr - i di, inv = 1 / |D|^2.
+// Amplitude k, A = h / D with a real numerator h, from the shared factors: di of D = dr - i di,
 template <typename T, typename V>
-__device__ __forceinline__ void ls_amp(const LsTables<T>& t, int k, const V* sc, const V* gc, const V* hc, int stride,
-                                       V& re, V& im, V& dr, V& di, V& inv) {
+__device__ __forceinline__ V ls_width(const LsTables<T>& t, int k, const V* gc, int stride) {
+  return lsv::mul(lsv::splat(V{}, t.res[k].c1), gc[t.res[k].group * stride]);
+}
+// 1 / D = gr + i gi, and di,
+template <typename T, typename V>
+__device__ __forceinline__ void ls_propagator(const LsTables<T>& t, int k, const V* sc, const V* gc, int stride, V& gr,
+                                              V& gi, V& di) {
   using namespace lsv;
   const typename LsTables<T>::Res& R = t.res[k];
-  const int g = R.group, p = g / 3;
-  dr = sub(splat(V{}, R.m0sq), sc[p * stride]);
-  di = mul(splat(V{}, R.c1), gc[g * stride]);
-  inv = rcp(fma(dr, dr, mul(di, di)));
-  const V scale = g == 3 * p ? inv : mul(mul(splat(V{}, R.c2), hc[g * stride]), inv);  // L = 0: h = c2 = 1
-  re = mul(dr, scale);
-  im = mul(di, scale);
+  const V dr = sub(splat(V{}, R.m0sq), sc[R.group / 3 * stride]);
+  di = ls_width<T, V>(t, k, gc, stride);
+  const V inv = rcp(fma(dr, dr, mul(di, di)));
+  gr = mul(dr, inv);
+  gi = mul(di, inv);
+}
+// and h.
+template <typename T, typename V>
+__device__ __forceinline__ V ls_numerator(const LsTables<T>& t, int k, const V* hc, int stride) {
+  using namespace lsv;
+  const typename LsTables<T>::Res& R = t.res[k];
+  return mul(splat(V{}, R.c2), hc[R.group * stride]);
+}
+template <typename T, typename V>
+__device__ __forceinline__ void ls_amp(const LsTables<T>& t, int k, const V* sc, const V* gc, const V* hc, int stride,
+                                       V& re, V& im) {
+  using namespace lsv;
+  V gr, gi, di;
+  ls_propagator<T, V>(t, k, sc, gc, stride, gr, gi, di);
+  const V h = ls_numerator<T, V>(t, k, hc, stride);
+  re = mul(gr, h);
+  im = mul(gi, h);
 }
 
 // Threads per block of the kernels that keep the shared factors in shared memory: 21 values per
