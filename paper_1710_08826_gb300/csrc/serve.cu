@@ -474,9 +474,12 @@ __global__ void __launch_bounds__(kBlock, 2) srv_nll_kernel(const SrvEval* __res
         if (bb) atomicAdd(&results[fit].bad, bb);
       }
     }
-    __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(&fit_ticket[fit], 1u) == (unsigned)(ft.x - 1);
+    // the barrier orders the block's partial sums before thread 0's fence and ticket
+    if (threadIdx.x == 0) {
+      __threadfence();
+      s_last = atomicAdd(&fit_ticket[fit], 1u) == (unsigned)(ft.x - 1);
+    }
     __syncthreads();
     if (!s_last) continue;
     __threadfence();
