@@ -7,7 +7,7 @@
 // 32 products; one block of 384 threads per SM (the sums fill the register file), the SMs
 // divided over the tiles in proportion to their products.  One block per row that re-read the whole
 // cache for every row and added with scalar Kahan sums took 128 us for 1M points of 9
-// amplitudes, this kernel 35 us (64 MB: 9.4 us; some 14 us are launch, reduction and result); the three 16 x 16 matrices of the time-dependent
+// amplitudes, this kernel 32 us (64 MB: 9.4 us; some 14 us are launch, reduction and result); the three 16 x 16 matrices of the time-dependent
 // three-body model, one block per element with FP64 sums before, 16 ms, now 0.9 ms.
 //
 // FP32: sums of 16 events run in registers (plain FMAs) and are then added, Kahan compensated, to the

@@ -44,8 +44,8 @@
 // The lanes per event are X, Y, Z and the bracket without its G^2 R, each over R; the last block
 // applies the constant factors (time_gradient).  The kernels are bound by their instructions (FP32)
 // or FP64 slots: summing the derivatives as series too and branching between two erfcx calls cost
-// 2M events FP32 64.1 us (four-body) and 114.5 us (three-body), now 59.3 and 97.3 us; 1M events
-// FP64 four-body 1222 us, now 872 us.
+// 2M events FP32 64.1 us (four-body) and 114.5 us (three-body), this 59.3 and 97.3 us; 1M events
+// FP64 four-body 1222 us, this 872 us (the kernels' later figures stand beside them).
 #pragma once
 
 #include <cmath>
