@@ -32,45 +32,42 @@ BYTES_PER_EVENT_F64 = 24
 # in "profile"): DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) and, for the FP64
 # kernels, the FP64 pipe's active fraction (sm__pipe_fp64_cycles_active).  A record is used
 # only while the kernel's sources still hash to the captured value; bytes scale with events.
-_SOP_SRC = ['paper_1710_08826_gb300/csrc/tree.cu', 'paper_1710_08826_gb300/csrc/sop_kernels.cuh', 'paper_1710_08826_gb300/csrc/jit.cu', 'paper_1710_08826_gb300/csrc/common.cuh', 'paper_1710_08826_gb300/csrc/model.cuh']
-_COH_SRC = ['paper_1710_08826_gb300/csrc/dalitz.cu', 'paper_1710_08826_gb300/csrc/dalitz.cuh', 'paper_1710_08826_gb300/csrc/common.cuh', 'paper_1710_08826_gb300/csrc/model.cuh']
-_TD4_SRC = ['paper_1710_08826_gb300/csrc/td4.cu', 'paper_1710_08826_gb300/csrc/dalitz.cuh', 'paper_1710_08826_gb300/csrc/common.cuh', 'paper_1710_08826_gb300/csrc/model.cuh', 'paper_1710_08826_gb300/csrc/timeterms.cuh']
+_SOP_SRC = ['paper_1710_08826_gb300/csrc/tree.cu', 'paper_1710_08826_gb300/csrc/sop_kernels.cuh', 'paper_1710_08826_gb300/csrc/sop64.cuh', 'paper_1710_08826_gb300/csrc/fp64.cuh', 'paper_1710_08826_gb300/csrc/jit.cu', 'paper_1710_08826_gb300/csrc/common.cuh', 'paper_1710_08826_gb300/csrc/model.cuh']
+_COH_SRC = ['paper_1710_08826_gb300/csrc/dalitz.cu', 'paper_1710_08826_gb300/csrc/dalitz.cuh', 'paper_1710_08826_gb300/csrc/lineshape.cuh', 'paper_1710_08826_gb300/csrc/fp64.cuh', 'paper_1710_08826_gb300/csrc/common.cuh', 'paper_1710_08826_gb300/csrc/model.cuh']
+_TD4_SRC = ['paper_1710_08826_gb300/csrc/td4.cu', 'paper_1710_08826_gb300/csrc/fp64.cuh', 'paper_1710_08826_gb300/csrc/common.cuh', 'paper_1710_08826_gb300/csrc/model.cuh', 'paper_1710_08826_gb300/csrc/timeterms.cuh']
 _TD3_SRC = _COH_SRC + ['paper_1710_08826_gb300/csrc/timeterms.cuh']
 # warp-instruction issue peak of a GB300: 152 SMs x 4 schedulers x 2.07 GHz (one warp
 # instruction per scheduler per cycle)
 ISSUE_PEAK = 152 * 4 * 2.07e9
 
 NCU_RECORDS = {
-    "sop_nll_grad_f32": {"bytes": 127_851_008, "events": 10_000_000, "duration_ns": 40864, "warp_inst": 21_770_696, "issue_active": 0.5403,
-        "sources": _SOP_SRC, "sha256": "510948a29bee9a77654bc84a7a3df5014e9aba8eb1fb4f7f3c6495b38be33291",
-        "profile": "profiles/sop_event2_kernel_f32_c2_10M.md"},
-    "sop_nll_f64": {"bytes": 243_686_912, "events": 10_000_000, "duration_ns": 2504160, "fp64_pipe": 0.8625, "fp64_ops": {"dfma": 649_995_818, "dadd": 340_076_105, "dmul": 259_998_770},
-        "sources": _SOP_SRC, "sha256": "510948a29bee9a77654bc84a7a3df5014e9aba8eb1fb4f7f3c6495b38be33291",
-        "profile": "profiles/sop_event_kernel_f64_c2_10M.md"},
-    "coh_nll_grad_f32": {"bytes": 323_078_912, "events": 5_000_000, "duration_ns": 62912, "warp_inst": 30_962_164, "issue_active": 0.4583,
-        "sources": _COH_SRC, "sha256": "e6dd74780f809bce3110cf47365aa77f11795ed20f00040bf6bdb22689ec5c10",
-        "profile": "profiles/coh_nll_staged_kernel_f32_c3_5M.md"},
-    "coh_nll_f64": {"bytes": 643_060_224, "events": 5_000_000, "duration_ns": 773056, "fp64_pipe": 0.8699, "fp64_ops": {"dfma": 165_155_649, "dadd": 135_077_825, "dmul": 105_000_000},
-        "sources": _COH_SRC, "sha256": "e6dd74780f809bce3110cf47365aa77f11795ed20f00040bf6bdb22689ec5c10",
-        "profile": "profiles/coh_nll_kernel_f64_c3_5M.md"},
-    "coh_ls_mc_f32": {"bytes": 8_068_608, "events": 1_000_000, "duration_ns": 91424, "warp_inst": 65_097_718, "issue_active": 0.6327,
-        "sources": _COH_SRC, "sha256": "e6dd74780f809bce3110cf47365aa77f11795ed20f00040bf6bdb22689ec5c10",
-        "profile": "profiles/coh_ls_kernel_f32_c3_floating_5M.md"},
-    "coh_ls_grad_f32": {"bytes": 40_095_744, "events": 5_000_000, "duration_ns": 423008, "warp_inst": 313_878_490, "issue_active": 0.6404,
-        "sources": _COH_SRC, "sha256": "e6dd74780f809bce3110cf47365aa77f11795ed20f00040bf6bdb22689ec5c10",
-        "profile": "profiles/coh_ls_kernel_f32_c3_floating_5M.md"},
-    "td3_nll_grad_f32": {"bytes": 523_792_384, "events": 2_000_000, "duration_ns": 123872, "warp_inst": 57_684_324, "issue_active": 0.4858,
-        "sources": _TD3_SRC, "sha256": "6ed9dd3bdcc23857eee61afd5ccf6fea65229ed5889dce989198cfbc3c23a7cc",
-        "profile": "profiles/td3_nll_kernel_td3_2M.md"},
-    "td3_nll_f64": {"bytes": 979_099_392, "events": 2_000_000, "duration_ns": 1546976, "fp64_pipe": 0.8508, "fp64_ops": {"dfma": 365_298_265, "dadd": 152_012_483, "dmul": 204_519_536},
-        "sources": _TD3_SRC, "sha256": "6ed9dd3bdcc23857eee61afd5ccf6fea65229ed5889dce989198cfbc3c23a7cc",
-        "profile": "profiles/td3_nll_kernel_td3_2M.md"},
-    "td4_nll_grad_f32": {"bytes": 170_933_248, "events": 2_000_000, "duration_ns": 65632, "warp_inst": 40_895_064, "issue_active": 0.6042,
-        "sources": _TD4_SRC, "sha256": "898395f56ed8fefb846f9ef3fb08867f16fcc8eb6ff15e61bc5de84b41a27fd9",
-        "profile": "profiles/td4_nll_f32_kernel_c4_2M.md"},
-    "td4_nll_f64": {"bytes": 339_106_816, "events": 2_000_000, "duration_ns": 1312992, "fp64_pipe": 0.8540, "fp64_ops": {"dfma": 325_287_209, "dadd": 112_011_018, "dmul": 164_442_328},
-        "sources": _TD4_SRC, "sha256": "898395f56ed8fefb846f9ef3fb08867f16fcc8eb6ff15e61bc5de84b41a27fd9",
-        "profile": "profiles/td4_nll_f64_kernel_c4_2M.md"},
+    "sop_nll_grad_f32": {"bytes": 123_068_160, "events": 10_000_000, "duration_ns": 40608, "warp_inst": 22_805_711, "issue_active": 0.5646,
+        "sources": _SOP_SRC, "sha256": "124950dcf5c5c94ec2e141d3f8f9b3cd0cbe1678cb7458087434a4cf52c03f98",
+        "profile": "profiles/likelihood_kernels.md"},
+    "sop_nll_f64": {"bytes": 243_111_680, "events": 10_000_000, "duration_ns": 913568, "fp64_pipe": 0.8516, "fp64_ops": {"dfma": 191_320_056, "dadd": 110_777_259, "dmul": 140_310_804},
+        "sources": _SOP_SRC, "sha256": "124950dcf5c5c94ec2e141d3f8f9b3cd0cbe1678cb7458087434a4cf52c03f98",
+        "profile": "profiles/likelihood_kernels.md"},
+    "coh_nll_grad_f32": {"bytes": 323_097_344, "events": 5_000_000, "duration_ns": 56800, "warp_inst": 27_167_220, "issue_active": 0.4435,
+        "sources": _COH_SRC, "sha256": "85ed9ad5153e8447601fa8515abd76e6c72e04a5a34ad367f3e52048f017d7ed",
+        "profile": "profiles/likelihood_kernels.md"},
+    "coh_nll_f64": {"bytes": 643_084_544, "events": 5_000_000, "duration_ns": 345728, "fp64_pipe": 0.8457, "fp64_ops": {"dfma": 166_323_009, "dadd": 778241, "dmul": 10_311_296},
+        "sources": _COH_SRC, "sha256": "85ed9ad5153e8447601fa8515abd76e6c72e04a5a34ad367f3e52048f017d7ed",
+        "profile": "profiles/likelihood_kernels.md"},
+    "coh_ls_grad_f32": {"bytes": 48_058_880, "events": 5_000_000, "duration_ns": 138848, "warp_inst": 87_844_859, "issue_active": 0.5679,
+        "sources": _COH_SRC, "sha256": "85ed9ad5153e8447601fa8515abd76e6c72e04a5a34ad367f3e52048f017d7ed",
+        "profile": "profiles/likelihood_kernels.md"},
+    "td3_nll_grad_f32": {"bytes": 523_144_704, "events": 2_000_000, "duration_ns": 85952, "warp_inst": 45_199_736, "issue_active": 0.4852,
+        "sources": _TD3_SRC, "sha256": "a673576e0ae4f32c52273e72077ed5265ab443ec1d2d1065a1aea6814d7e7645",
+        "profile": "profiles/likelihood_kernels.md"},
+    "td3_nll_f64": {"bytes": 979_168_512, "events": 2_000_000, "duration_ns": 845248, "fp64_pipe": 0.8468, "fp64_ops": {"dfma": 347_196_472, "dadd": 12_249_169, "dmul": 59_299_278},
+        "sources": _TD3_SRC, "sha256": "a673576e0ae4f32c52273e72077ed5265ab443ec1d2d1065a1aea6814d7e7645",
+        "profile": "profiles/likelihood_kernels.md"},
+    "td4_nll_grad_f32": {"bytes": 171_081_216, "events": 2_000_000, "duration_ns": 45024, "warp_inst": 20_464_799, "issue_active": 0.4573,
+        "sources": _TD4_SRC, "sha256": "63198b66e68e67608efd5fa465112bd2e4605b3a1cfc9324f22d06d841b6b1a9",
+        "profile": "profiles/likelihood_kernels.md"},
+    "td4_nll_f64": {"bytes": 371_114_496, "events": 2_000_000, "duration_ns": 540128, "fp64_pipe": 0.8479, "fp64_ops": {"dfma": 188_172_375, "dadd": 12_716_574, "dmul": 59_611_103},
+        "sources": _TD4_SRC, "sha256": "63198b66e68e67608efd5fa465112bd2e4605b3a1cfc9324f22d06d841b6b1a9",
+        "profile": "profiles/likelihood_kernels.md"},
 }
 
 
@@ -1145,11 +1142,11 @@ def run_profile(args):
 
     c2: 4 FP32+grad evaluations (one event kernel each: the kernel specialised for the model
         at run time, normalising the grid itself), then one FP64 evaluation (grid kernel, then
-        the scalar event kernel), 10M events.
+        the FP64 event kernel), 10M events.
     c3: amplitude caches and Gram (first call), then 4 FP32+grad and 1 FP64 coherent
         evaluations on 5M events generated on the device.
-    c3f: the same events with floating lineshapes: 4 FP32+grad evaluations (an MC pass and an
-        event pass each), then 1 FP64 evaluation.
+    c3f: the same events with floating lineshapes: 4 FP32+grad evaluations (one launch each), then
+        1 FP64 evaluation.
     c4: amplitude caches and Gram (first call), then 4 FP32+grad and 1 FP64 time-dependent
         four-body evaluations on 2M events.
     td3: amplitude caches and Gram matrices (first call), then 4 FP32+grad and 1 FP64
