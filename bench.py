@@ -852,8 +852,8 @@ def c3_measure(goo, ctx, stream, steps, n_events=5_000_000, n_mc=1_000_000, fma6
 
 
 def c3_floating_measure(goo, ctx, stream, model, ds, theta, flush, steps, n_events, n_mc):
-    """The same events with the resonance masses and widths free: every evaluation runs an MC
-    pass and an event pass that evaluate all amplitudes and their lineshape derivatives."""
+    """The same events with the resonance masses and widths free: every evaluation is one
+    launch over the MC sample and the events that evaluates all amplitudes and their derivatives."""
     import numpy as np
     import torch
 
@@ -969,7 +969,7 @@ def c4_measure(goo, ctx, stream, steps, n_events=2_000_000, n_mc=3_000_000, fma6
             "bound": "hbm" if grad else "fp64", "ncu": ncu_record(name, n_events),
             "roofline": None if grad or fma64 is None else fp64_roofline(name, n_events, per, fma64),
             "what": ("goo_nll_grad, FP32 amplitude cache (80 B/event) + time, adjoint gradient" if grad
-                     else "goo_nll, FP64 amplitude cache (160 B/event) + time")}
+                     else "goo_nll, FP64 amplitude cache (160 B/event, and 16 of B) + time")}
     out["parity_this_run"] = {"nll_f32": nll["f32"], "nll_f64": nll["f64"],
                               "rel": abs(nll["f32"] - nll["f64"]) / abs(nll["f64"])}
     # no fit is timed here: these events are phase-space points, not drawn from the model
