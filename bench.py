@@ -42,31 +42,31 @@ ISSUE_PEAK = 152 * 4 * 2.07e9
 
 NCU_RECORDS = {
     "sop_nll_grad_f32": {"bytes": 123_068_160, "events": 10_000_000, "duration_ns": 40608, "warp_inst": 22_805_711, "issue_active": 0.5646,
-        "sources": _SOP_SRC, "sha256": "124950dcf5c5c94ec2e141d3f8f9b3cd0cbe1678cb7458087434a4cf52c03f98",
+        "sources": _SOP_SRC, "sha256": "8c76b3c11bcc170ffcde57bc1ec90479a95fba091734604320cc23ba4d4ef2cb",
         "profile": "profiles/likelihood_kernels.md"},
     "sop_nll_f64": {"bytes": 243_111_680, "events": 10_000_000, "duration_ns": 913568, "fp64_pipe": 0.8516, "fp64_ops": {"dfma": 191_320_056, "dadd": 110_777_259, "dmul": 140_310_804},
-        "sources": _SOP_SRC, "sha256": "124950dcf5c5c94ec2e141d3f8f9b3cd0cbe1678cb7458087434a4cf52c03f98",
+        "sources": _SOP_SRC, "sha256": "8c76b3c11bcc170ffcde57bc1ec90479a95fba091734604320cc23ba4d4ef2cb",
         "profile": "profiles/likelihood_kernels.md"},
     "coh_nll_grad_f32": {"bytes": 323_097_344, "events": 5_000_000, "duration_ns": 56800, "warp_inst": 27_167_220, "issue_active": 0.4435,
-        "sources": _COH_SRC, "sha256": "85ed9ad5153e8447601fa8515abd76e6c72e04a5a34ad367f3e52048f017d7ed",
+        "sources": _COH_SRC, "sha256": "50df3928891bc82ae89a996ee33e106fca4a78927da9c62d7d7dedc7045d8823",
         "profile": "profiles/likelihood_kernels.md"},
     "coh_nll_f64": {"bytes": 643_084_544, "events": 5_000_000, "duration_ns": 345728, "fp64_pipe": 0.8457, "fp64_ops": {"dfma": 166_323_009, "dadd": 778241, "dmul": 10_311_296},
-        "sources": _COH_SRC, "sha256": "85ed9ad5153e8447601fa8515abd76e6c72e04a5a34ad367f3e52048f017d7ed",
+        "sources": _COH_SRC, "sha256": "50df3928891bc82ae89a996ee33e106fca4a78927da9c62d7d7dedc7045d8823",
         "profile": "profiles/likelihood_kernels.md"},
     "coh_ls_grad_f32": {"bytes": 48_058_880, "events": 5_000_000, "duration_ns": 138848, "warp_inst": 87_844_859, "issue_active": 0.5679,
-        "sources": _COH_SRC, "sha256": "85ed9ad5153e8447601fa8515abd76e6c72e04a5a34ad367f3e52048f017d7ed",
+        "sources": _COH_SRC, "sha256": "50df3928891bc82ae89a996ee33e106fca4a78927da9c62d7d7dedc7045d8823",
         "profile": "profiles/likelihood_kernels.md"},
     "td3_nll_grad_f32": {"bytes": 523_144_704, "events": 2_000_000, "duration_ns": 85952, "warp_inst": 45_199_736, "issue_active": 0.4852,
-        "sources": _TD3_SRC, "sha256": "a673576e0ae4f32c52273e72077ed5265ab443ec1d2d1065a1aea6814d7e7645",
+        "sources": _TD3_SRC, "sha256": "402ac1225fb418591f8bf2cb5246ab23f064850c04bf77f38956b1359b72b968",
         "profile": "profiles/likelihood_kernels.md"},
     "td3_nll_f64": {"bytes": 979_168_512, "events": 2_000_000, "duration_ns": 845248, "fp64_pipe": 0.8468, "fp64_ops": {"dfma": 347_196_472, "dadd": 12_249_169, "dmul": 59_299_278},
-        "sources": _TD3_SRC, "sha256": "a673576e0ae4f32c52273e72077ed5265ab443ec1d2d1065a1aea6814d7e7645",
+        "sources": _TD3_SRC, "sha256": "402ac1225fb418591f8bf2cb5246ab23f064850c04bf77f38956b1359b72b968",
         "profile": "profiles/likelihood_kernels.md"},
     "td4_nll_grad_f32": {"bytes": 171_081_216, "events": 2_000_000, "duration_ns": 45024, "warp_inst": 20_464_799, "issue_active": 0.4573,
-        "sources": _TD4_SRC, "sha256": "63198b66e68e67608efd5fa465112bd2e4605b3a1cfc9324f22d06d841b6b1a9",
+        "sources": _TD4_SRC, "sha256": "0687c1d783437bbd6d92b9172be3f0b394d31ca9cce7d76ce2ec0f281d014318",
         "profile": "profiles/likelihood_kernels.md"},
     "td4_nll_f64": {"bytes": 371_114_496, "events": 2_000_000, "duration_ns": 540128, "fp64_pipe": 0.8479, "fp64_ops": {"dfma": 188_172_375, "dadd": 12_716_574, "dmul": 59_611_103},
-        "sources": _TD4_SRC, "sha256": "63198b66e68e67608efd5fa465112bd2e4605b3a1cfc9324f22d06d841b6b1a9",
+        "sources": _TD4_SRC, "sha256": "0687c1d783437bbd6d92b9172be3f0b394d31ca9cce7d76ce2ec0f281d014318",
         "profile": "profiles/likelihood_kernels.md"},
 }
 

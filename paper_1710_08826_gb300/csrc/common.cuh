@@ -740,14 +740,4 @@ __device__ __forceinline__ void reduce_partials(const float2* partials, int nslo
   __syncthreads();
 }
 
-// The ticket and the reduction by every thread; returns true in the last block, which also
-// resets the ticket.
-__device__ __forceinline__ bool last_block_reduce(const float2* partials, int nslots, int nblocks,
-                                                  unsigned* ticket, double* out, ddf* smem) {
-  if (!last_block_ticket(ticket, nblocks)) return false;
-  reduce_partials(partials, nslots, nblocks, out, smem, blockDim.x);
-  if (threadIdx.x == 0) *ticket = 0u;
-  return true;
-}
-
 }  // namespace goo
