@@ -300,9 +300,16 @@ struct TdMath<double> {
     if (ha < 0x40180000) return mul_rn(gauss, herfcx_tab(__hiloint2double(ha, __double2loint(u)), tab.erfcx));
     return hu < 0 ? 0.0 : mul_rn(gauss, 0.5 * erfcx(u));
   }
-  // on the integer pipe (nonneg: false for -0, where both forms agree; below: to 2^-20)
+  // on the integer pipe (nonneg: false for -0, where both forms agree).  below: a double's high word with
+  // the other bits of a negative one flipped is a signed integer that orders as the doubles do, whatever their signs
+  // (t < 0 and the limit -inf, "never", among them); where the words are equal, t within 2^-20 of
+  // the limit, the answer is no.
   __device__ __forceinline__ static bool nonneg(double u) { return __double2hiint(u) >= 0; }
-  __device__ __forceinline__ static bool below(double t, double limit) { return __double2hiint(t) < __double2hiint(limit); }
+  __device__ __forceinline__ static int ordered_high(double x) {
+    const int h = __double2hiint(x);
+    return h ^ ((h >> 31) & 0x7fffffff);
+  }
+  __device__ __forceinline__ static bool below(double t, double limit) { return ordered_high(t) < ordered_high(limit); }
 };
 
 // E(g) for real g (gauss = exp(-t^2/2s^2)): with h = gauss erfcx(|u|) / 2, u = (g s^2 - t) / (s sqrt 2),
