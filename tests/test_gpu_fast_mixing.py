@@ -64,8 +64,7 @@ def test_negative_times_past_the_series_limit(goo, ctx, bodies, point, precision
     rnll, rg = ref.nll_grad(data, ref.amplitudes(mc) if bodies == 4 else mc, theta)
     assert abs(nll - rnll) <= TOL_NLL[precision] * max(abs(rnll), t.size), (nll, rnll)
     assert np.max(np.abs(g - rg)) <= TOL_GRAD[precision] * np.max(np.abs(rg)), (g, rg)
-    if precision == "f64":
-        assert model.nll(ds, theta, precision) == pytest.approx(nll, rel=1e-12)
+    assert model.nll(ds, theta, precision) == pytest.approx(nll, rel=1e-12)
     if bodies == 4:
         logf = model.eval_logf(ds, theta, precision).cpu().numpy()
         assert abs(-logf.sum() - rnll) <= TOL_NLL[precision] * max(abs(rnll), t.size)
