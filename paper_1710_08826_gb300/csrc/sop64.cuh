@@ -23,9 +23,13 @@
 
 namespace goo {
 
-// exp(-x) for x >= 0, 0 from 704 on (below 2^-1015 of the term it is added to)
+// exp(-x) for x >= 0, 0 from 704 on (below 2^-1015 of the term it is added to).  NaN stays NaN: a present
+// product whose exponent is NaN or +inf (its integral is negative, or vanishes) makes a difference of exponents
+// NaN, and the event then has no density, whatever the other products are.
 __device__ __forceinline__ double exp_neg(double x, const ExpTable& tab) {
-  return __double2hiint(x) >= 0x40860000 ? 0.0 : exp_tab(-x, tab);
+  const int h = __double2hiint(x);
+  if (h >= 0x40860000) return h > 0x7ff00000 ? x : 0.0;
+  return exp_tab(-x, tab);
 }
 
 // On the integer pipe: x is not zero; the largest exponent of an event's products is a number, not an
@@ -194,7 +198,7 @@ __global__ void __launch_bounds__(kBlock, 1)
         lp.mul(S);
       }
       invS = rcp64(S);
-    } else if (S > 0.0 && M > -1e29) {  // subnormal or infinite
+    } else if (S > 0.0 && M > -1e29 && M < HUGE_VAL) {  // S subnormal or infinite
       acc += wi * (M + log(S));
       invS = 1.0 / S;
     } else {
