@@ -23,12 +23,13 @@
 
 namespace goo {
 
-// exp(-x) for x >= 0, 0 from 704 on (below 2^-1015 of the term it is added to).  NaN stays NaN: a present
+// exp(-x) for x >= 0, 0 from 746 on (where exp() gives 0 too: a product that far below another one is all
+// there is where the other's weight is 0).  NaN stays NaN: a present
 // product whose exponent is NaN or +inf (its integral is negative, or vanishes) makes a difference of exponents
 // NaN, and the event then has no density, whatever the other products are.
 __device__ __forceinline__ double exp_neg(double x, const ExpTable& tab) {
   const int h = __double2hiint(x);
-  if (h >= 0x40860000) return h > 0x7ff00000 ? x : 0.0;
+  if (h >= 0x40875000) return h > 0x7ff00000 ? x : 0.0;
   return exp_tab(-x, tab);
 }
 
