@@ -60,7 +60,6 @@ struct DalitzModel {
   LsTables<double> ls64{};         // the lineshape constants of lineshape.cuh, passed by value
   LsTables<float> ls32{};
   // Gram matrices (K x K complex, row-major, FP64) per precision, with their keys
-  double* gram_dev[2] = {nullptr, nullptr};
   double gram_host[2][kMaxAmp * kMaxAmp * 2];
   uint64_t gram_key[2] = {0, 0};
   const goo_dataset* mc = nullptr;
@@ -1256,8 +1255,8 @@ static int ensure_gram(goo_model* m, int precision, const goo_dataset* ds = null
   const void* cache = nullptr;
   GOO_TRY(ensure_cache(m, d.mc, precision, &cache));
   if (d.mc->n < 1) return set_error(GOO_ERR_ARG, "the MC normalisation sample is empty");
-  GOO_TRY(gram_matrices(m->ctx, precision, false, 1, &cache, &cache, d.mc->n, d.nbw, d.K, d.gram_dev[pi],
-                        d.gram_host[pi], pi == 0 ? "gram_f32" : "gram_f64", [&]() -> int {
+  GOO_TRY(gram_matrices(m->ctx, precision, false, 1, &cache, &cache, d.mc->n, d.nbw, d.K, d.gram_host[pi],
+                        pi == 0 ? "gram_f32" : "gram_f64", [&]() -> int {
                           const void* c = nullptr;
                           return ds ? ensure_cache(m, ds, precision, &c, false, true) : GOO_OK;
                         }));
@@ -1495,7 +1494,7 @@ static int ensure_td_grams(goo_model* m, int precision, const goo_dataset* ds = 
   GOO_TRY(ensure_cache(m, d.mc, precision, &ca));
   GOO_TRY(ensure_cache(m, d.mc, precision, &cb, true));
   const void *x[3] = {ca, cb, ca}, *y[3] = {ca, cb, cb};
-  GOO_TRY(gram_matrices(ctx, precision, true, 3, x, y, d.mc->n, d.nbw, d.K, nullptr, d.gram3_host[pi],
+  GOO_TRY(gram_matrices(ctx, precision, true, 3, x, y, d.mc->n, d.nbw, d.K, d.gram3_host[pi],
                         pi == 0 ? "td3_gram_f32" : "td3_gram_f64", [&]() -> int {
                           const void* c = nullptr;
                           if (!ds) return GOO_OK;
@@ -1740,9 +1739,7 @@ int build_dalitz_model(goo_ctx* ctx, const goo_node* nodes, int n_nodes, int n_p
                      d->m3);
   (void)lo;
   (void)hi;
-  if (cudaMalloc(&d->dev, sizeof(DalitzDev)) != cudaSuccess ||
-      cudaMalloc(&d->gram_dev[0], sizeof(double) * 2 * kMaxAmp * kMaxAmp) != cudaSuccess ||
-      cudaMalloc(&d->gram_dev[1], sizeof(double) * 2 * kMaxAmp * kMaxAmp) != cudaSuccess) {
+  if (cudaMalloc(&d->dev, sizeof(DalitzDev)) != cudaSuccess) {
     cudaGetLastError();
     return set_error(GOO_ERR_OOM, "cannot allocate the amplitude model");
   }
@@ -1769,8 +1766,6 @@ void dalitz_free(goo_model* m) {
   DalitzModel* d = m->dalitz;
   if (!d) return;
   if (d->dev) cudaFree(d->dev);
-  for (int i = 0; i < 2; ++i)
-    if (d->gram_dev[i]) cudaFree(d->gram_dev[i]);
   delete d;
   m->dalitz = nullptr;
 }
@@ -1937,7 +1932,6 @@ int dalitz_server_info(goo_model* m, const double* theta, AmpModelInfo* info) {
   GOO_TRY(dalitz_dev(m));
   const DalitzModel& d = *m->dalitz;
   info->dalitz_dev = d.dev;
-  info->gram_dev = d.gram_dev[0];
   info->gram_host = d.gram_host[0];
   info->K = d.K;
   info->nbw = d.nbw;

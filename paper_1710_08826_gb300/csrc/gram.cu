@@ -8,7 +8,7 @@
 namespace goo {
 
 template <typename T, bool EXACT>
-static int launch_gram_tiles(goo_ctx* ctx, GramArgs& A, double* out, double* out_host, const char* name) {
+static int launch_gram_tiles(goo_ctx* ctx, GramArgs& A, double* out_host, const char* name) {
   const void* fn = (const void*)gram_tile_kernel<T, EXACT>;
   GOO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmem<T>));
   int blocks = 0;
@@ -16,13 +16,13 @@ static int launch_gram_tiles(goo_ctx* ctx, GramArgs& A, double* out, double* out
   GOO_TRY(ensure_partials(ctx, (size_t)blocks * kGramAll));
   LaunchScope ls(ctx, name);
   GOO_CUDA_TRY(launch_early(gram_tile_kernel<T, EXACT>, blocks, kGramBlock<T>, kGramSmem<T>, ctx->stream, A,
-                            ctx->scratch.partials, ctx->scratch.counters, out, out_host));
+                            ctx->scratch.partials, ctx->scratch.counters, out_host));
   GOO_CUDA_TRY(cudaGetLastError());
   return GOO_OK;
 }
 
 int gram_matrices(goo_ctx* ctx, int precision, bool exact, int nmat, const void* const* x, const void* const* y,
-                  int64_t n, int nbw, int K, double* out, double* host, const char* name,
+                  int64_t n, int nbw, int K, double* host, const char* name,
                   const std::function<int()>& behind) {
   const int fields = nmat * 2 * K * K;
   if (nmat > 3 || fields > kGramRecord) return set_error(GOO_ERR_STATE, "Gram matrices of %d fields", fields);
@@ -71,9 +71,9 @@ int gram_matrices(goo_ctx* ctx, int precision, bool exact, int nmat, const void*
       A.tile[t].nblk = (int)std::max<int64_t>(1, std::min<int64_t>(most, (int64_t)ctx->num_sms * work[t] / total));
       blk += A.tile[t].nblk;
     }
-    if (precision == GOO_F64) GOO_TRY((launch_gram_tiles<double, false>(ctx, A, out, s.gram_host, name)));
-    else if (exact) GOO_TRY((launch_gram_tiles<float, true>(ctx, A, out, s.gram_host, name)));
-    else GOO_TRY((launch_gram_tiles<float, false>(ctx, A, out, s.gram_host, name)));
+    if (precision == GOO_F64) GOO_TRY((launch_gram_tiles<double, false>(ctx, A, s.gram_host, name)));
+    else if (exact) GOO_TRY((launch_gram_tiles<float, true>(ctx, A, s.gram_host, name)));
+    else GOO_TRY((launch_gram_tiles<float, false>(ctx, A, s.gram_host, name)));
   }
   const int queued = behind ? behind() : GOO_OK;
   GOO_TRY(read_mapped(ctx, s.gram_host, fields, host));  // in any case: the kernel writes the record

@@ -239,11 +239,10 @@ __device__ __forceinline__ void gram_tile_sums(const GramArgs& A, const GramArgs
   }
 }
 
-// out[src]: the K x K matrices (re, im interleaved) on the device (null: not stored there), and in mapped
-// host memory.
+// out_host[src]: the K x K matrices (re, im interleaved), in mapped host memory.
 template <typename T, bool EXACT>
 __global__ void __launch_bounds__(kGramBlock<T>, 1) gram_tile_kernel(const __grid_constant__ GramArgs A, float2* partials,
-                                                              unsigned* counters, double* out, double* out_host) {
+                                                              unsigned* counters, double* out_host) {
   extern __shared__ __align__(16) unsigned char s_gram[];
   __shared__ double s_out[kGramAll];
   __shared__ ddf s_red[kGramBlock<T> / 32];
@@ -275,7 +274,6 @@ __global__ void __launch_bounds__(kGramBlock<T>, 1) gram_tile_kernel(const __gri
   const size_t o = (size_t)t.src * 2 * A.K * A.K;
   auto put = [&](int k, int l, int im, double m) {
     const size_t e = o + 2 * (k * A.K + l) + im;
-    if (out) out[e] = m;
     *(volatile double*)(out_host + e) = m;
   };
   if (threadIdx.x < kGramLanes) {
@@ -298,12 +296,12 @@ __global__ void __launch_bounds__(kGramBlock<T>, 1) gram_tile_kernel(const __gri
 }
 
 // Sums the nmat (1..3) K x K matrices of the caches x[q], y[q] over n events into `host` (nmat x K x K
-// complex) and, one Hermitian matrix only, `out` on the device (or null): launches the kernel, queues
+// complex): launches the kernel, queues
 // what `behind` queues (device work that does not need the matrices, so that it runs while the host
 // waits for them and launches what does), and waits for the mapped record.  A matrix of two different caches
 // needs both caches' own matrices in the same call.  exact: see above (FP32).
 int gram_matrices(goo_ctx* ctx, int precision, bool exact, int nmat, const void* const* x, const void* const* y,
-                  int64_t n, int nbw, int K, double* out, double* host, const char* name,
+                  int64_t n, int nbw, int K, double* host, const char* name,
                   const std::function<int()>& behind = {});
 
 }  // namespace goo

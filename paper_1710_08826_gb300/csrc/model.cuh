@@ -138,8 +138,7 @@ namespace goo {
 // constants and FP32-path Gram matrix at theta, amplitude/parameter layout and the box.
 struct AmpModelInfo {
   const void* dalitz_dev;   // DalitzDev*
-  const double* gram_dev;   // K x K complex, FP64 (from the float32 MC cache)
-  const double* gram_host;  // the same on the host
+  const double* gram_host;  // K x K complex, FP64 (from the float32 MC cache), on the host
   int K, nbw, has_nr;
   int par_re[16], par_im[16];
   double lo12, hi12, lo13, hi13;

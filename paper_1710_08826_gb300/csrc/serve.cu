@@ -1443,8 +1443,7 @@ int goo_server_create(goo_model* model, const double* theta_gen, const int* free
   SrvModel sm{};
   sm.nbw = info.nbw;
   sm.has_ref = 1;
-  std::vector<double> G(2 * info.K * info.K);
-  GOO_CUDA_TRY(cudaMemcpy(G.data(), info.gram_dev, G.size() * sizeof(double), cudaMemcpyDeviceToHost));
+  const double* G = info.gram_host;
   auto slot_of = [&](int m) { return m < info.nbw ? m : kSrvKB; };
   for (int a = 0; a < info.K; ++a)
     for (int b = 0; b < info.K; ++b) {

@@ -580,7 +580,6 @@ struct Td4Model {
   double br[kTdMaxAmp], bi[kTdMaxAmp];
   Td4Dev host{};
   Td4Dev* dev = nullptr;
-  double* gram_dev[2] = {nullptr, nullptr};
   double gram_host[2][kTdMaxAmp * kTdMaxAmp * 2];
   uint64_t gram_key[2] = {0, 0};
   const goo_dataset* mc = nullptr;
@@ -655,8 +654,7 @@ int build_td4_model(goo_ctx* ctx, const goo_node* nodes, int n_nodes, int n_para
   const unsigned char* bytes = (const unsigned char*)&h;
   for (size_t i = 0; i < sizeof(Td4Dev); ++i) key = (key ^ bytes[i]) * 1099511628211ull;
   d->key = key;
-  if (cudaMalloc(&d->dev, sizeof(Td4Dev)) != cudaSuccess || cudaMalloc(&d->gram_dev[0], sizeof(double) * 2 * kTdMaxAmp * kTdMaxAmp) != cudaSuccess ||
-      cudaMalloc(&d->gram_dev[1], sizeof(double) * 2 * kTdMaxAmp * kTdMaxAmp) != cudaSuccess) {
+  if (cudaMalloc(&d->dev, sizeof(Td4Dev)) != cudaSuccess) {
     cudaGetLastError();
     return set_error(GOO_ERR_OOM, "goo_model_build: four-body model tables");
   }
@@ -670,8 +668,6 @@ void td4_free(goo_model* m) {
   Td4Model* d = m->td4;
   if (!d) return;
   if (d->dev) cudaFree(d->dev);
-  for (auto& g : d->gram_dev)
-    if (g) cudaFree(g);
   delete d;
   m->td4 = nullptr;
 }
@@ -751,7 +747,7 @@ static int td4_ensure_gram(goo_model* m, int precision) {
   if (d.mc->n < 1) return set_error(GOO_ERR_ARG, "the MC normalisation sample is empty");
   const void* cache = nullptr;
   GOO_TRY(td4_cache(m, d.mc, precision, &cache));
-  GOO_TRY(gram_matrices(m->ctx, precision, false, 1, &cache, &cache, d.mc->n, d.K, d.K, d.gram_dev[pi], d.gram_host[pi],
+  GOO_TRY(gram_matrices(m->ctx, precision, false, 1, &cache, &cache, d.mc->n, d.K, d.K, d.gram_host[pi],
                         pi == 0 ? "td4_gram_f32" : "td4_gram_f64"));
   d.gram_key[pi] = key;
   return GOO_OK;
