@@ -135,6 +135,8 @@ struct CacheSlot {
   void* ptr = nullptr;
   size_t bytes = 0;
   uint64_t key = 0;
+  // FP64 four-body cache: B = sum b_k a_k in the plane behind the amplitudes; it was to have that plane
+  bool has_b = false, asked_b = false;
 };
 }  // namespace goo
 

@@ -685,7 +685,8 @@ int td4_set_norm(goo_model* m, const goo_norm_spec* spec) {
 // Bytes of the FP64 cache with B's plane.
 static size_t td4_bytes_b(const Td4Model& d, int64_t n) { return (size_t)(d.K + 1) * (size_t)n * sizeof(double2); }
 
-static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, const void** out) {
+// with_b: keep B in the FP64 cache where there is room (the events; nothing reads it from the MC sample's)
+static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, bool with_b, const void** out) {
   goo_dataset* ds = const_cast<goo_dataset*>(ds_c);
   Td4Model& d = *m->td4;
   goo_ctx* ctx = m->ctx;
@@ -695,15 +696,17 @@ static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, const
   CacheSlot& slot = ds->cache[pi];
   const int64_t n = ds->n;
   const size_t bytes = pi == 0 ? (size_t)((d.K + 1) / 2) * (size_t)n * sizeof(float4) : (size_t)d.K * (size_t)n * sizeof(double2);
-  if (slot.ptr && slot.key == key && slot.bytes >= bytes) {
+  const bool same = slot.ptr && slot.key == key && slot.bytes >= bytes;
+  if (same && (pi == 0 || !with_b || slot.asked_b)) {
     *out = slot.ptr;
     return GOO_OK;
   }
-  if (!slot.ptr || slot.bytes < bytes) {
+  // same: an MC sample's cache that is now evaluated as events
+  if (!slot.ptr || slot.bytes < bytes || same) {
     if (slot.ptr) cudaFree(slot.ptr);
     slot.ptr = nullptr;
     slot.bytes = 0;
-    size_t got = pi == 1 ? td4_bytes_b(d, n) : bytes;
+    size_t got = pi == 1 && with_b ? td4_bytes_b(d, n) : bytes;
     cudaError_t e = cudaMalloc(&slot.ptr, got > 0 ? got : 16);
     if (e != cudaSuccess && got > bytes) {  // no room for B's plane: the evaluation forms B itself
       cudaGetLastError();
@@ -717,6 +720,8 @@ static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, const
     }
     slot.bytes = got;
   }
+  slot.asked_b = with_b;
+  slot.has_b = pi == 1 && with_b && slot.bytes >= td4_bytes_b(d, n);
   if (n > 0) {
     const int nb = grid_blocks(ctx, n, 4);
     if (pi == 0) {
@@ -728,7 +733,7 @@ static int td4_cache(goo_model* m, const goo_dataset* ds_c, int precision, const
       Td4Cols<double> c{};
       for (int j = 0; j < 5; ++j) c.c[j] = ds->d64[j];
       LaunchScope ls(ctx, "td4_cache_f64");
-      td4_cache_kernel<double><<<nb, kBlock, 0, ctx->stream>>>(d.dev, c, n, slot.ptr, slot.bytes >= td4_bytes_b(d, n));
+      td4_cache_kernel<double><<<nb, kBlock, 0, ctx->stream>>>(d.dev, c, n, slot.ptr, slot.has_b);
     }
     GOO_CUDA_TRY(cudaGetLastError());
   }
@@ -746,7 +751,7 @@ static int td4_ensure_gram(goo_model* m, int precision) {
   if (d.gram_key[pi] == key) return GOO_OK;
   if (d.mc->n < 1) return set_error(GOO_ERR_ARG, "the MC normalisation sample is empty");
   const void* cache = nullptr;
-  GOO_TRY(td4_cache(m, d.mc, precision, &cache));
+  GOO_TRY(td4_cache(m, d.mc, precision, false, &cache));
   GOO_TRY(gram_matrices(m->ctx, precision, false, 1, &cache, &cache, d.mc->n, d.K, d.K, d.gram_host[pi],
                         pi == 0 ? "td4_gram_f32" : "td4_gram_f64"));
   d.gram_key[pi] = key;
@@ -879,7 +884,7 @@ static int launch_td4_f64(goo_model* m, const void* cache, const goo_dataset* ds
   goo_ctx* ctx = m->ctx;
   Td4Args<double> a;
   td4_args<double>(m, theta, ds->n, a);
-  a.has_b = ds->cache[1].bytes >= td4_bytes_b(*m->td4, ds->n);
+  a.has_b = ds->cache[1].has_b;
   td4_norm_terms<double>(m, GOO_F64, a);
   const Fp64Tables* tables = nullptr;
   GOO_TRY(fp64_tables(ctx, &tables));
@@ -922,7 +927,7 @@ int td4_nll(goo_model* m, const goo_dataset* ds, int64_t begin, int64_t end, con
     return GOO_OK;
   }
   const void* cache = nullptr;
-  GOO_TRY(td4_cache(m, ds, precision, &cache));
+  GOO_TRY(td4_cache(m, ds, precision, true, &cache));
   GOO_TRY((grad ? td4_launch<true>(m, cache, ds, begin, end, theta, precision, out_mode)
                 : td4_launch<false>(m, cache, ds, begin, end, theta, precision, out_mode)));
   return read_result_mapped(ctx, nout, out);
@@ -973,7 +978,7 @@ int td4_eval_logf(goo_model* m, const goo_dataset* ds, const double* theta, int 
   if (ds->n == 0) return GOO_OK;
   const double logN = std::log(td4_norm_host(m, theta, precision));
   const void* cache = nullptr;
-  GOO_TRY(td4_cache(m, ds, precision, &cache));
+  GOO_TRY(td4_cache(m, ds, precision, true, &cache));
   const int nb = grid_blocks(ctx, ds->n, 4);
   LaunchScope ls(ctx, "td4_logf");
   const bool small = m->td4->K <= 10;
@@ -986,7 +991,7 @@ int td4_eval_logf(goo_model* m, const goo_dataset* ds, const double* theta, int 
   } else {
     Td4Args<double> a;
     td4_args<double>(m, theta, ds->n, a);
-    a.has_b = ds->cache[1].bytes >= td4_bytes_b(*m->td4, ds->n);
+    a.has_b = ds->cache[1].has_b;
     const Fp64Tables* tables = nullptr;
     GOO_TRY(fp64_tables(ctx, &tables));
     const double2* amps = (const double2*)cache;
@@ -1007,7 +1012,7 @@ int td4_gram(goo_model* m, int precision, double* out, int* K_out) {
 
 int td4_amplitudes(goo_model* m, const goo_dataset* ds, int precision, const void** cache, int* n_amp) {
   if (ds->ncols < 5) return set_error(GOO_ERR_ARG, "the four-body model needs the five phase-space columns");
-  GOO_TRY(td4_cache(m, ds, precision, cache));
+  GOO_TRY(td4_cache(m, ds, precision, true, cache));
   GOO_CUDA_TRY(cudaStreamSynchronize(m->ctx->stream));
   *n_amp = m->td4->K;
   return GOO_OK;
