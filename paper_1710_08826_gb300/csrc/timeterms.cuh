@@ -155,6 +155,7 @@ struct TimeCoef {
   // criterion: K - 1 when that covers every event the dataset's time range admits
   int ku;
   T t_series;
+  T t_gauss;                   // below it the FP32 Gaussian is subnormal
   T is2, is2h, ir2s;           // 1 / s^2, 1 / (2 s^2), 1 / (s sqrt 2): no event divides by them
   T k_phi;                     // 1 / (s sqrt(2 pi))
   T s2, Gs2, hG2s2;            // s^2, G s^2, G^2 s^2 / 2
@@ -195,6 +196,7 @@ inline void fill_time_coef(TimeCoef<T>& c, double x64, double y64, double tau, d
   c.qy = (T)(2.0 * G * G * y);
   c.Gx2 = (T)(G * G * x * x);
   c.Gy2 = (T)(G * G * y * y);
+  c.t_gauss = (T)(-s * std::sqrt(2.0 * 87.3));
   double fact = 1.0;  // (2m)!
   for (int m = 0; m <= K; ++m) {
     const double sg = (m & 1) ? -1.0 : 1.0;
@@ -262,7 +264,9 @@ struct TdMath<float> {
   __device__ __forceinline__ static bool below(float t, float limit) { return t < limit; }
 };
 // Two events: exp from the hardware's 2^x of x log2(e) rounded once, the product's rounding error (an FMA gives
-// it) applied as a factor; erfcx from its table in shared memory.
+// it) applied as a factor; erfcx from its table in shared memory.  2^x is 0 below 2^-126: where a result
+// there matters (the Gaussian of an event 13.2 resolutions below zero, the exponential 87 lifetimes above, whose
+// rates are normal numbers) expf() takes over (exp_tail, for arguments below -87.3).
 template <>
 struct TdMath<float2> {
   const Fp32Tables& tab;
@@ -271,6 +275,10 @@ struct TdMath<float2> {
     const float2 e = fma_rn(v, pk::splat(kLog2eLo), fma_rn(v, pk::splat(kLog2eHi), np));
     const float2 y = make_float2(pk::ex2(-np.x), pk::ex2(-np.y));
     return fma_rn(mul_rn(y, e), pk::splat(kLn2Hi), y);
+  }
+  __device__ __forceinline__ static void exp_tail(float2 v, float2& y) {
+    if (v.x < -87.3f) y.x = expf(v.x);
+    if (v.y < -87.3f) y.y = expf(v.y);
   }
   // gauss erfcx(|u|) / 2; where u <= -6 it is below 2^-52 of the exponential it is subtracted from
   // (conv_real) and is left out
@@ -320,7 +328,12 @@ __device__ __forceinline__ V conv_real(const TdMath<V>& F, T g, T gs2, T hg2s2, 
   const V z{};
   const V u = mul_rn(sub_rn(in(z, gs2), t), in(z, ir2s));
   const V h = F.gauss_herfcx(gauss, u);
-  const V x = sub_rn(F.exp(fma_rn(in(z, -g), t, in(z, hg2s2))), h);
+  const V a = fma_rn(in(z, -g), t, in(z, hg2s2));
+  V e = F.exp(a);
+  if constexpr (sizeof(V) > sizeof(T)) {
+    if (fminf(a.x, a.y) < -87.3f) F.exp_tail(a, e);
+  }
+  const V x = sub_rn(e, h);
   if constexpr (sizeof(V) > sizeof(T)) return make_float2(u.x >= 0.f ? h.x : x.x, u.y >= 0.f ? h.y : x.y);
   else return F.nonneg(u) ? h : x;
 }
@@ -422,7 +435,9 @@ __device__ __forceinline__ void time_terms_g(const TdMath<T>& F, const TimeCoef<
 // The same for two events, packed; an event above the series' limit goes through the scalar code.
 __device__ __forceinline__ void time_terms_pair(const TdMath<float2>& F, const TimeCoef<float>& c, const float* wa,
                                                 int wN, float wL, float2 t, TimeTerms<float2>& R) {
-  const float2 gauss = F.exp(mul_rn(mul_rn(mul_rn(t, pk::splat(-1.f)), t), pk::splat(c.is2h)));
+  const float2 q = mul_rn(mul_rn(mul_rn(t, pk::splat(-1.f)), t), pk::splat(c.is2h));
+  float2 gauss = F.exp(q);
+  if (fminf(t.x, t.y) < c.t_gauss) F.exp_tail(q, gauss);
   R.phi = mul_rn(pk::splat(c.k_phi), gauss);
   if (c.ku == TimeCoef<float>::K) time_terms_series<float2, float, TimeCoef<float>::K>(F, c, t, gauss, R);
   else time_terms_series<float2, float, TimeCoef<float>::K - 1>(F, c, t, gauss, R);
