@@ -8,7 +8,9 @@ normalisation, per-event evaluation, log, accumulation, adjoint gradient and the
 reduction, through goo_nll_grad with FP32 per-event arithmetic and compensated accumulation.
 The FP64 plain form (goo_nll in float64) is timed beside it.
 
-Prints ONE JSON line on rank 0.  With --impl reference it times the FP64 CPU oracle on
+Prints ONE JSON line on rank 0: the benchmark's own figures and one number or two of each other workload,
+short enough (MAX_LINE) to be read back whole from the end of a log.  Everything that was measured goes to
+standard error, one JSON object per part, and with --record to a file.  With --impl reference it times the FP64 CPU oracle on
 the host cores instead (bounded samples of the same workload).
 """
 import argparse
@@ -28,6 +30,7 @@ METRIC = "NLL evals/s (events/s) FP64 plain vs FP32+grad; toy fits/s, p50/p99 la
 UNIT = "events/s"
 BYTES_PER_EVENT_F32 = 12   # three float32 columns
 BYTES_PER_EVENT_F64 = 24
+MAX_LINE = 2600            # characters of the JSON line
 # Counters of one launch of each timed kernel from one ncu capture (the profiles/ file named
 # in "profile"): DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) and, for the FP64
 # kernels, the FP64 pipe's active fraction (sm__pipe_fp64_cycles_active).  A record is used
@@ -117,6 +120,40 @@ def fp64_roofline(kernel, n_events, kernel_ms, fma64_per_s):
             "profile": rec["profile"]}
 
 
+# the parts of the full record that the JSON line gives in full, and what it takes of the others
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+             "vs_baseline", "dtype", "data", "config", "gpu_launches", "clocks")
+PART_KEYS = {"e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "ms_per_step"),
+             "fp64_plain": ("events_per_s", "ms_per_eval"), "parity_this_run": ("rel",),
+             "roofline": ("bound", "kernel", "achieved", "peak", "unit", "frac", "launch_ms"),
+             "c5_serving": ("toys", "fits_per_s", "latency_p50_s", "latency_p99_s", "converged"),
+             "c5_serving_poisson": ("arrival", "fits_per_s", "latency_p50_s", "latency_p99_s"),
+             "cpu_baseline": ("value", "unit", "cores", "kind")}
+FORM_KEYS = ("c1_1d", "c3_dalitz", "c4_td4", "td3_dalitz")
+
+
+def short_line(line):
+    """The printed line: LINE_KEYS and PART_KEYS of the full record, floats to seven digits, and events/s of the
+    other workloads' forms.  Parts are left out from the last one on where it would exceed MAX_LINE."""
+    def short(v):
+        if isinstance(v, float):
+            return float(f"{v:.7g}")
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return [short(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+    out = {k: short(line[k]) for k in LINE_KEYS if k in line}
+    parts = {k: short({q: line[k][q] for q in keys if q in line[k]}) for k, keys in PART_KEYS.items()
+             if isinstance(line.get(k), dict)}
+    for k in FORM_KEYS:
+        forms = line.get(k) or {}
+        parts[k + "_events_per_s"] = {q: short(forms[q]["events_per_s"]) for q in ("f32_grad", "f64_plain") if q in forms}
+    for k, v in parts.items():
+        if v and (k == "e2e" or len(json.dumps({**out, k: v})) <= MAX_LINE):
+            out[k] = v
+    return out
+
+
 def idle_gpu_wait(cycles=200_000):
     """Keeps the current stream busy for about 0.1 ms without touching memory, so that a
     synchronous evaluation issued meanwhile starts right after its start event (tight event
@@ -144,6 +181,7 @@ def parse():
     ap.add_argument("--no-extra", action="store_true", help="skip the Dalitz and serving measurements")
     ap.add_argument("--toys", type=int, default=4096)
     ap.add_argument("--rate", type=float, default=1000.0, help="Poisson arrival rate of the second serving run")
+    ap.add_argument("--record", help="file for the full record as JSON")
     ap.add_argument("--profile", action="store_true", help="short fixed launch sequence for ncu captures")
     ap.add_argument("--profile-workload", default="c2", choices=["c2", "c3", "c3f", "c4", "c5", "td3"])
     return ap.parse_args()
@@ -729,7 +767,13 @@ def run_ours(args):
                 base["host"] = host
                 line[key]["cpu_baseline"] = base
     if rank == 0:
-        print(json.dumps(line))
+        for key, part in line.items():
+            print(json.dumps({key: part}), file=sys.stderr)
+        if args.record:
+            with open(args.record, "w") as f:
+                json.dump(line, f, indent=1)
+        sys.stderr.flush()
+        print(json.dumps(short_line(line)))
     if pg is not None:
         pg.barrier()
         pg.destroy_process_group()
