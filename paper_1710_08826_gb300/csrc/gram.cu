@@ -10,12 +10,12 @@ namespace goo {
 template <typename T, bool EXACT>
 static int launch_gram_tiles(goo_ctx* ctx, GramArgs& A, double* out_host, const char* name) {
   const void* fn = (const void*)gram_tile_kernel<T, EXACT>;
-  GOO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmem<T>));
+  GOO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGramSmem<T, EXACT>));
   int blocks = 0;
   for (int t = 0; t < A.ntiles; ++t) blocks += A.tile[t].nblk;
-  GOO_TRY(ensure_partials(ctx, (size_t)blocks * kGramAll));
+  GOO_TRY(ensure_partials(ctx, (size_t)blocks * kGramAll<T, EXACT>));
   LaunchScope ls(ctx, name);
-  GOO_CUDA_TRY(launch_early(gram_tile_kernel<T, EXACT>, blocks, kGramBlock<T>, kGramSmem<T>, ctx->stream, A,
+  GOO_CUDA_TRY(launch_early(gram_tile_kernel<T, EXACT>, blocks, kGramBlock<T, EXACT>, kGramSmem<T, EXACT>, ctx->stream, A,
                             ctx->scratch.partials, ctx->scratch.counters, out_host));
   GOO_CUDA_TRY(cudaGetLastError());
   return GOO_OK;
@@ -39,20 +39,22 @@ int gram_matrices(goo_ctx* ctx, int precision, bool exact, int nmat, const void*
   A.K = K;
   // the record comes back through mapped host memory, polled field by field (read_result_mapped)
   arm_mapped(s.gram_host, fields);
+  const int cols = precision == GOO_F32 && !exact ? kGramCols<float, false> : kGramCols<double, false>;
+  static_assert(kGramCols<float, true> == kGramCols<double, false>, "two widths of tiles");
   int work[kGramTiles], total = 0;
   for (int q = 0; q < nmat; ++q) {
     A.x[q] = x[q];
     A.y[q] = y[q];
     const bool hermitian = x[q] == y[q];
     for (int r0 = 0; r0 < nbw; r0 += kGramRows)
-      for (int c0 = hermitian ? r0 : 0; c0 < nbw; c0 += kGramCols) {
+      for (int c0 = hermitian ? r0 : 0; c0 < nbw; c0 += cols) {
         GramArgs::Tile& t = A.tile[A.ntiles];
         t.src = q;
         t.r0 = r0;
         t.c0 = c0;
         t.diag = hermitian && c0 == r0;
         // its products, and about the cost of six more for reading an event
-        work[A.ntiles] = kGramRows * std::min(kGramCols, nbw - c0) - (t.diag ? 6 : 0) + 6;
+        work[A.ntiles] = kGramRows * std::min(cols, nbw - c0) - (t.diag ? 6 : 0) + 6;
         total += work[A.ntiles++];
       }
     if (nbw < K && (!hermitian || nbw == 0))  // the constant amplitude's fields, which no tile writes
@@ -63,7 +65,7 @@ int gram_matrices(goo_ctx* ctx, int precision, bool exact, int nmat, const void*
         }
   }
   if (A.ntiles > 0) {
-    const int block = precision == GOO_F64 ? kGramBlock<double> : kGramBlock<float>;
+    const int block = precision == GOO_F64 ? kGramBlock<double, false> : exact ? kGramBlock<float, true> : kGramBlock<float, false>;
     const int64_t most = (n + block - 1) / block;
     int blk = 0;
     for (int t = 0; t < A.ntiles; ++t) {

@@ -2,19 +2,20 @@
 // G_kl = mean over the sample of X_k conj(Y_l), X and Y two caches of the same events (the same one
 // for a Hermitian matrix, of which only the upper triangle is summed).
 //
-// The matrix is cut into tiles of 4 rows and 8 columns.  A block takes one tile and a share of the events and
-// keeps the tile's 32 complex sums in registers, so an event's 12 amplitudes are read once for
-// 32 products; one block of 384 threads per SM (the sums fill the register file), the SMs
+// The matrix is cut into tiles of 4 rows and 8 columns (FP32: 4 and 4).  A block takes one tile and a share of
+// the events and keeps the tile's complex sums in registers, so an event's amplitudes are read once for
+// all of the tile's products; one block per SM (the sums fill the register file), the SMs
 // divided over the tiles in proportion to their products.  One block per row that re-read the whole
 // cache for every row and added with scalar Kahan sums took 128 us for 1M points of 9
-// amplitudes, this kernel 32 us (64 MB: 9.4 us; some 14 us are launch, reduction and result); the three 16 x 16 matrices of the time-dependent
+// amplitudes, this kernel 35 us (64 MB: 9.4 us; some 14 us are launch, reduction and result); the three 16 x 16 matrices of the time-dependent
 // three-body model, one block per element with FP64 sums before, 16 ms, now 0.9 ms.
 //
-// FP32: sums of 16 events run in registers (plain FMAs) and are then added, Kahan compensated, to the
-// thread's totals in shared memory: compensated for every event the sums take three times the instructions, and
-// the error (that of the FP32 amplitudes, 9e-8) was the same.  EXACT (the
-// time-dependent three-body model, whose sums were FP64): every product and its rounding
-// error (an FMA gives it) is added with compensation in registers, so the result is that of
+// FP32: every event's product is added with Kahan's compensation, real and imaginary part as one packed pair
+// (sums and remainders of a 4 x 4 tile take 64 registers), so the sums' error is that of the products'
+// rounding, 1e-10 of the mean magnitude at 1M points.  Sums of 16 events run in plain FMAs before a
+// compensated addition in shared memory were 8 us faster per scan of three points (320 against 328) and off by
+// 1e-9 to 3e-9.  EXACT (the time-dependent three-body model, whose sums were FP64): every product and its rounding
+// error (an FMA gives it) is added with compensation, so the result is that of
 // FP64 products and sums to 2^-45.  FP64: FMA chains (bound by the FP64 pipe).
 // Each tile's last block adds its blocks' sums in block order; results are bitwise repeatable.
 #pragma once
@@ -25,21 +26,24 @@
 
 namespace goo {
 
-constexpr int kGramRows = 4, kGramCols = 8;
+constexpr int kGramRows = 4;
+template <typename T, bool EXACT>
+constexpr int kGramCols = sizeof(T) == 4 && !EXACT ? 4 : 8;
 constexpr int kGramTiles = 24;
-constexpr int kGramLanes = 2 * kGramRows * kGramCols;  // lane 2 (k kGramCols + l) + (0: re, 1: im)
-constexpr int kGramAll = kGramLanes + 2 * kGramRows;   // then the rows' own sums (the constant amplitude's column)
+template <typename T, bool EXACT>
+constexpr int kGramLanes = 2 * kGramRows * kGramCols<T, EXACT>;  // lane 2 (k kGramCols + l) + (0: re, 1: im)
+// then the rows' own sums (the constant amplitude's column)
+template <typename T, bool EXACT>
+constexpr int kGramAll = kGramLanes<T, EXACT> + 2 * kGramRows;
 constexpr int kGramTickets = 16;  // the tiles' tickets: counters[kGramTickets ..)
-constexpr int kGramRun = 16;      // FP32: events summed in registers at a time
-// FP32: events requested ahead.  Two in flight per thread of one block per SM held 37 KB per SM, which at
-// the memory's latency is 3/4 of its bandwidth
-template <bool DIAG>
-constexpr int kGramAhead = DIAG ? 4 : 2;
-// threads per block: FP32 the most whose lanes fit in shared memory, FP64 the most whose sums fit in registers
-template <typename T>
-constexpr int kGramBlock = sizeof(T) == 4 ? 384 : 256;
-template <typename T>
-constexpr size_t kGramSmem = (size_t)kGramAll * kGramBlock<T> * sizeof(ddf);
+// FP32: events requested ahead; a diagonal tile's third and fourth cost registers that 16 warps do not have
+// (333 us per scan)
+constexpr int kGramAhead = 2;
+// threads per block: the most whose sums fit in registers (FP32 in 384 threads: 333 us per scan)
+template <typename T, bool EXACT>
+constexpr int kGramBlock = sizeof(T) == 8 ? 256 : EXACT ? 384 : 512;
+template <typename T, bool EXACT>
+constexpr size_t kGramSmem = (size_t)kGramAll<T, EXACT> * kGramBlock<T, EXACT> * sizeof(ddf);
 
 struct GramArgs {
   const void *x[3], *y[3];  // caches of up to three matrices
@@ -89,16 +93,19 @@ template <typename T, bool EXACT>
 struct GramSum;
 template <>
 struct GramSum<float, false> {
-  float re, im;
-  __device__ __forceinline__ void clear() { re = im = 0.f; }
+  float2 s, c;  // (re, im): the sums, and what their roundings left out
+  __device__ __forceinline__ void clear() { s = c = make_float2(0.f, 0.f); }
+  __device__ __forceinline__ void step(float2 y) {
+    const float2 t = pk::add(s, y);
+    c = pk::sub(y, pk::sub(t, s));
+    s = t;
+  }
   __device__ __forceinline__ void mul_add(float2 x, float2 y) {
-    re = fmaf(x.x, y.x, fmaf(x.y, y.y, re));
-    im = fmaf(x.y, y.x, fmaf(-x.x, y.y, im));
+    step(pk::fma(pk::splat(x.y), make_float2(y.y, y.x), pk::fma(pk::splat(x.x), make_float2(y.x, -y.y), c)));
   }
-  __device__ __forceinline__ void add(float2 x) {
-    re += x.x;
-    im += x.y;
-  }
+  __device__ __forceinline__ void add(float2 x) { step(pk::add(x, c)); }
+  __device__ __forceinline__ ddf dre() const { return dd_make(s.x, c.x); }
+  __device__ __forceinline__ ddf dim() const { return dd_make(s.y, c.y); }
 };
 template <>
 struct GramSum<float, true> {
@@ -140,30 +147,30 @@ struct GramSum<double, false> {
 
 template <typename T, bool EXACT>
 struct GramAcc {
-  GramSum<T, EXACT> m[kGramRows][kGramCols], row[kGramRows];
+  GramSum<T, EXACT> m[kGramRows][kGramCols<T, EXACT>], row[kGramRows];
   __device__ __forceinline__ void clear() {
 #pragma unroll
     for (int k = 0; k < kGramRows; ++k) {
       row[k].clear();
 #pragma unroll
-      for (int l = 0; l < kGramCols; ++l) m[k][l].clear();
+      for (int l = 0; l < kGramCols<T, EXACT>; ++l) m[k][l].clear();
     }
   }
 };
 
-// The thread's sums over its events into its column of s (kGramAll lanes of kGramBlock<T> double-floats).
+// The thread's sums over its events into its column of s (kGramAll lanes of kGramBlock<T, EXACT> double-floats).
 template <typename T, bool EXACT, bool DIAG>
 __device__ __forceinline__ void gram_tile_sums(const GramArgs& A, const GramArgs::Tile& t, int64_t i, int64_t stride,
                                                ddf* s) {
   using V = typename GramAmp<T>::V;
-  constexpr bool RUNS = sizeof(T) == 4 && !EXACT;
+  constexpr int COLS = kGramCols<T, EXACT>;
   const void *xc = A.x[t.src], *yc = A.y[t.src];
   GramAcc<T, EXACT> acc;
   acc.clear();
-  auto lane = [&](int j) -> ddf& { return s[j * kGramBlock<T>]; };
+  auto lane = [&](int j) -> ddf& { return s[j * kGramBlock<T, EXACT>]; };
   // the D events ahead are requested before this one's products; a diagonal tile's rows are its first columns
-  constexpr int D = kGramAhead<DIAG>;
-  V nx[D][kGramRows], ny[D][kGramCols];
+  constexpr int D = sizeof(T) == 4 && !EXACT ? kGramAhead : 1;
+  V nx[D][kGramRows], ny[D][COLS];
   auto fetch = [&](int b, int64_t j) {
     if (j >= A.n) return;
     if (!DIAG) GramAmp<T>::load(xc, A.n, j, t.r0, A.nbw, nx[b]);
@@ -171,7 +178,7 @@ __device__ __forceinline__ void gram_tile_sums(const GramArgs& A, const GramArgs
   };
   auto event = [&](int b) {
 #pragma unroll
-    for (int l = 0; l < kGramCols; ++l) {
+    for (int l = 0; l < COLS; ++l) {
       if (t.c0 + l >= A.nbw) break;  // uniform
 #pragma unroll
       for (int k = 0; k < kGramRows; ++k)
@@ -182,92 +189,66 @@ __device__ __forceinline__ void gram_tile_sums(const GramArgs& A, const GramArgs
       for (int k = 0; k < kGramRows; ++k) acc.row[k].add(ny[b][k]);
     }
   };
-  if constexpr (RUNS) {
-    for (int j = 0; j < kGramAll; ++j) lane(j) = ddf{0.f, 0.f};
-    // (hi, lo) holds a Kahan sum and its compensation
-    auto flush = [&]() {
-      auto put = [&](int j, float v) {
-        const ddf o = lane(j);
-        const float y = v - o.lo, h = o.hi + y;
-        lane(j) = ddf{h, (h - o.hi) - y};
-      };
-#pragma unroll
-      for (int k = 0; k < kGramRows; ++k) {
-#pragma unroll
-        for (int l = 0; l < kGramCols; ++l) {
-          if (DIAG && l < k) continue;
-          put(2 * (k * kGramCols + l), acc.m[k][l].re);
-          put(2 * (k * kGramCols + l) + 1, acc.m[k][l].im);
-        }
-        if (DIAG) {
-          put(kGramLanes + 2 * k, acc.row[k].re);
-          put(kGramLanes + 2 * k + 1, acc.row[k].im);
-        }
-      }
-      acc.clear();
-    };
+  if constexpr (D > 1) {
 #pragma unroll
     for (int e = 0; e < D; ++e) fetch(e, i + e * stride);
-    while (i < A.n) {
 #pragma unroll 1
-      for (int r = 0; r < kGramRun / D && i < A.n; ++r, i += D * stride) {
+    for (; i < A.n; i += D * stride) {
 #pragma unroll
-        for (int e = 0; e < D; ++e) {
-          if (i + e * stride >= A.n) break;
-          event(e);
-          fetch(e, i + (D + e) * stride);
-        }
+      for (int e = 0; e < D; ++e) {
+        if (i + e * stride >= A.n) break;
+        event(e);
+        fetch(e, i + (D + e) * stride);
       }
-      flush();
     }
-    for (int j = 0; j < kGramAll; ++j) lane(j) = dd_make(lane(j).hi, -lane(j).lo);
   } else {
     for (; i < A.n; i += stride) {
       fetch(0, i);
       event(0);
     }
+  }
 #pragma unroll
-    for (int k = 0; k < kGramRows; ++k) {
+  for (int k = 0; k < kGramRows; ++k) {
 #pragma unroll
-      for (int l = 0; l < kGramCols; ++l) {
-        lane(2 * (k * kGramCols + l)) = acc.m[k][l].dre();
-        lane(2 * (k * kGramCols + l) + 1) = acc.m[k][l].dim();
-      }
-      lane(kGramLanes + 2 * k) = acc.row[k].dre();
-      lane(kGramLanes + 2 * k + 1) = acc.row[k].dim();
+    for (int l = 0; l < COLS; ++l) {
+      lane(2 * (k * COLS + l)) = acc.m[k][l].dre();
+      lane(2 * (k * COLS + l) + 1) = acc.m[k][l].dim();
     }
+    lane(kGramLanes<T, EXACT> + 2 * k) = acc.row[k].dre();
+    lane(kGramLanes<T, EXACT> + 2 * k + 1) = acc.row[k].dim();
   }
 }
 
 // out_host[src]: the K x K matrices (re, im interleaved), in mapped host memory.
 template <typename T, bool EXACT>
-__global__ void __launch_bounds__(kGramBlock<T>, 1) gram_tile_kernel(const __grid_constant__ GramArgs A, float2* partials,
+__global__ void __launch_bounds__(kGramBlock<T, EXACT>, 1) gram_tile_kernel(const __grid_constant__ GramArgs A, float2* partials,
                                                               unsigned* counters, double* out_host) {
+  constexpr int COLS = kGramCols<T, EXACT>, LANES = kGramLanes<T, EXACT>, ALL = kGramAll<T, EXACT>;
   extern __shared__ __align__(16) unsigned char s_gram[];
-  __shared__ double s_out[kGramAll];
-  __shared__ ddf s_red[kGramBlock<T> / 32];
+  __shared__ double s_out[ALL];
+  __shared__ ddf s_red[kGramBlock<T, EXACT> / 32];
   int ti = 0;
   while (ti + 1 < A.ntiles && (int)blockIdx.x >= A.tile[ti + 1].blk0) ++ti;
   const GramArgs::Tile t = A.tile[ti];  // in registers
   const int b = blockIdx.x - t.blk0;
   ddf* buf = reinterpret_cast<ddf*>(s_gram);
-  const int64_t i0 = b * (int64_t)kGramBlock<T> + threadIdx.x, stride = (int64_t)t.nblk * kGramBlock<T>;
+  const int64_t i0 = b * (int64_t)kGramBlock<T, EXACT> + threadIdx.x, stride = (int64_t)t.nblk * kGramBlock<T, EXACT>;
   grid_dep_wait();  // the caches' kernel
   if (t.diag) gram_tile_sums<T, EXACT, true>(A, t, i0, stride, buf + threadIdx.x);
   else gram_tile_sums<T, EXACT, false>(A, t, i0, stride, buf + threadIdx.x);
   grid_dep_launch();  // what is queued behind may take the SMs that are done
   __syncthreads();
   // lane sums over the threads: one warp per lane at a time, then the warp's tree
-  float2* part = partials + (size_t)t.blk0 * kGramAll;
+  float2* part = partials + (size_t)t.blk0 * ALL;
   const int warp = threadIdx.x / 32, w = threadIdx.x % 32;
-  for (int lane = warp; lane < kGramAll; lane += kGramBlock<T> / 32) {
-    ddf v = buf[lane * kGramBlock<T> + w];
-    for (int j = w + 32; j < kGramBlock<T>; j += 32) v = dd_add(v, buf[lane * kGramBlock<T> + j]);
+  for (int lane = warp; lane < ALL; lane += kGramBlock<T, EXACT> / 32) {
+    ddf v = buf[lane * kGramBlock<T, EXACT> + w];
+    for (int j = w + 32; j < kGramBlock<T, EXACT>; j += 32) v = dd_add(v, buf[lane * kGramBlock<T, EXACT> + j]);
     v = dd_warp_sum(v);
-    if (w == 0) part[(size_t)b * kGramAll + lane] = make_float2(v.hi, v.lo);
+    if (w == 0) part[(size_t)b * ALL + lane] = make_float2(v.hi, v.lo);
   }
   if (!last_block_ticket(counters + kGramTickets + ti, t.nblk)) return;
-  reduce_partials(part, kGramAll, t.nblk, s_out, s_red, kGramBlock<T>);
+  reduce_partials(part, ALL, t.nblk, s_out, s_red, kGramBlock<T, EXACT>);
   if (threadIdx.x == 0) counters[kGramTickets + ti] = 0u;
   const double inv_n = 1.0 / (double)A.n;
   const bool hermitian = A.x[t.src] == A.y[t.src];
@@ -276,22 +257,22 @@ __global__ void __launch_bounds__(kGramBlock<T>, 1) gram_tile_kernel(const __gri
     const size_t e = o + 2 * (k * A.K + l) + im;
     *(volatile double*)(out_host + e) = m;
   };
-  if (threadIdx.x < kGramLanes) {
+  if (threadIdx.x < LANES) {
     const int p = threadIdx.x / 2, im = threadIdx.x & 1;
-    const int k = t.r0 + p / kGramCols, l = t.c0 + p % kGramCols;
+    const int k = t.r0 + p / COLS, l = t.c0 + p % COLS;
     if (k < A.nbw && l < A.nbw && !(t.diag && l < k)) {
       const double m = (hermitian && im && k == l) ? 0.0 : s_out[threadIdx.x] * inv_n;
       put(k, l, im, m);
       if (hermitian && k != l) put(l, k, im, im ? -m : m);
     }
-  } else if (threadIdx.x < kGramAll) {
-    const int k = t.r0 + (threadIdx.x - kGramLanes) / 2, im = threadIdx.x & 1;
+  } else if (threadIdx.x < ALL) {
+    const int k = t.r0 + (threadIdx.x - LANES) / 2, im = threadIdx.x & 1;
     if (t.diag && A.K > A.nbw && k < A.nbw) {  // the constant amplitude: G_k,nbw = mean X_k
       const double m = s_out[threadIdx.x] * inv_n;
       put(k, A.nbw, im, m);
       put(A.nbw, k, im, im ? -m : m);
     }
-    if (t.diag && A.K > A.nbw && t.r0 == 0 && threadIdx.x < kGramLanes + 2) put(A.nbw, A.nbw, im, im ? 0.0 : 1.0);
+    if (t.diag && A.K > A.nbw && t.r0 == 0 && threadIdx.x < LANES + 2) put(A.nbw, A.nbw, im, im ? 0.0 : 1.0);
   }
 }
 
