@@ -667,9 +667,8 @@ struct GradMap {
 // Completion word of a result record (kResultFlag): every thread of the last block calls
 // this after its last write to `result`; thread 0 sets the word.  A host that polls a mapped
 // record watches its fields (kResultSentinel), so no system-scope fence is needed here (one
-// cost about 1.5 us at the end of every evaluation); `writers` is kept for the call sites.
-__device__ __forceinline__ void result_complete(double* result, int writers = 1 << 30) {
-  (void)writers;
+// cost about 1.5 us at the end of every evaluation).
+__device__ __forceinline__ void result_complete(double* result) {
   __syncthreads();
   if (threadIdx.x == 0) *(volatile double*)(result + kResultFlag) = 1.0;
 }

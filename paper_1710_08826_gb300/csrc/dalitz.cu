@@ -246,7 +246,7 @@ __device__ __forceinline__ void coh_finish(const CohArgs<T>& a, CohAcc<T, KB>& a
       result[2] = nb;
     }
   }
-  result_complete(result, P > 1 ? P : 1);
+  result_complete(result);
 }
 
 template <typename T, int KB>
@@ -528,7 +528,6 @@ static uint64_t lineshape_key(const DalitzModel& d, const double* theta) {
   return h ? h : 1;
 }
 
-// Lineshape constants for the current theta (FP64, once per lineshape version).
 // ---------------------------------------------------------------------------------------
 // floating lineshapes (masses and widths free; paper Sec. 4: the cache is then invalid at
 // every step).  No amplitude cache: each evaluation evaluates every Breit-Wigner amplitude of the
@@ -559,7 +558,7 @@ static uint64_t lineshape_key(const DalitzModel& d, const double* theta) {
 template <typename T>
 struct LsConst {
   T cr[kMaxAmp], ci[kMaxAmp];          // coefficients by slot: resonances, then the NR in slot KB
-  T ncr[kMaxAmp], nci[kMaxAmp];        // minus these
+  T nci[kMaxAmp];                      // -ci
   double rho[kMaxAmp], kappa[kMaxAmp], two_m0[kMaxAmp], inv_g0[kMaxAmp];
 };
 
@@ -925,7 +924,7 @@ __device__ __forceinline__ void td3_finish(const Td3Args<T>& a, ddf lf, const T 
       out[2] = nb;
     }
   }
-  result_complete(out, P > 1 ? P : 1);
+  result_complete(out);
 }
 
 // FP32: all amplitude planes of the event are requested before any is used (loads
@@ -1119,6 +1118,7 @@ static void fill_ls_tables(const DalitzModel& d, LsTables<T>& t) {
   }
 }
 
+// Lineshape constants for the current theta (FP64, once per lineshape version).
 static int dalitz_constants(goo_model* m, const double* theta) {
   DalitzModel& d = *m->dalitz;
   const uint64_t key = lineshape_key(d, theta);
@@ -1405,7 +1405,6 @@ static void fill_ls(const DalitzModel& d, const double* theta, LsConst<T>& c) {
     coef(d, theta, k, re, im);
     c.cr[k] = (T)re;
     c.ci[k] = (T)im;
-    c.ncr[k] = -c.cr[k];
     c.nci[k] = -c.ci[k];
     double mA, mB, mC;
     pair_masses(d, d.pair[k], mA, mB, mC);

@@ -323,7 +323,6 @@ struct EvNorm {
 struct MdFin {
   const ModelDev* __restrict__ md;
   int nK;
-  static constexpr bool kOwnNorm = false;
   __device__ int n_params() const { return md->n_params; }
   __device__ double w(int k) const { return k < nK ? md->comp[k].w : 0.0; }
   __device__ double dw(int k, int p) const { return md->dw[k][p]; }
@@ -331,15 +330,13 @@ struct MdFin {
   __device__ int par(int k, int l, int j) const {
     return (k < nK && l < md->comp[k].n_leaf) ? md->leaf[k * kMaxLeaf + l].par[j] : -1;
   }
-  __device__ double term(int, int, int) const { return 0.0; }
 };
 
 
 // Block reduction, last-block reduction over the blocks and the final FP64 combination
 // (lanes -> NLL and d NLL / d theta), shared by the event kernels:
-//   d NLL / d theta_p = sum_k [w_k C_k dlogN_kp - C_k dw_kp] - sum_{k,l,j: par = p} w_k A_klj,
-// with dlogN_kp = sum_{l,j: par = p} t_klj for a block's own normalisation terms.  Thread p
-// takes parameter p and gathers its terms in a fixed order.  The constants are loaded before
+//   d NLL / d theta_p = sum_k [w_k C_k dlogN_kp - C_k dw_kp] - sum_{k,l,j: par = p} w_k A_klj;
+// thread p takes parameter p and gathers its terms in a fixed order.  The constants are loaded before
 // the block's reduction, so that their latency overlaps it; the last block alone combines.
 template <int K, int L, bool GRAD, unsigned long long SIG, typename Fin>
 __device__ __forceinline__ void event_finish(ddf (&v)[EventLanes<float, K, L, GRAD, SIG>::NS], unsigned bad,
@@ -357,7 +354,7 @@ __device__ __forceinline__ void event_finish(ddf (&v)[EventLanes<float, K, L, GR
     for (int k = 0; k < K; ++k) {
       const bool on = p < P && k < nK;
       dwp[k] = on ? F.dw(k, p) : 0.0;
-      dlp[k] = (on && !Fin::kOwnNorm) ? F.dlogN(k, p) : 0.0;
+      dlp[k] = on ? F.dlogN(k, p) : 0.0;
     }
     for (int t = threadIdx.x; t < K * L * 3; t += blockDim.x) {
       const int k = t / (L * 3), l = (t / 3) % L, jj = t % 3;
@@ -402,8 +399,7 @@ __device__ __forceinline__ void event_finish(ddf (&v)[EventLanes<float, K, L, GR
 #pragma unroll
           for (int jj = 0; jj < 3; ++jj)
             if (a_present<K, L, SIG>(k, l, jj) && s_par[k][l][jj] == p)
-              gp += s_w[k] * ((Fin::kOwnNorm ? s_out[1 + k] * F.term(k, l, jj) : 0.0) -
-                              s_out[a_lane<K, L, SIG>(k, l, jj)]);
+              gp -= s_w[k] * s_out[a_lane<K, L, SIG>(k, l, jj)];
     }
     result[off + p] = gp;
   }
@@ -423,7 +419,7 @@ __device__ __forceinline__ void event_finish(ddf (&v)[EventLanes<float, K, L, GR
       result[2] = nb;
     }
   }
-  result_complete(result, P > 1 ? P : 1);
+  result_complete(result);
 }
 
 // Resident blocks per SM the event kernel is compiled for: the FP32 form of the small shape
@@ -926,7 +922,7 @@ __device__ __forceinline__ void event_finish_fused(const ddf (&v)[EventLanes<flo
       result[2] = nb;
     }
   }
-  result_complete(result, P > 1 ? P : 1);
+  result_complete(result);
 }
 
 template <int K, int L, bool GRAD>

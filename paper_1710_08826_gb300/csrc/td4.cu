@@ -280,7 +280,7 @@ __device__ __forceinline__ void td4_finish(const Td4Args<T>& a, TdAcc<T, KB>& ac
       result[2] = nb;
     }
   }
-  result_complete(result, P > 1 ? P : 1);
+  result_complete(result);
 }
 
 // The FP64 sums A = sum c_k a_k and B = sum b_k a_k of event i; B comes from the cache where it holds it.
