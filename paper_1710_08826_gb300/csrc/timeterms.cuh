@@ -179,7 +179,9 @@ inline void fill_time_coef(TimeCoef<T>& c, double x64, double y64, double tau, d
   const double x = (double)c.x, y = (double)c.y, G = (double)c.G, s = (double)c.s;
   const double zs = std::fmax(std::fabs(x), std::fabs(y)) * G;
   c.is2 = (T)(1.0 / (s * s));
-  c.is2h = (T)(0.5 / (s * s));
+  // FP32: t^2 times it stays finite up to the end of the range (the two-event exponential has no use for an
+  // infinite argument); the Gaussian is 0 there all the same
+  c.is2h = sizeof(T) == 4 ? (T)std::fmin(0.5 / (s * s), 3e38 / std::fmax(t_hi * t_hi, 1e-30)) : (T)(0.5 / (s * s));
   c.ir2s = (T)(0.70710678118654752440 / s);
   c.k_phi = (T)(0.39894228040143267794 / s);
   c.s2 = (T)(s * s);
