@@ -645,10 +645,16 @@ __device__ __forceinline__ void ls_weight(bool mc, float2 s2, bool v0, bool v1, 
   }
   const bool ok0 = s2.x > 0.f, ok1 = s2.y > 0.f;
   bad += (unsigned)(v0 && !ok0) + (unsigned)(v1 && !ok1);
-  constexpr float kMin = 1.17549435e-38f;  // the hardware functions flush smaller values to 0
-  const float2 s = make_float2(fmaxf(s2.x, kMin), fmaxf(s2.y, kMin)), r = lsv::rcp(s);
+  float2 r, l;
+  if (fminf(s2.x, s2.y) >= 1.17549435e-38f) {
+    r = lsv::rcp(s2);
+    l = make_float2(pk::lg2(s2.x), pk::lg2(s2.y));
+  } else {  // the hardware functions take a subnormal number for 0
+    r = make_float2(1.f / s2.x, 1.f / s2.y);
+    l = make_float2(log2f(s2.x), log2f(s2.y));
+  }
   w = make_float2(v0 && ok0 ? r.x : 0.f, v1 && ok1 ? r.y : 0.f);
-  term = make_float2(v0 && ok0 ? pk::lg2(s.x) : 0.f, v1 && ok1 ? pk::lg2(s.y) : 0.f);
+  term = make_float2(v0 && ok0 ? l.x : 0.f, v1 && ok1 ? l.y : 0.f);
 }
 __device__ __forceinline__ void ls_weight(bool mc, double s2, bool, bool, double& w, double& term, unsigned& bad) {
   if (mc) {
