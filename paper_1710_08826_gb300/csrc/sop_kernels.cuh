@@ -682,11 +682,19 @@ __device__ __forceinline__ void eval_event2(const EvConst<float, K, L>& P, const
   float2 M = ak[0];
 #pragma unroll
   for (int k = 1; k < K; ++k) M = make_float2(fmaxf(M.x, ak[k].x), fmaxf(M.y, ak[k].y));
+  // weighted: where a product's weight is 0 (a fraction at its limit) a subnormal share of another one may be all
+  // there is, which the hardware's exponential and logarithm take for 0
+  bool limit = false;
+  if (WEIGHTED) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) limit = limit || (k < P.nK && P.w_hi[k] == 0.f);
+  }
   float2 S = splat(0.f);
 #pragma unroll
   for (int k = 0; k < K; ++k) {
     const float2 t = sub(ak[k], M);
-    const float2 e = make_float2(ex2(t.x), ex2(t.y));
+    float2 e = make_float2(ex2(t.x), ex2(t.y));
+    if (limit) e = make_float2(exp2f(t.x), exp2f(t.y));
     if (SIG == 0 || sig_product_has_r(SIG, k, L)) {
       rq[k] = mul(rq[k], e);  // the product's value without its PQ factor
       rk[k] = sig_product_poly_q(SIG, k, L) ? mul(rq[k], rp[k]) : rq[k];
@@ -699,7 +707,9 @@ __device__ __forceinline__ void eval_event2(const EvConst<float, K, L>& P, const
   // has r = 0 or w = 0.  The logarithm of a lane with S <= 0 is not used.
   ok0 = S.x > 0.f;
   ok1 = S.y > 0.f;
-  logf = add(M, make_float2(lg2(S.x), lg2(S.y)));
+  float2 lS = make_float2(lg2(S.x), lg2(S.y));
+  if (limit) lS = make_float2(log2f(S.x), log2f(S.y));
+  logf = add(M, lS);
   if constexpr (GRAD) {
     float2 invS = rcp(S);
     // weighted: finite where S is subnormal (the larger product's fraction at its limit 0)
