@@ -10,6 +10,9 @@
 //   - log S is a running product (LogProduct), 1/S, 1/u and 1/r are third-order reciprocals, exp
 //     and log come from shared-memory tables;
 //   - a polynomial r that is its product's only one needs no reciprocal: c_k / r is the other factors;
+//     an event where a polynomial is exactly 0 is left out of its lanes all the same, like the rest of the product
+//     (x times the other factors over S may be any number: where a narrow signal is all that is left, it leaves
+//     the float range of the block sums, and to carry the exponent that far costs 10 registers, 448 -> 471 us);
 //   - the constant factors of the lanes (1/sigma, 2/m0) are applied once per thread, and the Argus endpoint's
 //     derivative is formed from the sums of c_k / u, c_k and c_k u.
 // The three-dimensional signal + background model takes 76 slots per event (counted) with the
