@@ -340,26 +340,47 @@ __device__ __forceinline__ V conv_real(const TdMath<V>& F, T g, T gs2, T hg2s2, 
   else return F.nonneg(u) ? h : x;
 }
 
+// The Faddeeva function as above, each operation rounded as written (see mul_rn).
+template <typename T>
+__device__ __forceinline__ void faddeeva_rn(T zr, T zi, const T* a, int N, T L, T& wr, T& wi) {
+  const T dr = add_rn(L, zi), inv = T(1) / fma_rn(dr, dr, mul_rn(zr, zr));
+  const T ir = mul_rn(dr, inv), ii = mul_rn(zr, inv);
+  const T nr = sub_rn(L, zi);
+  const T Zr = fma_rn(nr, ir, -mul_rn(zr, ii)), Zi = fma_rn(nr, ii, mul_rn(zr, ir));
+  T pr = a[N - 1], pi = T(0);
+  for (int j = N - 2; j >= 0; --j) {
+    const T tr = fma_rn(pr, Zr, fma_rn(-pi, Zi, a[j]));
+    pi = fma_rn(pr, Zi, mul_rn(pi, Zr));
+    pr = tr;
+  }
+  const T qr = fma_rn(T(2), fma_rn(pr, ir, -mul_rn(pi, ii)), T(0.56418958354775628695));
+  const T qi = mul_rn(T(2), fma_rn(pr, ii, mul_rn(pi, ir)));
+  wr = fma_rn(ir, qr, -mul_rn(ii, qi));
+  wi = fma_rn(ir, qi, mul_rn(ii, qr));
+}
+
 // E(g) for complex g = (gr, gi)
 template <typename T>
-__device__ __forceinline__ void conv_complex(const TdMath<T>& F, T gr, T gi, T t, T s, T gauss, const T* wa, int wN,
-                                             T wL, T& Er, T& Ei) {
-  const T c = T(0.70710678118654752440) / s;
-  const T ur = (gr * s * s - t) * c, ui = gi * s * s * c;
+__device__ __forceinline__ void conv_complex(const TdMath<T>& F, T gr, T gi, T t, T s, T ir2s, T gauss, const T* wa,
+                                             int wN, T wL, T& Er, T& Ei) {
+  const T grs = mul_rn(gr, s), gis = mul_rn(gi, s);
+  const T ur = mul_rn(fma_rn(grs, s, -t), ir2s), ui = mul_rn(mul_rn(gis, s), ir2s);
+  const T hg = mul_rn(T(0.5), gauss);
   T wr, wi;
   if (ur >= T(0)) {
-    faddeeva<T>(-ui, ur, wa, wN, wL, wr, wi);  // w(i u)
-    Er = T(0.5) * gauss * wr;
-    Ei = T(0.5) * gauss * wi;
+    faddeeva_rn<T>(-ui, ur, wa, wN, wL, wr, wi);  // w(i u)
+    Er = mul_rn(hg, wr);
+    Ei = mul_rn(hg, wi);
   } else {
-    faddeeva<T>(ui, -ur, wa, wN, wL, wr, wi);  // w(-i u)
-    const T er = T(0.5) * (gr * gr - gi * gi) * s * s - gr * t, ei = gr * gi * s * s - gi * t;
+    faddeeva_rn<T>(ui, -ur, wa, wN, wL, wr, wi);  // w(-i u)
+    const T er = fma_rn(T(0.5), fma_rn(grs, grs, -mul_rn(gis, gis)), -mul_rn(gr, t));
+    const T ei = fma_rn(grs, gis, -mul_rn(gi, t));
     const T mag = F.exp(er);
     T sn, cs;
     if constexpr (sizeof(T) == 4) sincosf(ei, &sn, &cs);
     else sincos(ei, &sn, &cs);
-    Er = mag * cs - T(0.5) * gauss * wr;
-    Ei = mag * sn - T(0.5) * gauss * wi;
+    Er = fma_rn(mag, cs, -mul_rn(hg, wr));
+    Ei = fma_rn(mag, sn, -mul_rn(hg, wi));
   }
 }
 
@@ -368,27 +389,17 @@ __device__ __forceinline__ void conv_complex(const TdMath<T>& F, T gr, T gi, T t
 template <typename T>
 __device__ __forceinline__ void time_terms_direct(const TdMath<T>& F, const TimeCoef<T>& c, const T* wa, int wN, T wL,
                                                   T t, T gauss, TimeTerms<T>& R) {
-  const T gp = c.G * (T(1) - c.y), gm = c.G * (T(1) + c.y);
-  const T Ep = conv_real(F, gp, gp * c.s2, T(0.5) * gp * gp * c.s2, c.ir2s, t, gauss);
-  const T Em = conv_real(F, gm, gm * c.s2, T(0.5) * gm * gm * c.s2, c.ir2s, t, gauss);
+  const T gp = mul_rn(c.G, sub_rn(T(1), c.y)), gm = mul_rn(c.G, add_rn(T(1), c.y));
+  const T gps = mul_rn(gp, c.s2), gms = mul_rn(gm, c.s2);
+  const T Ep = conv_real(F, gp, gps, mul_rn(mul_rn(T(0.5), gp), gps), c.ir2s, t, gauss);
+  const T Em = conv_real(F, gm, gms, mul_rn(mul_rn(T(0.5), gm), gms), c.ir2s, t, gauss);
   T Ecr, Eci;
-  conv_complex<T>(F, c.G, -c.G * c.x, t, c.s, gauss, wa, wN, wL, Ecr, Eci);
-  const T Tch = T(0.5) * (Ep + Em);
-  R.P = T(0.5) * (Tch + Ecr);
-  R.Q = T(0.5) * (Tch - Ecr);
-  R.Tsh = T(0.5) * (Ep - Em);
+  conv_complex<T>(F, c.G, -mul_rn(c.G, c.x), t, c.s, c.ir2s, gauss, wa, wN, wL, Ecr, Eci);
+  const T Tch = mul_rn(T(0.5), add_rn(Ep, Em));
+  R.P = mul_rn(T(0.5), add_rn(Tch, Ecr));
+  R.Q = mul_rn(T(0.5), sub_rn(Tch, Ecr));
+  R.Tsh = mul_rn(T(0.5), sub_rn(Ep, Em));
   R.Ts = Eci;
-}
-
-// The pair form's (time_terms_pair), out of line: the compiler fuses products and sums in it as it likes, so one
-// copy serves the four-body kernels with and without the gradient, which return the same NLL (inlined into
-// each, it differed by 2e-9).  The three-body kernel's two forms agree inlined, and a call in its loop
-// costs it registers (2M events: 94 -> 129 us).
-static __device__ __noinline__ float4 time_terms_direct32(const TimeCoef<float>& c, const float* wa, int wN, float wL,
-                                                          float t, float gauss) {
-  TimeTerms<float> R;
-  time_terms_direct<float>(TdMath<float>{}, c, wa, wN, wL, t, gauss, R);
-  return make_float4(R.P, R.Q, R.Tsh, R.Ts);
 }
 
 // The decay-time terms by the moment series of order KU (small mixing; see the top of this
@@ -448,11 +459,12 @@ __device__ __forceinline__ void time_terms_pair(const TdMath<float2>& F, const T
     for (int e = 0; e < 2; ++e) {
       const float te = e ? t.y : t.x;
       if (te < c.t_series) continue;
-      const float4 d = time_terms_direct32(c, wa, wN, wL, te, expf(mul_rn(mul_rn(-te, te), c.is2h)));
-      (e ? R.P.y : R.P.x) = d.x;
-      (e ? R.Q.y : R.Q.x) = d.y;
-      (e ? R.Tsh.y : R.Tsh.x) = d.z;
-      (e ? R.Ts.y : R.Ts.x) = d.w;
+      TimeTerms<float> S;
+      time_terms_direct<float>(TdMath<float>{}, c, wa, wN, wL, te, expf(mul_rn(mul_rn(-te, te), c.is2h)), S);
+      (e ? R.P.y : R.P.x) = S.P;
+      (e ? R.Q.y : R.Q.x) = S.Q;
+      (e ? R.Tsh.y : R.Tsh.x) = S.Tsh;
+      (e ? R.Ts.y : R.Ts.x) = S.Ts;
     }
   }
 }
