@@ -163,6 +163,9 @@ struct TimeCoef {
   T hx, hy, fx, fy;            // s^2 G x / 2, s^2 G y / 2, and twice these
   T Gx, Gy, qx, qy;            // G x, G y, 2 G^2 x, 2 G^2 y
   T Gx2, Gy2;                  // (G x)^2, (G y)^2
+  // the Faddeeva path's: g = G (1 -+ y), g s^2 and g^2 s^2 / 2 of each; of g = G (1 - i x) the real part of
+  // g^2 s^2 / 2 and the imaginary part of u
+  T gp, gps2, hgp2s2, gm, gms2, hgm2s2, hgc2s2, ui;
 };
 
 #ifndef __CUDACC_RTC__
@@ -198,6 +201,15 @@ inline void fill_time_coef(TimeCoef<T>& c, double x64, double y64, double tau, d
   c.qy = (T)(2.0 * G * G * y);
   c.Gx2 = (T)(G * G * x * x);
   c.Gy2 = (T)(G * G * y * y);
+  const double gp = G * (1.0 - y), gm = G * (1.0 + y);
+  c.gp = (T)gp;
+  c.gps2 = (T)(gp * s * s);
+  c.hgp2s2 = (T)(0.5 * gp * gp * s * s);
+  c.gm = (T)gm;
+  c.gms2 = (T)(gm * s * s);
+  c.hgm2s2 = (T)(0.5 * gm * gm * s * s);
+  c.hgc2s2 = (T)(0.5 * G * G * s * s * (1.0 - x * x));
+  c.ui = (T)(-G * x * s * 0.70710678118654752440);
   c.t_gauss = (T)(-s * std::sqrt(2.0 * 87.3));
   double fact = 1.0;  // (2m)!
   for (int m = 0; m <= K; ++m) {
@@ -359,42 +371,27 @@ __device__ __forceinline__ void faddeeva_rn(T zr, T zi, const T* a, int N, T L, 
   wi = fma_rn(ir, qi, mul_rn(ii, qr));
 }
 
-// E(g) for complex g = (gr, gi)
-template <typename T>
-__device__ __forceinline__ void conv_complex(const TdMath<T>& F, T gr, T gi, T t, T s, T ir2s, T gauss, const T* wa,
-                                             int wN, T wL, T& Er, T& Ei) {
-  const T grs = mul_rn(gr, s), gis = mul_rn(gi, s);
-  const T ur = mul_rn(fma_rn(grs, s, -t), ir2s), ui = mul_rn(mul_rn(gis, s), ir2s);
-  const T hg = mul_rn(T(0.5), gauss);
-  T wr, wi;
-  if (ur >= T(0)) {
-    faddeeva_rn<T>(-ui, ur, wa, wN, wL, wr, wi);  // w(i u)
-    Er = mul_rn(hg, wr);
-    Ei = mul_rn(hg, wi);
-  } else {
-    faddeeva_rn<T>(ui, -ur, wa, wN, wL, wr, wi);  // w(-i u)
-    const T er = fma_rn(T(0.5), fma_rn(grs, grs, -mul_rn(gis, gis)), -mul_rn(gr, t));
-    const T ei = fma_rn(grs, gis, -mul_rn(gi, t));
-    const T mag = F.exp(er);
-    T sn, cs;
-    if constexpr (sizeof(T) == 4) sincosf(ei, &sn, &cs);
-    else sincos(ei, &sn, &cs);
-    Er = fma_rn(mag, cs, -mul_rn(hg, wr));
-    Ei = fma_rn(mag, sn, -mul_rn(hg, wi));
-  }
-}
-
 // The decay-time terms at the observed time t from the convolved exponentials (Faddeeva
-// path, any mixing); gauss = exp(-t^2 / 2 s^2).
+// path, any mixing); gauss = exp(-t^2 / 2 s^2).  E of the complex g = G (1 - i x) by the same two forms as
+// conv_real, u = (g s^2 - t) / (s sqrt 2).
 template <typename T>
 __device__ __forceinline__ void time_terms_direct(const TdMath<T>& F, const TimeCoef<T>& c, const T* wa, int wN, T wL,
                                                   T t, T gauss, TimeTerms<T>& R) {
-  const T gp = mul_rn(c.G, sub_rn(T(1), c.y)), gm = mul_rn(c.G, add_rn(T(1), c.y));
-  const T gps = mul_rn(gp, c.s2), gms = mul_rn(gm, c.s2);
-  const T Ep = conv_real(F, gp, gps, mul_rn(mul_rn(T(0.5), gp), gps), c.ir2s, t, gauss);
-  const T Em = conv_real(F, gm, gms, mul_rn(mul_rn(T(0.5), gm), gms), c.ir2s, t, gauss);
-  T Ecr, Eci;
-  conv_complex<T>(F, c.G, -mul_rn(c.G, c.x), t, c.s, c.ir2s, gauss, wa, wN, wL, Ecr, Eci);
+  const T Ep = conv_real(F, c.gp, c.gps2, c.hgp2s2, c.ir2s, t, gauss);
+  const T Em = conv_real(F, c.gm, c.gms2, c.hgm2s2, c.ir2s, t, gauss);
+  const T v = sub_rn(t, c.Gs2), ur = mul_rn(-v, c.ir2s);
+  const bool right = ur >= T(0);
+  T wr, wi;  // w(i u), or w(-i u)
+  faddeeva_rn<T>(right ? -c.ui : c.ui, right ? ur : -ur, wa, wN, wL, wr, wi);
+  T Ecr = mul_rn(mul_rn(T(0.5), gauss), wr), Eci = mul_rn(mul_rn(T(0.5), gauss), wi);
+  if (!right) {
+    const T mag = F.exp(fma_rn(-c.G, t, c.hgc2s2)), ei = mul_rn(c.Gx, v);
+    T sn, cs;
+    if constexpr (sizeof(T) == 4) sincosf(ei, &sn, &cs);
+    else sincos(ei, &sn, &cs);
+    Ecr = fma_rn(mag, cs, -Ecr);
+    Eci = fma_rn(mag, sn, -Eci);
+  }
   const T Tch = mul_rn(T(0.5), add_rn(Ep, Em));
   R.P = mul_rn(T(0.5), add_rn(Tch, Ecr));
   R.Q = mul_rn(T(0.5), sub_rn(Tch, Ecr));
