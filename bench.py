@@ -44,32 +44,32 @@ _TD3_SRC = _COH_SRC + ['paper_1710_08826_gb300/csrc/timeterms.cuh']
 ISSUE_PEAK = 152 * 4 * 2.07e9
 
 NCU_RECORDS = {
-    "sop_nll_grad_f32": {"bytes": 123_068_160, "events": 10_000_000, "duration_ns": 40608, "warp_inst": 22_805_711, "issue_active": 0.5646,
-        "sources": _SOP_SRC, "sha256": "8c76b3c11bcc170ffcde57bc1ec90479a95fba091734604320cc23ba4d4ef2cb",
+    "sop_nll_grad_f32": {"bytes": 123_161_856, "events": 10_000_000, "duration_ns": 39008, "warp_inst": 22_805_707, "issue_active": 0.5703,
+        "sources": _SOP_SRC, "sha256": "ce89d75c759e7b5b5a992106a2f106feb7b29c8603745c242569e3655369c6cd",
         "profile": "profiles/likelihood_kernels.md"},
-    "sop_nll_f64": {"bytes": 243_111_680, "events": 10_000_000, "duration_ns": 913568, "fp64_pipe": 0.8516, "fp64_ops": {"dfma": 191_320_056, "dadd": 110_777_259, "dmul": 140_310_804},
-        "sources": _SOP_SRC, "sha256": "8c76b3c11bcc170ffcde57bc1ec90479a95fba091734604320cc23ba4d4ef2cb",
+    "sop_nll_f64": {"bytes": 243_199_232, "events": 10_000_000, "duration_ns": 913888, "fp64_pipe": 0.8514, "fp64_ops": {"dfma": 191_320_056, "dadd": 110_777_259, "dmul": 140_310_804},
+        "sources": _SOP_SRC, "sha256": "ce89d75c759e7b5b5a992106a2f106feb7b29c8603745c242569e3655369c6cd",
         "profile": "profiles/likelihood_kernels.md"},
-    "coh_nll_grad_f32": {"bytes": 323_097_344, "events": 5_000_000, "duration_ns": 56800, "warp_inst": 27_167_220, "issue_active": 0.4435,
-        "sources": _COH_SRC, "sha256": "50df3928891bc82ae89a996ee33e106fca4a78927da9c62d7d7dedc7045d8823",
+    "coh_nll_grad_f32": {"bytes": 323_064_832, "events": 5_000_000, "duration_ns": 57184, "warp_inst": 27_167_220, "issue_active": 0.4416,
+        "sources": _COH_SRC, "sha256": "411018c9e640fabcf18d75e6fa92446dd9e07fa260f339ea916a0c37f7692ee0",
         "profile": "profiles/likelihood_kernels.md"},
-    "coh_nll_f64": {"bytes": 643_084_544, "events": 5_000_000, "duration_ns": 345728, "fp64_pipe": 0.8457, "fp64_ops": {"dfma": 166_323_009, "dadd": 778241, "dmul": 10_311_296},
-        "sources": _COH_SRC, "sha256": "50df3928891bc82ae89a996ee33e106fca4a78927da9c62d7d7dedc7045d8823",
+    "coh_nll_f64": {"bytes": 643_040_768, "events": 5_000_000, "duration_ns": 342976, "fp64_pipe": 0.8459, "fp64_ops": {"dfma": 166_323_009, "dadd": 778241, "dmul": 10_311_296},
+        "sources": _COH_SRC, "sha256": "411018c9e640fabcf18d75e6fa92446dd9e07fa260f339ea916a0c37f7692ee0",
         "profile": "profiles/likelihood_kernels.md"},
-    "coh_ls_grad_f32": {"bytes": 48_058_880, "events": 5_000_000, "duration_ns": 138848, "warp_inst": 87_844_859, "issue_active": 0.5679,
-        "sources": _COH_SRC, "sha256": "50df3928891bc82ae89a996ee33e106fca4a78927da9c62d7d7dedc7045d8823",
+    "coh_ls_grad_f32": {"bytes": 48_060_416, "events": 5_000_000, "duration_ns": 137408, "warp_inst": 88_311_178, "issue_active": 0.5731,
+        "sources": _COH_SRC, "sha256": "411018c9e640fabcf18d75e6fa92446dd9e07fa260f339ea916a0c37f7692ee0",
         "profile": "profiles/likelihood_kernels.md"},
-    "td3_nll_grad_f32": {"bytes": 523_144_704, "events": 2_000_000, "duration_ns": 85952, "warp_inst": 45_199_736, "issue_active": 0.4852,
-        "sources": _TD3_SRC, "sha256": "402ac1225fb418591f8bf2cb5246ab23f064850c04bf77f38956b1359b72b968",
+    "td3_nll_grad_f32": {"bytes": 522_721_792, "events": 2_000_000, "duration_ns": 87616, "warp_inst": 45_343_452, "issue_active": 0.4812,
+        "sources": _TD3_SRC, "sha256": "4869c17847fbcfe9517d1fe33420425e4fcb4ca5668aea7d67a33c398297fa46",
         "profile": "profiles/likelihood_kernels.md"},
-    "td3_nll_f64": {"bytes": 979_168_512, "events": 2_000_000, "duration_ns": 845248, "fp64_pipe": 0.8468, "fp64_ops": {"dfma": 347_196_472, "dadd": 12_249_169, "dmul": 59_299_278},
-        "sources": _TD3_SRC, "sha256": "402ac1225fb418591f8bf2cb5246ab23f064850c04bf77f38956b1359b72b968",
+    "td3_nll_f64": {"bytes": 979_187_456, "events": 2_000_000, "duration_ns": 839424, "fp64_pipe": 0.8470, "fp64_ops": {"dfma": 347_896_888, "dadd": 12_871_761, "dmul": 57_898_446},
+        "sources": _TD3_SRC, "sha256": "4869c17847fbcfe9517d1fe33420425e4fcb4ca5668aea7d67a33c398297fa46",
         "profile": "profiles/likelihood_kernels.md"},
-    "td4_nll_grad_f32": {"bytes": 171_081_216, "events": 2_000_000, "duration_ns": 45024, "warp_inst": 20_464_799, "issue_active": 0.4573,
-        "sources": _TD4_SRC, "sha256": "0687c1d783437bbd6d92b9172be3f0b394d31ca9cce7d76ce2ec0f281d014318",
+    "td4_nll_grad_f32": {"bytes": 171_087_616, "events": 2_000_000, "duration_ns": 45248, "warp_inst": 20_615_388, "issue_active": 0.4825,
+        "sources": _TD4_SRC, "sha256": "0b32bcce10f2e59f5efb1ef0568e170c6e5f4223d86a035479cada30b3b738b8",
         "profile": "profiles/likelihood_kernels.md"},
-    "td4_nll_f64": {"bytes": 371_114_496, "events": 2_000_000, "duration_ns": 540128, "fp64_pipe": 0.8479, "fp64_ops": {"dfma": 188_172_375, "dadd": 12_716_574, "dmul": 59_611_103},
-        "sources": _TD4_SRC, "sha256": "0687c1d783437bbd6d92b9172be3f0b394d31ca9cce7d76ce2ec0f281d014318",
+    "td4_nll_f64": {"bytes": 371_125_504, "events": 2_000_000, "duration_ns": 535488, "fp64_pipe": 0.8497, "fp64_ops": {"dfma": 187_899_991, "dadd": 12_872_222, "dmul": 57_898_975},
+        "sources": _TD4_SRC, "sha256": "0b32bcce10f2e59f5efb1ef0568e170c6e5f4223d86a035479cada30b3b738b8",
         "profile": "profiles/likelihood_kernels.md"},
 }
 

@@ -553,7 +553,8 @@ static uint64_t lineshape_key(const DalitzModel& d, const double* theta) {
 // works on two points at a time; the first blocks of the one launch take the MC sample and the others the events, so that neither waits for the
 // other's reduction.  5M events and 1M MC points, 8 resonances: 495 us in two launches with every
 // resonance evaluated by itself, 144 us with the amplitudes formed a second time for the lanes, now
-// 131 us (217 KB of shared memory; issue slots 59 %, FMA pipe 54 %, shared memory 53 % busy).
+// 131 us in repeated calls and 137 us under ncu, a call 146 us (217 KB of shared memory; issue slots 57 %, FMA pipe 54 %,
+// shared memory 53 % busy).
 // ---------------------------------------------------------------------------------------
 template <typename T>
 struct LsConst {

@@ -1034,7 +1034,7 @@ __host__ __device__ constexpr int cols_col(unsigned long long cols, int slot) { 
 // warp that completes the count refills the buffer with the tile kEventStages ahead.  No
 // block barrier separates tiles, so a warp that is fast on one tile runs ahead on the next
 // instead of waiting for the slowest warp.
-// WEIGHTED (the interpreter only: a fit's evaluations would not pay for a compilation): the
+// WEIGHTED (the interpreter only; the other forms are compiled for the model at run time): the
 // weights are staged as one more column behind the observables.
 // Dynamic shared memory: kEventStages * n_obs (+ 1 when weighted) * TE floats.
 template <int K, int L, bool GRAD, unsigned long long SIG = 0, unsigned long long COLS = 0, bool DIRECT = false,
